@@ -254,8 +254,9 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   return 0;
 }
 
-int aqt_quantize(const float* x, int64_t rows, int64_t cols, int64_t ld, int bits, int axis, int rounding, int pack,
-                 void* q_out, float* scale_out, void* stream) {
+// partial: nullptr, or max_partials words of scratch that save the whole-tensor scale a launch.
+static int quantize_entry(const float* x, int64_t rows, int64_t cols, int64_t ld, int bits, int axis, int rounding, int pack,
+                          void* q_out, float* scale_out, void* stream, float* partial, int64_t max_partials) {
   if (rows < 0 || cols < 0 || ld < cols || !quant_bits_ok(bits)) return AQT_ERR_BADARG;
   if (axis != AQT_AXIS_ROW && axis != AQT_AXIS_COL && axis != AQT_AXIS_TENSOR) return AQT_ERR_BADARG;
   if (rounding != AQT_ROUND_HALF_UP_FLOOR && rounding != AQT_ROUND_NEAREST_EVEN) return AQT_ERR_BADARG;
@@ -269,11 +270,16 @@ int aqt_quantize(const float* x, int64_t rows, int64_t cols, int64_t ld, int bit
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int qmax = qmax_of(bits);
   if (rounding == AQT_ROUND_HALF_UP_FLOOR) {
-    return pack ? launch_quantize_axis<AQT_ROUND_HALF_UP_FLOOR, true>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st)
-                : launch_quantize_axis<AQT_ROUND_HALF_UP_FLOOR, false>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st);
+    return pack ? launch_quantize_axis<AQT_ROUND_HALF_UP_FLOOR, true>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st, partial, max_partials)
+                : launch_quantize_axis<AQT_ROUND_HALF_UP_FLOOR, false>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st, partial, max_partials);
   }
-  return pack ? launch_quantize_axis<AQT_ROUND_NEAREST_EVEN, true>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st)
-              : launch_quantize_axis<AQT_ROUND_NEAREST_EVEN, false>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st);
+  return pack ? launch_quantize_axis<AQT_ROUND_NEAREST_EVEN, true>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st, partial, max_partials)
+              : launch_quantize_axis<AQT_ROUND_NEAREST_EVEN, false>(x, rows, cols, ld, qmax, axis, q_out, scale_out, st, partial, max_partials);
+}
+
+int aqt_quantize(const float* x, int64_t rows, int64_t cols, int64_t ld, int bits, int axis, int rounding, int pack,
+                 void* q_out, float* scale_out, void* stream) {
+  return quantize_entry(x, rows, cols, ld, bits, axis, rounding, pack, q_out, scale_out, stream, nullptr, 0);
 }
 
 int aqt_pack_int4(const int8_t* q, int64_t rows, int64_t cols, uint8_t* packed, void* stream) {
@@ -525,7 +531,9 @@ int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w
   // Step 1 (Fig. 2): dynamic quantization of the activations over K; 4-bit codes stay in int8
   // containers between the two kernels, which is what the figure's cast produces.
   const int axis = a_scale_kind == AQT_SCALE_ROW ? AQT_AXIS_ROW : AQT_AXIS_TENSOR;
-  rc = aqt_quantize(x, M, K, ldx, bits_a, axis, rounding, 0, codes, s_x, stream);
+  // (one scale: the other M - 1 words of its area are scratch for the quantizer)
+  const bool one_scale = a_scale_kind == AQT_SCALE_TENSOR;
+  rc = quantize_entry(x, M, K, ldx, bits_a, axis, rounding, 0, codes, s_x, stream, one_scale && M > 1 ? s_x + 1 : nullptr, M - 1);
   if (rc != AQT_OK) return rc;
   // Step 2: integer matmul + de-quantizing epilogue.
   return qmatmul_i8a(codes, s_x, a_scale_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y,

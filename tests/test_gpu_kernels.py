@@ -75,6 +75,28 @@ def test_quantize_col_and_tensor_axes_bit_exact(axis, bits, shape):
         assert np.array_equal(qp.cpu().numpy(), orc.pack_int4(orc.quantize(x, 4, axis)[0]))
 
 
+@pytest.mark.parametrize("rows,cols,ld,std", [(17, 4096, 4096, 1.0), (1025, 64, 64, 1.0), (129, 512, 520, 1.0), (4737, 512, 512, 1.0),
+                                              (300, 1000, 1004, 1e-30), (70, 1024, 1024, 0.0)])
+@pytest.mark.parametrize("bits,pack", [(8, False), (4, True)])
+def test_quantize_tensor_axis_beyond_one_block(rows, cols, ld, std, bits, pack):
+    """One scale for a tensor of more than 64 K elements read as float4s: dense and with a row pitch, a
+    remainder in the last block, scales outside the short quotient sequence's range, a tensor of
+    zeros.  aqt_linear_fwd finds the same scale through its own scratch words (exact: y is compared
+    bit for bit)."""
+    x = np.full((rows, ld), 7e9, np.float32)  # the padding must not be seen
+    x[:, :cols] = gen.normal(11, 3, rows, cols, std=std)
+    q_ref, s_ref = orc.quantize(x[:, :cols], bits, orc.AXIS_TENSOR)
+    xd = _dev(x)[:, :cols]
+    q, s = aqt.aqt_quantize(xd, bits, aqt.AXIS_TENSOR, pack=pack)
+    assert np.array_equal(s.cpu().numpy(), s_ref)
+    assert np.array_equal(q.cpu().numpy().view(np.uint8), orc.pack_int4(q_ref) if pack else q_ref.view(np.uint8))
+    if cols % 16 == 0:
+        wq, s_w = orc.quantize(gen.weight(11, 4, cols, 64), 8, orc.AXIS_ROW)
+        y = aqt.aqt_linear_fwd(xd, _dev(wq), _dev(s_w), bits_a=bits, a_scale_kind=aqt.SCALE_TENSOR)
+        y_ref = orc.linear_fwd(np.ascontiguousarray(x[:, :cols]), wq, s_w, bits_a=bits, a_scale_kind=orc.SCALE_TENSOR)
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), y_ref.view(np.uint32))
+
+
 def test_quantize_heavy_tailed_rows():
     x = gen.student_t3(0, 77, 256, 1024)
     q_ref, s_ref = orc.quantize(x, 8, orc.AXIS_ROW)
