@@ -1,5 +1,9 @@
 """Thin Python binding of the C ABI in include/aqt.h: same names, argument marshalling only.
 
+The entry points on the per-layer path are called through the extension module `_fastcall` (plain
+integers for arguments, see csrc/host/fastcall.c), the others and the pre-marshalled forms through
+ctypes; both reach the same libaqt.so.
+
 Every step of the quantized linear layer runs in the CUDA library; torch is used here for device
 memory and the current stream.  There is no CPU fallback: if the shared library is missing the
 import of any entry point fails with an error that says how to build it.
@@ -39,6 +43,7 @@ class AqtError(RuntimeError):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_fast = None
 
 
 def lib() -> ctypes.CDLL:
@@ -56,6 +61,21 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _fc():
+    """The extension module of the per-layer entry points, opened on libaqt.so.  Never falls back."""
+    global _fast
+    if _fast is None:
+        lib()
+        try:
+            from . import _fastcall
+        except ImportError as e:
+            raise ImportError("extension module %s is missing or does not load (%s); build it with "
+                              "`python -m paper_2203_15952_b200.build`" % (_build.FASTCALL_PATH, e))
+        _fastcall.open(_build.LIB_PATH)
+        _fast = _fastcall
+    return _fast
+
+
 def status_string(status: int) -> str:
     return lib().aqt_status_string(int(status)).decode()
 
@@ -71,6 +91,13 @@ def _ptr(t: Optional[torch.Tensor]):
 
 def _i64(v) -> ctypes.c_int64:
     return ctypes.c_int64(int(v))
+
+
+def _raw_stream(stream) -> int:
+    """The cudaStream_t of `stream`, or of the current stream of the current device."""
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _stream(stream=None):
@@ -145,7 +172,7 @@ def aqt_version() -> int:
 
 
 def aqt_workspace_bytes(op: int, M: int, N: int, K: int, bits_a: int, bits_w: int) -> int:
-    return int(lib().aqt_workspace_bytes(int(op), _i64(M), _i64(N), _i64(K), int(bits_a), int(bits_w)))
+    return _fc().workspace_bytes(op, M, N, K, bits_a, bits_w)
 
 
 def aqt_plan_qmatmul(M: int, N: int, K: int, bits_a: int = 8, bits_w: int = 8, act: int = ACT_NONE, float_kind: bool = False,
@@ -203,8 +230,10 @@ def aqt_quantize(x: torch.Tensor, bits: int, axis: int = AXIS_ROW, rounding: int
     n_scale = rows if axis == AXIS_ROW else (cols if axis == AXIS_COL else 1)
     if scale_out is None:
         scale_out = torch.empty(n_scale, dtype=torch.float32, device=x.device)
-    _check("aqt_quantize", lib().aqt_quantize(_ptr(x), _i64(rows), _i64(cols), _i64(ld), int(bits), int(axis), int(rounding),
-                                              int(bool(pack)), _ptr(q_out), _ptr(scale_out), _stream(stream)))
+    st = _fc().quantize(x.data_ptr(), rows, cols, ld, bits, axis, rounding, bool(pack), q_out.data_ptr(), scale_out.data_ptr(),
+                        _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_quantize", st)
     return q_out, scale_out
 
 
@@ -226,12 +255,23 @@ def aqt_unpack_int4(packed: torch.Tensor, cols: int, out: Optional[torch.Tensor]
     return out
 
 
-def _workspace(need: int, workspace: Optional[torch.Tensor], device) -> Optional[torch.Tensor]:
-    if need == 0:
-        return workspace
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=device)
-    return workspace
+def _workspace(op: int, M: int, N: int, K: int, bits_a: int, bits_w: int, device) -> Optional[torch.Tensor]:
+    """Scratch for a caller that brought none (None where the call needs none)."""
+    need = aqt_workspace_bytes(op, M, N, K, bits_a, bits_w)
+    return torch.empty(need, dtype=torch.uint8, device=device) if need else None
+
+
+def _addr(t: Optional[torch.Tensor]):
+    return None if t is None else t.data_ptr()
+
+
+def _area(t: Optional[torch.Tensor]) -> Tuple[int, int]:
+    """Address and size of a workspace tensor."""
+    return (0, 0) if t is None else (t.data_ptr(), t.numel())
+
+
+def _pitch(t: Optional[torch.Tensor]) -> int:
+    return 0 if t is None else t.stride(0)
 
 
 def aqt_qmatmul(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s_w: torch.Tensor,
@@ -246,16 +286,21 @@ def aqt_qmatmul(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s_w: torc
     n_out = _n_out(N, act)
     if y is None:
         y = torch.empty((M, n_out), dtype=torch.float32, device=xq.device)
-    need = aqt_workspace_bytes(OP_QMATMUL, M, N, K, bits_a, bits_w)
-    workspace = _workspace(need, workspace, xq.device)
-    args = (_ptr(xq), _ptr(s_x), int(s_x_kind), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
-            _i64(residual.stride(0) if residual is not None else 0), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K),
-            int(bits_a), int(bits_w), int(act), _ptr(y), _i64(y.stride(0)), _ptr(acc_debug), _ptr(workspace),
-            ctypes.c_size_t(0 if workspace is None else workspace.numel()), _stream(stream))
+    if workspace is None:
+        workspace = _workspace(OP_QMATMUL, M, N, K, bits_a, bits_w, xq.device)
     if plan is None:
-        _check("aqt_qmatmul", lib().aqt_qmatmul(*args))
+        ws, ws_bytes = _area(workspace)
+        st = _fc().qmatmul(xq.data_ptr(), s_x.data_ptr(), s_x_kind, wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual),
+                           _pitch(residual), residual_scale, M, N, K, bits_a, bits_w, act, y.data_ptr(), y.stride(0), _addr(acc_debug),
+                           ws, ws_bytes, _raw_stream(stream))
+        if st != AQT_OK:
+            raise AqtError("aqt_qmatmul", st)
     else:
-        _check("aqt_qmatmul_with_plan", lib().aqt_qmatmul_with_plan(ctypes.c_char_p(plan.encode()), *args))
+        _check("aqt_qmatmul_with_plan", lib().aqt_qmatmul_with_plan(
+            ctypes.c_char_p(plan.encode()), _ptr(xq), _ptr(s_x), int(s_x_kind), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
+            _i64(_pitch(residual)), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K), int(bits_a), int(bits_w), int(act), _ptr(y),
+            _i64(y.stride(0)), _ptr(acc_debug), _ptr(workspace), ctypes.c_size_t(0 if workspace is None else workspace.numel()),
+            _stream(stream)))
     return y
 
 
@@ -276,14 +321,14 @@ def aqt_qmatmul_requant(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s
         s_out = torch.empty((M,), dtype=torch.float32, device=xq.device)
     if y is None and (want_y or residual is not None):
         y = torch.empty((M, n_out), dtype=torch.float32, device=xq.device)
-    need = aqt_workspace_bytes(OP_QMATMUL_REQUANT, M, N, K, bits_a, bits_w)
-    workspace = _workspace(need, workspace, xq.device)
-    _check("aqt_qmatmul_requant", lib().aqt_qmatmul_requant(
-        _ptr(xq), _ptr(s_x), int(s_x_kind), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
-        _i64(residual.stride(0) if residual is not None else 0), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K),
-        int(bits_a), int(bits_w), int(act), int(bits_out), int(rounding), int(bool(pack_out)), _ptr(q_out), _ptr(s_out),
-        _ptr(y), _i64(y.stride(0) if y is not None else 0), _ptr(workspace),
-        ctypes.c_size_t(0 if workspace is None else workspace.numel()), _stream(stream)))
+    if workspace is None:
+        workspace = _workspace(OP_QMATMUL_REQUANT, M, N, K, bits_a, bits_w, xq.device)
+    ws, ws_bytes = _area(workspace)
+    st = _fc().qmatmul_requant(xq.data_ptr(), s_x.data_ptr(), s_x_kind, wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual),
+                               _pitch(residual), residual_scale, M, N, K, bits_a, bits_w, act, bits_out, rounding, bool(pack_out),
+                               q_out.data_ptr(), s_out.data_ptr(), _addr(y), _pitch(y), ws, ws_bytes, _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_qmatmul_requant", st)
     return q_out, s_out, y
 
 
@@ -315,13 +360,14 @@ def aqt_linear_fwd(x: torch.Tensor, wq: torch.Tensor, s_w: torch.Tensor, bias: O
     n_out = _n_out(N, act)
     if y is None:
         y = torch.empty((M, n_out), dtype=torch.float32, device=x.device)
-    need = aqt_workspace_bytes(OP_LINEAR_FWD, M, N, K, bits_a, bits_w)
-    workspace = _workspace(need, workspace, x.device)
-    _check("aqt_linear_fwd", lib().aqt_linear_fwd(
-        _ptr(x), _i64(x.stride(0)), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
-        _i64(residual.stride(0) if residual is not None else 0), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K),
-        int(bits_a), int(bits_w), int(a_scale_kind), int(rounding), int(act), _ptr(y), _i64(y.stride(0)), _ptr(workspace),
-        ctypes.c_size_t(workspace.numel()), _stream(stream)))
+    if workspace is None:
+        workspace = _workspace(OP_LINEAR_FWD, M, N, K, bits_a, bits_w, x.device)
+    ws, ws_bytes = _area(workspace)
+    st = _fc().linear_fwd(x.data_ptr(), x.stride(0), wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual), _pitch(residual),
+                          residual_scale, M, N, K, bits_a, bits_w, a_scale_kind, rounding, act, y.data_ptr(), y.stride(0), ws, ws_bytes,
+                          _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_linear_fwd", st)
     return y
 
 
@@ -336,13 +382,14 @@ def aqt_linear_fwd_weight_only(x: torch.Tensor, wq: torch.Tensor, s_w: torch.Ten
     N = wq.shape[0]
     if y is None:
         y = torch.empty((M, _n_out(N, act)), dtype=torch.float32, device=x.device)
-    need = aqt_workspace_bytes(OP_LINEAR_WEIGHT_ONLY_X2 if precision == FLOAT_TF32X2 else OP_LINEAR_WEIGHT_ONLY, M, N, K, 0, bits_w)
-    workspace = _workspace(need, workspace, x.device)
-    _check("aqt_linear_fwd_weight_only", lib().aqt_linear_fwd_weight_only(
-        _ptr(x), _i64(x.stride(0)), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
-        _i64(residual.stride(0) if residual is not None else 0), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K),
-        int(bits_w), int(precision), int(act), _ptr(y), _i64(y.stride(0)), _ptr(workspace), ctypes.c_size_t(workspace.numel()),
-        _stream(stream)))
+    if workspace is None:
+        workspace = _workspace(OP_LINEAR_WEIGHT_ONLY_X2 if precision == FLOAT_TF32X2 else OP_LINEAR_WEIGHT_ONLY, M, N, K, 0, bits_w, x.device)
+    ws, ws_bytes = _area(workspace)
+    st = _fc().linear_fwd_weight_only(x.data_ptr(), x.stride(0), wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual),
+                                      _pitch(residual), residual_scale, M, N, K, bits_w, precision, act, y.data_ptr(), y.stride(0), ws,
+                                      ws_bytes, _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_linear_fwd_weight_only", st)
     return y
 
 
@@ -358,12 +405,13 @@ def aqt_linear_bwd(dy: torch.Tensor, xq: Optional[torch.Tensor], s_x: Optional[t
     dx = torch.empty((M, K), **f32) if want_dx else None
     dw = torch.empty((N, K), **f32) if want_dw else None
     db = torch.empty((N,), **f32) if want_dbias else None
-    need = aqt_workspace_bytes(OP_LINEAR_BWD, M, N, K, 0, 0)
-    workspace = _workspace(need, workspace, dy.device)
-    _check("aqt_linear_bwd", lib().aqt_linear_bwd(
-        _ptr(dy), _i64(dy.stride(0)), _ptr(xq), _ptr(s_x), int(s_x_kind), int(bits_a), _ptr(wq), _ptr(s_w), int(bits_w),
-        _i64(M), _i64(N), _i64(K), _ptr(dx), _i64(K), _ptr(dw), _i64(K), _ptr(db), _ptr(workspace),
-        ctypes.c_size_t(0 if workspace is None else workspace.numel()), _stream(stream)))
+    if workspace is None:
+        workspace = _workspace(OP_LINEAR_BWD, M, N, K, 0, 0, dy.device)
+    ws, ws_bytes = _area(workspace)
+    st = _fc().linear_bwd(dy.data_ptr(), dy.stride(0), _addr(xq), _addr(s_x), s_x_kind, bits_a, _addr(wq), _addr(s_w), bits_w, M, N, K,
+                          _addr(dx), K, _addr(dw), K, _addr(db), ws, ws_bytes, _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_linear_bwd", st)
     return dx, dw, db
 
 
@@ -404,12 +452,16 @@ def bind_ffn_fwd(x, w1q, s_w1, bits_w1, w2q, s_w2, bits_w2, y, workspace, *, bit
                 _ptr(workspace), ctypes.c_size_t(workspace.numel()), _stream(stream))
 
 
-def aqt_ffn_fwd(x, w1q, s_w1, bits_w1, w2q, s_w2, bits_w2, y, workspace=None, **kw):
+def aqt_ffn_fwd(x, w1q, s_w1, bits_w1, w2q, s_w2, bits_w2, y, workspace=None, *, bits_a=8, rounding=ROUND_NEAREST_EVEN, act=ACT_SWISH,
+                stream=None):
     """y = W2 . act(W1 . x) through two quantized layers (aqt_ffn_fwd); x / y may be pinned host tensors."""
     M, d = x.shape
     ff = w1q.shape[0]
     if workspace is None:
-        workspace = torch.empty(aqt_workspace_bytes(OP_FFN_FWD, M, ff, d, kw.get("bits_a", 8), 4), dtype=torch.uint8,
-                                device=w1q.device)
-    bind_ffn_fwd(x, w1q, s_w1, bits_w1, w2q, s_w2, bits_w2, y, workspace, **kw)()
+        workspace = _workspace(OP_FFN_FWD, M, ff, d, bits_a, 4, w1q.device)
+    ws, ws_bytes = _area(workspace)
+    st = _fc().ffn_fwd(x.data_ptr(), not x.is_cuda, w1q.data_ptr(), s_w1.data_ptr(), None, bits_w1, w2q.data_ptr(), s_w2.data_ptr(), None,
+                       bits_w2, M, d, ff, bits_a, rounding, act, y.data_ptr(), not y.is_cuda, ws, ws_bytes, _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_ffn_fwd", st)
     return y
