@@ -249,6 +249,45 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
                 void* stream);
 
 /*
+ * aqt_chain_fwd -- a chain of quantized layers on a few rows (streaming: a step of some frames
+ * through a whole encoder) in one launch.  (No counterpart in the paper: layer by layer this is
+ * aqt_quantize + aqt_qmatmul, with the same arithmetic and the same bits; a step of a few rows is
+ * bound by the number of dependent kernels, not by their work.)
+ *   c_0 = quantize(x, rows, layers[0].bits_a);  h = x
+ *   layer i:  a = act(fma(float(acc) * s, s_w, bias)),  acc = c . wq^T
+ *             o = a, or with AQT_CHAIN_ADD  o = fma(residual_scale, a, h);  h = o
+ *             y = o where y is given
+ *             unless AQT_CHAIN_SIDE: the next layer's input is quantize(o, rows, its bits_a);
+ *             after a side layer the next layer reads the same input again
+ * x         fp32 [M, layers[0].K], row pitch ldx (a multiple of 4 floats), 16-byte aligned.
+ * layers    host array, read during the call.  wq, s_w, bias, N, K, bits_w, act as for aqt_qmatmul;
+ *           y fp32 [M, N_out] with row pitch ldy (16-byte aligned, ldy % 4 == 0) or NULL.
+ * M         any, but the call is meant for at most AQT_CHAIN_MAX_ROWS rows: from there on layer by
+ *           layer is faster.
+ * Limits (AQT_ERR_UNSUPPORTED otherwise, nothing enqueued): at most AQT_CHAIN_MAX_LAYERS layers; N and
+ * N_out multiples of 128, N <= 8192, N_out <= 4096; K a multiple of 128, K <= 8192; layers that read the
+ * same input agree in bits_a and in whether their weights are packed; layers with AQT_CHAIN_ADD have
+ * N_out equal to layers[0].K.
+ */
+#define AQT_CHAIN_SIDE 1
+#define AQT_CHAIN_ADD 2
+#define AQT_CHAIN_MAX_LAYERS 256
+#define AQT_CHAIN_MAX_ROWS 224
+typedef struct aqt_chain_layer {
+  const void* wq;
+  const float* s_w;
+  const float* bias;
+  float* y;
+  int64_t ldy;
+  int32_t N, K;
+  int32_t bits_w, bits_a;
+  int32_t act, flags;
+  float residual_scale;
+  int32_t reserved;
+} aqt_chain_layer;
+int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer* layers, int n_layers, int rounding, void* stream);
+
+/*
  * aqt_linear_fwd_weight_only -- the layer of the weight-only configurations of Section 4.1 (I8W
  * and I4W: 8- or 4-bit weight codes against unquantized binary32 activations; the section notes
  * that the codes have to be turned back into floats when the layer runs).  Activations are not quantized; the stored

@@ -32,8 +32,9 @@ STATIC_WEIGHTS = 0x100  # OR into bits_w: the weights were complete before the p
 EXPORTS = ("aqt_version", "aqt_status_string", "aqt_quantize", "aqt_pack_int4", "aqt_unpack_int4", "aqt_qmatmul",
            "aqt_linear_fwd", "aqt_linear_fwd_host", "aqt_workspace_bytes", "aqt_device_status", "aqt_qmatmul_w4_noalloc",
            "aqt_selftest_bounded_wait", "aqt_qmatmul_requant", "aqt_linear_fwd_weight_only", "aqt_linear_bwd",
-           "aqt_plan_qmatmul", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_selftest_sfu_rate")
+           "aqt_plan_qmatmul", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_chain_fwd", "aqt_selftest_sfu_rate")
 NOALLOC_MAX_WEIGHT_BYTES = 4 << 20
+CHAIN_MAX_ROWS = 224
 
 
 class AqtError(RuntimeError):
@@ -413,6 +414,34 @@ def aqt_linear_bwd(dy: torch.Tensor, xq: Optional[torch.Tensor], s_x: Optional[t
     if st != AQT_OK:
         raise AqtError("aqt_linear_bwd", st)
     return dx, dw, db
+
+
+def _chain_input_ok(x: torch.Tensor) -> bool:
+    return (0 < x.shape[0] <= CHAIN_MAX_ROWS and x.is_cuda and x.dtype == torch.float32 and x.dim() == 2 and x.stride(1) == 1
+            and x.stride(0) % 4 == 0 and x.data_ptr() % 16 == 0)
+
+
+def chain_ffn(x: torch.Tensor, first, second, y: torch.Tensor, rounding: int, stream=None) -> bool:
+    """y = W2 . act(W1 . x) of two encoder.QuantLinear layers in one launch (aqt_chain_fwd), for a few rows.
+    False, and nothing done, where the shape does not allow it."""
+    if not _chain_input_ok(x):
+        return False
+    st = _fc().chain_ffn(x.data_ptr(), x.stride(0), x.shape[0], first, second, y.data_ptr(), y.stride(0), rounding, _raw_stream(stream))
+    if st not in (AQT_OK, -2, -3):
+        raise AqtError("aqt_chain_fwd", st)
+    return st == AQT_OK
+
+
+def chain_encoder(x: torch.Tensor, blocks, qkv: torch.Tensor, out: torch.Tensor, rounding: int, stream=None) -> bool:
+    """The layers of encoder.EncoderStack's blocks in one launch (aqt_chain_fwd), for a few rows.  False, and
+    nothing done, where a shape does not allow it."""
+    if not _chain_input_ok(x):
+        return False
+    st = _fc().chain_encoder(x.data_ptr(), x.stride(0), x.shape[0], blocks, qkv.data_ptr(), qkv.stride(0), out.data_ptr(), out.stride(0),
+                             rounding, _raw_stream(stream))
+    if st not in (AQT_OK, -2, -3):
+        raise AqtError("aqt_chain_fwd", st)
+    return st == AQT_OK
 
 
 def linear_fwd_host_workspace_bytes(M: int, N: int, K: int, bits_a: int, bits_w: int, act: int,

@@ -7,6 +7,7 @@
 #include "qgemm_requant_sm100.cuh"
 #include "qgemv_small_m.cuh"
 #include "quantize.cuh"
+#include "chain_small_m.cuh"
 
 using namespace aqt;
 
@@ -570,6 +571,63 @@ int aqt_linear_fwd_host(const float* x, int x_on_host, const void* wq, const flo
   return AQT_OK;
 }
 
+int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer* layers, int n_layers, int rounding, void* stream) {
+  if (M < 0 || n_layers < 0 || (n_layers > 0 && layers == nullptr)) return AQT_ERR_BADARG;
+  if (rounding != AQT_ROUND_HALF_UP_FLOOR && rounding != AQT_ROUND_NEAREST_EVEN) return AQT_ERR_BADARG;
+  if (M == 0 || n_layers == 0) return AQT_OK;
+  if (n_layers > AQT_CHAIN_MAX_LAYERS || M >= (1ll << 24)) return AQT_ERR_UNSUPPORTED;
+  if (x == nullptr) return AQT_ERR_BADARG;
+  if (!is_aligned(x, 16) || ldx % 4 != 0) return AQT_ERR_ALIGN;
+  ChainParams<kChainMaxSteps> p;
+  p.x = x;
+  p.ldx = ldx;
+  p.M = (int32_t)M;
+  p.K0 = layers[0].K;
+  p.n_steps = n_layers;
+  p.rounding = rounding;
+  p.in_qmax = qmax_of(layers[0].bits_a);
+  p.h_cols = 0;
+  if (ldx < p.K0) return AQT_ERR_BADARG;
+  int64_t width = p.K0;  // of the current input
+  int head = 0;          // first layer that reads it
+  int feeder = -1;       // layer whose output it is
+  for (int i = 0; i < n_layers; ++i) {
+    const aqt_chain_layer& l = layers[i];
+    int rc = validate_matmul_shape(M, l.N, l.K, l.bits_a, l.bits_w, l.act, AQT_SCALE_ROW);
+    if (rc != AQT_OK) return rc;
+    const int64_t n_out = is_glu(l.act) ? l.N / 2 : l.N;
+    if (!quant_bits_ok(l.bits_a) || l.K != width || l.N == 0) return AQT_ERR_BADARG;
+    if (l.wq == nullptr || l.s_w == nullptr || (l.y != nullptr && l.ldy < n_out)) return AQT_ERR_BADARG;
+    if (!is_aligned(l.wq, 16) || !is_aligned(l.s_w, 4) || (l.y != nullptr && (!is_aligned(l.y, 16) || l.ldy % 4 != 0))) return AQT_ERR_ALIGN;
+    ChainStep& s = p.steps[i];
+    s.w = reinterpret_cast<const uint8_t*>(l.wq);
+    s.s_w = l.s_w;
+    s.bias = l.bias;
+    s.y = l.y;
+    s.ldy = (int32_t)l.ldy;
+    s.N = l.N;
+    s.K = l.K;
+    s.rs = l.residual_scale;
+    s.flags = (uint32_t)l.act | (is_packed(l.bits_w) ? kChainPacked : 0u) | ((l.flags & AQT_CHAIN_SIDE) ? kChainSide : 0u) |
+              ((l.flags & AQT_CHAIN_ADD) ? kChainAdd : 0u);
+    if (l.ldy >= (1ll << 31) || !chain_step_ok(s)) return AQT_ERR_UNSUPPORTED;
+    if (l.bits_a != layers[head].bits_a || is_packed(l.bits_w) != is_packed(layers[head].bits_w)) return AQT_ERR_UNSUPPORTED;
+    if (i == head && feeder >= 0 && l.bits_a == 4) p.steps[feeder].flags |= kChainOut4;
+    if (l.flags & AQT_CHAIN_ADD) {
+      if (n_out != p.K0) return AQT_ERR_UNSUPPORTED;
+      p.h_cols = p.K0 / kChainCtas;
+    }
+    if (!(l.flags & AQT_CHAIN_SIDE)) {
+      width = n_out;
+      head = i + 1;
+      feeder = i;
+    }
+  }
+  int rc = check_device();
+  if (rc != AQT_OK) return rc;
+  return launch_chain(p, reinterpret_cast<cudaStream_t>(stream));
+}
+
 int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w1, const float* bias1, int bits_w1,
                 const void* w2q, const float* s_w2, const float* bias2, int bits_w2, int64_t M, int64_t d, int64_t ff,
                 int bits_a, int rounding, int act, float* y, int y_on_host, void* workspace, size_t workspace_bytes,
@@ -601,6 +659,15 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
   float* s1 = reinterpret_cast<float*>(ws + L.s1);
   int8_t* q2 = reinterpret_cast<int8_t*>(ws + L.q2);
   float* s2 = reinterpret_cast<float*>(ws + L.s2);
+  if (M <= AQT_CHAIN_MAX_ROWS) {
+    // a few rows: both layers in one launch
+    const aqt_chain_layer pair[2] = {
+        {w1q, s_w1, bias1, nullptr, 0, (int32_t)ff, (int32_t)d, bits_w1, bits_a, act, 0, 0.0f, 0},
+        {w2q, s_w2, bias2, y_dev, d, (int32_t)d, (int32_t)ff, bits_w2, bits_a, AQT_ACT_NONE, 0, 0.0f, 0}};
+    rc = aqt_chain_fwd(x_dev, d, M, pair, 2, rounding, stream);
+    if (rc == AQT_OK && y_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(y, y_dev, (size_t)M * d * 4, cudaMemcpyDeviceToHost, st));
+    if (rc != AQT_ERR_UNSUPPORTED && rc != AQT_ERR_ALIGN) return rc;
+  }
   const size_t mm_bytes = L.total - L.mm;
   // Fig. 2 on the input rows; first matmul with the rows of u = act(W1 x) quantized in its epilogue
   // (4-bit codes stay in int8 containers between the kernels); second matmul.

@@ -1,0 +1,494 @@
+// A chain of quantized layers on a few rows (a streaming step of some frames through a whole encoder)
+// in one launch.
+//
+// What bounds such a step is not work but the number of dependent kernels: an eight-row step through
+// the 17-block d = 512 encoder reads 67 MB of weights (10 us of HBM time) in 187 launches of 2 to
+// 11 us each (1276 us).  Here one thread-block cluster of sixteen CTAs carries up to 32 rows through
+// every layer; clusters take different rows and do not interact (rows are independent under per-row
+// scales).  Within a cluster:
+//   * CTA r owns 1/16 of every layer's output channels and with it 1/16 of the weights, which stream
+//     from L2 / HBM into registers, one chunk (eight 16-byte loads a lane) ahead of use across layer
+//     boundaries, L2 prefetches two layers ahead;
+//   * every CTA holds the codes of all rows of the current activations in shared memory; the products
+//     are mma.sync m16n8k32 (int8): 16 rows fill its M, where a tcgen05 tile would spend 128 rows on
+//     16 and first want the weights unpacked in shared memory;
+//   * the output rows are quantized for the next layer in place (Fig. 2): row maxima go to all sixteen
+//     CTAs' shared memory, a cluster barrier, then each CTA writes its share of the codes to all
+//     sixteen, a second barrier.  Nothing but requested outputs is written to global memory, and the
+//     residual stream stays in shared memory with the CTA that owns its columns.
+// All exchange is through distributed shared memory and the hardware's cluster barrier: no CTA polls
+// memory, and a cluster is scheduled as a whole, so nothing has to be resident beside it.
+// The arithmetic is that of the per-layer kernels operation by operation (exact int32 sums, the same
+// de-quantization, activation and quantizer), so the results are the same bits.
+#pragma once
+
+#include "aqt_common.cuh"
+#include "pack.cuh"
+#include "qgemv_small_m.cuh"
+#include "quantize.cuh"
+
+namespace aqt {
+
+constexpr int kChainCtas = 16;     // CTAs of a cluster (beyond the portable eight: allowed per function)
+constexpr int kChainWarps = 16;
+constexpr int kChainThreads = 32 * kChainWarps;
+constexpr int kChainChunk = 8;     // 16-byte weight loads per lane in flight
+constexpr int kChainMaxSteps = 256;
+constexpr int kChainMaxN = 16 * kChainThreads;  // one scale per thread
+constexpr int kChainMaxCols = 256;              // output columns per CTA: eight floats per lane and row
+
+struct ChainStep {
+  const uint8_t* w;   // codes [N, K] int8, or packed [N, K/2]
+  const float* s_w;
+  const float* bias;
+  float* y;           // fp32 output [M, N_out] or null
+  int32_t N, K, ldy;
+  float rs;           // residual scale
+  uint32_t flags;
+};
+enum : uint32_t {
+  kChainActMask = 3u,
+  kChainPacked = 4u,  // 4-bit weights, two per byte
+  kChainSide = 8u,    // the output only goes to y: the next step reads the same input
+  kChainAdd = 16u,    // output = residual stream + rs * act(z), and is the new residual stream
+  kChainOut4 = 32u    // the next layer's input is quantized to 4 bits
+};
+
+template <int MAXS>
+struct ChainParams {
+  const float* x;
+  int64_t ldx;
+  int32_t M, K0, n_steps, rounding;
+  int32_t in_qmax;     // of the first step's input
+  int32_t code_bytes;  // shared memory for the activation codes
+  int32_t part_bytes;  // for the partial sums
+  int32_t h_cols;      // residual-stream columns per CTA (0: no step adds)
+  ChainStep steps[MAXS];
+};
+
+// Activation codes: row pitch by the consumer's weight width, so that the eight lanes of a 128-bit
+// shared-memory phase (two rows, four lanes each) touch all banks once: a lane reads 32 codes per
+// 128 with packed weights, 16 per 64 with int8 weights.
+__host__ __device__ inline int chain_pitch(int K, bool packed) { return K + (packed ? 16 : 64); }
+// n8-tiles per CTA (value and gate tiles for GLU) and the split of K over warps.
+__host__ __device__ inline int chain_tiles(int N) { return N / (8 * kChainCtas); }
+__host__ __device__ inline int chain_ksplit(int tiles, int K) {
+  if (tiles >= kChainWarps) return 1;
+  const int by_warps = kChainWarps / tiles, by_k = K / 128;
+  return by_warps < by_k ? by_warps : by_k;
+}
+
+__device__ __forceinline__ void mma_s8_16x8x32(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t chain_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t chain_mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void chain_st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void chain_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Four codes of a row as one word.
+template <int ROUNDING>
+__device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax) {
+  if (c.fast)
+    return pack4_i8(quantize_fast<ROUNDING>(v[0], c.s, c.r), quantize_fast<ROUNDING>(v[1], c.s, c.r), quantize_fast<ROUNDING>(v[2], c.s, c.r),
+                    quantize_fast<ROUNDING>(v[3], c.s, c.r));
+  return pack4_i8(quantize_elem<ROUNDING>(v[0], c, qmax), quantize_elem<ROUNDING>(v[1], c, qmax), quantize_elem<ROUNDING>(v[2], c, qmax),
+                  quantize_elem<ROUNDING>(v[3], c, qmax));
+}
+__device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax, int rounding) {
+  return rounding == AQT_ROUND_HALF_UP_FLOOR ? chain_codes4<AQT_ROUND_HALF_UP_FLOOR>(v, c, qmax)
+                                             : chain_codes4<AQT_ROUND_NEAREST_EVEN>(v, c, qmax);
+}
+__device__ __forceinline__ float chain_max4(float m, const float (&v)[4]) {
+  return fmaxf(m, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
+}
+
+// MT: 16-row tiles per cluster.
+template <int MT, int MAXS>
+__global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const __grid_constant__ ChainParams<MAXS> p) {
+  constexpr int R = 16 * MT;
+  extern __shared__ __align__(128) uint8_t chain_smem[];
+  __shared__ __align__(16) float sw_s[2][kChainThreads], bias_s[2][kChainThreads];
+  __shared__ uint32_t amax_s[R][kChainCtas];  // bit patterns of the row maxima of every CTA's columns
+  uint8_t* codes = chain_smem;
+  int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes);
+  float* h = reinterpret_cast<float*>(chain_smem + p.code_bytes + p.part_bytes);  // [R][h_cols]
+
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, kq = lane & 3;
+  const uint32_t rank = cluster_ctarank();
+  const int row0 = (int)(blockIdx.x / kChainCtas) * R;
+  const int rows = min(R, p.M - row0);
+
+  grid_dependency_wait();
+
+  // ---- weight chunks of this warp in program order: (step, unit, first load of the chunk)
+  int it_step = 0, it_u = warp, it_i = 0;
+  uint4 nxt[kChainChunk];
+  auto unit_loads = [&](const ChainStep& st, int u) {  // 16-byte loads per lane of unit u
+    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7, ks = u / tiles;
+    const int blocks = (ks + 1) * k128 / ks_n - ks * k128 / ks_n;
+    return (st.flags & kChainPacked) ? blocks : 2 * blocks;
+  };
+  auto skip_idle_steps = [&]() {
+    while (it_step < p.n_steps) {
+      const int tiles = chain_tiles(p.steps[it_step].N);
+      if (it_u < tiles * chain_ksplit(tiles, p.steps[it_step].K)) break;
+      ++it_step;
+      it_u = warp;
+    }
+  };
+  auto load_next = [&]() {  // the chunk the iterator stands on -> nxt, then advance
+    if (it_step >= p.n_steps) return;
+    const ChainStep& st = p.steps[it_step];
+    const bool packed = (st.flags & kChainPacked) != 0;
+    const uint32_t act = st.flags & kChainActMask;
+    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7;
+    const int tile = it_u % tiles, ks = it_u / tiles;
+    int n = (int)rank * (st.N / kChainCtas) + tile * 8 + g;
+    if (act >= AQT_ACT_GLU) {  // value tiles, then the gate tiles of the same output columns
+      const int half = tiles >> 1, gate = tile >= half;
+      n = gate * (st.N >> 1) + (int)rank * (st.N / (2 * kChainCtas)) + (tile - gate * half) * 8 + g;
+    }
+    const int64_t row_bytes = packed ? st.K >> 1 : st.K;
+    const uint8_t* src = st.w + n * row_bytes + (int64_t)(ks * k128 / ks_n) * (packed ? 64 : 128) + it_i * 64 + kq * 16;
+    const int left = unit_loads(st, it_u) - it_i;
+#pragma unroll
+    for (int j = 0; j < kChainChunk; ++j)
+      if (j < left) nxt[j] = __ldg(reinterpret_cast<const uint4*>(src + j * 64));
+    it_i += kChainChunk;
+    if (left <= kChainChunk) {
+      it_i = 0;
+      it_u += kChainWarps;
+      skip_idle_steps();
+    }
+  };
+  auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
+    wv = bv = 0.0f;
+    if (s >= p.n_steps) return;
+    const ChainStep& st = p.steps[s];
+    const int per_cta = st.N / kChainCtas, c = threadIdx.x;
+    if (c >= per_cta) return;
+    int n = (int)rank * per_cta + c;
+    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
+      const int cols = per_cta >> 1, gate = c >= cols;
+      n = gate * (st.N >> 1) + (int)rank * cols + c - gate * cols;
+    }
+    wv = __ldg(st.s_w + n);
+    if (st.bias != nullptr) bv = __ldg(st.bias + n);
+  };
+  auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2
+    if (threadIdx.x != 0 || s >= p.n_steps || blockIdx.x >= kChainCtas) return;
+    const ChainStep& st = p.steps[s];
+    const int64_t row_bytes = (st.flags & kChainPacked) ? st.K >> 1 : st.K;
+    const int per_cta = st.N / kChainCtas;
+    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
+      const int cols = per_cta >> 1;
+#pragma unroll 1
+      for (int gate = 0; gate < 2; ++gate)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st.w + (gate * (int64_t)(st.N >> 1) + (int64_t)rank * cols) * row_bytes),
+                     "r"((uint32_t)(cols * row_bytes))
+                     : "memory");
+    } else {
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st.w + (int64_t)rank * per_cta * row_bytes), "r"((uint32_t)(per_cta * row_bytes))
+                   : "memory");
+    }
+  };
+
+  skip_idle_steps();
+  load_next();
+  prefetch_slice(1);
+  {
+    float wv, bv;
+    load_scales(0, wv, bv);
+    sw_s[0][threadIdx.x] = wv;
+    bias_s[0][threadIdx.x] = bv;
+  }
+
+  // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
+  float sx[MT];  // input scales of this warp's rows (warp, warp + 16)
+  {
+    const int pitch = chain_pitch(p.K0, (p.steps[0].flags & kChainPacked) != 0);
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      const int r = warp + 16 * t;
+      sx[t] = 0.0f;
+      if (r >= rows) continue;
+      const float4* xr = reinterpret_cast<const float4*>(p.x + (int64_t)(row0 + r) * p.ldx);
+      float amax = 0.0f;
+      for (int c = lane; c < p.K0 / 4; c += 32) {
+        const float4 f = __ldg(xr + c);
+        const float v[4] = {f.x, f.y, f.z, f.w};
+        amax = chain_max4(amax, v);
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
+      const ScaleCtx sc = make_scale_ctx(amax, p.in_qmax);
+      sx[t] = sc.s;
+      for (int c = lane; c < p.K0 / 4; c += 32) {
+        const float4 f = __ldg(xr + c);
+        const float v[4] = {f.x, f.y, f.z, f.w};
+        *reinterpret_cast<uint32_t*>(codes + r * pitch + 4 * c) = chain_codes4(v, sc, p.in_qmax, p.rounding);
+      }
+      for (int c = lane; c < p.h_cols / 4; c += 32)
+        *reinterpret_cast<float4*>(h + r * p.h_cols + 4 * c) = __ldg(xr + (int)rank * (p.h_cols / 4) + c);
+    }
+  }
+  chain_cluster_sync();  // codes ready; every CTA of the cluster runs (its shared memory may be written)
+
+  for (int s = 0; s < p.n_steps; ++s) {
+    const ChainStep& st = p.steps[s];
+    const bool packed = (st.flags & kChainPacked) != 0;
+    const uint32_t act = st.flags & kChainActMask;
+    const int per_cta = st.N / kChainCtas;
+    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7;
+    const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 8;
+    prefetch_slice(s + 2);
+    float wv, bv;
+    load_scales(s + 1, wv, bv);
+
+    // ---- integer products of this warp's units (tile, share of K)
+    for (int u = warp; u < tiles * ks_n; u += kChainWarps) {
+      const int tile = u % tiles, ks = u / tiles;
+      const int n_loads = unit_loads(st, u);
+      int acc[MT][2][4];
+#pragma unroll
+      for (int t = 0; t < MT; ++t)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[t][j >> 2][j & 3] = 0;
+      const uint8_t* a_row = codes + g * pitch + (ks * k128 / ks_n) * 128 + kq * (packed ? 32 : 16);
+      for (int i0 = 0; i0 < n_loads; i0 += kChainChunk) {
+        uint4 cur[kChainChunk];
+#pragma unroll
+        for (int j = 0; j < kChainChunk; ++j) cur[j] = nxt[j];
+        load_next();
+        const uint8_t* a0 = a_row + i0 * (packed ? 128 : 64);
+        if (packed) {
+#pragma unroll
+          for (int j = 0; j < kChainChunk; ++j) {
+            if (i0 + j >= n_loads) break;
+            uint32_t b[8];
+            unpack_word(cur[j].x, b[0], b[1]);
+            unpack_word(cur[j].y, b[2], b[3]);
+            unpack_word(cur[j].z, b[4], b[5]);
+            unpack_word(cur[j].w, b[6], b[7]);
+#pragma unroll
+            for (int t = 0; t < MT; ++t) {
+              const uint8_t* a = a0 + t * 16 * pitch + j * 128;
+              const uint4 l0 = *reinterpret_cast<const uint4*>(a), l1 = *reinterpret_cast<const uint4*>(a + 16);
+              uint4 h0 = make_uint4(0u, 0u, 0u, 0u), h1 = h0;
+              if (rows > 8 + 16 * t) {
+                h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
+                h1 = *reinterpret_cast<const uint4*>(a + 8 * pitch + 16);
+              }
+              mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, b[0], b[1]);
+              mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, b[2], b[3]);
+              mma_s8_16x8x32(acc[t][0], l1.x, h1.x, l1.y, h1.y, b[4], b[5]);
+              mma_s8_16x8x32(acc[t][1], l1.z, h1.z, l1.w, h1.w, b[6], b[7]);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < kChainChunk; ++j) {
+            if (i0 + j >= n_loads) break;
+#pragma unroll
+            for (int t = 0; t < MT; ++t) {
+              const uint8_t* a = a0 + t * 16 * pitch + j * 64;
+              const uint4 l0 = *reinterpret_cast<const uint4*>(a);
+              uint4 h0 = make_uint4(0u, 0u, 0u, 0u);
+              if (rows > 8 + 16 * t) h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
+              mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, cur[j].x, cur[j].y);
+              mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, cur[j].z, cur[j].w);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < MT; ++t) {
+        int* dst = part + (ks * R + 16 * t + g) * part_pitch + tile * 8 + 2 * kq;
+        *reinterpret_cast<int2*>(dst) = make_int2(acc[t][0][0] + acc[t][1][0], acc[t][0][1] + acc[t][1][1]);
+        *reinterpret_cast<int2*>(dst + 8 * part_pitch) = make_int2(acc[t][0][2] + acc[t][1][2], acc[t][0][3] + acc[t][1][3]);
+      }
+    }
+    sw_s[(s + 1) & 1][threadIdx.x] = wv;
+    bias_s[(s + 1) & 1][threadIdx.x] = bv;
+    __syncthreads();
+
+    // ---- epilogue: warp w owns rows w and w + 16, a lane four consecutive columns at a time
+    const bool glu = act >= AQT_ACT_GLU;
+    const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
+    const bool side = (st.flags & kChainSide) != 0, last = s + 1 == p.n_steps;
+    float v[MT][2][4];
+    float amax[MT];
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      amax[t] = 0.0f;
+      const int r = warp + 16 * t;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int c = 4 * lane + 128 * j;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[t][j][e] = 0.0f;
+        if (r >= rows || c >= cols) continue;
+        auto dequant = [&](int cc, float (&z)[4]) {
+          int4 a = make_int4(0, 0, 0, 0);
+          for (int ks = 0; ks < ks_n; ++ks) {
+            const int4 q = *reinterpret_cast<const int4*>(part + (ks * R + r) * part_pitch + cc);
+            a.x += q.x; a.y += q.y; a.z += q.z; a.w += q.w;
+          }
+          const float4 w4 = *reinterpret_cast<const float4*>(&sw_s[s & 1][cc]);
+          const float4 b4 = *reinterpret_cast<const float4*>(&bias_s[s & 1][cc]);
+          z[0] = __fmaf_rn(__fmul_rn(__int2float_rn(a.x), sx[t]), w4.x, b4.x);
+          z[1] = __fmaf_rn(__fmul_rn(__int2float_rn(a.y), sx[t]), w4.y, b4.y);
+          z[2] = __fmaf_rn(__fmul_rn(__int2float_rn(a.z), sx[t]), w4.z, b4.z);
+          z[3] = __fmaf_rn(__fmul_rn(__int2float_rn(a.w), sx[t]), w4.w, b4.w);
+        };
+        float (&o)[4] = v[t][j];
+        dequant(c, o);
+        if (glu) {
+          float zg[4];
+          dequant(cols + c, zg);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(zg[e]));
+        }
+        if (act == AQT_ACT_SWISH || act == AQT_ACT_GLU_SWISH) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(o[e]));
+        }
+        if (st.flags & kChainAdd) {
+          float4* hr = reinterpret_cast<float4*>(h + r * p.h_cols + c);
+          const float4 r4 = *hr;
+          o[0] = __fmaf_rn(st.rs, o[0], r4.x);
+          o[1] = __fmaf_rn(st.rs, o[1], r4.y);
+          o[2] = __fmaf_rn(st.rs, o[2], r4.z);
+          o[3] = __fmaf_rn(st.rs, o[3], r4.w);
+          *hr = make_float4(o[0], o[1], o[2], o[3]);
+        }
+        if (st.y != nullptr)
+          *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + (int)rank * cols + c) = make_float4(o[0], o[1], o[2], o[3]);
+        amax[t] = chain_max4(amax[t], o);
+      }
+    }
+    if (last) break;
+    if (side) {
+      __syncthreads();  // the partial sums have been read
+      continue;
+    }
+
+    // ---- quantize the output rows for the next step
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      const int r = warp + 16 * t;
+      if (r >= rows) continue;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) amax[t] = fmaxf(amax[t], __shfl_xor_sync(0xffffffffu, amax[t], off));
+      if (lane < kChainCtas) chain_st_cluster(chain_mapa(chain_smem_u32(&amax_s[r][rank]), lane), __float_as_uint(amax[t]));
+    }
+    chain_cluster_sync();  // all maxima have arrived; nobody reads the old codes any more
+    const int n_out = glu ? st.N >> 1 : st.N;
+    const int qmax = (st.flags & kChainOut4) ? 7 : 127;
+    const int out_pitch = chain_pitch(n_out, (p.steps[s + 1].flags & kChainPacked) != 0);
+#pragma unroll
+    for (int t = 0; t < MT; ++t) {
+      const int r = warp + 16 * t;
+      if (r >= rows) continue;
+      uint32_t m = lane < kChainCtas ? amax_s[r][lane] : 0u;
+      m = __reduce_max_sync(0xffffffffu, m);
+      const ScaleCtx sc = make_scale_ctx(__uint_as_float(m), qmax);
+      sx[t] = sc.s;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int c = 4 * lane + 128 * j;
+        if (c >= cols) continue;
+        const uint32_t word = chain_codes4(v[t][j], sc, qmax, p.rounding);
+        const uint32_t dst = chain_smem_u32(codes + r * out_pitch + (int)rank * cols + c);
+#pragma unroll
+        for (uint32_t k = 0; k < (uint32_t)kChainCtas; ++k) chain_st_cluster(chain_mapa(dst, (rank + k) & (kChainCtas - 1)), word);
+      }
+    }
+    chain_cluster_sync();  // the next step's codes are complete
+  }
+  grid_dependents_launch();
+  chain_cluster_sync();  // no CTA leaves while its shared memory may still be written
+}
+
+// ------------------------------------------------------------------------------------------------
+// Host side
+
+// True if the chain kernel can run this step at all.
+static bool chain_step_ok(const ChainStep& st) {
+  const bool glu = (st.flags & kChainActMask) >= AQT_ACT_GLU;
+  const int n_out = glu ? st.N / 2 : st.N;
+  if (st.N % (8 * kChainCtas) != 0 || n_out % (8 * kChainCtas) != 0 || st.K % 128 != 0) return false;
+  return st.N <= kChainMaxN && n_out <= kChainMaxCols * kChainCtas && st.K <= 8192;
+}
+
+struct ChainSizes {
+  int code_bytes, part_bytes, h_bytes;
+  int smem(void) const { return code_bytes + part_bytes + h_bytes; }
+};
+static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
+  int code = 0, part = 0, h = 0;
+  for (int i = 0; i < n; ++i) {
+    const ChainStep& st = steps[i];
+    const int tiles = chain_tiles(st.N);
+    const int c = R * (st.K + 64), q = chain_ksplit(tiles, st.K) * R * (st.N / kChainCtas + 8) * 4;
+    if (c > code) code = c;
+    if (q > part) part = q;
+    if ((st.flags & kChainAdd) && R * (st.N / kChainCtas) * 4 > h) h = R * (st.N / kChainCtas) * 4;
+  }
+  ChainSizes z;
+  z.code_bytes = (int)round_up(code, 128);
+  z.part_bytes = (int)round_up(part, 128);
+  z.h_bytes = (int)round_up(h, 128);
+  return z;
+}
+
+constexpr int kChainMaxSmem = 200 * 1024;
+
+// 16-row clusters that run at the same time (the part schedules seven or eight of sixteen CTAs each).
+constexpr int kChainClusters = 7;
+
+template <int MT, int MAXS>
+static int launch_chain_inst(const ChainParams<kChainMaxSteps>& full, int smem, cudaStream_t st) {
+  ChainParams<MAXS> p;
+  memcpy(static_cast<void*>(&p), &full, offsetof(ChainParams<MAXS>, steps) + (size_t)full.n_steps * sizeof(ChainStep));
+  auto kernel = chain_small_m_kernel<MT, MAXS>;
+  static std::atomic<uint64_t> opted_in{0}, wide{0};
+  int rc = ensure_dynamic_smem(kernel, kChainMaxSmem, opted_in);
+  if (rc != AQT_OK) return rc;
+  rc = ensure_wide_clusters(kernel, wide);
+  if (rc != AQT_OK) return rc;
+  const unsigned clusters = (unsigned)ceil_div(full.M, 16 * MT);
+  return launch_pdl(kernel, dim3(clusters * kChainCtas, 1, 1), dim3(kChainThreads, 1, 1), (size_t)smem, st, kChainCtas, p);
+}
+
+// p: everything but the shared-memory sizes.  AQT_ERR_UNSUPPORTED if the kernel cannot take the chain.
+static int launch_chain(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
+  if (p.M <= 0 || p.n_steps <= 0 || p.n_steps > kChainMaxSteps) return AQT_ERR_UNSUPPORTED;
+  // sixteen rows per cluster while the clusters fit the part side by side, then 32
+  int mt = p.M <= 16 * kChainClusters ? 1 : 2;
+  ChainSizes z = chain_sizes(p.steps, p.n_steps, 16 * mt);
+  if (mt == 2 && z.smem() > kChainMaxSmem) {
+    mt = 1;
+    z = chain_sizes(p.steps, p.n_steps, 16);
+  }
+  if (z.smem() > kChainMaxSmem) return AQT_ERR_UNSUPPORTED;
+  p.code_bytes = z.code_bytes;
+  p.part_bytes = z.part_bytes;
+  if (p.n_steps <= 16) return mt == 1 ? launch_chain_inst<1, 16>(p, z.smem(), st) : launch_chain_inst<2, 16>(p, z.smem(), st);
+  return mt == 1 ? launch_chain_inst<1, kChainMaxSteps>(p, z.smem(), st) : launch_chain_inst<2, kChainMaxSteps>(p, z.smem(), st);
+}
+
+}  // namespace aqt

@@ -212,6 +212,8 @@ class FfnPair:
         self.u = torch.empty((M, layers[0].spec.n_out), dtype=torch.float32, device=device) if self.keep_u else None
 
     def forward(self, x: torch.Tensor, y: torch.Tensor) -> torch.Tensor:
+        if self._chains() and aqt.chain_ffn(x, *self.layers, y, self.run.rounding):
+            return y
         if not self.fused:
             self.run(self.layers[0], x, self.u)
             return self.run(self.layers[1], self.u, y)
@@ -220,9 +222,13 @@ class FfnPair:
         uq, us = self.run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u)
         return self.run.matmul(l1, uq, us, y)
 
+    def _chains(self) -> bool:
+        """True if a step is small enough for both layers to run in one launch (shape permitting)."""
+        return self.fused and not self.keep_u and self.run.M <= aqt.CHAIN_MAX_ROWS
+
     @property
     def launches_per_step(self) -> int:
-        """Kernels of the library launched by one forward()."""
+        """Kernels of the library launched by one forward() of a batch (a few rows take one)."""
         l0, l1 = self.layers
         return 3 if self.fused else 4
 
@@ -364,7 +370,13 @@ class EncoderStack:
         self.h1 = torch.empty((M, d), dtype=torch.float32, device=device)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        """x is read only; the result lives in one of the stack's own buffers."""
+        """x is read only; the result lives in one of the stack's own buffers.  A streaming step of a few
+        rows goes through all blocks in one launch (aqt_chain_fwd, the same bits)."""
+        run = self.block.run
+        if x.shape[0] <= aqt.CHAIN_MAX_ROWS and x.shape == self.h0.shape and run.a_scale_kind == aqt.SCALE_ROW:
+            out = self.h0 if len(self.blocks) % 2 == 1 else self.h1
+            if aqt.chain_encoder(x, self.blocks, self.block.qkv, out, run.rounding):
+                return out
         src, codes = x, None
         for b, layers in enumerate(self.blocks):
             dst = self.h0 if b % 2 == 0 else self.h1
