@@ -12,12 +12,17 @@
 //   * every CTA holds the codes of all rows of the current activations in shared memory; the products
 //     are mma.sync m16n8k32 (int8): 16 rows fill its M, where a tcgen05 tile would spend 128 rows on
 //     16 and first want the weights unpacked in shared memory;
-//   * the output rows are quantized for the next layer in place (Fig. 2): row maxima go to all sixteen
-//     CTAs' shared memory, a cluster barrier, then each CTA writes its share of the codes to all
-//     sixteen, a second barrier.  Nothing but requested outputs is written to global memory, and the
-//     residual stream stays in shared memory with the CTA that owns its columns.
-// All exchange is through distributed shared memory and the hardware's cluster barrier: no CTA polls
-// memory, and a cluster is scheduled as a whole, so nothing has to be resident beside it.
+//   * the output rows are quantized for the next layer in place (Fig. 2): every warp sends the maxima of
+//     its rows over the CTA's columns to all sixteen CTAs, waits for the other fifteen of each row,
+//     and sends its share of the codes to all sixteen.  Nothing but requested outputs is written
+//     to global memory, and the residual stream stays in shared memory with the CTA that owns its columns.
+// All exchange is by asynchronous stores to distributed shared memory that complete on the receiver's
+// mbarrier: a receiver waits for the bytes it needs (one one-way latency each, where cluster barriers
+// cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
+// scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
+// wait of the library.
+// What a layer then costs is a chain of latencies, so the loops hold no integer division and no
+// dependent parameter load: the step table sits in shared memory with everything derived from the sizes.
 // The arithmetic is that of the per-layer kernels operation by operation (exact int32 sums, the same
 // de-quantization, activation and quantizer), so the results are the same bits.
 #pragma once
@@ -45,7 +50,11 @@ struct ChainStep {
   int32_t N, K, ldy;
   float rs;           // residual scale
   uint32_t flags;
+  // derived by the host (chain_derive)
+  uint16_t tiles, ks_n;          // n8-tiles per CTA (value and gate tiles for GLU), shares of K
+  uint32_t inv_tiles, inv_ks;    // ceil(65536 / .): quotients of the small numbers below by a multiply and a shift
 };
+static_assert(sizeof(ChainStep) == 64, "copied to shared memory as 16-byte words");
 enum : uint32_t {
   kChainActMask = 3u,
   kChainPacked = 4u,  // 4-bit weights, two per byte
@@ -71,8 +80,8 @@ struct ChainParams {
 // 128 with packed weights, 16 per 64 with int8 weights.
 __host__ __device__ inline int chain_pitch(int K, bool packed) { return K + (packed ? 16 : 64); }
 // n8-tiles per CTA (value and gate tiles for GLU) and the split of K over warps.
-__host__ __device__ inline int chain_tiles(int N) { return N / (8 * kChainCtas); }
-__host__ __device__ inline int chain_ksplit(int tiles, int K) {
+static inline int chain_tiles(int N) { return N / (8 * kChainCtas); }
+static inline int chain_ksplit(int tiles, int K) {
   if (tiles >= kChainWarps) return 1;
   const int by_warps = kChainWarps / tiles, by_k = K / 128;
   return by_warps < by_k ? by_warps : by_k;
@@ -83,14 +92,36 @@ __device__ __forceinline__ void mma_s8_16x8x32(int (&c)[4], uint32_t a0, uint32_
                : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t chain_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t chain_mapa(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void chain_st_cluster(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+// Store to another CTA's shared memory that counts its bytes on that CTA's mbarrier when it lands.
+__device__ __forceinline__ void chain_st_async(uint32_t addr, uint32_t v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+// mbar_wait with cluster-scope acquire (the data come from other CTAs).
+__device__ __forceinline__ void chain_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint64_t t_start) {
+  for (uint32_t spin = 1;; ++spin) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity), "r"(kTryWaitSuspendNs)
+        : "memory");
+    if (done) return;
+    if ((spin & 0x3) == 0) {
+      if (*abort_flag) return;
+      if (global_timer_ns() - t_start > kWaitLimitNs) {
+        *abort_flag = 1;
+        atomicExch(&g_device_status, AQT_ERR_TIMEOUT);
+        return;
+      }
+    }
+  }
 }
 __device__ __forceinline__ void chain_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -119,94 +150,107 @@ template <int MT, int MAXS>
 __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const __grid_constant__ ChainParams<MAXS> p) {
   constexpr int R = 16 * MT;
   extern __shared__ __align__(128) uint8_t chain_smem[];
-  __shared__ __align__(16) float sw_s[2][kChainThreads], bias_s[2][kChainThreads];
+  __shared__ __align__(16) ChainStep steps[MAXS];
+  __shared__ __align__(16) float sw_s[3][kChainThreads], bias_s[3][kChainThreads];  // a step's slot is read while the one after next's is filled
   __shared__ uint32_t amax_s[R][kChainCtas];  // bit patterns of the row maxima of every CTA's columns
+  __shared__ uint64_t amax_bar[R];            // a row's sixteen maxima have arrived
+  __shared__ uint64_t codes_bar;              // all codes of the next input have arrived
+  __shared__ int abort_flag;
   uint8_t* codes = chain_smem;
-  int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes);
-  float* h = reinterpret_cast<float*>(chain_smem + p.code_bytes + p.part_bytes);  // [R][h_cols]
+  float* h = reinterpret_cast<float*>(chain_smem + p.code_bytes + 2 * p.part_bytes);  // [R][h_cols]
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, kq = lane & 3;
-  const uint32_t rank = cluster_ctarank();
+  const int rank = (int)cluster_ctarank();
   const int row0 = (int)(blockIdx.x / kChainCtas) * R;
   const int rows = min(R, p.M - row0);
+  const int n_steps = p.n_steps, rounding = p.rounding, h_cols = p.h_cols;
+  const uint64_t t_start = global_timer_ns();
 
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int r = 0; r < R; ++r) mbar_init(smem_u32(&amax_bar[r]), 1);
+    mbar_init(smem_u32(&codes_bar), 1);
+    fence_barrier_init();
+  }
+  for (int i = threadIdx.x; i < n_steps * 4; i += kChainThreads)
+    reinterpret_cast<uint4*>(steps)[i] = reinterpret_cast<const uint4*>(p.steps)[i];
+  __syncthreads();
   grid_dependency_wait();
 
-  // ---- weight chunks of this warp in program order: (step, unit, first load of the chunk)
-  int it_step = 0, it_u = warp, it_i = 0;
+  // ---- weight chunks of this warp in program order, each asked for one chunk ahead of its use
+  int it_step = 0, it_u = warp, it_left = 0;
+  const uint8_t* it_src = nullptr;
   uint4 nxt[kChainChunk];
-  auto unit_loads = [&](const ChainStep& st, int u) {  // 16-byte loads per lane of unit u
-    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7, ks = u / tiles;
-    const int blocks = (ks + 1) * k128 / ks_n - ks * k128 / ks_n;
-    return (st.flags & kChainPacked) ? blocks : 2 * blocks;
+  // (tile, first 128 of K, 16-byte loads per lane) of unit u: tiles fastest, then shares of K
+  auto unit_of = [&](const ChainStep& st, int u, int& tile, int& ks, int& kb0) {
+    const int tiles = st.tiles, k128 = st.K >> 7;
+    tile = u;
+    ks = 0;
+    kb0 = 0;
+    int kb1 = k128;
+    if (st.ks_n > 1) {
+      ks = (int)((uint32_t)u * st.inv_tiles >> 16);
+      tile = u - ks * tiles;
+      kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks >> 16);
+      kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks >> 16);
+    }
+    return (kb1 - kb0) << ((st.flags & kChainPacked) ? 0 : 1);
   };
-  auto skip_idle_steps = [&]() {
-    while (it_step < p.n_steps) {
-      const int tiles = chain_tiles(p.steps[it_step].N);
-      if (it_u < tiles * chain_ksplit(tiles, p.steps[it_step].K)) break;
+  auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
+    while (it_step < n_steps && it_u >= steps[it_step].tiles * steps[it_step].ks_n) {
       ++it_step;
       it_u = warp;
     }
-  };
-  auto load_next = [&]() {  // the chunk the iterator stands on -> nxt, then advance
-    if (it_step >= p.n_steps) return;
-    const ChainStep& st = p.steps[it_step];
-    const bool packed = (st.flags & kChainPacked) != 0;
-    const uint32_t act = st.flags & kChainActMask;
-    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7;
-    const int tile = it_u % tiles, ks = it_u / tiles;
-    int n = (int)rank * (st.N / kChainCtas) + tile * 8 + g;
-    if (act >= AQT_ACT_GLU) {  // value tiles, then the gate tiles of the same output columns
-      const int half = tiles >> 1, gate = tile >= half;
-      n = gate * (st.N >> 1) + (int)rank * (st.N / (2 * kChainCtas)) + (tile - gate * half) * 8 + g;
+    if (it_step >= n_steps) return;
+    const ChainStep& st = steps[it_step];
+    int tile, ks, kb0;
+    it_left = unit_of(st, it_u, tile, ks, kb0);
+    const uint32_t packed = (st.flags & kChainPacked) ? 1u : 0u;
+    int n = rank * (st.N >> 4) + tile * 8 + g;
+    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value tiles, then the gate tiles of the same output columns
+      const int half = st.tiles >> 1, gate = tile >= half ? 1 : 0;
+      n = gate * (st.N >> 1) + rank * (st.N >> 5) + (tile - gate * half) * 8 + g;
     }
-    const int64_t row_bytes = packed ? st.K >> 1 : st.K;
-    const uint8_t* src = st.w + n * row_bytes + (int64_t)(ks * k128 / ks_n) * (packed ? 64 : 128) + it_i * 64 + kq * 16;
-    const int left = unit_loads(st, it_u) - it_i;
+    it_src = st.w + (int64_t)n * (st.K >> packed) + (kb0 << (7 - packed)) + kq * 16;
+  };
+  auto load_next = [&]() {
+    if (it_step >= n_steps) return;
 #pragma unroll
     for (int j = 0; j < kChainChunk; ++j)
-      if (j < left) nxt[j] = __ldg(reinterpret_cast<const uint4*>(src + j * 64));
-    it_i += kChainChunk;
-    if (left <= kChainChunk) {
-      it_i = 0;
+      if (j < it_left) nxt[j] = __ldg(reinterpret_cast<const uint4*>(it_src + j * 64));
+    it_src += kChainChunk * 64;
+    it_left -= kChainChunk;
+    if (it_left <= 0) {
       it_u += kChainWarps;
-      skip_idle_steps();
+      open_unit();
     }
   };
   auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
     wv = bv = 0.0f;
-    if (s >= p.n_steps) return;
-    const ChainStep& st = p.steps[s];
-    const int per_cta = st.N / kChainCtas, c = threadIdx.x;
+    if (s >= n_steps) return;
+    const ChainStep& st = steps[s];
+    const int per_cta = st.N >> 4, c = threadIdx.x;
     if (c >= per_cta) return;
-    int n = (int)rank * per_cta + c;
+    int n = rank * per_cta + c;
     if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
-      const int cols = per_cta >> 1, gate = c >= cols;
-      n = gate * (st.N >> 1) + (int)rank * cols + c - gate * cols;
+      const int cols = per_cta >> 1, gate = c >= cols ? 1 : 0;
+      n = gate * (st.N >> 1) + rank * cols + c - gate * cols;
     }
     wv = __ldg(st.s_w + n);
     if (st.bias != nullptr) bv = __ldg(st.bias + n);
   };
-  auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2
-    if (threadIdx.x != 0 || s >= p.n_steps || blockIdx.x >= kChainCtas) return;
-    const ChainStep& st = p.steps[s];
-    const int64_t row_bytes = (st.flags & kChainPacked) ? st.K >> 1 : st.K;
-    const int per_cta = st.N / kChainCtas;
-    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
-      const int cols = per_cta >> 1;
-#pragma unroll 1
-      for (int gate = 0; gate < 2; ++gate)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st.w + (gate * (int64_t)(st.N >> 1) + (int64_t)rank * cols) * row_bytes),
-                     "r"((uint32_t)(cols * row_bytes))
-                     : "memory");
-    } else {
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(st.w + (int64_t)rank * per_cta * row_bytes), "r"((uint32_t)(per_cta * row_bytes))
-                   : "memory");
-    }
+  auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2 (the last thread: it has no row of a single row tile)
+    if (threadIdx.x != kChainThreads - 1 || s >= n_steps || blockIdx.x >= kChainCtas) return;
+    const ChainStep& st = steps[s];
+    const bool glu = (st.flags & kChainActMask) >= AQT_ACT_GLU;
+    const int row_bytes = (st.flags & kChainPacked) ? st.K >> 1 : st.K, rows_here = st.N >> (glu ? 5 : 4);
+    const uint8_t* src = st.w + (int64_t)rank * rows_here * row_bytes;
+    for (int gate = 0; gate <= (glu ? 1 : 0); ++gate, src += (int64_t)(st.N >> 1) * row_bytes)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(rows_here * row_bytes)) : "memory");
   };
 
-  skip_idle_steps();
+  open_unit();
   load_next();
   prefetch_slice(1);
   {
@@ -219,7 +263,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
   float sx[MT];  // input scales of this warp's rows (warp, warp + 16)
   {
-    const int pitch = chain_pitch(p.K0, (p.steps[0].flags & kChainPacked) != 0);
+    const int pitch = chain_pitch(p.K0, (steps[0].flags & kChainPacked) != 0);
 #pragma unroll
     for (int t = 0; t < MT; ++t) {
       const int r = warp + 16 * t;
@@ -239,45 +283,54 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       for (int c = lane; c < p.K0 / 4; c += 32) {
         const float4 f = __ldg(xr + c);
         const float v[4] = {f.x, f.y, f.z, f.w};
-        *reinterpret_cast<uint32_t*>(codes + r * pitch + 4 * c) = chain_codes4(v, sc, p.in_qmax, p.rounding);
+        *reinterpret_cast<uint32_t*>(codes + r * pitch + 4 * c) = chain_codes4(v, sc, p.in_qmax, rounding);
       }
-      for (int c = lane; c < p.h_cols / 4; c += 32)
-        *reinterpret_cast<float4*>(h + r * p.h_cols + 4 * c) = __ldg(xr + (int)rank * (p.h_cols / 4) + c);
+      for (int c = lane; c < h_cols / 4; c += 32)
+        *reinterpret_cast<float4*>(h + r * h_cols + 4 * c) = __ldg(xr + rank * (h_cols / 4) + c);
     }
   }
-  chain_cluster_sync();  // codes ready; every CTA of the cluster runs (its shared memory may be written)
+  chain_cluster_sync();  // own codes ready; every CTA's barriers exist
 
-  for (int s = 0; s < p.n_steps; ++s) {
-    const ChainStep& st = p.steps[s];
+  uint32_t exchange_parity = 0;  // of the exchange in progress (steps that are no side steps)
+  bool fresh = false;            // the codes of this step's input come from the exchange before it
+  int slot = 0;                  // of sw_s / bias_s
+  for (int s = 0; s < n_steps; ++s) {
+    const ChainStep st = steps[s];
     const bool packed = (st.flags & kChainPacked) != 0;
     const uint32_t act = st.flags & kChainActMask;
-    const int per_cta = st.N / kChainCtas;
-    const int tiles = chain_tiles(st.N), ks_n = chain_ksplit(tiles, st.K), k128 = st.K >> 7;
+    const bool glu = act >= AQT_ACT_GLU;
+    const int per_cta = st.N >> 4, units = st.tiles * st.ks_n, ks_n = st.ks_n;
+    const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
+    const int n_out = glu ? st.N >> 1 : st.N;
     const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 8;
+    const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
+    // two buffers of partial sums: after a side step the next products are written while these are read
+    int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
     prefetch_slice(s + 2);
     float wv, bv;
     load_scales(s + 1, wv, bv);
+    const int next_slot = slot == 2 ? 0 : slot + 1;
+    if (fresh) chain_wait(smem_u32(&codes_bar), exchange_parity ^ 1u, &abort_flag, t_start);
 
     // ---- integer products of this warp's units (tile, share of K)
-    for (int u = warp; u < tiles * ks_n; u += kChainWarps) {
-      const int tile = u % tiles, ks = u / tiles;
-      const int n_loads = unit_loads(st, u);
+    for (int u = warp; u < units; u += kChainWarps) {
+      int tile, ks, kb0;
+      const int n_loads = unit_of(st, u, tile, ks, kb0);
       int acc[MT][2][4];
 #pragma unroll
       for (int t = 0; t < MT; ++t)
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[t][j >> 2][j & 3] = 0;
-      const uint8_t* a_row = codes + g * pitch + (ks * k128 / ks_n) * 128 + kq * (packed ? 32 : 16);
-      for (int i0 = 0; i0 < n_loads; i0 += kChainChunk) {
+      const uint8_t* a0 = codes + g * pitch + kb0 * 128 + kq * (packed ? 32 : 16);
+      for (int left = n_loads; left > 0; left -= kChainChunk) {
         uint4 cur[kChainChunk];
 #pragma unroll
         for (int j = 0; j < kChainChunk; ++j) cur[j] = nxt[j];
         load_next();
-        const uint8_t* a0 = a_row + i0 * (packed ? 128 : 64);
         if (packed) {
 #pragma unroll
           for (int j = 0; j < kChainChunk; ++j) {
-            if (i0 + j >= n_loads) break;
+            if (j >= left) break;
             uint32_t b[8];
             unpack_word(cur[j].x, b[0], b[1]);
             unpack_word(cur[j].y, b[2], b[3]);
@@ -298,10 +351,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
               mma_s8_16x8x32(acc[t][1], l1.z, h1.z, l1.w, h1.w, b[6], b[7]);
             }
           }
+          a0 += kChainChunk * 128;
         } else {
 #pragma unroll
           for (int j = 0; j < kChainChunk; ++j) {
-            if (i0 + j >= n_loads) break;
+            if (j >= left) break;
 #pragma unroll
             for (int t = 0; t < MT; ++t) {
               const uint8_t* a = a0 + t * 16 * pitch + j * 64;
@@ -312,6 +366,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
               mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, cur[j].z, cur[j].w);
             }
           }
+          a0 += kChainChunk * 64;
         }
       }
 #pragma unroll
@@ -321,34 +376,35 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         *reinterpret_cast<int2*>(dst + 8 * part_pitch) = make_int2(acc[t][0][2] + acc[t][1][2], acc[t][0][3] + acc[t][1][3]);
       }
     }
-    sw_s[(s + 1) & 1][threadIdx.x] = wv;
-    bias_s[(s + 1) & 1][threadIdx.x] = bv;
+    sw_s[next_slot][threadIdx.x] = wv;
+    bias_s[next_slot][threadIdx.x] = bv;
     __syncthreads();
+    if (*(volatile int*)&abort_flag) break;  // a wait gave up: every thread leaves here
 
     // ---- epilogue: warp w owns rows w and w + 16, a lane four consecutive columns at a time
-    const bool glu = act >= AQT_ACT_GLU;
-    const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
-    const bool side = (st.flags & kChainSide) != 0, last = s + 1 == p.n_steps;
     float v[MT][2][4];
-    float amax[MT];
+    if (threadIdx.x == 0 && !side && !last) mbar_arrive_expect_tx(smem_u32(&codes_bar), (uint32_t)(rows * n_out));
 #pragma unroll
     for (int t = 0; t < MT; ++t) {
-      amax[t] = 0.0f;
+      float amax = 0.0f;
       const int r = warp + 16 * t;
+      if (r >= rows) continue;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int c = 4 * lane + 128 * j;
 #pragma unroll
         for (int e = 0; e < 4; ++e) v[t][j][e] = 0.0f;
-        if (r >= rows || c >= cols) continue;
+        if (c >= cols) continue;
         auto dequant = [&](int cc, float (&z)[4]) {
-          int4 a = make_int4(0, 0, 0, 0);
-          for (int ks = 0; ks < ks_n; ++ks) {
-            const int4 q = *reinterpret_cast<const int4*>(part + (ks * R + r) * part_pitch + cc);
+          const int* src = part + r * part_pitch + cc;
+          int4 a = *reinterpret_cast<const int4*>(src);
+          for (int ks = 1; ks < ks_n; ++ks) {
+            src += R * part_pitch;
+            const int4 q = *reinterpret_cast<const int4*>(src);
             a.x += q.x; a.y += q.y; a.z += q.z; a.w += q.w;
           }
-          const float4 w4 = *reinterpret_cast<const float4*>(&sw_s[s & 1][cc]);
-          const float4 b4 = *reinterpret_cast<const float4*>(&bias_s[s & 1][cc]);
+          const float4 w4 = *reinterpret_cast<const float4*>(&sw_s[slot][cc]);
+          const float4 b4 = *reinterpret_cast<const float4*>(&bias_s[slot][cc]);
           z[0] = __fmaf_rn(__fmul_rn(__int2float_rn(a.x), sx[t]), w4.x, b4.x);
           z[1] = __fmaf_rn(__fmul_rn(__int2float_rn(a.y), sx[t]), w4.y, b4.y);
           z[2] = __fmaf_rn(__fmul_rn(__int2float_rn(a.z), sx[t]), w4.z, b4.z);
@@ -367,7 +423,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
           for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(o[e]));
         }
         if (st.flags & kChainAdd) {
-          float4* hr = reinterpret_cast<float4*>(h + r * p.h_cols + c);
+          float4* hr = reinterpret_cast<float4*>(h + r * h_cols + c);
           const float4 r4 = *hr;
           o[0] = __fmaf_rn(st.rs, o[0], r4.x);
           o[1] = __fmaf_rn(st.rs, o[1], r4.y);
@@ -376,48 +432,46 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
           *hr = make_float4(o[0], o[1], o[2], o[3]);
         }
         if (st.y != nullptr)
-          *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + (int)rank * cols + c) = make_float4(o[0], o[1], o[2], o[3]);
-        amax[t] = chain_max4(amax[t], o);
+          *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + rank * cols + c) = make_float4(o[0], o[1], o[2], o[3]);
+        amax = chain_max4(amax, o);
       }
+      if (side || last) continue;
+      const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative floats order like their bit patterns
+      const uint32_t bar = smem_u32(&amax_bar[r]);
+      if (lane == 0) mbar_arrive_expect_tx(bar, kChainCtas * 4);
+      if (lane < kChainCtas) chain_st_async(chain_mapa(smem_u32(&amax_s[r][rank]), lane), m, chain_mapa(bar, lane));
     }
+    slot = next_slot;
     if (last) break;
-    if (side) {
-      __syncthreads();  // the partial sums have been read
-      continue;
-    }
+    fresh = !side;
+    if (side) continue;
 
-    // ---- quantize the output rows for the next step
-#pragma unroll
-    for (int t = 0; t < MT; ++t) {
-      const int r = warp + 16 * t;
-      if (r >= rows) continue;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) amax[t] = fmaxf(amax[t], __shfl_xor_sync(0xffffffffu, amax[t], off));
-      if (lane < kChainCtas) chain_st_cluster(chain_mapa(chain_smem_u32(&amax_s[r][rank]), lane), __float_as_uint(amax[t]));
-    }
-    chain_cluster_sync();  // all maxima have arrived; nobody reads the old codes any more
-    const int n_out = glu ? st.N >> 1 : st.N;
+    // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
+    // CTA has finished its products, so nobody reads the old codes any more.
     const int qmax = (st.flags & kChainOut4) ? 7 : 127;
-    const int out_pitch = chain_pitch(n_out, (p.steps[s + 1].flags & kChainPacked) != 0);
+    const int out_pitch = chain_pitch(n_out, (steps[s + 1].flags & kChainPacked) != 0);
 #pragma unroll
     for (int t = 0; t < MT; ++t) {
       const int r = warp + 16 * t;
       if (r >= rows) continue;
-      uint32_t m = lane < kChainCtas ? amax_s[r][lane] : 0u;
-      m = __reduce_max_sync(0xffffffffu, m);
+      chain_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
+      const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
       const ScaleCtx sc = make_scale_ctx(__uint_as_float(m), qmax);
       sx[t] = sc.s;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         const int c = 4 * lane + 128 * j;
         if (c >= cols) continue;
-        const uint32_t word = chain_codes4(v[t][j], sc, qmax, p.rounding);
-        const uint32_t dst = chain_smem_u32(codes + r * out_pitch + (int)rank * cols + c);
+        const uint32_t word = chain_codes4(v[t][j], sc, qmax, rounding);
+        const uint32_t dst = smem_u32(codes + r * out_pitch + rank * cols + c), bar = smem_u32(&codes_bar);
 #pragma unroll
-        for (uint32_t k = 0; k < (uint32_t)kChainCtas; ++k) chain_st_cluster(chain_mapa(dst, (rank + k) & (kChainCtas - 1)), word);
+        for (int k = 0; k < kChainCtas; ++k) {
+          const uint32_t to = (uint32_t)(rank + k) & (kChainCtas - 1);
+          chain_st_async(chain_mapa(dst, to), word, chain_mapa(bar, to));
+        }
       }
     }
-    chain_cluster_sync();  // the next step's codes are complete
+    exchange_parity ^= 1u;
   }
   grid_dependents_launch();
   chain_cluster_sync();  // no CTA leaves while its shared memory may still be written
@@ -434,9 +488,16 @@ static bool chain_step_ok(const ChainStep& st) {
   return st.N <= kChainMaxN && n_out <= kChainMaxCols * kChainCtas && st.K <= 8192;
 }
 
+static void chain_derive(ChainStep& st) {
+  st.tiles = (uint16_t)chain_tiles(st.N);
+  st.ks_n = (uint16_t)chain_ksplit(st.tiles, st.K);
+  st.inv_tiles = (65536u + st.tiles - 1) / st.tiles;  // exact: dividends < 16 * 64, divisors <= 16
+  st.inv_ks = (65536u + st.ks_n - 1) / st.ks_n;
+}
+
 struct ChainSizes {
   int code_bytes, part_bytes, h_bytes;
-  int smem(void) const { return code_bytes + part_bytes + h_bytes; }
+  int smem(void) const { return code_bytes + 2 * part_bytes + h_bytes; }
 };
 static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
   int code = 0, part = 0, h = 0;
@@ -455,7 +516,7 @@ static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
   return z;
 }
 
-constexpr int kChainMaxSmem = 200 * 1024;
+constexpr int kChainMaxSmem = 180 * 1024;  // beside the step table and the exchange words
 
 // 16-row clusters that run at the same time (the part schedules seven or eight of sixteen CTAs each).
 constexpr int kChainClusters = 7;
@@ -478,6 +539,7 @@ static int launch_chain_inst(const ChainParams<kChainMaxSteps>& full, int smem, 
 static int launch_chain(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
   if (p.M <= 0 || p.n_steps <= 0 || p.n_steps > kChainMaxSteps) return AQT_ERR_UNSUPPORTED;
   // sixteen rows per cluster while the clusters fit the part side by side, then 32
+  for (int i = 0; i < p.n_steps; ++i) chain_derive(p.steps[i]);
   int mt = p.M <= 16 * kChainClusters ? 1 : 2;
   ChainSizes z = chain_sizes(p.steps, p.n_steps, 16 * mt);
   if (mt == 2 && z.smem() > kChainMaxSmem) {
