@@ -21,8 +21,12 @@
 // cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
 // scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
 // wait of the library.
-// What a layer then costs is a chain of latencies, so the loops hold no integer division and no
-// dependent parameter load: the step table sits in shared memory with everything derived from the sizes.
+// What a layer then costs is a chain of latencies and of instructions that every warp issues once: no
+// integer division and no dependent parameter load in the loops (the step table sits in shared memory
+// with everything derived from the sizes), the next layer's weights, scales and prefetches are asked
+// for while the row maxima are under way, and packed weights are used as sixteen times their codes
+// (a nibble in the upper half of a byte; the sums are shifted back, exact), two instructions per four
+// codes instead of eleven per eight, against activation codes stored in the same even / odd order.
 // The arithmetic is that of the per-layer kernels operation by operation (exact int32 sums, the same
 // de-quantization, activation and quantizer), so the results are the same bits.
 #pragma once
@@ -52,7 +56,8 @@ struct ChainStep {
   uint32_t flags;
   // derived by the host (chain_derive)
   uint16_t tiles, ks_n;          // n8-tiles per CTA (value and gate tiles for GLU), shares of K
-  uint32_t inv_tiles, inv_ks;    // ceil(65536 / .): quotients of the small numbers below by a multiply and a shift
+  uint32_t inv_tiles;            // ceil(65536 / tiles), ceil(65536 / ks_n): quotients of small numbers by a multiply and a shift
+  uint16_t inv_ks_lo, units;     // (ks_n == 1 is not divided by)
 };
 static_assert(sizeof(ChainStep) == 64, "copied to shared memory as 16-byte words");
 enum : uint32_t {
@@ -101,31 +106,21 @@ __device__ __forceinline__ uint32_t chain_mapa(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void chain_st_async(uint32_t addr, uint32_t v, uint32_t bar) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
 }
-// mbar_wait with cluster-scope acquire (the data come from other CTAs).
-__device__ __forceinline__ void chain_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint64_t t_start) {
-  for (uint32_t spin = 1;; ++spin) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity), "r"(kTryWaitSuspendNs)
-        : "memory");
-    if (done) return;
-    if ((spin & 0x3) == 0) {
-      if (*abort_flag) return;
-      if (global_timer_ns() - t_start > kWaitLimitNs) {
-        *abort_flag = 1;
-        atomicExch(&g_device_status, AQT_ERR_TIMEOUT);
-        return;
-      }
-    }
-  }
+__device__ __forceinline__ void chain_st_async_v2(uint32_t addr, uint32_t v0, uint32_t v1, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v0), "r"(v1), "r"(bar)
+               : "memory");
 }
 __device__ __forceinline__ void chain_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Eight consecutive codes (two words) in the order the consumer's weights have them: as they are for
+// int8 weights, the even ones and then the odd ones for packed weights.
+__device__ __forceinline__ void chain_order8(bool packed, uint32_t& w0, uint32_t& w1) {
+  const uint32_t even = __byte_perm(w0, w1, 0x6420), odd = __byte_perm(w0, w1, 0x7531);
+  w0 = packed ? even : w0;
+  w1 = packed ? odd : w1;
 }
 
 // Four codes of a row as one word.
@@ -151,7 +146,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   constexpr int R = 16 * MT;
   extern __shared__ __align__(128) uint8_t chain_smem[];
   __shared__ __align__(16) ChainStep steps[MAXS];
-  __shared__ __align__(16) float sw_s[3][kChainThreads], bias_s[3][kChainThreads];  // a step's slot is read while the one after next's is filled
+  __shared__ __align__(16) float sw_s[2][kChainThreads], bias_s[2][kChainThreads];
   __shared__ uint32_t amax_s[R][kChainCtas];  // bit patterns of the row maxima of every CTA's columns
   __shared__ uint64_t amax_bar[R];            // a row's sixteen maxima have arrived
   __shared__ uint64_t codes_bar;              // all codes of the next input have arrived
@@ -178,60 +173,52 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   __syncthreads();
   grid_dependency_wait();
 
-  // ---- weight chunks of this warp in program order, each asked for one chunk ahead of its use
-  int it_step = 0, it_u = warp, it_left = 0;
-  const uint8_t* it_src = nullptr;
+  // ---- This warp's products in program order: units (an n8-tile and a share of K), each in items of up to
+  // kChainChunk 16-byte loads per lane.  The next item's loads are in nxt (zeros beyond its end).
+  int it_step = 0, it_u = warp;  // unit of the item
+  int u_left = 0;                // loads from the item to the end of the unit
+  int u_a = 0, u_part = 0;       // this lane's first activation code (byte offset), first partial sum (index)
+  bool u_first = true;
+  const uint8_t* u_src = nullptr;
   uint4 nxt[kChainChunk];
-  // (tile, first 128 of K, 16-byte loads per lane) of unit u: tiles fastest, then shares of K
-  auto unit_of = [&](const ChainStep& st, int u, int& tile, int& ks, int& kb0) {
-    const int tiles = st.tiles, k128 = st.K >> 7;
-    tile = u;
-    ks = 0;
-    kb0 = 0;
-    int kb1 = k128;
-    if (st.ks_n > 1) {
-      ks = (int)((uint32_t)u * st.inv_tiles >> 16);
-      tile = u - ks * tiles;
-      kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks >> 16);
-      kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks >> 16);
-    }
-    return (kb1 - kb0) << ((st.flags & kChainPacked) ? 0 : 1);
-  };
   auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
-    while (it_step < n_steps && it_u >= steps[it_step].tiles * steps[it_step].ks_n) {
+    while (it_step < n_steps && it_u >= steps[it_step].units) {
       ++it_step;
       it_u = warp;
     }
+    u_left = 0;
     if (it_step >= n_steps) return;
     const ChainStep& st = steps[it_step];
-    int tile, ks, kb0;
-    it_left = unit_of(st, it_u, tile, ks, kb0);
-    const uint32_t packed = (st.flags & kChainPacked) ? 1u : 0u;
+    const int k128 = st.K >> 7;
+    const bool packed = (st.flags & kChainPacked) != 0;
+    int tile = it_u, kb0 = 0, kb1 = k128, ks = 0;  // tiles fastest, then shares of K
+    if (st.ks_n > 1) {
+      ks = (int)((uint32_t)it_u * st.inv_tiles >> 16);
+      tile = it_u - ks * st.tiles;
+      kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks_lo >> 16);
+      kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks_lo >> 16);
+    }
     int n = rank * (st.N >> 4) + tile * 8 + g;
     if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value tiles, then the gate tiles of the same output columns
       const int half = st.tiles >> 1, gate = tile >= half ? 1 : 0;
       n = gate * (st.N >> 1) + rank * (st.N >> 5) + (tile - gate * half) * 8 + g;
     }
-    it_src = st.w + (int64_t)n * (st.K >> packed) + (kb0 << (7 - packed)) + kq * 16;
+    const int shift = packed ? 1 : 0;
+    u_left = (kb1 - kb0) << (1 - shift);
+    u_src = st.w + (int64_t)n * (st.K >> shift) + (kb0 << (7 - shift)) + kq * 16;
+    u_a = g * chain_pitch(st.K, packed) + kb0 * 128 + kq * (16 << shift);
+    u_part = (ks * R + g) * ((st.N >> 4) + 8) + tile * 8 + 2 * kq;
+    u_first = true;
   };
-  auto load_next = [&]() {
-    if (it_step >= n_steps) return;
-#pragma unroll
-    for (int j = 0; j < kChainChunk; ++j)
-      if (j < it_left) nxt[j] = __ldg(reinterpret_cast<const uint4*>(it_src + j * 64));
-    it_src += kChainChunk * 64;
-    it_left -= kChainChunk;
-    if (it_left <= 0) {
-      it_u += kChainWarps;
-      open_unit();
-    }
+  auto load_item = [&](int j) {
+    nxt[j] = j < u_left ? __ldg(reinterpret_cast<const uint4*>(u_src + j * 64)) : make_uint4(0u, 0u, 0u, 0u);
   };
   auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
     wv = bv = 0.0f;
     if (s >= n_steps) return;
     const ChainStep& st = steps[s];
     const int per_cta = st.N >> 4, c = threadIdx.x;
-    if (c >= per_cta) return;
+    if (c - lane >= per_cta || c >= per_cta) return;
     int n = rank * per_cta + c;
     if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
       const int cols = per_cta >> 1, gate = c >= cols ? 1 : 0;
@@ -251,14 +238,11 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   };
 
   open_unit();
-  load_next();
+#pragma unroll
+  for (int j = 0; j < kChainChunk; ++j) load_item(j);
   prefetch_slice(1);
-  {
-    float wv, bv;
-    load_scales(0, wv, bv);
-    sw_s[0][threadIdx.x] = wv;
-    bias_s[0][threadIdx.x] = bv;
-  }
+  float wv, bv;  // scale and bias of this thread's channel of the next step, on their way to sw_s / bias_s
+  load_scales(0, wv, bv);
 
   // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
   float sx[MT];  // input scales of this warp's rows (warp, warp + 16)
@@ -280,10 +264,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
       const ScaleCtx sc = make_scale_ctx(amax, p.in_qmax);
       sx[t] = sc.s;
-      for (int c = lane; c < p.K0 / 4; c += 32) {
-        const float4 f = __ldg(xr + c);
-        const float v[4] = {f.x, f.y, f.z, f.w};
-        *reinterpret_cast<uint32_t*>(codes + r * pitch + 4 * c) = chain_codes4(v, sc, p.in_qmax, rounding);
+      for (int c = lane; c < p.K0 / 8; c += 32) {
+        const float4 f0 = __ldg(xr + 2 * c), f1 = __ldg(xr + 2 * c + 1);
+        const float v0[4] = {f0.x, f0.y, f0.z, f0.w}, v1[4] = {f1.x, f1.y, f1.z, f1.w};
+        uint32_t w0 = chain_codes4(v0, sc, p.in_qmax, rounding), w1 = chain_codes4(v1, sc, p.in_qmax, rounding);
+        chain_order8((steps[0].flags & kChainPacked) != 0, w0, w1);
+        *reinterpret_cast<uint2*>(codes + r * pitch + 8 * c) = make_uint2(w0, w1);
       }
       for (int c = lane; c < h_cols / 4; c += 32)
         *reinterpret_cast<float4*>(h + r * h_cols + 4 * c) = __ldg(xr + rank * (h_cols / 4) + c);
@@ -291,93 +277,106 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   }
   chain_cluster_sync();  // own codes ready; every CTA's barriers exist
 
+  // lane l sends its warp's row maxima to CTA l of the cluster
+  const uint32_t to_amax = chain_mapa(smem_u32(&amax_s[0][rank]), lane & 15), to_amax_bar = chain_mapa(smem_u32(&amax_bar[0]), lane & 15);
   uint32_t exchange_parity = 0;  // of the exchange in progress (steps that are no side steps)
   bool fresh = false;            // the codes of this step's input come from the exchange before it
-  int slot = 0;                  // of sw_s / bias_s
   for (int s = 0; s < n_steps; ++s) {
     const ChainStep st = steps[s];
     const bool packed = (st.flags & kChainPacked) != 0;
     const uint32_t act = st.flags & kChainActMask;
     const bool glu = act >= AQT_ACT_GLU;
-    const int per_cta = st.N >> 4, units = st.tiles * st.ks_n, ks_n = st.ks_n;
+    const int per_cta = st.N >> 4, units = st.units, ks_n = st.ks_n;
     const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
     const int n_out = glu ? st.N >> 1 : st.N;
     const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 8;
     const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
     // two buffers of partial sums: after a side step the next products are written while these are read
     int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
-    prefetch_slice(s + 2);
-    float wv, bv;
-    load_scales(s + 1, wv, bv);
-    const int next_slot = slot == 2 ? 0 : slot + 1;
-    if (fresh) chain_wait(smem_u32(&codes_bar), exchange_parity ^ 1u, &abort_flag, t_start);
+    const int slot = s & 1;  // of sw_s / bias_s
+    if (fresh) mbar_wait(smem_u32(&codes_bar), exchange_parity ^ 1u, &abort_flag, t_start);
 
-    // ---- integer products of this warp's units (tile, share of K)
-    for (int u = warp; u < units; u += kChainWarps) {
-      int tile, ks, kb0;
-      const int n_loads = unit_of(st, u, tile, ks, kb0);
-      int acc[MT][2][4];
+    // ---- integer products
+    bool used = false;
+    int acc[MT][2][4];
+    while (it_step == s) {
+      const int n = u_left, part0 = u_part;
+      const uint8_t* a0 = codes + u_a;
+      if (u_first) {
 #pragma unroll
-      for (int t = 0; t < MT; ++t)
+        for (int t = 0; t < MT; ++t)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[t][j >> 2][j & 3] = 0;
-      const uint8_t* a0 = codes + g * pitch + kb0 * 128 + kq * (packed ? 32 : 16);
-      for (int left = n_loads; left > 0; left -= kChainChunk) {
-        uint4 cur[kChainChunk];
+          for (int j = 0; j < 8; ++j) acc[t][j >> 2][j & 3] = 0;
+      }
+      // the next item: loaded slot by slot below if it belongs to this step, else while the maxima are under way
+      bool more = true;
+      if (n > kChainChunk) {
+        u_left -= kChainChunk;
+        u_src += kChainChunk * 64;
+        u_a += kChainChunk * (packed ? 128 : 64);
+        u_first = false;
+      } else {
+        it_u += kChainWarps;
+        more = it_u < units;
+        if (more) open_unit();
+        else used = true;
+      }
 #pragma unroll
-        for (int j = 0; j < kChainChunk; ++j) cur[j] = nxt[j];
-        load_next();
-        if (packed) {
+      for (int jj = 0; jj < kChainChunk; jj += 2) {
+        if (jj < n) {
 #pragma unroll
-          for (int j = 0; j < kChainChunk; ++j) {
-            if (j >= left) break;
-            uint32_t b[8];
-            unpack_word(cur[j].x, b[0], b[1]);
-            unpack_word(cur[j].y, b[2], b[3]);
-            unpack_word(cur[j].z, b[4], b[5]);
-            unpack_word(cur[j].w, b[6], b[7]);
+          for (int j = jj; j < jj + 2; ++j) {
+            const uint4 w = nxt[j];
+            if (packed) {
+              // sixteen times the codes: the even ones' nibbles moved up, the odd ones' in place
+              const uint32_t b[8] = {(w.x << 4) & 0xF0F0F0F0u, w.x & 0xF0F0F0F0u, (w.y << 4) & 0xF0F0F0F0u, w.y & 0xF0F0F0F0u,
+                                     (w.z << 4) & 0xF0F0F0F0u, w.z & 0xF0F0F0F0u, (w.w << 4) & 0xF0F0F0F0u, w.w & 0xF0F0F0F0u};
 #pragma unroll
-            for (int t = 0; t < MT; ++t) {
-              const uint8_t* a = a0 + t * 16 * pitch + j * 128;
-              const uint4 l0 = *reinterpret_cast<const uint4*>(a), l1 = *reinterpret_cast<const uint4*>(a + 16);
-              uint4 h0 = make_uint4(0u, 0u, 0u, 0u), h1 = h0;
-              if (rows > 8 + 16 * t) {
-                h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
-                h1 = *reinterpret_cast<const uint4*>(a + 8 * pitch + 16);
+              for (int t = 0; t < MT; ++t) {
+                const uint8_t* a = a0 + t * 16 * pitch + j * 128;
+                const uint4 l0 = *reinterpret_cast<const uint4*>(a), l1 = *reinterpret_cast<const uint4*>(a + 16);
+                uint4 h0 = make_uint4(0u, 0u, 0u, 0u), h1 = h0;
+                if (rows > 8 + 16 * t) {
+                  h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
+                  h1 = *reinterpret_cast<const uint4*>(a + 8 * pitch + 16);
+                }
+                mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, b[0], b[1]);
+                mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, b[2], b[3]);
+                mma_s8_16x8x32(acc[t][0], l1.x, h1.x, l1.y, h1.y, b[4], b[5]);
+                mma_s8_16x8x32(acc[t][1], l1.z, h1.z, l1.w, h1.w, b[6], b[7]);
               }
-              mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, b[0], b[1]);
-              mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, b[2], b[3]);
-              mma_s8_16x8x32(acc[t][0], l1.x, h1.x, l1.y, h1.y, b[4], b[5]);
-              mma_s8_16x8x32(acc[t][1], l1.z, h1.z, l1.w, h1.w, b[6], b[7]);
+            } else {
+#pragma unroll
+              for (int t = 0; t < MT; ++t) {
+                const uint8_t* a = a0 + t * 16 * pitch + j * 64;
+                const uint4 l0 = *reinterpret_cast<const uint4*>(a);
+                uint4 h0 = make_uint4(0u, 0u, 0u, 0u);
+                if (rows > 8 + 16 * t) h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
+                mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, w.x, w.y);
+                mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, w.z, w.w);
+              }
             }
           }
-          a0 += kChainChunk * 128;
-        } else {
-#pragma unroll
-          for (int j = 0; j < kChainChunk; ++j) {
-            if (j >= left) break;
-#pragma unroll
-            for (int t = 0; t < MT; ++t) {
-              const uint8_t* a = a0 + t * 16 * pitch + j * 64;
-              const uint4 l0 = *reinterpret_cast<const uint4*>(a);
-              uint4 h0 = make_uint4(0u, 0u, 0u, 0u);
-              if (rows > 8 + 16 * t) h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
-              mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, cur[j].x, cur[j].y);
-              mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, cur[j].z, cur[j].w);
-            }
-          }
-          a0 += kChainChunk * 64;
+        }
+        if (more) {
+          load_item(jj);
+          load_item(jj + 1);
         }
       }
+      if (n <= kChainChunk) {  // the unit's last item
+        const int shift = packed ? 4 : 0;
 #pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        int* dst = part + (ks * R + 16 * t + g) * part_pitch + tile * 8 + 2 * kq;
-        *reinterpret_cast<int2*>(dst) = make_int2(acc[t][0][0] + acc[t][1][0], acc[t][0][1] + acc[t][1][1]);
-        *reinterpret_cast<int2*>(dst + 8 * part_pitch) = make_int2(acc[t][0][2] + acc[t][1][2], acc[t][0][3] + acc[t][1][3]);
+        for (int t = 0; t < MT; ++t) {
+          int* dst = part + part0 + 16 * t * part_pitch;
+          *reinterpret_cast<int2*>(dst) = make_int2((acc[t][0][0] + acc[t][1][0]) >> shift, (acc[t][0][1] + acc[t][1][1]) >> shift);
+          *reinterpret_cast<int2*>(dst + 8 * part_pitch) =
+              make_int2((acc[t][0][2] + acc[t][1][2]) >> shift, (acc[t][0][3] + acc[t][1][3]) >> shift);
+        }
       }
+      if (!more) break;
     }
-    sw_s[next_slot][threadIdx.x] = wv;
-    bias_s[next_slot][threadIdx.x] = bv;
+    sw_s[slot][threadIdx.x] = wv;
+    bias_s[slot][threadIdx.x] = bv;
     __syncthreads();
     if (*(volatile int*)&abort_flag) break;  // a wait gave up: every thread leaves here
 
@@ -437,38 +436,61 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       }
       if (side || last) continue;
       const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative floats order like their bit patterns
-      const uint32_t bar = smem_u32(&amax_bar[r]);
-      if (lane == 0) mbar_arrive_expect_tx(bar, kChainCtas * 4);
-      if (lane < kChainCtas) chain_st_async(chain_mapa(smem_u32(&amax_s[r][rank]), lane), m, chain_mapa(bar, lane));
+      if (lane == 0) mbar_arrive_expect_tx(smem_u32(&amax_bar[r]), kChainCtas * 4);
+      if (lane < kChainCtas) chain_st_async(to_amax + r * (kChainCtas * 4), m, to_amax_bar + r * 8);
     }
-    slot = next_slot;
     if (last) break;
+
+    // ---- what the next step needs from memory, asked for while the maxima are under way
+    if (used) {
+      open_unit();
+#pragma unroll
+      for (int j = 0; j < kChainChunk; ++j) load_item(j);
+    }
+    load_scales(s + 1, wv, bv);
+    prefetch_slice(s + 2);
     fresh = !side;
     if (side) continue;
 
     // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
     // CTA has finished its products, so nobody reads the old codes any more.
     const int qmax = (st.flags & kChainOut4) ? 7 : 127;
-    const int out_pitch = chain_pitch(n_out, (steps[s + 1].flags & kChainPacked) != 0);
+    const bool next_packed = (steps[s + 1].flags & kChainPacked) != 0;
+    const int out_pitch = chain_pitch(n_out, next_packed);
 #pragma unroll
     for (int t = 0; t < MT; ++t) {
       const int r = warp + 16 * t;
       if (r >= rows) continue;
-      chain_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
+      mbar_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
       const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
       const ScaleCtx sc = make_scale_ctx(__uint_as_float(m), qmax);
       sx[t] = sc.s;
+      uint32_t word[2] = {0u, 0u};
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const int c = 4 * lane + 128 * j;
-        if (c >= cols) continue;
-        const uint32_t word = chain_codes4(v[t][j], sc, qmax, rounding);
-        const uint32_t dst = smem_u32(codes + r * out_pitch + rank * cols + c), bar = smem_u32(&codes_bar);
-#pragma unroll
-        for (int k = 0; k < kChainCtas; ++k) {
-          const uint32_t to = (uint32_t)(rank + k) & (kChainCtas - 1);
-          chain_st_async(chain_mapa(dst, to), word, chain_mapa(bar, to));
-        }
+        if (4 * lane + 128 * j >= cols) continue;
+        word[j] = chain_codes4(v[t][j], sc, qmax, rounding);
+      }
+      // to all sixteen CTAs, eight codes per lane and store: `span` lanes (a power of two) cover the row's share,
+      // so a store instruction is 32 / span runs of consecutive bytes (the interconnect is paid per run: 250 clocks
+      // for a store scattered over sixteen CTAs)
+      const int span_bits = cols <= 16 ? 1 : 32 - __clz((cols >> 3) - 1), span = 1 << span_bits, i = lane & (span - 1);
+      uint32_t w0, w1;
+      if (cols <= 128) {
+        w0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31);
+        w1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
+      } else {  // columns from 128 on sit in the lanes' second word
+        const uint32_t x0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31), x1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
+        const uint32_t y0 = __shfl_sync(0xffffffffu, word[1], (2 * i) & 31), y1 = __shfl_sync(0xffffffffu, word[1], (2 * i + 1) & 31);
+        w0 = i < 16 ? x0 : y0;
+        w1 = i < 16 ? x1 : y1;
+      }
+      chain_order8(next_packed, w0, w1);
+      const uint32_t dst = smem_u32(codes) + (uint32_t)(r * out_pitch + rank * cols + 8 * i);
+      const uint32_t bar_off = smem_u32(&codes_bar) - dst;  // the same distance in every CTA's window
+      for (int to = lane >> span_bits; to < kChainCtas; to += 32 >> span_bits) {
+        const uint32_t remote = chain_mapa(dst, (uint32_t)(rank + to) & (kChainCtas - 1));
+        if (8 * i < cols) chain_st_async_v2(remote, w0, w1, remote + bar_off);
       }
     }
     exchange_parity ^= 1u;
@@ -492,7 +514,8 @@ static void chain_derive(ChainStep& st) {
   st.tiles = (uint16_t)chain_tiles(st.N);
   st.ks_n = (uint16_t)chain_ksplit(st.tiles, st.K);
   st.inv_tiles = (65536u + st.tiles - 1) / st.tiles;  // exact: dividends < 16 * 64, divisors <= 16
-  st.inv_ks = (65536u + st.ks_n - 1) / st.ks_n;
+  st.inv_ks_lo = (uint16_t)((65536u + st.ks_n - 1) / st.ks_n);
+  st.units = (uint16_t)(st.tiles * st.ks_n);
 }
 
 struct ChainSizes {
