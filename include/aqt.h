@@ -265,7 +265,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
  * M         any, but the call is meant for at most AQT_CHAIN_MAX_ROWS rows: from there on layer by
  *           layer is faster.
  * Limits (AQT_ERR_UNSUPPORTED otherwise, nothing enqueued): at most AQT_CHAIN_MAX_LAYERS layers; N and
- * N_out multiples of 128, N <= 8192, N_out <= 4096; K a multiple of 128, K <= 8192; layers that read the
+ * N_out multiples of 128, N <= 4096; K a multiple of 128, K <= 8192; layers that read the
  * same input agree in bits_a and in whether their weights are packed; layers with AQT_CHAIN_ADD have
  * N_out equal to layers[0].K.
  */

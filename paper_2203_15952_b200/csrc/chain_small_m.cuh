@@ -10,8 +10,10 @@
 //     from L2 / HBM into registers, one chunk (eight 16-byte loads a lane) ahead of use across layer
 //     boundaries, L2 prefetches two layers ahead;
 //   * every CTA holds the codes of all rows of the current activations in shared memory; the products
-//     are mma.sync m16n8k32 (int8): 16 rows fill its M, where a tcgen05 tile would spend 128 rows on
-//     16 and first want the weights unpacked in shared memory;
+//     are mma.sync m16n8k32 (int8) with sixteen output channels as its M and eight activation rows as
+//     its N, so that eight rows waste nothing (a tcgen05 tile would first want the weights unpacked in
+//     shared memory; this part issues an m16n8k32 every sixteen clocks per scheduler, which is what the
+//     feed-forward layers' products cost);
 //   * the output rows are quantized for the next layer in place (Fig. 2): every warp sends the maxima of
 //     its rows over the CTA's columns to all sixteen CTAs, waits for the other fifteen of each row,
 //     and sends its share of the codes to all sixteen.  Nothing but requested outputs is written
@@ -24,7 +26,7 @@
 // What a layer then costs is a chain of latencies and of instructions that every warp issues once: no
 // integer division and no dependent parameter load in the loops (the step table sits in shared memory
 // with everything derived from the sizes), the next layer's weights, scales and prefetches are asked
-// for while the row maxima are under way, and packed weights are used as sixteen times their codes
+// for while the row maxima are under way, eight warps instead of sixteen, and packed weights are used as sixteen times their codes
 // (a nibble in the upper half of a byte; the sums are shifted back, exact), two instructions per four
 // codes instead of eleven per eight, against activation codes stored in the same even / odd order.
 // The arithmetic is that of the per-layer kernels operation by operation (exact int32 sums, the same
@@ -39,11 +41,11 @@
 namespace aqt {
 
 constexpr int kChainCtas = 16;     // CTAs of a cluster (beyond the portable eight: allowed per function)
-constexpr int kChainWarps = 16;
+constexpr int kChainWarps = 8;
 constexpr int kChainThreads = 32 * kChainWarps;
-constexpr int kChainChunk = 8;     // 16-byte weight loads per lane in flight
+constexpr int kChainChunk = 8;     // pieces (two 16-byte weight loads per lane) in flight
 constexpr int kChainMaxSteps = 256;
-constexpr int kChainMaxN = 16 * kChainThreads;  // one scale per thread
+constexpr int kChainMaxN = kChainCtas * kChainThreads;  // one scale per thread
 constexpr int kChainMaxCols = 256;              // output columns per CTA: eight floats per lane and row
 
 struct ChainStep {
@@ -55,7 +57,7 @@ struct ChainStep {
   float rs;           // residual scale
   uint32_t flags;
   // derived by the host (chain_derive)
-  uint16_t tiles, ks_n;          // n8-tiles per CTA (value and gate tiles for GLU), shares of K
+  uint16_t tiles, ks_n;          // 16-channel tiles per CTA, shares of K
   uint32_t inv_tiles;            // ceil(65536 / tiles), ceil(65536 / ks_n): quotients of small numbers by a multiply and a shift
   uint16_t inv_ks_lo, units;     // (ks_n == 1 is not divided by)
 };
@@ -84,8 +86,8 @@ struct ChainParams {
 // shared-memory phase (two rows, four lanes each) touch all banks once: a lane reads 32 codes per
 // 128 with packed weights, 16 per 64 with int8 weights.
 __host__ __device__ inline int chain_pitch(int K, bool packed) { return K + (packed ? 16 : 64); }
-// n8-tiles per CTA (value and gate tiles for GLU) and the split of K over warps.
-static inline int chain_tiles(int N) { return N / (8 * kChainCtas); }
+// Tiles of sixteen channels per CTA (the last one may be half empty) and the split of K over warps.
+static inline int chain_tiles(int N) { return (N / kChainCtas + 15) / 16; }
 static inline int chain_ksplit(int tiles, int K) {
   if (tiles >= kChainWarps) return 1;
   const int by_warps = kChainWarps / tiles, by_k = K / 128;
@@ -140,10 +142,11 @@ __device__ __forceinline__ float chain_max4(float m, const float (&v)[4]) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
 }
 
-// MT: 16-row tiles per cluster.
-template <int MT, int MAXS>
+// NT: 8-row tiles per cluster.
+template <int NT, int MAXS>
 __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const __grid_constant__ ChainParams<MAXS> p) {
-  constexpr int R = 16 * MT;
+  constexpr int R = 8 * NT;
+  constexpr int SETS = NT == 1 ? 2 : 1;  // independent accumulators per row tile (the products of one set depend on one another)
   extern __shared__ __align__(128) uint8_t chain_smem[];
   __shared__ __align__(16) ChainStep steps[MAXS];
   __shared__ __align__(16) float sw_s[2][kChainThreads], bias_s[2][kChainThreads];
@@ -173,14 +176,15 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   __syncthreads();
   grid_dependency_wait();
 
-  // ---- This warp's products in program order: units (an n8-tile and a share of K), each in items of up to
-  // kChainChunk 16-byte loads per lane.  The next item's loads are in nxt (zeros beyond its end).
+  // ---- This warp's products in program order: units (sixteen channels and a share of K), each in items of up to
+  // kChainChunk pieces (16 bytes of two channels' weights per lane: 128 of K packed, 64 of K int8).  The next
+  // item's pieces are in nxt (zeros beyond its end).
   int it_step = 0, it_u = warp;  // unit of the item
-  int u_left = 0;                // loads from the item to the end of the unit
+  int u_left = 0;                // pieces from the item to the end of the unit
   int u_a = 0, u_part = 0;       // this lane's first activation code (byte offset), first partial sum (index)
-  bool u_first = true;
-  const uint8_t* u_src = nullptr;
-  uint4 nxt[kChainChunk];
+  bool u_first = true, u_both = true;  // the unit's first item; its upper eight channels exist
+  const uint8_t *u_src0 = nullptr, *u_src1 = nullptr;
+  uint4 nxt[kChainChunk][2];
   auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
     while (it_step < n_steps && it_u >= steps[it_step].units) {
       ++it_step;
@@ -189,8 +193,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     u_left = 0;
     if (it_step >= n_steps) return;
     const ChainStep& st = steps[it_step];
-    const int k128 = st.K >> 7;
-    const bool packed = (st.flags & kChainPacked) != 0;
+    const int k128 = st.K >> 7, per_cta = st.N >> 4;
+    const int shift = (st.flags & kChainPacked) ? 1 : 0;
     int tile = it_u, kb0 = 0, kb1 = k128, ks = 0;  // tiles fastest, then shares of K
     if (st.ks_n > 1) {
       ks = (int)((uint32_t)it_u * st.inv_tiles >> 16);
@@ -198,20 +202,29 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks_lo >> 16);
       kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks_lo >> 16);
     }
-    int n = rank * (st.N >> 4) + tile * 8 + g;
-    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value tiles, then the gate tiles of the same output columns
-      const int half = st.tiles >> 1, gate = tile >= half ? 1 : 0;
-      n = gate * (st.N >> 1) + rank * (st.N >> 5) + (tile - gate * half) * 8 + g;
+    const int c0 = tile * 16 + g;  // this lane's channels among the CTA's: c0 and c0 + 8
+    u_both = tile * 16 + 8 < per_cta;
+    const int c1 = u_both ? c0 + 8 : c0;
+    int n0 = rank * per_cta + c0, n1 = rank * per_cta + c1;
+    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value channels, then the gate channels of the same output columns
+      const int cols = per_cta >> 1, gate_off = (st.N >> 1) - cols;
+      n0 = rank * cols + c0 + (c0 >= cols ? gate_off : 0);
+      n1 = rank * cols + c1 + (c1 >= cols ? gate_off : 0);
     }
-    const int shift = packed ? 1 : 0;
     u_left = (kb1 - kb0) << (1 - shift);
-    u_src = st.w + (int64_t)n * (st.K >> shift) + (kb0 << (7 - shift)) + kq * 16;
-    u_a = g * chain_pitch(st.K, packed) + kb0 * 128 + kq * (16 << shift);
-    u_part = (ks * R + g) * ((st.N >> 4) + 8) + tile * 8 + 2 * kq;
+    const uint8_t* w = st.w + (kb0 << (7 - shift)) + kq * 16;
+    u_src0 = w + (int64_t)n0 * (st.K >> shift);
+    u_src1 = w + (int64_t)n1 * (st.K >> shift);
+    u_a = g * chain_pitch(st.K, shift != 0) + kb0 * 128 + kq * (16 << shift);
+    u_part = (ks * R + 2 * kq) * (per_cta + 4) + c0;
     u_first = true;
   };
-  auto load_item = [&](int j) {
-    nxt[j] = j < u_left ? __ldg(reinterpret_cast<const uint4*>(u_src + j * 64)) : make_uint4(0u, 0u, 0u, 0u);
+  auto load_piece = [&](int j) {
+    nxt[j][0] = nxt[j][1] = make_uint4(0u, 0u, 0u, 0u);
+    if (j < u_left) {
+      nxt[j][0] = __ldg(reinterpret_cast<const uint4*>(u_src0 + j * 64));
+      nxt[j][1] = __ldg(reinterpret_cast<const uint4*>(u_src1 + j * 64));
+    }
   };
   auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
     wv = bv = 0.0f;
@@ -239,18 +252,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
 
   open_unit();
 #pragma unroll
-  for (int j = 0; j < kChainChunk; ++j) load_item(j);
+  for (int j = 0; j < kChainChunk; ++j) load_piece(j);
   prefetch_slice(1);
   float wv, bv;  // scale and bias of this thread's channel of the next step, on their way to sw_s / bias_s
   load_scales(0, wv, bv);
 
   // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
-  float sx[MT];  // input scales of this warp's rows (warp, warp + 16)
+  float sx[NT];  // input scales of this warp's rows (warp, warp + 8, ...)
   {
     const int pitch = chain_pitch(p.K0, (steps[0].flags & kChainPacked) != 0);
 #pragma unroll
-    for (int t = 0; t < MT; ++t) {
-      const int r = warp + 16 * t;
+    for (int t = 0; t < NT; ++t) {
+      const int r = warp + 8 * t;
       sx[t] = 0.0f;
       if (r >= rows) continue;
       const float4* xr = reinterpret_cast<const float4*>(p.x + (int64_t)(row0 + r) * p.ldx);
@@ -289,7 +302,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     const int per_cta = st.N >> 4, units = st.units, ks_n = st.ks_n;
     const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
     const int n_out = glu ? st.N >> 1 : st.N;
-    const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 8;
+    const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 4;
     const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
     // two buffers of partial sums: after a side step the next products are written while these are read
     int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
@@ -298,21 +311,23 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
 
     // ---- integer products
     bool used = false;
-    int acc[MT][2][4];
+    int acc[NT][SETS][4];
     while (it_step == s) {
       const int n = u_left, part0 = u_part;
+      const bool both = u_both;
       const uint8_t* a0 = codes + u_a;
       if (u_first) {
 #pragma unroll
-        for (int t = 0; t < MT; ++t)
+        for (int t = 0; t < NT; ++t)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) acc[t][j >> 2][j & 3] = 0;
+          for (int j = 0; j < 4 * SETS; ++j) acc[t][j >> 2][j & 3] = 0;
       }
-      // the next item: loaded slot by slot below if it belongs to this step, else while the maxima are under way
+      // the next item: loaded piece by piece below if it belongs to this step, else while the maxima are under way
       bool more = true;
       if (n > kChainChunk) {
         u_left -= kChainChunk;
-        u_src += kChainChunk * 64;
+        u_src0 += kChainChunk * 64;
+        u_src1 += kChainChunk * 64;
         u_a += kChainChunk * (packed ? 128 : 64);
         u_first = false;
       } else {
@@ -326,51 +341,52 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         if (jj < n) {
 #pragma unroll
           for (int j = jj; j < jj + 2; ++j) {
-            const uint4 w = nxt[j];
+            const uint4 w0 = nxt[j][0], w1 = nxt[j][1];
             if (packed) {
               // sixteen times the codes: the even ones' nibbles moved up, the odd ones' in place
-              const uint32_t b[8] = {(w.x << 4) & 0xF0F0F0F0u, w.x & 0xF0F0F0F0u, (w.y << 4) & 0xF0F0F0F0u, w.y & 0xF0F0F0F0u,
-                                     (w.z << 4) & 0xF0F0F0F0u, w.z & 0xF0F0F0F0u, (w.w << 4) & 0xF0F0F0F0u, w.w & 0xF0F0F0F0u};
+              constexpr uint32_t kHigh = 0xF0F0F0F0u;
+              const uint32_t e[8] = {(w0.x << 4) & kHigh, (w1.x << 4) & kHigh, (w0.y << 4) & kHigh, (w1.y << 4) & kHigh,
+                                     (w0.z << 4) & kHigh, (w1.z << 4) & kHigh, (w0.w << 4) & kHigh, (w1.w << 4) & kHigh};
+              const uint32_t o[8] = {w0.x & kHigh, w1.x & kHigh, w0.y & kHigh, w1.y & kHigh, w0.z & kHigh, w1.z & kHigh, w0.w & kHigh, w1.w & kHigh};
 #pragma unroll
-              for (int t = 0; t < MT; ++t) {
-                const uint8_t* a = a0 + t * 16 * pitch + j * 128;
-                const uint4 l0 = *reinterpret_cast<const uint4*>(a), l1 = *reinterpret_cast<const uint4*>(a + 16);
-                uint4 h0 = make_uint4(0u, 0u, 0u, 0u), h1 = h0;
-                if (rows > 8 + 16 * t) {
-                  h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
-                  h1 = *reinterpret_cast<const uint4*>(a + 8 * pitch + 16);
-                }
-                mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, b[0], b[1]);
-                mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, b[2], b[3]);
-                mma_s8_16x8x32(acc[t][0], l1.x, h1.x, l1.y, h1.y, b[4], b[5]);
-                mma_s8_16x8x32(acc[t][1], l1.z, h1.z, l1.w, h1.w, b[6], b[7]);
+              for (int t = 0; t < NT; ++t) {
+                const uint8_t* a = a0 + t * 8 * pitch + j * 128;
+                const uint4 x0 = *reinterpret_cast<const uint4*>(a), x1 = *reinterpret_cast<const uint4*>(a + 16);
+                mma_s8_16x8x32(acc[t][0], e[0], e[1], o[0], o[1], x0.x, x0.y);
+                mma_s8_16x8x32(acc[t][SETS - 1], e[2], e[3], o[2], o[3], x0.z, x0.w);
+                mma_s8_16x8x32(acc[t][0], e[4], e[5], o[4], o[5], x1.x, x1.y);
+                mma_s8_16x8x32(acc[t][SETS - 1], e[6], e[7], o[6], o[7], x1.z, x1.w);
               }
             } else {
 #pragma unroll
-              for (int t = 0; t < MT; ++t) {
-                const uint8_t* a = a0 + t * 16 * pitch + j * 64;
-                const uint4 l0 = *reinterpret_cast<const uint4*>(a);
-                uint4 h0 = make_uint4(0u, 0u, 0u, 0u);
-                if (rows > 8 + 16 * t) h0 = *reinterpret_cast<const uint4*>(a + 8 * pitch);
-                mma_s8_16x8x32(acc[t][0], l0.x, h0.x, l0.y, h0.y, w.x, w.y);
-                mma_s8_16x8x32(acc[t][1], l0.z, h0.z, l0.w, h0.w, w.z, w.w);
+              for (int t = 0; t < NT; ++t) {
+                const uint4 x0 = *reinterpret_cast<const uint4*>(a0 + t * 8 * pitch + j * 64);
+                mma_s8_16x8x32(acc[t][0], w0.x, w1.x, w0.y, w1.y, x0.x, x0.y);
+                mma_s8_16x8x32(acc[t][SETS - 1], w0.z, w1.z, w0.w, w1.w, x0.z, x0.w);
               }
             }
           }
         }
         if (more) {
-          load_item(jj);
-          load_item(jj + 1);
+          load_piece(jj);
+          load_piece(jj + 1);
         }
       }
       if (n <= kChainChunk) {  // the unit's last item
         const int shift = packed ? 4 : 0;
 #pragma unroll
-        for (int t = 0; t < MT; ++t) {
-          int* dst = part + part0 + 16 * t * part_pitch;
-          *reinterpret_cast<int2*>(dst) = make_int2((acc[t][0][0] + acc[t][1][0]) >> shift, (acc[t][0][1] + acc[t][1][1]) >> shift);
-          *reinterpret_cast<int2*>(dst + 8 * part_pitch) =
-              make_int2((acc[t][0][2] + acc[t][1][2]) >> shift, (acc[t][0][3] + acc[t][1][3]) >> shift);
+        for (int t = 0; t < NT; ++t) {
+          int* dst = part + part0 + 8 * t * part_pitch;
+          if (SETS == 2) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[t][0][j] += acc[t][SETS - 1][j];
+          }
+          dst[0] = acc[t][0][0] >> shift;
+          dst[part_pitch] = acc[t][0][1] >> shift;
+          if (both) {
+            dst[8] = acc[t][0][2] >> shift;
+            dst[part_pitch + 8] = acc[t][0][3] >> shift;
+          }
         }
       }
       if (!more) break;
@@ -380,13 +396,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     __syncthreads();
     if (*(volatile int*)&abort_flag) break;  // a wait gave up: every thread leaves here
 
-    // ---- epilogue: warp w owns rows w and w + 16, a lane four consecutive columns at a time
-    float v[MT][2][4];
+    // ---- epilogue: warp w owns rows w, w + 8, ..., a lane four consecutive columns at a time
+    float v[NT][2][4];
     if (threadIdx.x == 0 && !side && !last) mbar_arrive_expect_tx(smem_u32(&codes_bar), (uint32_t)(rows * n_out));
 #pragma unroll
-    for (int t = 0; t < MT; ++t) {
+    for (int t = 0; t < NT; ++t) {
       float amax = 0.0f;
-      const int r = warp + 16 * t;
+      const int r = warp + 8 * t;
       if (r >= rows) continue;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
@@ -445,7 +461,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     if (used) {
       open_unit();
 #pragma unroll
-      for (int j = 0; j < kChainChunk; ++j) load_item(j);
+      for (int j = 0; j < kChainChunk; ++j) load_piece(j);
     }
     load_scales(s + 1, wv, bv);
     prefetch_slice(s + 2);
@@ -458,8 +474,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     const bool next_packed = (steps[s + 1].flags & kChainPacked) != 0;
     const int out_pitch = chain_pitch(n_out, next_packed);
 #pragma unroll
-    for (int t = 0; t < MT; ++t) {
-      const int r = warp + 16 * t;
+    for (int t = 0; t < NT; ++t) {
+      const int r = warp + 8 * t;
       if (r >= rows) continue;
       mbar_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
       const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
@@ -527,7 +543,7 @@ static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
   for (int i = 0; i < n; ++i) {
     const ChainStep& st = steps[i];
     const int tiles = chain_tiles(st.N);
-    const int c = R * (st.K + 64), q = chain_ksplit(tiles, st.K) * R * (st.N / kChainCtas + 8) * 4;
+    const int c = R * (st.K + 64), q = chain_ksplit(tiles, st.K) * R * (st.N / kChainCtas + 4) * 4;
     if (c > code) code = c;
     if (q > part) part = q;
     if ((st.flags & kChainAdd) && R * (st.N / kChainCtas) * 4 > h) h = R * (st.N / kChainCtas) * 4;
@@ -541,39 +557,40 @@ static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
 
 constexpr int kChainMaxSmem = 180 * 1024;  // beside the step table and the exchange words
 
-// 16-row clusters that run at the same time (the part schedules seven or eight of sixteen CTAs each).
+// Clusters that run at the same time (the part schedules seven or eight of sixteen CTAs each).
 constexpr int kChainClusters = 7;
 
-template <int MT, int MAXS>
+template <int NT, int MAXS>
 static int launch_chain_inst(const ChainParams<kChainMaxSteps>& full, int smem, cudaStream_t st) {
   ChainParams<MAXS> p;
   memcpy(static_cast<void*>(&p), &full, offsetof(ChainParams<MAXS>, steps) + (size_t)full.n_steps * sizeof(ChainStep));
-  auto kernel = chain_small_m_kernel<MT, MAXS>;
+  auto kernel = chain_small_m_kernel<NT, MAXS>;
   static std::atomic<uint64_t> opted_in{0}, wide{0};
   int rc = ensure_dynamic_smem(kernel, kChainMaxSmem, opted_in);
   if (rc != AQT_OK) return rc;
   rc = ensure_wide_clusters(kernel, wide);
   if (rc != AQT_OK) return rc;
-  const unsigned clusters = (unsigned)ceil_div(full.M, 16 * MT);
+  const unsigned clusters = (unsigned)ceil_div(full.M, 8 * NT);
   return launch_pdl(kernel, dim3(clusters * kChainCtas, 1, 1), dim3(kChainThreads, 1, 1), (size_t)smem, st, kChainCtas, p);
+}
+template <int NT>
+static int launch_chain_rows(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
+  const ChainSizes z = chain_sizes(p.steps, p.n_steps, 8 * NT);
+  if (z.smem() > kChainMaxSmem) return AQT_ERR_UNSUPPORTED;
+  p.code_bytes = z.code_bytes;
+  p.part_bytes = z.part_bytes;
+  return p.n_steps <= 16 ? launch_chain_inst<NT, 16>(p, z.smem(), st) : launch_chain_inst<NT, kChainMaxSteps>(p, z.smem(), st);
 }
 
 // p: everything but the shared-memory sizes.  AQT_ERR_UNSUPPORTED if the kernel cannot take the chain.
 static int launch_chain(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
   if (p.M <= 0 || p.n_steps <= 0 || p.n_steps > kChainMaxSteps) return AQT_ERR_UNSUPPORTED;
-  // sixteen rows per cluster while the clusters fit the part side by side, then 32
   for (int i = 0; i < p.n_steps; ++i) chain_derive(p.steps[i]);
-  int mt = p.M <= 16 * kChainClusters ? 1 : 2;
-  ChainSizes z = chain_sizes(p.steps, p.n_steps, 16 * mt);
-  if (mt == 2 && z.smem() > kChainMaxSmem) {
-    mt = 1;
-    z = chain_sizes(p.steps, p.n_steps, 16);
-  }
-  if (z.smem() > kChainMaxSmem) return AQT_ERR_UNSUPPORTED;
-  p.code_bytes = z.code_bytes;
-  p.part_bytes = z.part_bytes;
-  if (p.n_steps <= 16) return mt == 1 ? launch_chain_inst<1, 16>(p, z.smem(), st) : launch_chain_inst<2, 16>(p, z.smem(), st);
-  return mt == 1 ? launch_chain_inst<1, kChainMaxSteps>(p, z.smem(), st) : launch_chain_inst<2, kChainMaxSteps>(p, z.smem(), st);
+  // the fewest rows per cluster with which all clusters run at once
+  if (p.M <= 8 * kChainClusters) return launch_chain_rows<1>(p, st);
+  if (p.M <= 16 * kChainClusters) return launch_chain_rows<2>(p, st);
+  const int rc = launch_chain_rows<4>(p, st);
+  return rc == AQT_ERR_UNSUPPORTED ? launch_chain_rows<2>(p, st) : rc;
 }
 
 }  // namespace aqt
