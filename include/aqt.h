@@ -272,7 +272,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
 #define AQT_CHAIN_SIDE 1
 #define AQT_CHAIN_ADD 2
 #define AQT_CHAIN_MAX_LAYERS 256
-#define AQT_CHAIN_MAX_ROWS 224
+#define AQT_CHAIN_MAX_ROWS 112
 typedef struct aqt_chain_layer {
   const void* wq;
   const float* s_w;

@@ -34,7 +34,7 @@ EXPORTS = ("aqt_version", "aqt_status_string", "aqt_quantize", "aqt_pack_int4", 
            "aqt_selftest_bounded_wait", "aqt_qmatmul_requant", "aqt_linear_fwd_weight_only", "aqt_linear_bwd",
            "aqt_plan_qmatmul", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_chain_fwd", "aqt_selftest_sfu_rate")
 NOALLOC_MAX_WEIGHT_BYTES = 4 << 20
-CHAIN_MAX_ROWS = 224
+CHAIN_MAX_ROWS = 112
 
 
 class AqtError(RuntimeError):

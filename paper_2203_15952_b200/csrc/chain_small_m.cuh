@@ -3,7 +3,7 @@
 //
 // What bounds such a step is not work but the number of dependent kernels: an eight-row step through
 // the 17-block d = 512 encoder reads 67 MB of weights (10 us of HBM time) in 187 launches of 2 to
-// 11 us each (1276 us).  Here one thread-block cluster of sixteen CTAs carries up to 32 rows through
+// 11 us each (1276 us).  Here one thread-block cluster of sixteen CTAs carries up to 16 rows through
 // every layer; clusters take different rows and do not interact (rows are independent under per-row
 // scales).  Within a cluster:
 //   * CTA r owns 1/16 of every layer's output channels and with it 1/16 of the weights, which stream
@@ -23,6 +23,10 @@
 // cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
 // scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
 // wait of the library.
+// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 425 vs 1250 us, 32 rows
+// 427 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 626 vs 1340; beyond, a
+// second wave of clusters or 32 rows per cluster lose to the per-layer kernels at d = 1024 (860 vs 700
+// us for 8 blocks at 113 rows), which is where AQT_CHAIN_MAX_ROWS lies.
 // What a layer then costs is a chain of latencies and of instructions that every warp issues once: no
 // integer division and no dependent parameter load in the loops (the step table sits in shared memory
 // with everything derived from the sizes), the next layer's weights, scales and prefetches are asked
@@ -463,10 +467,12 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
 #pragma unroll
       for (int j = 0; j < kChainChunk; ++j) load_piece(j);
     }
-    load_scales(s + 1, wv, bv);
-    prefetch_slice(s + 2);
     fresh = !side;
-    if (side) continue;
+    if (side) {
+      load_scales(s + 1, wv, bv);
+      prefetch_slice(s + 2);
+      continue;
+    }
 
     // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
     // CTA has finished its products, so nobody reads the old codes any more.
@@ -509,6 +515,8 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         if (8 * i < cols) chain_st_async_v2(remote, w0, w1, remote + bar_off);
       }
     }
+    load_scales(s + 1, wv, bv);
+    prefetch_slice(s + 2);
     exchange_parity ^= 1u;
   }
   grid_dependents_launch();
@@ -588,9 +596,7 @@ static int launch_chain(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
   for (int i = 0; i < p.n_steps; ++i) chain_derive(p.steps[i]);
   // the fewest rows per cluster with which all clusters run at once
   if (p.M <= 8 * kChainClusters) return launch_chain_rows<1>(p, st);
-  if (p.M <= 16 * kChainClusters) return launch_chain_rows<2>(p, st);
-  const int rc = launch_chain_rows<4>(p, st);
-  return rc == AQT_ERR_UNSUPPORTED ? launch_chain_rows<2>(p, st) : rc;
+  return launch_chain_rows<2>(p, st);
 }
 
 }  // namespace aqt

@@ -35,11 +35,10 @@ def _layer_by_layer(stack, x):
 
 @pytest.mark.parametrize("M,d,ff,blocks,bits", [
     (1, 512, 2048, 2, (4, 8, 8)), (8, 512, 2048, 3, (4, 8, 8)), (9, 256, 1024, 2, (8, 4, 4)), (16, 384, 1536, 2, (4, 4, 8)),
-    (17, 512, 2048, 1, (8, 8, 8)), (112, 512, 2048, 1, (4, 8, 8)), (113, 256, 1024, 1, (4, 4, 4)), (224, 512, 2048, 1, (4, 8, 4)),
-    (5, 1024, 4096, 1, (4, 4, 8)), (130, 1024, 4096, 1, (4, 8, 8)), (3, 256, 1024, 27, (4, 8, 8))])
+    (17, 512, 2048, 1, (8, 8, 8)), (56, 512, 2048, 1, (4, 8, 4)), (57, 256, 1024, 1, (4, 4, 4)), (112, 512, 2048, 1, (4, 8, 8)),
+    (5, 1024, 4096, 1, (4, 4, 8)), (90, 1024, 4096, 1, (4, 8, 8)), (3, 256, 1024, 27, (4, 8, 8))])
 def test_encoder_chain_gives_the_per_layer_bits(M, d, ff, blocks, bits):
-    """Row counts around the 8- and 16-row halves of a tile, one and two row tiles per cluster, several
-    clusters, every mix of packed and int8 weights, a stack longer than one launch takes; some rows zero or tiny."""
+    """Row counts around an 8-row tile, one and two tiles per cluster, several clusters, every mix of packed and int8 weights, a stack longer than one launch takes; some rows zero or tiny."""
     stack, x = _stack(M, d, ff, blocks, bits, M + d, bias=True, rounding=aqt.ROUND_HALF_UP_FLOOR if M % 2 else aqt.ROUND_NEAREST_EVEN)
     if M > 2:
         x[1] = 0.0
@@ -54,7 +53,7 @@ def test_encoder_chain_gives_the_per_layer_bits(M, d, ff, blocks, bits):
     assert aqt.aqt_device_status() == 0
 
 
-@pytest.mark.parametrize("M,d,ff,bits_w,bits_a", [(1, 256, 1024, 4, 8), (8, 512, 2048, 4, 8), (30, 640, 2560, 8, 4), (200, 768, 3072, 4, 8),
+@pytest.mark.parametrize("M,d,ff,bits_w,bits_a", [(1, 256, 1024, 4, 8), (8, 512, 2048, 4, 8), (30, 640, 2560, 8, 4), (100, 768, 3072, 4, 8),
                                                   (16, 1024, 4096, 8, 8)])
 def test_ffn_chain_gives_the_per_layer_bits(M, d, ff, bits_w, bits_a):
     g = torch.Generator(device=DEV).manual_seed(M + d)
