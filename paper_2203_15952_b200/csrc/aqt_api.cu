@@ -4,6 +4,7 @@
 #include "backward.cuh"
 #include "pack.cuh"
 #include "qgemm_sm100.cuh"
+#include "dw_split_sm100.cuh"
 #include "qgemm_requant_sm100.cuh"
 #include "qgemv_small_m.cuh"
 #include "quantize.cuh"
@@ -46,14 +47,14 @@ size_t ws_weight_only(int64_t M, int64_t N, int64_t K, int precision) {
   return round_up((size_t)N * (size_t)K * 4, 256);
 }
 
-// Backward workspace: [ones K | column-sum partials | s_w-scaled W^T [K, N] | dy^T | s_x-scaled xq^T | dw partials].
+// Backward workspace of the tf32 form: [column-sum partials | s_w-scaled W^T [K, N] | dy^T | s_x-scaled xq^T | dw partials].
 // The weight gradient is an [N, K] output with a contraction of M: few, very deep tiles.  Its
 // contraction is therefore cut into `batches` chunks of `chunk` rows (a multiple of 32), each
 // batch a matmul of its own in the same launch (GemmParams::batch_tiles_m), and the batches'
 // outputs are added in order.  The split is chosen for the 148 SMs of the one device this library
 // is built for, so that the layout (and aqt_workspace_bytes) needs no CUDA call.
 struct BwdLayout {
-  size_t ones, partial, wt, dyt, xt, dwp, total;
+  size_t partial, wt, dyt, xt, dwp, total;
   int64_t batches, chunk, n_pad;  // batches == 1: chunk is the padded pitch of the transposed operands
 };
 BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K) {
@@ -70,8 +71,7 @@ BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K) {
     L.chunk = round_up((size_t)ceil_div(M, batches), kTrRows);
     L.batches = ceil_div(M, L.chunk);
   }
-  L.ones = 0;
-  L.partial = L.ones + round_up((size_t)K * 4, 256);
+  L.partial = 0;
   // column-sum partials: one row of N per 128-row block of the transpose (or per 2048-row chunk of the stand-alone sum)
   L.wt = L.partial + round_up((size_t)(transpose_row_blocks(L.batches * L.chunk) + colsum_chunks(M)) * (size_t)N * 4, 256);
   L.dyt = L.wt + round_up((size_t)K * (size_t)N * 4, 256);
@@ -81,11 +81,52 @@ BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K) {
   return L;
 }
 
+// Weight gradient on split operands: [codes of x transposed, bf16 [K, m_pitch] | column-sum partials | dw partials], behind
+// the scaled transposed weights of the other product.  Its contraction over M is cut into `batches` of `chunk` rows (a
+// multiple of 32): the tiles are few and very deep, and they fill the SM pairs that the other product leaves free, so
+// smaller ones end more evenly (half a tile's time, at 0.39 us a K-block of 32 rows, plus 3 us a tile to start it)
+// against 5 TB/s for adding the partial products.  For the 74 pairs of the one part this library is built for, so that
+// the layout needs no CUDA call.
+struct DwLayout {
+  size_t wt, xt, colsum, dwp, total;
+  int64_t m_pitch, batches, chunk, n_pad;
+};
+DwLayout dw_layout(int64_t M, int64_t N, int64_t K) {
+  DwLayout L;
+  const int64_t tiles = ceil_div(N, 256) * ceil_div(K, 256), pairs = kDefaultSms / 2;
+  L.m_pitch = (int64_t)round_up((size_t)M, 8);
+  L.n_pad = (int64_t)round_up((size_t)N, 256);
+  L.batches = 1;
+  double best = 1e300;
+  for (int64_t b = 1; b <= 16 && (b == 1 || M / b >= 256); ++b) {
+    const double tile_us = 0.39 * (double)ceil_div(ceil_div(M, b), 32) + 3.0;
+    const double rounds = (double)(tiles * b) / (double)pairs;
+    const double main_us = tile_us * (rounds < 1.0 ? 1.0 : rounds + 0.5);
+    const double sum_us = b > 1 ? 2.0 + ((double)b + 1.0) * (double)N * (double)K * 4.0 / 5e6 : 0.0;
+    if (main_us + sum_us < best) {
+      best = main_us + sum_us;
+      L.batches = b;
+    }
+  }
+  L.chunk = (int64_t)round_up((size_t)ceil_div(M, L.batches), 32);
+  L.batches = ceil_div(M, L.chunk);
+  L.wt = 0;
+  L.xt = L.wt + round_up((size_t)K * (size_t)N * 4, 256);
+  L.colsum = L.xt + round_up((size_t)K * L.m_pitch * 2, 256);
+  L.dwp = L.colsum + round_up((size_t)(L.batches * DwCfg::kGroups) * N * 4, 256);
+  L.total = L.dwp + (L.batches > 1 ? round_up((size_t)L.batches * L.n_pad * K * 4, 256) : 0);
+  return L;
+}
+size_t bwd_workspace(int64_t M, int64_t N, int64_t K) {
+  const size_t tf32_form = bwd_layout(M, N, K).total, split_form = dw_layout(M, N, K).total;
+  return tf32_form > split_form ? tf32_form : split_form;
+}
+
 // y[r][c] = sum_j a[r][j] * b[c][j] on the float kind of the GEMM (no scale, bias or activation).
 // batches > 1: a holds `batches` stacked [rows / batches, depth] blocks, b as many stacked [cols, depth] blocks,
 // and y receives the stacked [rows / batches, cols] products.
-int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int64_t cols, int64_t depth, const float* ones, float* y,
-                  int64_t ldy, cudaStream_t st, int64_t batches = 1) {
+int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int64_t cols, int64_t depth, float* y, int64_t ldy,
+                  cudaStream_t st, int64_t batches = 1, bool early_trigger = false) {
   GemmParams p;
   if (batches > 1) {
     p.batch_tiles_m = (int)(rows / batches / kBM);  // rows per batch are a multiple of the tile height
@@ -93,7 +134,7 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
     p.b_rows = batches * cols;
   }
   p.s_x = nullptr;
-  p.s_w = ones;
+  p.s_w = nullptr;
   p.bias = nullptr;
   p.residual = nullptr;
   p.acc_debug = nullptr;
@@ -109,6 +150,7 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
   p.n_out = (int)cols;
   p.tiles_m = p.tiles_n = p.k_blocks = 0;
   p.small_acc = 0;
+  p.early_trigger = early_trigger ? 1 : 0;
   return launch_qgemm(reinterpret_cast<const int8_t*>(a), b, false, y, ldy, p, st);
 }
 
@@ -249,7 +291,7 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   if (op == AQT_OP_LINEAR_FWD) return ws_linear(M, N, K, bits_w);
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return ws_weight_only(0, N, K, AQT_FLOAT_TF32);
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY_X2) return ws_weight_only(M, N, K, AQT_FLOAT_TF32X2);
-  if (op == AQT_OP_LINEAR_BWD) return bwd_layout(M, N, K).total;
+  if (op == AQT_OP_LINEAR_BWD) return bwd_workspace(M, N, K);
   if (op == AQT_OP_FFN_FWD) return ffn_layout(M, K, N, bits_w, bits_w).total;
   if (op == AQT_OP_QMATMUL_REQUANT) return round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256) + requant_exchange_bytes(M, N);
   return 0;
@@ -746,6 +788,55 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
   return launch_qgemm(reinterpret_cast<const int8_t*>(a_f), w_f, false, y, ldy, p, st);
 }
 
+// The weight gradient takes the split operands from 256 rows on (20.1 vs 27.0 us at 1100 x 2048 x 512, 64.5 vs 120 us at
+// 12 800 x 2048 x 512, 1084 vs 1413 us at 65 536 x 4096 x 1024, with the bias gradient; below, its contraction is a few
+// K-blocks and the tf32 form's narrow tiles occupy more SMs).
+static bool dw_split_applies(int64_t M, int64_t N, int64_t K) { return M >= 256 && N >= 128 && K >= 128; }
+
+// The backward with the weight gradient on split operands: the scale of x multiplies dy while it is split, the codes stay
+// exact, and dy is read in place.  The other product stays on the tf32 form, which needs no conversion in the kernel (62.6
+// vs 65.0 us at 12 800 x 2048 x 512, 729 vs 850 us at 65 536 x 4096 x 1024); the two run side by side (166 against 83 + 109
+// us at 65 536 x 512 x 512).
+static int linear_bwd_split(const float* dy, int64_t lddy, const void* xq, const float* s_x, int s_x_kind, int bits_a, const void* wq,
+                            const float* s_w, int bits_w, int64_t M, int64_t N, int64_t K, float* dx, int64_t lddx, float* dw, int64_t lddw,
+                            float* dbias, uint8_t* ws, cudaStream_t st) {
+  const DwLayout L = dw_layout(M, N, K);
+  float* colsum = reinterpret_cast<float*>(ws + L.colsum);
+  float* wt = reinterpret_cast<float*>(ws + L.wt);
+  uint16_t* xt = reinterpret_cast<uint16_t*>(ws + L.xt);
+  int rc;
+  if (dx != nullptr) {
+    rc = launch_transpose_scale_codes(wq, is_packed(bits_w), s_w, true, N, K, wt, N, N, K, st);
+    if (rc != AQT_OK) return rc;
+  }
+  rc = launch_transpose_codes_bf16(xq, is_packed(bits_a), M, K, xt, L.m_pitch, st);
+  if (rc != AQT_OK) return rc;
+  if (dx != nullptr) {
+    // dx = dy . (s_w wq): rows m, columns k, contraction n
+    rc = float_gemm_nt(dy, lddy, wt, M, K, N, dx, lddx, st, 1, true);
+    if (rc != AQT_OK) return rc;
+  }
+  // dw = (diag(s_x) dy)^T . xq: rows n, columns k, contraction m, cut into batches
+  DwParams p = {};
+  p.a_scale = s_x;
+  p.a_scale_step = s_x_kind == AQT_SCALE_ROW ? 1 : 0;
+  p.colsum = dbias != nullptr ? colsum : nullptr;
+  p.M = (int)N;
+  p.N = (int)K;
+  p.K = (int)M;
+  p.batch_k = (int)L.chunk;
+  p.beside_previous = dx != nullptr ? 1 : 0;
+  float* dwp = reinterpret_cast<float*>(ws + L.dwp);
+  const bool one = L.batches == 1;
+  rc = launch_dw_split(dy, lddy, xt, L.m_pitch, one ? dw : dwp, one ? N : L.batches * L.n_pad, one ? lddw : K, p, (int)L.batches, st);
+  if (rc != AQT_OK) return rc;
+  if (!one) {
+    rc = launch_sum_batches(dwp, L.batches, L.n_pad, N, K, dw, lddw, st);
+    if (rc != AQT_OK) return rc;
+  }
+  return dbias != nullptr ? launch_colsum_stage2(colsum, L.batches * DwCfg::kGroups, N, dbias, st) : AQT_OK;
+}
+
 int aqt_linear_bwd(const float* dy, int64_t lddy, const void* xq, const float* s_x, int s_x_kind, int bits_a, const void* wq,
                    const float* s_w, int bits_w, int64_t M, int64_t N, int64_t K, float* dx, int64_t lddx, float* dw, int64_t lddw,
                    float* dbias, void* workspace, size_t workspace_bytes, void* stream) {
@@ -764,15 +855,14 @@ int aqt_linear_bwd(const float* dy, int64_t lddy, const void* xq, const float* s
   if (dbias != nullptr && !is_aligned(dbias, 4)) return AQT_ERR_ALIGN;
   if ((dx != nullptr && !is_aligned(wq, 16)) || (dw != nullptr && !is_aligned(xq, 16))) return AQT_ERR_ALIGN;
   const BwdLayout L = bwd_layout(M, N, K);
-  if (workspace == nullptr || workspace_bytes < L.total) return AQT_ERR_WORKSPACE;
+  if (workspace == nullptr || workspace_bytes < bwd_workspace(M, N, K)) return AQT_ERR_WORKSPACE;
   if (!is_aligned(workspace, 256)) return AQT_ERR_ALIGN;
   int rc = check_device();
   if (rc != AQT_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
-  float* ones = reinterpret_cast<float*>(ws + L.ones);
-  rc = launch_fill_f32(ones, K, 1.0f, st);
-  if (rc != AQT_OK) return rc;
+  if (dw != nullptr && dw_split_applies(M, N, K))
+    return linear_bwd_split(dy, lddy, xq, s_x, s_x_kind, bits_a, wq, s_w, bits_w, M, N, K, dx, lddx, dw, lddw, dbias, ws, st);
   if (dbias != nullptr && dw == nullptr) {  // with dw the column sums come out of the transpose of dy
     rc = launch_colsum(dy, lddy, M, N, reinterpret_cast<float*>(ws + L.partial), dbias, st);
     if (rc != AQT_OK) return rc;
@@ -782,7 +872,7 @@ int aqt_linear_bwd(const float* dy, int64_t lddy, const void* xq, const float* s
     float* wt = reinterpret_cast<float*>(ws + L.wt);
     rc = launch_transpose_scale_codes(wq, is_packed(bits_w), s_w, true, N, K, wt, N, N, K, st);
     if (rc != AQT_OK) return rc;
-    rc = float_gemm_nt(dy, lddy, wt, M, K, N, ones, dx, lddx, st);
+    rc = float_gemm_nt(dy, lddy, wt, M, K, N, dx, lddx, st);
     if (rc != AQT_OK) return rc;
   }
   if (dw != nullptr) {
@@ -796,11 +886,11 @@ int aqt_linear_bwd(const float* dy, int64_t lddy, const void* xq, const float* s
     rc = launch_transpose_scale_codes(xq, is_packed(bits_a), s_x, s_x_kind == AQT_SCALE_ROW, M, K, xt, m_pad, L.chunk, K, st);
     if (rc != AQT_OK) return rc;
     if (L.batches == 1) {
-      rc = float_gemm_nt(dyt, L.chunk, xt, N, K, L.chunk, ones, dw, lddw, st);
+      rc = float_gemm_nt(dyt, L.chunk, xt, N, K, L.chunk, dw, lddw, st);
       if (rc != AQT_OK) return rc;
     } else {
       float* dwp = reinterpret_cast<float*>(ws + L.dwp);
-      rc = float_gemm_nt(dyt, L.chunk, xt, L.batches * L.n_pad, K, L.chunk, ones, dwp, K, st, L.batches);
+      rc = float_gemm_nt(dyt, L.chunk, xt, L.batches * L.n_pad, K, L.chunk, dwp, K, st, L.batches);
       if (rc != AQT_OK) return rc;
       rc = launch_sum_batches(dwp, L.batches, L.n_pad, N, K, dw, lddw, st);
       if (rc != AQT_OK) return rc;

@@ -75,6 +75,57 @@ __global__ void __launch_bounds__(256) transpose_scale_codes_kernel(const uint8_
   }
 }
 
+// Four weight or activation codes -> bf16 values of the same integers: at most eight significant bits, so the lower
+// halves of the binary32 values are zero.
+__device__ __forceinline__ uint2 codes4_to_bf16(uint32_t w) {
+  const float a = (float)(int8_t)(w & 0xFF), b = (float)(int8_t)((w >> 8) & 0xFF), c = (float)(int8_t)((w >> 16) & 0xFF), d = (float)(int8_t)(w >> 24);
+  return make_uint2(__byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632), __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x7632));
+}
+// codes [R, C] -> out[c * pitch + r] = bf16(code[r][c]) (exact): the transposed operand of the split-operand product.
+// A block turns 128 rows x 64 columns: a thread transposes 4 x 4 bytes in registers, the tile goes through
+// shared memory as [column][row] bytes, and leaves in 256-byte runs.
+__global__ void __launch_bounds__(256) transpose_codes_bf16_kernel(const uint8_t* __restrict__ codes, bool packed, int64_t R, int64_t C,
+                                                                   uint16_t* __restrict__ out, int64_t pitch) {
+  __shared__ uint32_t tile[64][kTrRows / 4 + 1];
+  grid_dependency_wait();
+  const int64_t r0 = (int64_t)blockIdx.y * kTrRows, c0 = (int64_t)blockIdx.x * 64;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int item = threadIdx.x + 256 * j, cw = item & 15, rg = item >> 4;  // four columns, four rows
+    const int64_t c = c0 + 4 * cw;
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t r = r0 + 4 * rg + i;
+      w[i] = 0u;
+      if (r < R && c < C) {  // C is a multiple of 4: a word is inside the row or outside it
+        if (packed) {
+          uint32_t hi;
+          unpack_word((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(codes + r * (C / 2) + (c >> 1))), w[i], hi);
+        } else {
+          w[i] = __ldg(reinterpret_cast<const uint32_t*>(codes + r * C + c));
+        }
+      }
+    }
+    const uint32_t a = __byte_perm(w[0], w[1], 0x5140), b = __byte_perm(w[2], w[3], 0x5140);  // r0c0 r1c0 r0c1 r1c1
+    const uint32_t d = __byte_perm(w[0], w[1], 0x7362), e = __byte_perm(w[2], w[3], 0x7362);
+    tile[4 * cw + 0][rg] = __byte_perm(a, b, 0x5410);
+    tile[4 * cw + 1][rg] = __byte_perm(a, b, 0x7632);
+    tile[4 * cw + 2][rg] = __byte_perm(d, e, 0x5410);
+    tile[4 * cw + 3][rg] = __byte_perm(d, e, 0x7632);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int i = (threadIdx.x >> 4) + 16 * j, seg = threadIdx.x & 15;  // column of the tile, eight rows
+    const int64_t c = c0 + i, r = r0 + 8 * seg;
+    if (c >= C || r >= R) continue;
+    const uint2 lo = codes4_to_bf16(tile[i][2 * seg]), hi = codes4_to_bf16(tile[i][2 * seg + 1]);
+    *reinterpret_cast<uint4*>(out + c * pitch + r) = make_uint4(lo.x, lo.y, hi.x, hi.y);  // rows beyond R: zeros inside the pitch
+  }
+  grid_dependents_launch();
+}
+
 // x [R, C] floats with row pitch ldx -> value(r, c) = x[r][c] in the layout above.  If colsum_partial
 // is not null, the block also writes the sums of its 128 rows of each of its columns, added top
 // to bottom, to colsum_partial[blockIdx.y * C + c] (the first stage of a fixed-order column sum).
@@ -168,11 +219,6 @@ __global__ void __launch_bounds__(256) colsum_stage2_kernel(const float* __restr
   }
 }
 
-__global__ void __launch_bounds__(256) fill_f32_kernel(float* __restrict__ p, int64_t n, float v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
-}
-
 // r_pad: rows of the input covered, zeros beyond R (batches * chunk, or the padded pitch for one chunk).
 static int launch_transpose_scale_codes(const void* codes, bool packed, const float* scale, bool per_row, int64_t R, int64_t C, float* out,
                                         int64_t r_pad, int64_t chunk, int64_t rows_out, cudaStream_t st) {
@@ -180,6 +226,11 @@ static int launch_transpose_scale_codes(const void* codes, bool packed, const fl
   transpose_scale_codes_kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const uint8_t*>(codes), packed, scale, per_row, R, C, out, r_pad,
                                                      chunk, rows_out);
   return AQT_LAUNCH_STATUS();
+}
+// pitch: a multiple of 8, at least R.
+static int launch_transpose_codes_bf16(const void* codes, bool packed, int64_t R, int64_t C, uint16_t* out, int64_t pitch, cudaStream_t st) {
+  return launch_pdl(transpose_codes_bf16_kernel, dim3((unsigned)ceil_div(C, 64), (unsigned)ceil_div(R, kTrRows), 1), dim3(256, 1, 1), 0, st, 1,
+                    reinterpret_cast<const uint8_t*>(codes), packed, R, C, out, pitch);
 }
 // colsum_partial / colsum_out: null, or the column sums of x are produced on the way
 // (colsum_partial holds transpose_row_blocks(r_pad) * C floats).
@@ -210,10 +261,6 @@ static int launch_colsum(const float* x, int64_t ldx, int64_t R, int64_t C, floa
 }
 static int launch_colsum_stage2(const float* partial, int64_t chunks, int64_t C, float* out, cudaStream_t st) {
   colsum_stage2_kernel<<<(unsigned)ceil_div(C, kTrTile), 256, 0, st>>>(partial, chunks, C, out);
-  return AQT_LAUNCH_STATUS();
-}
-static int launch_fill_f32(float* p, int64_t n, float v, cudaStream_t st) {
-  fill_f32_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(p, n, v);
   return AQT_LAUNCH_STATUS();
 }
 

@@ -85,7 +85,7 @@ struct GemmCfg {
 
 struct GemmParams {
   const float* s_x;
-  const float* s_w;
+  const float* s_w;  // null (float kind only): 1
   const float* bias;
   const float* residual;
   int32_t* acc_debug;
@@ -120,6 +120,9 @@ struct GemmParams {
   // The weights (codes, scales, bias) were complete before the kernel ahead of this one in the stream
   // was enqueued, so a kernel may read them before that kernel has finished (see grid_dependency_wait).
   int static_w = 0;
+  // Float kind: the next launch on the stream does not read what this one writes and may start on SMs that fall free (it
+  // sees to it that it does not end first, see DwParams::beside_previous).
+  int early_trigger = 0;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -412,8 +415,8 @@ __device__ __forceinline__ void swish32(float (&a)[32]) {
   }
 }
 
-__device__ __forceinline__ float4 ld4_guard(const float* base, int n, int limit) {
-  if (base == nullptr) return make_float4(0.f, 0.f, 0.f, 0.f);
+__device__ __forceinline__ float4 ld4_guard(const float* base, int n, int limit, float if_null) {
+  if (base == nullptr) return make_float4(if_null, if_null, if_null, if_null);
   if (n + 3 < limit) return __ldg(reinterpret_cast<const float4*>(base + n));
   float4 r;
   r.x = n + 0 < limit ? __ldg(base + n + 0) : 0.f;
@@ -429,8 +432,8 @@ __device__ __forceinline__ void dequant32_gmem(const uint32_t (&acc)[32], float 
                                                int limit, float (&z)[32]) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const float4 w = ld4_guard(s_w, n0 + 4 * j, limit);
-    const float4 b = ld4_guard(bias, n0 + 4 * j, limit);
+    const float4 w = ld4_guard(s_w, n0 + 4 * j, limit, 1.0f);
+    const float4 b = ld4_guard(bias, n0 + 4 * j, limit, 0.0f);
     z[4 * j + 0] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 0]), sx), w.x, b.x);
     z[4 * j + 1] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 1]), sx), w.y, b.y);
     z[4 * j + 2] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 2]), sx), w.z, b.z);
@@ -544,6 +547,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
   }
   // everything above touched only this CTA's own state; from here on global memory is read
   grid_dependency_wait();
+  if (TF32 && p.early_trigger) grid_dependents_launch();
   // RQ: tag of this execution's exchange words (the call's tag mixed with the group's generation
   // counter, which the group's first CTA bumps when it has finished: a replayed graph repeats the call's tag)
   const int rq_group = RQ ? (int)(blockIdx.x >> 1) / p.tiles_n : 0;
@@ -562,7 +566,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
       }
       float wv = 0.0f, bv = 0.0f;
       if (n < limit) {
-        wv = __ldg(p.s_w + n);
+        wv = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + n);
         if (p.bias != nullptr) bv = __ldg(p.bias + n);
       }
       asm volatile("st.shared.f32 [%0], %1;" ::"r"(smem_scale + t * 4), "f"(wv) : "memory");
@@ -759,7 +763,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           const uint32_t off = c * slab_chunk_stride + lane * 4;
           float wv = 0.0f, bv = 0.0f;
           if (nv < n_value_limit) {
-            wv = __ldg(p.s_w + nv);
+            wv = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + nv);
             if (p.bias != nullptr) bv = __ldg(p.bias + nv);
           }
           asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + off), "f"(wv) : "memory");
@@ -768,7 +772,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             const int ng = p.N / 2 + out0 + col + lane;  // gate channel
             float wg = 0.0f, bg = 0.0f;
             if (ng < p.N) {
-              wg = __ldg(p.s_w + ng);
+              wg = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + ng);
               if (p.bias != nullptr) bg = __ldg(p.bias + ng);
             }
             asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + off + slab_gate_off), "f"(wg) : "memory");
@@ -1057,7 +1061,7 @@ static EncodeTiledFn get_encode_tiled() {
 }
 
 // 2-D row-major tensor [rows, cols] with `pitch_bytes` between rows; box [box_rows, box_cols];
-// swizzle_bytes: 128 or 32 (box_cols * element size must then be that many bytes), or 0 for none.
+// swizzle_bytes: 128, 64 or 32 (box_cols * element size must then be that many bytes), or 0 for none.
 static int make_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* base, uint64_t rows, uint64_t cols,
                        uint64_t pitch_bytes, uint32_t box_rows, uint32_t box_cols, int swizzle_bytes = 128) {
   EncodeTiledFn enc = get_encode_tiled();
@@ -1070,7 +1074,7 @@ static int make_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* bas
   cuuint32_t box[2] = {box_cols, box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, dt, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   swizzle_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (swizzle_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE),
+                   swizzle_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : swizzle_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE),
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS && debug_enabled())
@@ -1252,6 +1256,13 @@ static int plan_qgemm(const GemmShape& g, int sms) {
   const bool two_rounds_of_pairs = (!glu || f32) && ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256) >= 2 * pairs;
   // (float kind, measured: pairs win 6-10 % at M >= 25 600, lose 10 % at 12 800 x 2048 x 512)
   bool pairs_ok = f32 ? (two_rounds_of_pairs && g.M >= 2 * kBM * pairs) : (deep_k || (g.K >= 2048 && two_rounds_of_pairs));
+  // Float kind, up to three rounds of pair tiles: a pair moves 32 KB per k-block and CTA where a single CTA's tile moves
+  // 48 KB (measured: 22.4 vs 31.4 us at 4096 x 512 -> 2048 Swish, 25.8 vs 33.5 us at 9000 x 768 -> 768, 26.2 vs 31.8 us at
+  // 4096 x 2048 -> 512; below 32 tiles too few SMs are left with work, 11.9 vs 10.4 us at 2048 x 512 -> 512, and with more
+  // rounds the single-CTA tiles win again, 152 vs 209 us at 12 800 x 2048 -> 2048).
+  const int64_t pair_tiles = ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256);
+  const bool few_pair_rounds = f32 && pair_tiles >= 32 && pair_tiles <= 3 * pairs;
+  pairs_ok = pairs_ok || few_pair_rounds;
   if (tuning_env("AQT_NO_PAIRS") != nullptr) pairs_ok = false;
   if (tuning_env("AQT_FORCE_PAIRS") != nullptr) pairs_ok = true;
   if (!g.batched && g.M > kBM) {
@@ -1275,7 +1286,8 @@ static int plan_qgemm(const GemmShape& g, int sms) {
     // 65 536 x 1024 x 4096: 2753 vs 2671 TOPS burst, equal sustained; float kind 801 vs 752
     // TFLOP/s); at K = 2048 the eight-warp epilogue with four stages is 20-27 % faster (41.1 vs
     // 52.3 us at 37 888 x 512 x 2048, where the deep-K rule first applies; 83.1 vs 104.9 us at 65 536).
-    bool dp = deep_k && g.K >= 4096;
+    bool dp = deep_k && g.K >= 4096 && !few_pair_rounds;  // (float kind, few rounds: 60.0 vs 63.7 us at 12 800 x 2048 -> 512)
+    if (few_pair_rounds) bn2 = 256;
     if (const char* e = tuning_env("AQT_DEEP_PAIRS")) dp = atoi(e) != 0;
     if (bn2 == 256) return dp ? kPlanPair256S6E4 : kPlanPair256S4E8;
     return dp ? kPlanPair128S8E4 : kPlanPair128S6E8;

@@ -82,6 +82,35 @@ def test_backward_per_tensor_scale_padded_gradient_and_partial_outputs():
     assert np.all(np.abs(dw.cpu().numpy() - ref[1]) <= 2.0 ** -8 * ref[4] + 1e-30)
 
 
+@pytest.mark.parametrize("M,N,K,bits_a,bits_w,kind,pad", [
+    (255, 128, 128, 8, 8, aqt.SCALE_ROW, 0), (256, 128, 128, 8, 4, aqt.SCALE_ROW, 0), (256 + 31, 132, 388, 4, 4, aqt.SCALE_ROW, 4),
+    (1025, 516, 260, 8, 8, aqt.SCALE_TENSOR, 0), (5001, 260, 132, 8, 4, aqt.SCALE_ROW, 12), (2000, 384, 1028, 4, 8, aqt.SCALE_ROW, 0)])
+def test_backward_weight_gradient_on_split_operands(M, N, K, bits_a, bits_w, kind, pad):
+    """The weight gradient from 256 rows on (and one row below): contractions with a remainder of 32, one and several
+    batches of them, ragged tiles in both directions, a padded gradient, every code width.  The bound is the tf32
+    one; the split operands themselves are within 2^-16 of a term (two bf16 terms of a binary32 value), so the error of
+    dw also stays below (2^-15 + 2^-23 + M 2^-24) of the terms' magnitude."""
+    ex, ew = _check(M, N, K, bits_a, bits_w, seed=M, kind=kind, lddy=N + pad if pad else None)
+    if M >= 256:
+        tight = (2.0 ** -15 + 2.0 ** -23 + M * 2.0 ** -24) / (2.0 ** -9 + 2.0 ** -23 + M * 2.0 ** -24)
+        assert ew.max() <= tight
+
+
+@pytest.mark.parametrize("M", [300, 20000])
+def test_backward_partial_outputs_on_split_operands(M):
+    """Without dx, without dbias: the bits of the outputs do not depend on which others are asked for (nor on the
+    two products running side by side)."""
+    xq, wq, s_x, s_w, dy = _case(8, M, 384, 256, 8, 8)
+    a = [_dev(v) for v in (dy, xq, s_x, wq, s_w)]
+    dx, dw, db = aqt.aqt_linear_bwd(*a, K=256)
+    _, dw2, db2 = aqt.aqt_linear_bwd(*a, K=256, want_dx=False)
+    dx3, dw3, none = aqt.aqt_linear_bwd(*a, K=256, want_dbias=False)
+    dx4, none2, _ = aqt.aqt_linear_bwd(*a, K=256, want_dw=False)
+    assert aqt.aqt_device_status() == 0 and none is None and none2 is None
+    for g, h in ((dw, dw2), (db, db2), (dx, dx3), (dw, dw3), (dx, dx4)):
+        assert torch.equal(g.view(torch.int32), h.view(torch.int32))
+
+
 def test_backward_error_is_of_tf32_size():
     ex, ew = _check(512, 1024, 512, 8, 8, seed=4)
     assert np.median(ex) > 2.0 ** -14 and np.median(ew) > 2.0 ** -14   # the bound is not slack by orders of magnitude
