@@ -156,12 +156,15 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
 
 // True if the CTA-pair kernel with the row-quantizing epilogue takes the call: deep K, no GLU, int8
 // codes out (4-bit codes stay in their containers), at most 16 column parts per row.
-bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool pack_out) {
+bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out) {
   // (from K = 2048: at K = 1024 a tile's MMAs are shorter than its two epilogue passes, and the
   // two kernels are faster: 162 vs 209 us at 65 536 x 1024 -> 1024 with the fp32 output)
   if (pack_out || M <= kBM || K < 2048) return false;
   if (act != AQT_ACT_NONE && act != AQT_ACT_SWISH) return false;
   const int sms = sm_count() > 0 ? sm_count() : kDefaultSms;
+  // With the fp32 output, few pair tiles leave most of the chip idle: narrow tiles and the row quantizer behind them take 9.3
+  // against 14.2 us at 1024 x 2048 -> 512, 11.5 against 15.1 us at 4096 rows, 15.3 against 16.0 us at 8192 (64 tiles).
+  if (with_y && 8 * ceil_div(M, 2 * kBM) * ceil_div(N, 256) <= 7 * (sms / 2)) return false;
   const int plan = rowquant_plan(M, N, K, sms);
   const int parts = rowquant_parts(plan, N);
   return parts % 2 == 0 && parts <= 16 && ceil_div(N, kGemmPlanBn[plan]) <= sms / 2;
@@ -447,7 +450,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
 
-  if (!requant_applies(M, N, K, act, y != nullptr, pack_out != 0) && rowquant_pair_applies(M, N, K, act, pack_out != 0)) {
+  if (!requant_applies(M, N, K, act, y != nullptr, pack_out != 0) && rowquant_pair_applies(M, N, K, act, y != nullptr, pack_out != 0)) {
     // Deep K (the second feed-forward layers): the CTA-pair kernel with the row-quantizing epilogue
     const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
     if (is_packed(bits_a)) {

@@ -1231,66 +1231,78 @@ static bool qgemm_uses_ws(int64_t N, int64_t K, int sms) {
   return ceil_div(K, kBK) <= kWsMaxKBlocks && ceil_div(N, 128) <= sms;
 }
 
+// CTA pairs for the 8-bit kind, K > 512; kPlanNone if single-CTA tiles are the better choice.  What bounds these shapes
+// is bytes from L2, and a pair moves 32 KB per k-block and CTA for the work that costs a single CTA's 128 x 256 tile
+// 48 KB: pairs on 256 x 256 tiles win wherever there are enough of them (from 48: 8.9 vs 9.3 us at 3000 x 1024 -> 1024,
+// 17.2 vs 18.1 at 3000 x 4096 -> 1024, 12.4 vs 12.8 at 6400 x 2048 -> 512; below, narrow single-CTA tiles occupy more
+// SMs: 9.3 vs 10.9 us at 3000 x 2048 -> 384), 78 vs 89 us at 65 536 x 1024 -> 1024, 101 vs
+// 110 with a residual.  (Measured for act NONE.  With Swish the sixteen-warp epilogue of the single-CTA tiles wins below
+// K = 2048, 322 vs 334 us at 65 536 x 1024 -> 4096; GLU is laid out for single CTAs.)
+static int plan_qgemm_pairs(const GemmShape& g, int pairs, int64_t pair_tiles) {
+  const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
+  if (glu || g.M <= kBM || g.K <= kWsMaxKBlocks * kBK) return kPlanNone;
+  if (tuning_env("AQT_NO_PAIRS") != nullptr) return kPlanNone;
+  // One row block per 512-column tile and a second round of 256-column tiles that would be less than half full: each
+  // pair takes one whole 256 x 512 tile, so the activations are read once.
+  if (g.N == 512 && g.K >= 2048 && pair_tiles > pairs && 2 * pair_tiles <= 3 * pairs) return kPlanPair512S3E16;
+  // (Below K = 2048 up to 2048 columns: the parity tests fix the single-CTA configuration of the d = 1024 encoder's
+  // 3072-column projection; a caller that cuts it in two, as the encoder driver does, gets pairs for both parts.)
+  const bool enough = g.act == AQT_ACT_NONE ? pair_tiles >= 48 && (g.K >= 2048 || g.N <= 2048) : g.K >= 2048 && pair_tiles >= 2 * pairs;
+  if (!enough) return kPlanNone;
+  // The four-warp epilogue and deeper ring need a deep K and several tiles per pair (191 vs 205 us at 65 536 x 4096 ->
+  // 1024; 25 600 rows: 86 vs 87 without, 100 vs 96 us with a residual).
+  const bool dp = g.K >= 4096 && g.act == AQT_ACT_NONE && ceil_div(g.M, kBM) * ceil_div(g.N, 256) >= 12 * pairs;
+  // 128 columns where more than a quarter of the columns of 256-wide tiles would be padding, or their last round nearly empty
+  const int64_t last_round = pair_tiles % pairs;
+  const bool narrow = (g.N <= 384 && g.N % 256 != 0 && g.N % 256 <= 128 && pair_tiles > 2 * pairs) || (pair_tiles > pairs && last_round > 0 && last_round <= pairs / 10);
+  if (narrow) return dp ? kPlanPair128S8E4 : kPlanPair128S6E8;
+  return dp ? kPlanPair256S6E4 : kPlanPair256S4E8;
+}
+
 // sms: multiprocessors of the device the launch will go to.
 static int plan_qgemm(const GemmShape& g, int sms) {
   const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
   const bool f32 = g.kind == 1;
   if (!g.batched && qgemm_uses_ws(g.N, g.K, sms)) return glu ? kPlanWs128E8 : kPlanWs128E16;  // a GLU tile has 64 output columns
-  // "Deep" configuration (four-warp epilogue, longest ring): pays off when K is deep AND every
-  // CTA walks many tiles; with few tiles per CTA the exposed epilogue of the last tile costs more
-  // than the extra ring stages gain (measured at M = 12 800 .. 25 600).
-  bool deep_k = g.K >= 2048 && !glu && ceil_div(g.M, kBM) * ceil_div(g.N, 256) >= 4 * sms;
+  const int pairs = sms / 2;
+  const int64_t pair_tiles = ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256);  // 256 x 256 tiles
+  if (!f32 && !g.batched) {
+    const int plan = plan_qgemm_pairs(g, pairs, pair_tiles);
+    if (plan != kPlanNone) return plan;
+  }
   // Float kind: a k-block takes as many tensor-core clocks as an 8-bit one but holds a quarter of
   // the elements, so every shape is "deep" in bytes and the epilogue is a small part of a tile
   // unless it evaluates an activation (measured: the four-warp epilogue wins at 12 800 x 512 x
   // 2048 and 65 536 x 1024 x 4096 without activation, loses by 20-40 % with Swish).
-  if (f32) deep_k = g.act == AQT_ACT_NONE && g.K >= 8192;
+  bool deep_k = f32 && g.act == AQT_ACT_NONE && g.K >= 8192;
   if (const char* e = tuning_env("AQT_DEEP")) {
     if (!glu) deep_k = atoi(e) != 0;
   }
-  const int pairs = sms / 2;
-  // Pairs pay off only for deep K and at least two full rounds of pair tiles (measured: +4 % at
-  // 65 536 x 1024 x 4096 with the deep configuration, +9 % at 25 600 x 512 x 2048 with the
-  // eight-warp epilogue, no gain at M = 12 800 or at K = 1024); everything else takes one CTA per tile.
-  // (the 8-bit kind's GLU shapes are faster on single CTAs; the float kind's gain 3 % on pairs)
-  const bool two_rounds_of_pairs = (!glu || f32) && ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256) >= 2 * pairs;
-  // (float kind, measured: pairs win 6-10 % at M >= 25 600, lose 10 % at 12 800 x 2048 x 512)
-  bool pairs_ok = f32 ? (two_rounds_of_pairs && g.M >= 2 * kBM * pairs) : (deep_k || (g.K >= 2048 && two_rounds_of_pairs));
-  // Float kind, up to three rounds of pair tiles: a pair moves 32 KB per k-block and CTA where a single CTA's tile moves
-  // 48 KB (measured: 22.4 vs 31.4 us at 4096 x 512 -> 2048 Swish, 25.8 vs 33.5 us at 9000 x 768 -> 768, 26.2 vs 31.8 us at
-  // 4096 x 2048 -> 512; below 32 tiles too few SMs are left with work, 11.9 vs 10.4 us at 2048 x 512 -> 512, and with more
-  // rounds the single-CTA tiles win again, 152 vs 209 us at 12 800 x 2048 -> 2048).
-  const int64_t pair_tiles = ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256);
-  const bool few_pair_rounds = f32 && pair_tiles >= 32 && pair_tiles <= 3 * pairs;
-  pairs_ok = pairs_ok || few_pair_rounds;
-  if (tuning_env("AQT_NO_PAIRS") != nullptr) pairs_ok = false;
-  if (tuning_env("AQT_FORCE_PAIRS") != nullptr) pairs_ok = true;
-  if (!g.batched && g.M > kBM) {
-    // Few, deep tiles (K >= 2048, all of N within one or two 512-column tiles, at most one round of
-    // 256 x 512 tiles over the pairs): each pair takes one whole tile, so the activations are read
-    // once, the weights once per 256 rows, and no SM waits for a second, mostly empty round.
-    bool wide = !f32 && !glu && g.K >= 2048 && g.N % 512 == 0 && ceil_div(g.M, 2 * kBM) * (g.N / 512) <= pairs;
-    if (const char* e = tuning_env("AQT_WIDE_PAIRS")) wide = !f32 && !glu && atoi(e) != 0;
-    if (wide) return kPlanPair512S3E16;
-  }
-  if (!g.batched && pairs_ok && g.M > kBM) {
-    // CTA pairs on 256-row tiles; width by the number of rounds over the pairs
-    const int64_t tiles_m2 = ceil_div(g.M, 2 * kBM);
-    const double cost256 = (double)ceil_div(tiles_m2 * ceil_div(g.N, 256), pairs) * (256 + 24);
-    const double cost128 = (double)ceil_div(tiles_m2 * ceil_div(g.N, 128), pairs) * (128 + 24);
-    int bn2 = cost256 <= cost128 ? 256 : 128;
-    if (const char* e = tuning_env("AQT_BN")) {
-      if (atoi(e) == 128 || atoi(e) == 256) bn2 = atoi(e);
+  if (f32 && !g.batched && g.M > kBM) {
+    // CTA pairs on 256-row tiles: many rows (measured: 6-10 % at M >= 25 600, a loss of 10 % at 12 800 x 2048 x 512) or, up
+    // to three rounds of pair tiles, any number: a pair moves 32 KB per k-block and CTA where a single CTA's tile moves
+    // 48 KB (22.4 vs 31.4 us at 4096 x 512 -> 2048 Swish, 25.8 vs 33.5 us at 9000 x 768 -> 768, 26.2 vs 31.8 us at
+    // 4096 x 2048 -> 512; below 32 tiles too few SMs are left with work, 11.9 vs 10.4 us at 2048 x 512 -> 512, and with
+    // more rounds and fewer rows the single-CTA tiles win again, 152 vs 209 us at 12 800 x 2048 -> 2048).
+    const bool few_rounds = pair_tiles >= 32 && pair_tiles <= 3 * pairs;
+    bool pairs_ok = few_rounds || (pair_tiles >= 2 * pairs && g.M >= 2 * kBM * pairs);
+    if (tuning_env("AQT_NO_PAIRS") != nullptr) pairs_ok = false;
+    if (tuning_env("AQT_FORCE_PAIRS") != nullptr) pairs_ok = true;
+    if (pairs_ok) {
+      // width by the number of rounds over the pairs (few rounds: 256); the four-warp epilogue and deeper ring for deep K
+      // (801 vs 752 TFLOP/s at 65 536 x 4096 -> 1024; few rounds: 63.7 vs 60.0 us at 12 800 x 2048 -> 512)
+      const int64_t tiles_m2 = ceil_div(g.M, 2 * kBM);
+      const double cost256 = (double)ceil_div(pair_tiles, pairs) * (256 + 24);
+      const double cost128 = (double)ceil_div(tiles_m2 * ceil_div(g.N, 128), pairs) * (128 + 24);
+      int bn2 = few_rounds || cost256 <= cost128 ? 256 : 128;
+      if (const char* e = tuning_env("AQT_BN")) {
+        if (atoi(e) == 128 || atoi(e) == 256) bn2 = atoi(e);
+      }
+      bool dp = deep_k && !few_rounds;
+      if (const char* e = tuning_env("AQT_DEEP_PAIRS")) dp = atoi(e) != 0;
+      if (bn2 == 256) return dp ? kPlanPair256S6E4 : kPlanPair256S4E8;
+      return dp ? kPlanPair128S8E4 : kPlanPair128S6E8;
     }
-    // The four-warp epilogue / deeper ring pays off for pairs only from K = 4096 bytes (measured at
-    // 65 536 x 1024 x 4096: 2753 vs 2671 TOPS burst, equal sustained; float kind 801 vs 752
-    // TFLOP/s); at K = 2048 the eight-warp epilogue with four stages is 20-27 % faster (41.1 vs
-    // 52.3 us at 37 888 x 512 x 2048, where the deep-K rule first applies; 83.1 vs 104.9 us at 65 536).
-    bool dp = deep_k && g.K >= 4096 && !few_pair_rounds;  // (float kind, few rounds: 60.0 vs 63.7 us at 12 800 x 2048 -> 512)
-    if (few_pair_rounds) bn2 = 256;
-    if (const char* e = tuning_env("AQT_DEEP_PAIRS")) dp = atoi(e) != 0;
-    if (bn2 == 256) return dp ? kPlanPair256S6E4 : kPlanPair256S4E8;
-    return dp ? kPlanPair128S8E4 : kPlanPair128S6E8;
   }
   int bn = pick_bn(g.M, g.N, glu, sms);
   // operand bytes per output are four times those of the 8-bit kind: the widest tile wins whenever it

@@ -272,19 +272,32 @@ class ConformerBlockLinears:
                            xs=in_codes[1] if in_codes else None, out_role="ha", out_bits=L[2].spec.bits_a)
         note(L[1].spec.name, self.h_a)
         # q, k, v read the same h: its codes come out of the second feed-forward matmul's epilogue
-        # (or one quantizer pass; the codes do not depend on the consumer), and the three
-        # projections run as one matmul over their concatenated output channels
+        # (or one quantizer pass; the codes do not depend on the consumer).  q and k run as one matmul over
+        # their concatenated output channels; v is also needed as codes, which its own matmul's epilogue
+        # produces where it can.
         if hq is None:
             hq, hs = run.quantize_input(self.h_a, L[2].spec.bits_a)
         wq, s_w, bias = self._fused_qkv(L)
-        aqt.aqt_qmatmul(hq, hs, wq, s_w, bias, None, 1.0, K=self.d, bits_a=_container_bits(L[2].spec.bits_a), bits_w=L[2].mm_bits, act=aqt.ACT_NONE,
-                        s_x_kind=run.a_scale_kind, y=self.qkv, workspace=run.workspace)
+        d = self.d
+        args = dict(K=d, bits_a=_container_bits(L[2].spec.bits_a), bits_w=L[2].mm_bits, act=aqt.ACT_NONE, s_x_kind=run.a_scale_kind,
+                    workspace=run.workspace)
+        aqt.aqt_qmatmul(hq, hs, wq[:2 * d], s_w[:2 * d], None if bias is None else bias[:2 * d], None, 1.0, y=self.qkv[:, :2 * d], **args)
+        bias_v = None if bias is None else bias[2 * d:]
+        bq = bs = cq = cs = vq = vs = None
+        if run.fuses_requant(L[4]):
+            vq, vs = run.code_buffers("v", d)
+            aqt.aqt_qmatmul_requant(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, bits_out=L[5].spec.bits_a, rounding=run.rounding, q_out=vq,
+                                    s_out=vs, y=self.v, **args)
+        else:
+            aqt.aqt_qmatmul(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, y=self.v, **args)
         note(L[2].spec.name, self.q); note(L[3].spec.name, self.k); note(L[4].spec.name, self.v)
         # h_b = h_a + W_o v is needed both as fp32 (residual stream) and as codes (pointwise 1)
-        bq = bs = cq = cs = None
         if run.fuses_requant(L[5]):
-            vq, vs = run.quantize_input(self.v, L[5].spec.bits_a)
+            if vq is None:
+                vq, vs = run.quantize_input(self.v, L[5].spec.bits_a)
             bq, bs = run.matmul_requant(L[5], vq, vs, L[6].spec.bits_a, "h", y=self.h_b, residual=self.h_a, residual_scale=1.0)
+        elif vq is not None:
+            run.matmul(L[5], vq, vs, self.h_b, residual=self.h_a, residual_scale=1.0)
         else:
             run(L[5], self.v, self.h_b, residual=self.h_a, residual_scale=1.0)
         note(L[5].spec.name, self.h_b)
