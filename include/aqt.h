@@ -221,7 +221,8 @@ int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w
  *           256, plus 4*M*K rounded up to 256 if x_on_host, plus 4*M*N_out if y_on_host: the
  *           device copies of x and y are placed behind the layer's own scratch, in that order.
  * The call enqueues the host-to-device copy, the layer and the device-to-host copy on `stream`
- * and returns without synchronising.  Chaining two calls (host -> device, device -> host) runs a
+ * and returns without synchronising.  With per-row scales and 2 MB or more of pinned memory the rows go
+ * through in up to six pieces, whose copies overlap on two side streams forked from and joined to `stream`.  Chaining two calls (host -> device, device -> host) runs a
  * two-layer block with only its input and output crossing the bus.
  */
 int aqt_linear_fwd_host(const float* x, int x_on_host, const void* wq, const float* s_w, const float* bias,
@@ -234,7 +235,8 @@ int aqt_linear_fwd_host(const float* x, int x_on_host, const void* wq, const flo
  * de-quantization): aqt_quantize(x) -> aqt_qmatmul_requant (the hidden tensor u = act(W1 . x)
  * leaves the first matmul as codes and row scales and is never written as fp32) -> aqt_qmatmul.
  * x, y      fp32 [M, d] dense; host pointers if x_on_host / y_on_host != 0 (pinned memory makes
- *           the copies asynchronous), else device pointers.  The copies are enqueued on `stream`.
+ *           the copies asynchronous), else device pointers.  The copies are enqueued on `stream`, large ones
+ *           in pieces as in aqt_linear_fwd_host; kernels may read and write small pinned buffers in place.
  * w1q       W1^T codes [ff, d], s_w1 [ff], bias1 [ff] or NULL, bits_w1 as for aqt_qmatmul.
  * w2q       W2^T codes [d, ff], s_w2 [d], bias2 [d] or NULL, bits_w2.
  * bits_a    4 or 8: width both layers' activations are quantized to (per-row dynamic scales).

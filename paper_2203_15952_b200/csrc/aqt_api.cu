@@ -9,6 +9,7 @@
 #include "qgemv_small_m.cuh"
 #include "quantize.cuh"
 #include "chain_small_m.cuh"
+#include "host_copies.cuh"
 
 using namespace aqt;
 
@@ -601,19 +602,15 @@ int aqt_linear_fwd_host(const float* x, int x_on_host, const void* wq, const flo
   if (!is_aligned(workspace, 256)) return AQT_ERR_ALIGN;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
-  const float* x_dev = x;
-  float* y_dev = y;
-  if (x_on_host) {
-    float* xd = reinterpret_cast<float*>(ws + layer);
-    AQT_RETURN_IF_CUDA(cudaMemcpyAsync(xd, x, (size_t)M * K * 4, cudaMemcpyHostToDevice, st));
-    x_dev = xd;
-  }
-  if (y_on_host) y_dev = reinterpret_cast<float*>(ws + layer + xb);
-  rc = aqt_linear_fwd(x_dev, K, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, bits_a, bits_w, a_scale_kind, rounding, act, y_dev,
-                      n_out, ws, layer, stream);
-  if (rc != AQT_OK) return rc;
-  if (y_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(y, y_dev, (size_t)M * n_out * 4, cudaMemcpyDeviceToHost, st));
-  return AQT_OK;
+  float* x_copy = reinterpret_cast<float*>(ws + layer);
+  const float* x_dev = x_on_host ? x_copy : x;
+  float* y_dev = y_on_host ? reinterpret_cast<float*>(ws + layer + xb) : y;
+  // (one scale for the whole tensor needs every row before the first product)
+  return run_between_host_copies(x_on_host ? x : nullptr, x_copy, (size_t)K * 4, y_dev, y_on_host ? y : nullptr, (size_t)n_out * 4, M, st,
+                                 a_scale_kind == AQT_SCALE_ROW, [&](int64_t r0, int64_t rows) {
+                                   return aqt_linear_fwd(x_dev + r0 * K, K, wq, s_w, bias, nullptr, 0, 0.0f, rows, N, K, bits_a, bits_w,
+                                                         a_scale_kind, rounding, act, y_dev + r0 * n_out, n_out, ws, layer, stream);
+                                 });
 }
 
 int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer* layers, int n_layers, int rounding, void* stream) {
@@ -693,40 +690,50 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
   if (!requant_applies(M, ff, d, act, false, false)) return AQT_ERR_UNSUPPORTED;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
-  const float* x_dev = x;
-  float* y_dev = y;
-  if (x_on_host) {
-    AQT_RETURN_IF_CUDA(cudaMemcpyAsync(ws + L.x, x, (size_t)M * d * 4, cudaMemcpyHostToDevice, st));
-    x_dev = reinterpret_cast<const float*>(ws + L.x);
+  float* x_copy = reinterpret_cast<float*>(ws + L.x);
+  float* y_dev = y_on_host ? reinterpret_cast<float*>(ws + L.y) : y;
+  const bool chain = M <= AQT_CHAIN_MAX_ROWS;
+  if (x_on_host && (size_t)M * d * 4 < (chain ? kReadInPlaceBytesChain : kReadInPlaceBytes) && is_aligned(x, 16)) {
+    if (const void* mapped = pinned_on_device(x)) {
+      x = reinterpret_cast<const float*>(mapped);
+      x_on_host = 0;
+    }
   }
-  if (y_on_host) y_dev = reinterpret_cast<float*>(ws + L.y);
-  int8_t* q1 = reinterpret_cast<int8_t*>(ws + L.q1);
-  float* s1 = reinterpret_cast<float*>(ws + L.s1);
-  int8_t* q2 = reinterpret_cast<int8_t*>(ws + L.q2);
-  float* s2 = reinterpret_cast<float*>(ws + L.s2);
-  if (M <= AQT_CHAIN_MAX_ROWS) {
-    // a few rows: both layers in one launch
+  const float* x_dev = x_on_host ? x_copy : x;
+  if (chain) {
+    // a few rows: both layers in one launch, which writes the result over the bus itself (us a call, copied or not, d =
+    // 512: 16 rows 24 / 23, 64 rows 36 / 26)
+    float* y_out = y_on_host && is_aligned(y, 16) ? reinterpret_cast<float*>(pinned_on_device(y)) : nullptr;
+    const bool y_copied = y_on_host && y_out == nullptr;
+    if (y_out == nullptr) y_out = y_dev;
+    if (x_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(x_copy, x, (size_t)M * d * 4, cudaMemcpyHostToDevice, st));
     const aqt_chain_layer pair[2] = {
         {w1q, s_w1, bias1, nullptr, 0, (int32_t)ff, (int32_t)d, bits_w1, bits_a, act, 0, 0.0f, 0},
-        {w2q, s_w2, bias2, y_dev, d, (int32_t)d, (int32_t)ff, bits_w2, bits_a, AQT_ACT_NONE, 0, 0.0f, 0}};
+        {w2q, s_w2, bias2, y_out, d, (int32_t)d, (int32_t)ff, bits_w2, bits_a, AQT_ACT_NONE, 0, 0.0f, 0}};
     rc = aqt_chain_fwd(x_dev, d, M, pair, 2, rounding, stream);
-    if (rc == AQT_OK && y_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(y, y_dev, (size_t)M * d * 4, cudaMemcpyDeviceToHost, st));
+    if (rc == AQT_OK && y_copied) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(y, y_dev, (size_t)M * d * 4, cudaMemcpyDeviceToHost, st));
     if (rc != AQT_ERR_UNSUPPORTED && rc != AQT_ERR_ALIGN) return rc;
   }
   const size_t mm_bytes = L.total - L.mm;
-  // Fig. 2 on the input rows; first matmul with the rows of u = act(W1 x) quantized in its epilogue
-  // (4-bit codes stay in int8 containers between the kernels); second matmul.
-  rc = aqt_quantize(x_dev, M, d, d, bits_a, AQT_AXIS_ROW, rounding, 0, q1, s1, stream);
-  if (rc != AQT_OK) return rc;
   const int bits_mm = bits_a == 8 ? 8 : AQT_BITS_4_UNPACKED;
-  rc = aqt_qmatmul_requant(q1, s1, AQT_SCALE_ROW, w1q, s_w1, bias1, nullptr, 0, 0.0f, M, ff, d, bits_mm, bits_w1 | static_flag, act, bits_a, rounding, 0,
-                           q2, s2, nullptr, 0, ws + L.mm, mm_bytes, stream);
-  if (rc != AQT_OK) return rc;
-  rc = aqt_qmatmul(q2, s2, AQT_SCALE_ROW, w2q, s_w2, bias2, nullptr, 0, 0.0f, M, d, ff, bits_mm, bits_w2, AQT_ACT_NONE, y_dev, d, nullptr,
-                   ws + L.mm, mm_bytes, stream);
-  if (rc != AQT_OK) return rc;
-  if (y_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(y, y_dev, (size_t)M * d * 4, cudaMemcpyDeviceToHost, st));
-  return AQT_OK;
+  return run_between_host_copies(x_on_host ? x : nullptr, x_copy, (size_t)d * 4, y_dev, y_on_host ? y : nullptr, (size_t)d * 4, M, st, true,
+                                 [&](int64_t r0, int64_t rows) {
+    const float* xr = x_dev + r0 * d;
+    float* yr = y_dev + r0 * d;
+    // Fig. 2 on the input rows; first matmul with the rows of u = act(W1 x) quantized in its epilogue
+    // (4-bit codes stay in int8 containers between the kernels); second matmul.
+    int8_t* q1 = reinterpret_cast<int8_t*>(ws + L.q1) + r0 * d;
+    float* s1 = reinterpret_cast<float*>(ws + L.s1) + r0;
+    int8_t* q2 = reinterpret_cast<int8_t*>(ws + L.q2) + r0 * ff;
+    float* s2 = reinterpret_cast<float*>(ws + L.s2) + r0;
+    int rc = aqt_quantize(xr, rows, d, d, bits_a, AQT_AXIS_ROW, rounding, 0, q1, s1, stream);
+    if (rc != AQT_OK) return rc;
+    rc = aqt_qmatmul_requant(q1, s1, AQT_SCALE_ROW, w1q, s_w1, bias1, nullptr, 0, 0.0f, rows, ff, d, bits_mm, bits_w1 | static_flag, act, bits_a,
+                             rounding, 0, q2, s2, nullptr, 0, ws + L.mm, mm_bytes, stream);
+    if (rc != AQT_OK) return rc;
+    return aqt_qmatmul(q2, s2, AQT_SCALE_ROW, w2q, s_w2, bias2, nullptr, 0, 0.0f, rows, d, ff, bits_mm, bits_w2, AQT_ACT_NONE, yr, d, nullptr,
+                       ws + L.mm, mm_bytes, stream);
+  });
 }
 
 int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, const float* s_w, const float* bias,
