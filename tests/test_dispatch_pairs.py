@@ -9,12 +9,12 @@ from paper_2203_15952_b200 import inputs as gen
     (23 * 256, 512, 2048, gen.ACT_NONE, "stream64s5e8"), (23 * 256 + 1, 512, 2048, gen.ACT_NONE, "pair256s4e8"),  # 46 and 48 pair tiles
     (9472, 512, 2048, gen.ACT_NONE, "pair256s4e8"), (9473, 512, 2048, gen.ACT_NONE, "pair512s3e16"),   # one round of pairs, and more
     (14080, 512, 2048, gen.ACT_NONE, "pair512s3e16"), (14081, 512, 2048, gen.ACT_NONE, "pair256s4e8"),  # a second round half full
-    (12800, 2048, 1024, gen.ACT_NONE, "pair256s4e8"), (12800, 2064, 1024, gen.ACT_NONE, "stream256s3e16"),
+    (12800, 2048, 1024, gen.ACT_NONE, "pair256s4e8"), (12800, 2064, 1024, gen.ACT_NONE, "stream128s4e16"),
     (12544, 2064, 2048, gen.ACT_NONE, "pair256s4e8"),                                                  # any width from K = 2048
     (12800, 1024, 512, gen.ACT_NONE, "ws128e16"), (12800, 1024, 528, gen.ACT_NONE, "pair256s4e8"),
     (74 * 256, 256, 1024, gen.ACT_NONE, "pair256s4e8"), (81 * 256, 256, 1024, gen.ACT_NONE, "pair128s6e8"),  # a last round of 7 of 74
     (82 * 256, 256, 1024, gen.ACT_NONE, "pair256s4e8"),
-    (18944, 2048, 2048, gen.ACT_SWISH, "pair256s4e8"), (4000, 2048, 2048, gen.ACT_SWISH, "stream128s4e16"),
+    (18944, 2048, 2048, gen.ACT_SWISH, "pair256s4e8"), (4000, 2048, 2048, gen.ACT_SWISH, "stream256s3e16"),
 ])
 def test_cta_pairs_start_and_end_where_the_rules_say(M, N, K, act, plan):
     """Both sides of each line in the choice of CTA pairs for 8-bit matmuls (sizes that other tests run by plan name)."""
