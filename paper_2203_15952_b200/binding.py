@@ -289,19 +289,16 @@ def aqt_qmatmul(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s_w: torc
         y = torch.empty((M, n_out), dtype=torch.float32, device=xq.device)
     if workspace is None:
         workspace = _workspace(OP_QMATMUL, M, N, K, bits_a, bits_w, xq.device)
+    ws, ws_bytes = _area(workspace)
+    args = (xq.data_ptr(), s_x.data_ptr(), s_x_kind, wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual), _pitch(residual), residual_scale,
+            M, N, K, bits_a, bits_w, act, y.data_ptr(), y.stride(0), _addr(acc_debug), ws, ws_bytes, _raw_stream(stream))
     if plan is None:
-        ws, ws_bytes = _area(workspace)
-        st = _fc().qmatmul(xq.data_ptr(), s_x.data_ptr(), s_x_kind, wq.data_ptr(), s_w.data_ptr(), _addr(bias), _addr(residual),
-                           _pitch(residual), residual_scale, M, N, K, bits_a, bits_w, act, y.data_ptr(), y.stride(0), _addr(acc_debug),
-                           ws, ws_bytes, _raw_stream(stream))
-        if st != AQT_OK:
-            raise AqtError("aqt_qmatmul", st)
+        st = _fc().qmatmul(*args)
     else:
-        _check("aqt_qmatmul_with_plan", lib().aqt_qmatmul_with_plan(
-            ctypes.c_char_p(plan.encode()), _ptr(xq), _ptr(s_x), int(s_x_kind), _ptr(wq), _ptr(s_w), _ptr(bias), _ptr(residual),
-            _i64(_pitch(residual)), ctypes.c_float(residual_scale), _i64(M), _i64(N), _i64(K), int(bits_a), int(bits_w), int(act), _ptr(y),
-            _i64(y.stride(0)), _ptr(acc_debug), _ptr(workspace), ctypes.c_size_t(0 if workspace is None else workspace.numel()),
-            _stream(stream)))
+        name = ctypes.create_string_buffer(plan.encode())
+        st = _fc().qmatmul_with_plan(ctypes.addressof(name), *args)
+    if st != AQT_OK:
+        raise AqtError("aqt_qmatmul" if plan is None else "aqt_qmatmul_with_plan", st)
     return y
 
 

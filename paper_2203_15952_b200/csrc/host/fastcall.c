@@ -71,6 +71,8 @@ static int read_args(PyObject* const* args, Py_ssize_t nargs, const char* types,
 ENTRY(quantize, "iiiiiiiiiii", fn(P(0), I(1), I(2), I(3), N(4), N(5), N(6), N(7), P(8), P(9), P(10)))
 ENTRY(qmatmul, "iiiiiiiifiiiiiiiiiiii",
       fn(P(0), P(1), N(2), P(3), P(4), P(5), P(6), I(7), F(8), I(9), I(10), I(11), N(12), N(13), N(14), P(15), I(16), P(17), P(18), Z(19), P(20)))
+ENTRY(qmatmul_with_plan, "iiiiiiiiifiiiiiiiiiiii",
+      fn(P(0), P(1), P(2), N(3), P(4), P(5), P(6), P(7), I(8), F(9), I(10), I(11), I(12), N(13), N(14), N(15), P(16), I(17), P(18), P(19), Z(20), P(21)))
 ENTRY(qmatmul_requant, "iiiiiiiifiiiiiiiiiiiiiiii",
       fn(P(0), P(1), N(2), P(3), P(4), P(5), P(6), I(7), F(8), I(9), I(10), I(11), N(12), N(13), N(14), N(15), N(16), N(17), P(18), P(19),
          P(20), I(21), P(22), Z(23), P(24)))
@@ -223,6 +225,7 @@ static PyObject* w_open(PyObject* self, PyObject* path) {
   RESOLVE(linear_fwd_weight_only)
   RESOLVE(linear_bwd)
   RESOLVE(ffn_fwd)
+  RESOLVE(qmatmul_with_plan)
   RESOLVE(workspace_bytes)
   RESOLVE(chain_fwd)
   Py_RETURN_NONE;
@@ -237,6 +240,7 @@ static PyMethodDef methods[] = {{"open", w_open, METH_O, "Resolve the entry poin
                                 METHOD(linear_fwd_weight_only),
                                 METHOD(linear_bwd),
                                 METHOD(ffn_fwd),
+                                METHOD(qmatmul_with_plan),
                                 METHOD(workspace_bytes),
                                 METHOD(chain_ffn),
                                 METHOD(chain_encoder),
