@@ -10,6 +10,7 @@
 #include "quantize.cuh"
 #include "chain_small_m.cuh"
 #include "host_copies.cuh"
+#include "linear_small.cuh"
 
 using namespace aqt;
 
@@ -575,6 +576,12 @@ int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w
   int8_t* codes = reinterpret_cast<int8_t*>(ws);
   float* s_x = reinterpret_cast<float*>(ws + round_up((size_t)M * (size_t)K, 256));
   uint8_t* ws_mm = ws + round_up((size_t)M * (size_t)K, 256) + round_up((size_t)M * 4, 256);
+  if (M <= kLinSmallMaxRows) {
+    // a few rows: both steps in one launch
+    const LinSmallParams sp = {x, reinterpret_cast<const uint8_t*>(wq), s_w, bias, residual, y, ldx, ldr, ldy, residual_scale, (int32_t)M, (int32_t)N,
+                               (int32_t)K, act, qmax_of(bits_a), rounding, a_scale_kind == AQT_SCALE_TENSOR, 0, 0};
+    if (linear_small_applies(sp, is_packed(bits_w))) return launch_linear_small(sp, is_packed(bits_w), st);
+  }
   // Step 1 (Fig. 2): dynamic quantization of the activations over K; 4-bit codes stay in int8
   // containers between the two kernels, which is what the figure's cast produces.
   const int axis = a_scale_kind == AQT_SCALE_ROW ? AQT_AXIS_ROW : AQT_AXIS_TENSOR;
