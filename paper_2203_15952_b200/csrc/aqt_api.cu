@@ -681,7 +681,6 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
                 const void* w2q, const float* s_w2, const float* bias2, int bits_w2, int64_t M, int64_t d, int64_t ff,
                 int bits_a, int rounding, int act, float* y, int y_on_host, void* workspace, size_t workspace_bytes,
                 void* stream) {
-  const int static_flag = (bits_w1 | bits_w2) & AQT_STATIC_WEIGHTS;
   bits_w1 &= ~AQT_STATIC_WEIGHTS;
   bits_w2 &= ~AQT_STATIC_WEIGHTS;
   if (M < 0 || d <= 0 || ff <= 0 || !quant_bits_ok(bits_a) || !bits_ok(bits_w1) || !bits_ok(bits_w2)) return AQT_ERR_BADARG;
@@ -734,9 +733,10 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
     float* s1 = reinterpret_cast<float*>(ws + L.s1) + r0;
     int8_t* q2 = reinterpret_cast<int8_t*>(ws + L.q2) + r0 * ff;
     float* s2 = reinterpret_cast<float*>(ws + L.s2) + r0;
+    // (the work ahead of the first matmul is this quantizer, enqueued after the weights were complete or were ordered so)
     int rc = aqt_quantize(xr, rows, d, d, bits_a, AQT_AXIS_ROW, rounding, 0, q1, s1, stream);
     if (rc != AQT_OK) return rc;
-    rc = aqt_qmatmul_requant(q1, s1, AQT_SCALE_ROW, w1q, s_w1, bias1, nullptr, 0, 0.0f, rows, ff, d, bits_mm, bits_w1 | static_flag, act, bits_a,
+    rc = aqt_qmatmul_requant(q1, s1, AQT_SCALE_ROW, w1q, s_w1, bias1, nullptr, 0, 0.0f, rows, ff, d, bits_mm, bits_w1 | AQT_STATIC_WEIGHTS, act, bits_a,
                              rounding, 0, q2, s2, nullptr, 0, ws + L.mm, mm_bytes, stream);
     if (rc != AQT_OK) return rc;
     // The codes of u are still in L2: narrower tiles that read them twice, and start and drain sooner, then beat the tile

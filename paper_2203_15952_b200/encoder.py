@@ -180,13 +180,15 @@ class LayerRunner:
         return self._codes[role]
 
     def matmul_requant(self, layer: QuantLinear, xq: torch.Tensor, s_x: torch.Tensor, bits_out: int, role: str,
-                       y: Optional[torch.Tensor] = None, residual: Optional[torch.Tensor] = None, residual_scale: float = 1.0):
+                       y: Optional[torch.Tensor] = None, residual: Optional[torch.Tensor] = None, residual_scale: float = 1.0,
+                       static: bool = False):
         """`layer` on quantized activations, its output rows quantized to `bits_out` bits in the
-        epilogue.  Returns (codes, scales); y (fp32) is written too if given."""
+        epilogue.  Returns (codes, scales); y (fp32) is written too if given.  static: the kernel ahead on the
+        stream is one that the caller enqueued itself, after the weights were complete."""
         s = layer.spec
         q, sc = self.code_buffers(role, s.n_out)
         aqt.aqt_qmatmul_requant(xq, s_x, layer.mm_weight, layer.s_w, layer.bias, residual, residual_scale, K=s.K, bits_a=_container_bits(s.bits_a),
-                                bits_w=layer.mm_bits, act=s.act, s_x_kind=self.a_scale_kind, bits_out=bits_out,
+                                bits_w=layer.mm_bits | (aqt.STATIC_WEIGHTS if static else 0), act=s.act, s_x_kind=self.a_scale_kind, bits_out=bits_out,
                                 rounding=self.rounding, pack_out=False, q_out=q, s_out=sc, y=y, workspace=self.workspace)
         return q, sc
 
@@ -224,7 +226,7 @@ class FfnPair:
             return self.run(self.layers[1], self.u, y)
         l0, l1 = self.layers
         xq, xs = self.run.quantize_input(x, l0.spec.bits_a)
-        uq, us = self.run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u)
+        uq, us = self.run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u, static=True)
         return self.run.matmul(l1, uq, us, y, plan=self._plan)
 
     def _chains(self) -> bool:
@@ -260,12 +262,14 @@ class ConformerBlockLinears:
         self.h_b = torch.empty((M, d), **f32)
 
     def forward(self, layers: List[QuantLinear], h_in: torch.Tensor, h_out: torch.Tensor,
-                keep: Optional[Dict[str, torch.Tensor]] = None, in_codes=None, next_bits: Optional[int] = None):
+                keep: Optional[Dict[str, torch.Tensor]] = None, in_codes=None, next_bits: Optional[int] = None, first: bool = True):
         """h_in -> h_out (distinct buffers, neither h_a nor h_b).  `keep`, if given, receives
         clones of every intermediate keyed by layer name (for parity checks).  in_codes: (codes,
         scales) of h_in if the producer already quantized its rows.  next_bits: if given, the last
         matmul also quantizes the rows of h_out to that width for the next block, and the codes and
-        scales are returned with h_out (None where the shape does not allow it)."""
+        scales are returned with h_out (None where the shape does not allow it).  first: False if the work ahead on the
+        stream is another block of the same pass (then, and behind any kernel of this block, a matmul may fetch its weights
+        while the kernel ahead drains)."""
         L, run = layers, self.run
 
         def note(name, t):
@@ -274,7 +278,7 @@ class ConformerBlockLinears:
 
         parity = keep is not None  # then every fp32 intermediate is written as well
         hq, hs = self._ffn(L[0], L[1], h_in, self.h_a, 0.5, parity, note, xq=in_codes[0] if in_codes else None,
-                           xs=in_codes[1] if in_codes else None, out_role="ha", out_bits=L[2].spec.bits_a)
+                           xs=in_codes[1] if in_codes else None, out_role="ha", out_bits=L[2].spec.bits_a, static=not first or in_codes is None)
         note(L[1].spec.name, self.h_a)
         # q, k, v read the same h: its codes come out of the second feed-forward matmul's epilogue
         # (or one quantizer pass; the codes do not depend on the consumer).  q and k run as one matmul over
@@ -292,7 +296,7 @@ class ConformerBlockLinears:
         if run.fuses_requant(L[4]):
             vq, vs = run.code_buffers("v", d)
             aqt.aqt_qmatmul_requant(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, bits_out=L[5].spec.bits_a, rounding=run.rounding, q_out=vq,
-                                    s_out=vs, y=self.v, **args)
+                                    s_out=vs, y=self.v, **dict(args, bits_w=L[4].mm_bits | aqt.STATIC_WEIGHTS))
         else:
             aqt.aqt_qmatmul(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, y=self.v, **args)
         note(L[2].spec.name, self.q); note(L[3].spec.name, self.k); note(L[4].spec.name, self.v)
@@ -300,7 +304,7 @@ class ConformerBlockLinears:
         if run.fuses_requant(L[5]):
             if vq is None:
                 vq, vs = run.quantize_input(self.v, L[5].spec.bits_a)
-            bq, bs = run.matmul_requant(L[5], vq, vs, L[6].spec.bits_a, "h", y=self.h_b, residual=self.h_a, residual_scale=1.0)
+            bq, bs = run.matmul_requant(L[5], vq, vs, L[6].spec.bits_a, "h", y=self.h_b, residual=self.h_a, residual_scale=1.0, static=True)
         elif vq is not None:
             run.matmul(L[5], vq, vs, self.h_b, residual=self.h_a, residual_scale=1.0)
         else:
@@ -310,7 +314,7 @@ class ConformerBlockLinears:
         if not parity and run.fuses_requant(L[6], with_y=False):
             if bq is None:
                 bq, bs = run.quantize_input(self.h_b, L[6].spec.bits_a)
-            cq, cs = run.matmul_requant(L[6], bq, bs, L[7].spec.bits_a, "c")
+            cq, cs = run.matmul_requant(L[6], bq, bs, L[7].spec.bits_a, "c", static=True)
         elif bq is not None:
             run.matmul(L[6], bq, bs, self.c)
         else:
@@ -321,7 +325,7 @@ class ConformerBlockLinears:
         if run.fuses_requant(L[7]):
             if cq is None:
                 cq, cs = run.quantize_input(self.c, L[7].spec.bits_a)
-            aq, as_ = run.matmul_requant(L[7], cq, cs, L[8].spec.bits_a, "h", y=self.h_a, residual=self.h_b, residual_scale=1.0)
+            aq, as_ = run.matmul_requant(L[7], cq, cs, L[8].spec.bits_a, "h", y=self.h_a, residual=self.h_b, residual_scale=1.0, static=True)
             note(L[7].spec.name, self.h_a)
             out_codes = self._ffn(L[8], L[9], self.h_a, h_out, 0.5, parity, note, xq=aq, xs=as_, out_role="hb", out_bits=next_bits)
         else:
@@ -338,7 +342,7 @@ class ConformerBlockLinears:
 
     def _ffn(self, l0: QuantLinear, l1: QuantLinear, h: torch.Tensor, out: torch.Tensor, rs: float, parity: bool, note,
              xq: Optional[torch.Tensor] = None, xs: Optional[torch.Tensor] = None, out_role: str = "ha",
-             out_bits: Optional[int] = None):
+             out_bits: Optional[int] = None, static: bool = True):
         """out = h + rs * W_1 . Swish(W_0 . h); xq, xs: codes and scales of h if already at hand.
         out_bits: also quantize the rows of `out` to that width in the second matmul's epilogue
         where it can; returns (codes, scales) of out, or (None, None)."""
@@ -347,7 +351,7 @@ class ConformerBlockLinears:
         if run.fuses_requant(l0, with_y=parity):
             if xq is None:
                 xq, xs = run.quantize_input(h, l0.spec.bits_a)
-            uq, us = run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u if parity else None)
+            uq, us = run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u if parity else None, static=static)
             if parity:
                 note(l0.spec.name, self.u)
         else:
@@ -358,7 +362,7 @@ class ConformerBlockLinears:
             uq, us = run.code_buffers("u", l0.spec.n_out)
             aqt.aqt_quantize(self.u, l1.spec.bits_a, aqt.AXIS_ROW, run.rounding, q_out=uq, scale_out=us)
         if fuse_out:
-            return run.matmul_requant(l1, uq, us, out_bits, out_role, y=out, residual=h, residual_scale=rs)
+            return run.matmul_requant(l1, uq, us, out_bits, out_role, y=out, residual=h, residual_scale=rs, static=True)
         run.matmul(l1, uq, us, out, residual=h, residual_scale=rs)
         return None, None
 
@@ -400,10 +404,10 @@ class EncoderStack:
             dst = self.h0 if b % 2 == 0 else self.h1
             nxt = self.blocks[b + 1][0].spec.bits_a if b + 1 < len(self.blocks) else None
             if nxt is None:
-                self.block.forward(layers, src, dst, in_codes=codes)
+                self.block.forward(layers, src, dst, in_codes=codes, first=b == 0)
                 codes = None
             else:
-                _, codes = self.block.forward(layers, src, dst, in_codes=codes, next_bits=nxt)
+                _, codes = self.block.forward(layers, src, dst, in_codes=codes, next_bits=nxt, first=b == 0)
             src = dst
         return src
 
