@@ -11,6 +11,7 @@
 #include "chain_small_m.cuh"
 #include "host_copies.cuh"
 #include "linear_small.cuh"
+#include "weight_only_small.cuh"
 
 using namespace aqt;
 
@@ -769,6 +770,13 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
   int rc = check_device();
   if (rc != AQT_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  {
+    // few rows: one launch
+    const WoSmallParams sp = {x, reinterpret_cast<const uint8_t*>(wq), s_w, bias, residual, y, ldx, ldr, ldy, residual_scale, (int32_t)M, (int32_t)N,
+                              (int32_t)K, act};
+    const int terms = precision == AQT_FLOAT_TF32X2 ? 3 : 2;
+    if (weight_only_small_applies(sp, terms)) return launch_weight_only_small(sp, is_packed(bits_w), terms, st);
+  }
   // the weights converted to float (Section 4.1): the codes as binary32 integers, once per call;
   // the channel scales stay outside the sum and are applied to the accumulators.
   float* w_f = reinterpret_cast<float*>(workspace);
