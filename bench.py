@@ -782,7 +782,7 @@ def backward_ffn_layer(dev, steps: int = 20):
     ms = e0.elapsed_time(e1) / (steps * R)
     tflops = 4.0 * M * N * K / (ms * 1e-3) / 1e12
     return {"workload": "ffn_first_layer_M%d_N%d_K%d_w4a8_dx_dw_dbias" % (M, N, K), "value": tflops, "unit": "TFLOP/s", "ms_per_step": ms,
-            "dtype": "tf32", "gpu_launches_per_step": 9, "launch_mode": "cuda graph"}
+            "dtype": "tf32", "gpu_launches_per_step": 4, "launch_mode": "cuda graph"}
 
 
 def run_case(args):

@@ -834,11 +834,7 @@ static int linear_bwd_split(const float* dy, int64_t lddy, const void* xq, const
   float* wt = reinterpret_cast<float*>(ws + L.wt);
   uint16_t* xt = reinterpret_cast<uint16_t*>(ws + L.xt);
   int rc;
-  if (dx != nullptr) {
-    rc = launch_transpose_scale_codes(wq, is_packed(bits_w), s_w, true, N, K, wt, N, N, K, st);
-    if (rc != AQT_OK) return rc;
-  }
-  rc = launch_transpose_codes_bf16(xq, is_packed(bits_a), M, K, xt, L.m_pitch, st);
+  rc = launch_bwd_prep(wq, is_packed(bits_w), s_w, dx != nullptr ? wt : nullptr, xq, is_packed(bits_a), xt, L.m_pitch, M, N, K, st);
   if (rc != AQT_OK) return rc;
   if (dx != nullptr) {
     // dx = dy . (s_w wq): rows m, columns k, contraction n
@@ -859,11 +855,7 @@ static int linear_bwd_split(const float* dy, int64_t lddy, const void* xq, const
   const bool one = L.batches == 1;
   rc = launch_dw_split(dy, lddy, xt, L.m_pitch, one ? dw : dwp, one ? N : L.batches * L.n_pad, one ? lddw : K, p, (int)L.batches, st);
   if (rc != AQT_OK) return rc;
-  if (!one) {
-    rc = launch_sum_batches(dwp, L.batches, L.n_pad, N, K, dw, lddw, st);
-    if (rc != AQT_OK) return rc;
-  }
-  return dbias != nullptr ? launch_colsum_stage2(colsum, L.batches * DwCfg::kGroups, N, dbias, st) : AQT_OK;
+  return launch_bwd_finish(dwp, L.batches, L.n_pad, N, K, dw, lddw, colsum, L.batches * DwCfg::kGroups, dbias, st);
 }
 
 int aqt_linear_bwd(const float* dy, int64_t lddy, const void* xq, const float* s_x, int s_x_kind, int bits_a, const void* wq,

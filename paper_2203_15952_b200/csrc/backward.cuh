@@ -30,12 +30,11 @@ constexpr int kTrRows = 128;
 
 // codes [R, C] (int8, or nibble pairs along C if packed), scale [R] (or one value if !per_row)
 //   -> value(r, c) = scale[r] * float(code[r][c]) in the layout above.
-__global__ void __launch_bounds__(256) transpose_scale_codes_kernel(const uint8_t* __restrict__ codes, bool packed,
-                                                                    const float* __restrict__ scale, bool per_row, int64_t R,
-                                                                    int64_t C, float* __restrict__ out, int64_t r_pad, int64_t chunk,
-                                                                    int64_t rows_out) {
-  __shared__ float tile[kTrRows][kTrTile + 1];
-  const int64_t r0 = (int64_t)blockIdx.y * kTrRows, c0 = (int64_t)blockIdx.x * kTrTile;
+using TrScaleTile = float[kTrRows][kTrTile + 1];
+__device__ __forceinline__ void transpose_scale_codes_block(TrScaleTile& tile, int64_t bx, int64_t by, const uint8_t* __restrict__ codes, bool packed,
+                                                            const float* __restrict__ scale, bool per_row, int64_t R, int64_t C,
+                                                            float* __restrict__ out, int64_t r_pad, int64_t chunk, int64_t rows_out) {
+  const int64_t r0 = by * kTrRows, c0 = bx * kTrTile;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   // load: four codes (one 32-bit word, or two packed bytes) per thread and step; eight threads cover a row of the tile
 #pragma unroll
@@ -75,6 +74,14 @@ __global__ void __launch_bounds__(256) transpose_scale_codes_kernel(const uint8_
   }
 }
 
+__global__ void __launch_bounds__(256) transpose_scale_codes_kernel(const uint8_t* __restrict__ codes, bool packed,
+                                                                    const float* __restrict__ scale, bool per_row, int64_t R,
+                                                                    int64_t C, float* __restrict__ out, int64_t r_pad, int64_t chunk,
+                                                                    int64_t rows_out) {
+  __shared__ TrScaleTile tile;
+  transpose_scale_codes_block(tile, blockIdx.x, blockIdx.y, codes, packed, scale, per_row, R, C, out, r_pad, chunk, rows_out);
+}
+
 // Four weight or activation codes -> bf16 values of the same integers: at most eight significant bits, so the lower
 // halves of the binary32 values are zero.
 __device__ __forceinline__ uint2 codes4_to_bf16(uint32_t w) {
@@ -84,11 +91,10 @@ __device__ __forceinline__ uint2 codes4_to_bf16(uint32_t w) {
 // codes [R, C] -> out[c * pitch + r] = bf16(code[r][c]) (exact): the transposed operand of the split-operand product.
 // A block turns 128 rows x 64 columns: a thread transposes 4 x 4 bytes in registers, the tile goes through
 // shared memory as [column][row] bytes, and leaves in 256-byte runs.
-__global__ void __launch_bounds__(256) transpose_codes_bf16_kernel(const uint8_t* __restrict__ codes, bool packed, int64_t R, int64_t C,
-                                                                   uint16_t* __restrict__ out, int64_t pitch) {
-  __shared__ uint32_t tile[64][kTrRows / 4 + 1];
-  grid_dependency_wait();
-  const int64_t r0 = (int64_t)blockIdx.y * kTrRows, c0 = (int64_t)blockIdx.x * 64;
+using TrCodesTile = uint32_t[64][kTrRows / 4 + 1];
+__device__ __forceinline__ void transpose_codes_bf16_block(TrCodesTile& tile, int64_t bx, int64_t by, const uint8_t* __restrict__ codes, bool packed,
+                                                           int64_t R, int64_t C, uint16_t* __restrict__ out, int64_t pitch) {
+  const int64_t r0 = by * kTrRows, c0 = bx * 64;
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int item = threadIdx.x + 256 * j, cw = item & 15, rg = item >> 4;  // four columns, four rows
@@ -123,6 +129,32 @@ __global__ void __launch_bounds__(256) transpose_codes_bf16_kernel(const uint8_t
     const uint2 lo = codes4_to_bf16(tile[i][2 * seg]), hi = codes4_to_bf16(tile[i][2 * seg + 1]);
     *reinterpret_cast<uint4*>(out + c * pitch + r) = make_uint4(lo.x, lo.y, hi.x, hi.y);  // rows beyond R: zeros inside the pitch
   }
+}
+
+// Both operands of the split backward in one launch (the two are independent and each alone is a few microseconds of start and
+// drain: 12 800 x 512 and 2048 x 512 codes, 6.3 + 5.8 us one after the other): the first `scale_blocks` blocks transpose
+// and scale the weight codes, the others transpose the activation codes.
+struct BwdPrep {
+  const uint8_t *w, *x;
+  const float* s_w;
+  float* wt;
+  uint16_t* xt;
+  int64_t M, N, K, x_pitch;
+  int64_t scale_blocks;
+  bool w_packed, x_packed;
+};
+__global__ void __launch_bounds__(256) bwd_prep_kernel(const BwdPrep p) {
+  __shared__ union {
+    TrScaleTile scale;
+    TrCodesTile codes;
+  } tile;
+  grid_dependency_wait();
+  const int64_t b = blockIdx.x, scale_cols = (p.K + kTrTile - 1) / kTrTile, code_cols = (p.K + 63) / 64;
+  if (b < p.scale_blocks)
+    transpose_scale_codes_block(tile.scale, b % scale_cols, b / scale_cols, p.w, p.w_packed, p.s_w, true, p.N, p.K, p.wt, p.N, p.N, p.K);
+  else
+    transpose_codes_bf16_block(tile.codes, (b - p.scale_blocks) % code_cols, (b - p.scale_blocks) / code_cols, p.x, p.x_packed, p.M, p.K, p.xt,
+                               p.x_pitch);
   grid_dependents_launch();
 }
 
@@ -158,11 +190,11 @@ __global__ void __launch_bounds__(256) transpose_f32_kernel(const float* __restr
 }
 
 // out[n][k] (row pitch ldo) = sum over batches s of partial[(s * rows_p + n) * K + k], in order.
-__global__ void __launch_bounds__(256) sum_batches_kernel(const float* __restrict__ partial, int64_t batches, int64_t rows_p, int64_t N,
-                                                          int64_t K, float* __restrict__ out, int64_t ldo) {
+__device__ __forceinline__ void sum_batches_block(int64_t block, int64_t blocks, const float* __restrict__ partial, int64_t batches, int64_t rows_p,
+                                                  int64_t N, int64_t K, float* __restrict__ out, int64_t ldo) {
   const int64_t k4 = K >> 2, total = N * k4;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+  const int64_t stride = blocks * blockDim.x;
+  for (int64_t i = block * blockDim.x + threadIdx.x; i < total; i += stride) {
     const int64_t n = i / k4, c = i - n * k4;
     float4 t = __ldg(reinterpret_cast<const float4*>(partial + n * K) + c);
     for (int64_t s = 1; s < batches; ++s) {
@@ -174,6 +206,10 @@ __global__ void __launch_bounds__(256) sum_batches_kernel(const float* __restric
     }
     reinterpret_cast<float4*>(out + n * ldo)[c] = t;
   }
+}
+__global__ void __launch_bounds__(256) sum_batches_kernel(const float* __restrict__ partial, int64_t batches, int64_t rows_p, int64_t N,
+                                                          int64_t K, float* __restrict__ out, int64_t ldo) {
+  sum_batches_block(blockIdx.x, gridDim.x, partial, batches, rows_p, N, K, out, ldo);
 }
 
 // Column sums of x [R, C] in a fixed order (the same bits on every run): stage 1 sums the rows of
@@ -199,13 +235,13 @@ __global__ void __launch_bounds__(256) colsum_stage1_kernel(const float* __restr
     partial[(int64_t)blockIdx.y * C + c] = t;
   }
 }
-__global__ void __launch_bounds__(256) colsum_stage2_kernel(const float* __restrict__ partial, int64_t chunks, int64_t C,
-                                                            float* __restrict__ out) {
+__device__ __forceinline__ void colsum_stage2_block(int64_t block, const float* __restrict__ partial, int64_t chunks, int64_t C,
+                                                    float* __restrict__ out) {
   // 32 columns per block; thread (tx, ty) adds the chunks j = ty, ty + 8, ... of column tx in order,
   // then the eight sums of a column are added in order: a fixed grouping, the same bits on every run
   __shared__ float acc[8][kTrTile];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int64_t c = (int64_t)blockIdx.x * kTrTile + tx;
+  const int64_t c = block * kTrTile + tx;
   float t = 0.0f;
   if (c < C)
     for (int64_t j = ty; j < chunks; j += 8) t = __fadd_rn(t, __ldg(partial + j * C + c));
@@ -219,6 +255,24 @@ __global__ void __launch_bounds__(256) colsum_stage2_kernel(const float* __restr
   }
 }
 
+__global__ void __launch_bounds__(256) colsum_stage2_kernel(const float* __restrict__ partial, int64_t chunks, int64_t C,
+                                                            float* __restrict__ out) {
+  colsum_stage2_block(blockIdx.x, partial, chunks, C, out);
+}
+
+// The end of the split backward in one launch: the batches of dw added (the first `sum_blocks` blocks, none with one batch)
+// and the column sums (the others).
+struct BwdFinish {
+  const float *dwp, *colsum;
+  float *dw, *dbias;
+  int64_t batches, rows_p, N, K, lddw, sum_blocks, chunks;
+};
+__global__ void __launch_bounds__(256) bwd_finish_kernel(const BwdFinish p) {
+  grid_dependency_wait();
+  if (blockIdx.x < p.sum_blocks) sum_batches_block(blockIdx.x, p.sum_blocks, p.dwp, p.batches, p.rows_p, p.N, p.K, p.dw, p.lddw);
+  else colsum_stage2_block((int64_t)blockIdx.x - p.sum_blocks, p.colsum, p.chunks, p.N, p.dbias);
+}
+
 // r_pad: rows of the input covered, zeros beyond R (batches * chunk, or the padded pitch for one chunk).
 static int launch_transpose_scale_codes(const void* codes, bool packed, const float* scale, bool per_row, int64_t R, int64_t C, float* out,
                                         int64_t r_pad, int64_t chunk, int64_t rows_out, cudaStream_t st) {
@@ -227,10 +281,25 @@ static int launch_transpose_scale_codes(const void* codes, bool packed, const fl
                                                      chunk, rows_out);
   return AQT_LAUNCH_STATUS();
 }
-// pitch: a multiple of 8, at least R.
-static int launch_transpose_codes_bf16(const void* codes, bool packed, int64_t R, int64_t C, uint16_t* out, int64_t pitch, cudaStream_t st) {
-  return launch_pdl(transpose_codes_bf16_kernel, dim3((unsigned)ceil_div(C, 64), (unsigned)ceil_div(R, kTrRows), 1), dim3(256, 1, 1), 0, st, 1,
-                    reinterpret_cast<const uint8_t*>(codes), packed, R, C, out, pitch);
+// wt: null, or the scaled transposed weights are written too.  x_pitch: a multiple of 8, at least M.
+static int launch_bwd_prep(const void* wq, bool w_packed, const float* s_w, float* wt, const void* xq, bool x_packed, uint16_t* xt, int64_t x_pitch,
+                           int64_t M, int64_t N, int64_t K, cudaStream_t st) {
+  BwdPrep p = {reinterpret_cast<const uint8_t*>(wq), reinterpret_cast<const uint8_t*>(xq), s_w, wt, xt, M, N, K, x_pitch, 0, w_packed, x_packed};
+  if (wt != nullptr) p.scale_blocks = ceil_div(K, kTrTile) * ceil_div(N, kTrRows);
+  const int64_t blocks = p.scale_blocks + ceil_div(K, 64) * ceil_div(M, kTrRows);
+  if (blocks >= (1ll << 31)) return AQT_ERR_UNSUPPORTED;
+  return launch_pdl(bwd_prep_kernel, dim3((unsigned)blocks, 1, 1), dim3(256, 1, 1), 0, st, 1, p);
+}
+static int launch_bwd_finish(const float* dwp, int64_t batches, int64_t rows_p, int64_t N, int64_t K, float* dw, int64_t lddw, const float* colsum,
+                             int64_t chunks, float* dbias, cudaStream_t st) {
+  BwdFinish p = {dwp, colsum, dw, dbias, batches, rows_p, N, K, lddw, 0, chunks};
+  if (batches > 1) {
+    const int64_t want = ceil_div(N * K / 4, 256);
+    p.sum_blocks = want < 1 ? 1 : (want > 148 * 16 ? 148 * 16 : want);
+  }
+  const int64_t blocks = p.sum_blocks + (dbias != nullptr ? ceil_div(N, kTrTile) : 0);
+  if (blocks == 0) return AQT_OK;
+  return launch_pdl(bwd_finish_kernel, dim3((unsigned)blocks, 1, 1), dim3(256, 1, 1), 0, st, 1, p);
 }
 // colsum_partial / colsum_out: null, or the column sums of x are produced on the way
 // (colsum_partial holds transpose_row_blocks(r_pad) * C floats).
