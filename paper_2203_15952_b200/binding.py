@@ -226,11 +226,10 @@ def aqt_quantize(x: torch.Tensor, bits: int, axis: int = AXIS_ROW, rounding: int
     rows, cols = x.shape
     ld = x.stride(0) if rows > 1 else max(cols, 1)
     if q_out is None:
-        q_out = torch.empty((rows, cols // 2), dtype=torch.uint8, device=x.device) if pack else \
-            torch.empty((rows, cols), dtype=torch.int8, device=x.device)
+        q_out = x.new_empty(rows, cols // 2, dtype=torch.uint8) if pack else x.new_empty(rows, cols, dtype=torch.int8)
     n_scale = rows if axis == AXIS_ROW else (cols if axis == AXIS_COL else 1)
     if scale_out is None:
-        scale_out = torch.empty(n_scale, dtype=torch.float32, device=x.device)
+        scale_out = x.new_empty(n_scale)
     st = _fc().quantize(x.data_ptr(), rows, cols, ld, bits, axis, rounding, bool(pack), q_out.data_ptr(), scale_out.data_ptr(),
                         _raw_stream(stream))
     if st != AQT_OK:
@@ -286,7 +285,7 @@ def aqt_qmatmul(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s_w: torc
     M, N = xq.shape[0], wq.shape[0]
     n_out = _n_out(N, act)
     if y is None:
-        y = torch.empty((M, n_out), dtype=torch.float32, device=xq.device)
+        y = s_x.new_empty(M, n_out)
     if workspace is None:
         workspace = _workspace(OP_QMATMUL, M, N, K, bits_a, bits_w, xq.device)
     ws, ws_bytes = _area(workspace)
@@ -399,10 +398,9 @@ def aqt_linear_bwd(dy: torch.Tensor, xq: Optional[torch.Tensor], s_x: Optional[t
     dbias [N]), None for the ones not wanted.  dy fp32 [M, N]; codes and scales as in the forward."""
     assert dy.is_cuda and dy.dtype == torch.float32 and dy.dim() == 2 and dy.stride(1) == 1
     M, N = dy.shape
-    f32 = dict(dtype=torch.float32, device=dy.device)
-    dx = torch.empty((M, K), **f32) if want_dx else None
-    dw = torch.empty((N, K), **f32) if want_dw else None
-    db = torch.empty((N,), **f32) if want_dbias else None
+    dx = dy.new_empty(M, K) if want_dx else None
+    dw = dy.new_empty(N, K) if want_dw else None
+    db = dy.new_empty(N) if want_dbias else None
     if workspace is None:
         workspace = _workspace(OP_LINEAR_BWD, M, N, K, 0, 0, dy.device)
     ws, ws_bytes = _area(workspace)
