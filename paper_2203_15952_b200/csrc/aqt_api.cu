@@ -817,10 +817,11 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
   return launch_qgemm(reinterpret_cast<const int8_t*>(a_f), w_f, false, y, ldy, p, st);
 }
 
-// The weight gradient takes the split operands from 256 rows on (20.1 vs 27.0 us at 1100 x 2048 x 512, 64.5 vs 120 us at
-// 12 800 x 2048 x 512, 1084 vs 1413 us at 65 536 x 4096 x 1024, with the bias gradient; below, its contraction is a few
-// K-blocks and the tf32 form's narrow tiles occupy more SMs).
-static bool dw_split_applies(int64_t M, int64_t N, int64_t K) { return M >= 256 && N >= 128 && K >= 128; }
+// The weight gradient takes the split operands wherever its contraction fills a K-block of 32 rows and the output a fair
+// part of a tile: the tf32 form transposes dy and the scaled codes first, in launches of their own (both products, with
+// the bias gradient: 22.6 vs 11.9 us at 64 x 512 x 512, 64 vs 48 at 64 x 3776 x 2240, 36 vs 30 at 255 x 1024 x 4096, 64.5 vs
+// 120 us for dw alone at 12 800 x 2048 x 512).
+static bool dw_split_applies(int64_t M, int64_t N, int64_t K) { return M >= 32 && N >= 128 && K >= 128; }
 
 // The backward with the weight gradient on split operands: the scale of x multiplies dy while it is split, the codes stay
 // exact, and dy is read in place.  The other product stays on the tf32 form, which needs no conversion in the kernel (62.6
