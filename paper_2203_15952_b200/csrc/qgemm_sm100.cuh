@@ -1279,22 +1279,25 @@ static int plan_qgemm(const GemmShape& g, int sms) {
     if (!glu) deep_k = atoi(e) != 0;
   }
   if (f32 && !g.batched && g.M > kBM) {
-    // CTA pairs on 256-row tiles: many rows (measured: 6-10 % at M >= 25 600, a loss of 10 % at 12 800 x 2048 x 512) or, up
-    // to three rounds of pair tiles, any number: a pair moves 32 KB per k-block and CTA where a single CTA's tile moves
-    // 48 KB (22.4 vs 31.4 us at 4096 x 512 -> 2048 Swish, 25.8 vs 33.5 us at 9000 x 768 -> 768, 26.2 vs 31.8 us at
-    // 4096 x 2048 -> 512; below 32 tiles too few SMs are left with work, 11.9 vs 10.4 us at 2048 x 512 -> 512, and with
-    // more rounds and fewer rows the single-CTA tiles win again, 152 vs 209 us at 12 800 x 2048 -> 2048).
-    const bool few_rounds = pair_tiles >= 32 && pair_tiles <= 3 * pairs;
-    bool pairs_ok = few_rounds || (pair_tiles >= 2 * pairs && g.M >= 2 * kBM * pairs);
+    // CTA pairs on 256-row tiles, from 32 tiles on (below, too few SMs are left with work: 11.9 vs 10.4 us at 2048 x 512 ->
+    // 512): a pair moves 32 KB per k-block and CTA where a single CTA's tile moves 48 KB.  Pair / single, us, inputs not in
+    // L2: 12 800 x 512 -> 2048 Swish 60 / 73, 12 800 x 2048 -> 2048 144 / 159, 4096 x 1024 -> 4096 Swish 69 / 75, 65 536 x
+    // 4096 -> 1152 862 / 971.  Single tiles keep the sizes whose last round of pairs is nearly empty where theirs is not
+    // (7000 x 2048 -> 2048, four rounds against three: 106 / 91); to K = 512 pairs win there too (40 / 42 at N = 2048).
+    const bool few_rounds = pair_tiles <= 3 * pairs;
+    const int64_t pair_rounds = ceil_div(pair_tiles, pairs);
+    const int64_t single_rounds = ceil_div(ceil_div(g.M, kBM) * ceil_div(g.N, 256), sms);
+    bool pairs_ok = pair_tiles >= 32 && (g.K <= 512 || 8 * single_rounds >= 7 * pair_rounds);
     if (tuning_env("AQT_NO_PAIRS") != nullptr) pairs_ok = false;
     if (tuning_env("AQT_FORCE_PAIRS") != nullptr) pairs_ok = true;
     if (pairs_ok) {
-      // width by the number of rounds over the pairs (few rounds: 256); the four-warp epilogue and deeper ring for deep K
-      // (801 vs 752 TFLOP/s at 65 536 x 4096 -> 1024; few rounds: 63.7 vs 60.0 us at 12 800 x 2048 -> 512)
-      const int64_t tiles_m2 = ceil_div(g.M, 2 * kBM);
-      const double cost256 = (double)ceil_div(pair_tiles, pairs) * (256 + 24);
-      const double cost128 = (double)ceil_div(tiles_m2 * ceil_div(g.N, 128), pairs) * (128 + 24);
-      int bn2 = few_rounds || cost256 <= cost128 ? 256 : 128;
+      // Width by the number of rounds: one of 128-column tiles takes 0.7 of one of 256-column tiles, from K = 2048 on 0.8
+      // (256 / 128 wide, us: 65 536 x 4096 -> 1152 862 / 1349, 25 600 x 1024 -> 1024 97 / 120; 9500 x 4096 -> 384, two
+      // rounds either way, 116 / 91; 4096 x 2048 -> 512 38 / 32; 20 000 x 1024 -> 320, three against four, 56 / 52).  The
+      // four-warp epilogue and deeper ring for deep K (801 vs 752 TFLOP/s at 65 536 x 4096 -> 1024; few rounds: 63.7 vs
+      // 60.0 us at 12 800 x 2048 -> 512).
+      const int64_t narrow_rounds = ceil_div(ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 128), pairs);
+      int bn2 = 10 * pair_rounds <= (g.K >= 2048 ? 8 : 7) * narrow_rounds ? 256 : 128;
       if (const char* e = tuning_env("AQT_BN")) {
         if (atoi(e) == 128 || atoi(e) == 256) bn2 = atoi(e);
       }

@@ -216,3 +216,17 @@ def test_weight_only_argument_errors():
     assert call(0, 256, 128) == 0               # empty: no-op
     assert aqt.aqt_workspace_bytes(aqt.OP_LINEAR_WEIGHT_ONLY, 128, 256, 128, 0, 4) == 4 * 256 * 128
     assert aqt.aqt_workspace_bytes(aqt.OP_LINEAR_WEIGHT_ONLY_X2, 128, 256, 128, 0, 4) == 8 * 256 * 128 + 8 * 128 * 128
+
+
+@pytest.mark.parametrize("M,K,N,act", [
+    (12800, 64, 1536, orc.ACT_SWISH),   # 300 pair tiles, more than four rounds
+    (9473, 528, 320, orc.ACT_NONE),     # two rounds of pairs at either width: 128 columns, the last tile half empty
+    (4097, 64, 128, orc.ACT_NONE),      # 17 pair tiles: single CTAs
+    (8000, 64, 128, orc.ACT_NONE),      # 32 pair tiles, one row of tiles 128 wide
+    (9473, 64, 320, orc.ACT_GLU),       # 128 columns of a gated layer
+    (7000, 544, 2048, orc.ACT_NONE),    # four rounds of pairs against three of single CTAs
+    (7000, 512, 2048, orc.ACT_GLU),     # the same, to K = 512 on pairs
+])
+def test_pairs_and_their_width(M, K, N, act):
+    """Both sides of the lines between single CTAs, pairs on 128 columns and pairs on 256."""
+    _check(M, N, K, 8, act, seed=M)
