@@ -20,8 +20,10 @@ well (the residual stream, or a parity check; the GLU layer only fuses when it i
 """
 from __future__ import annotations
 
-from dataclasses import dataclass
-from typing import Dict, List, Optional
+import contextlib
+import weakref
+from dataclasses import dataclass, field
+from typing import Dict, Iterable, List, Optional
 
 import torch
 
@@ -37,12 +39,17 @@ def _container_bits(bits_a: int) -> int:
 @dataclass
 class QuantLinear:
     """Pre-quantized weights of one linear: codes W^T [N, K] (nibble-packed when 4-bit), one
-    fp32 scale per output channel (Section 2.2, channel-wise), optional fp32 bias."""
+    fp32 scale per output channel (Section 2.2, channel-wise), optional fp32 bias.
+
+    The forward passes of many rows read copies made from these (wq_unpacked, QkvStack), those of a few
+    rows read them directly: whoever writes into wq, s_w or bias afterwards calls refresh() behind the
+    writes, as WeightArena.quantize() does for the layers it handed out."""
     spec: LinearSpec
     wq: torch.Tensor
     s_w: torch.Tensor
     bias: Optional[torch.Tensor]
     wq_unpacked: Optional[torch.Tensor] = None
+    _stacks: list = field(default_factory=list, init=False, repr=False, compare=False)  # weak references to the QkvStacks it is in
 
     @classmethod
     def from_float(cls, spec: LinearSpec, wt: torch.Tensor, bias: Optional[torch.Tensor] = None,
@@ -62,6 +69,13 @@ class QuantLinear:
             self.wq_unpacked = aqt.aqt_unpack_int4(self.wq, s.K)
         return self
 
+    def refresh(self, stream=None) -> None:
+        """Bring the copies made from wq, s_w and bias up to date, in place, on `stream` (the one of the writes)."""
+        refresh_layers([self], stream)
+
+    def __getstate__(self):
+        return dict(self.__dict__, _stacks=[])
+
     @property
     def mm_weight(self) -> torch.Tensor:
         """The codes as handed to the matmul entry points."""
@@ -76,6 +90,39 @@ class QuantLinear:
         return self.wq.numel() + 4 * self.s_w.numel()
 
 
+class QkvStack:
+    """Codes, scales and bias of the q, k, v projections stacked along the output channels."""
+
+    def __init__(self, q: QuantLinear, k: QuantLinear, v: QuantLinear):
+        assert q.spec.bits_w == k.spec.bits_w == v.spec.bits_w and q.spec.act == k.spec.act == v.spec.act == aqt.ACT_NONE
+        self.layers = (q, k, v)
+        self.wq, self.s_w, self.bias = self._cat(None, None, None)
+        for l in self.layers:
+            l._stacks[:] = [r for r in l._stacks if r() is not None] + [weakref.ref(self)]
+
+    def _cat(self, wq, s_w, bias):
+        L = self.layers
+        return (torch.cat([l.mm_weight for l in L], out=wq), torch.cat([l.s_w for l in L], out=s_w),
+                None if L[0].bias is None else torch.cat([l.bias for l in L], out=bias))
+
+    def refresh(self) -> None:
+        self._cat(self.wq, self.s_w, self.bias)
+
+
+def refresh_layers(layers: Iterable[QuantLinear], stream=None) -> None:
+    """QuantLinear.refresh() of several layers."""
+    stacks: Dict[int, QkvStack] = {}
+    for l in layers:
+        if l.wq_unpacked is not None:
+            aqt.aqt_unpack_int4(l.wq, l.spec.K, out=l.wq_unpacked, stream=stream)
+        for s in (r() for r in l._stacks):
+            if s is not None:
+                stacks[id(s)] = s
+    with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+        for s in stacks.values():
+            s.refresh()
+
+
 class WeightArena:
     """The float weights W^T [N_i, K] of many linears kept in one tensor per (K, bit width), one
     below the other, so that re-quantizing all of them (every training step when the model is
@@ -83,7 +130,8 @@ class WeightArena:
     per weight: the quantizer reduces over K row by row (one scale per output channel), so the
     rows of different weights do not interact and the codes and scales are those of the
     per-weight calls.  `float_view(i)` is weight i's slice of the arena (the optimizer writes
-    there); `quantize()` fills the code and scale arenas; `linear(i)` wraps weight i's slices."""
+    there); `quantize()` fills the code and scale arenas; `linear(i)` wraps weight i's slices, and
+    the copies that such a layer keeps follow every later `quantize()`."""
 
     def __init__(self, specs: List[LinearSpec], device):
         self.specs = list(specs)
@@ -94,6 +142,7 @@ class WeightArena:
         self.code_arena: Dict[tuple, torch.Tensor] = {}
         self.scale_arena: Dict[tuple, torch.Tensor] = {}
         self._row0: Dict[int, int] = {}
+        self._linears: list = []  # weak references to the layers handed out
         for key, members in self.groups.items():
             K, bits = key
             rows = 0
@@ -105,6 +154,9 @@ class WeightArena:
                                                device=device)
             self.scale_arena[key] = torch.empty(rows, dtype=torch.float32, device=device)
 
+    def __getstate__(self):
+        return dict(self.__dict__, _linears=[])
+
     def _slice(self, arena: Dict[tuple, torch.Tensor], i: int) -> torch.Tensor:
         sp = self.specs[i]
         r0 = self._row0[i]
@@ -114,14 +166,19 @@ class WeightArena:
         return self._slice(self.float_arena, i)
 
     def quantize(self, rounding: int = aqt.ROUND_NEAREST_EVEN, stream=None) -> int:
-        """One quantizer call per group; returns the number of calls."""
+        """One quantizer call per group; returns the number of calls.  The copies kept by the layers that
+        linear() handed out are brought up to date behind them, on the same stream."""
         for key, wt in self.float_arena.items():
             aqt.aqt_quantize(wt, key[1], aqt.AXIS_ROW, rounding, pack=(key[1] == 4), q_out=self.code_arena[key],
                              scale_out=self.scale_arena[key], stream=stream)
+        if self._linears:
+            refresh_layers([l for l in (r() for r in self._linears) if l is not None], stream)
         return len(self.float_arena)
 
     def linear(self, i: int, bias: Optional[torch.Tensor] = None) -> "QuantLinear":
-        return QuantLinear(self.specs[i], self._slice(self.code_arena, i), self._slice(self.scale_arena, i), bias).prepare()
+        layer = QuantLinear(self.specs[i], self._slice(self.code_arena, i), self._slice(self.scale_arena, i), bias).prepare()
+        self._linears[:] = [r for r in self._linears if r() is not None] + [weakref.ref(layer)]
+        return layer
 
     @property
     def algorithmic_bytes(self) -> int:
@@ -256,7 +313,7 @@ class ConformerBlockLinears:
         # q, k, v come out of one GEMM over the concatenated projection weights (N = 3d)
         self.qkv = torch.empty((M, 3 * d), **f32)
         self.q, self.k, self.v = self.qkv[:, 0:d], self.qkv[:, d:2 * d], self.qkv[:, 2 * d:3 * d]
-        self._qkv_weights: Dict[int, tuple] = {}
+        self._qkv_stacks: Dict[tuple, QkvStack] = {}
         self.c = torch.empty((M, d), **f32)
         self.h_a = torch.empty((M, d), **f32)
         self.h_b = torch.empty((M, d), **f32)
@@ -367,16 +424,13 @@ class ConformerBlockLinears:
         return None, None
 
     def _fused_qkv(self, L: List[QuantLinear]):
-        """Codes, scales and bias of the q, k, v projections stacked along the output channels
-        (built once per block and kept)."""
-        key = id(L[2])
-        if key not in self._qkv_weights:
-            q, k, v = L[2], L[3], L[4]
-            assert q.spec.bits_w == k.spec.bits_w == v.spec.bits_w and q.spec.act == k.spec.act == v.spec.act == aqt.ACT_NONE
-            bias = None if q.bias is None else torch.cat([q.bias, k.bias, v.bias]).contiguous()
-            self._qkv_weights[key] = (torch.cat([q.mm_weight, k.mm_weight, v.mm_weight]).contiguous(),
-                                      torch.cat([q.s_w, k.s_w, v.s_w]).contiguous(), bias)
-        return self._qkv_weights[key]
+        """Codes, scales and bias of the q, k, v projections as one matrix each (built once per block and kept)."""
+        q, k, v = L[2], L[3], L[4]
+        key = (id(q), id(k), id(v))  # stays theirs: the stack keeps the layers
+        if key not in self._qkv_stacks:
+            self._qkv_stacks[key] = QkvStack(q, k, v)
+        s = self._qkv_stacks[key]
+        return s.wq, s.s_w, s.bias
 
     def ops(self, layers: List[QuantLinear]) -> int:
         return sum(2 * self.M * l.spec.N * l.spec.K for l in layers)

@@ -308,6 +308,44 @@ def test_weight_arena_quantizes_like_per_weight_calls_and_the_oracle():
         assert torch.equal(q_own.view(torch.uint8), lin.wq.view(torch.uint8)) and torch.equal(s_own, lin.s_w)
 
 
+@pytest.mark.parametrize("d,bits", [(256, (4, 8, 8)), (640, (4, 4, 8))])
+def test_requantized_arena_reaches_few_rows_and_many_alike(d, bits):
+    """After the arena has been quantized again, rows give the same bits in a small and in a large step, and those of
+    layers made afresh: every copy that a layer keeps (unpacked codes beyond K = 512, stacked q, k, v) follows."""
+    from paper_2203_15952_b200.encoder import QkvStack, WeightArena
+    specs = gen.block_linears(d, 4 * d, *bits)
+    arena = WeightArena(specs, DEV)
+    g = torch.Generator(device=DEV).manual_seed(d)
+    def refill():
+        for w in arena.float_arena.values():
+            w.normal_(std=0.5 * w.shape[1] ** -0.5, generator=g)
+    refill()
+    arena.quantize()
+    layers = [arena.linear(i) for i in range(len(specs))]
+    x = torch.randn((200, d), generator=g, device=DEV)
+    few, many = EncoderStack(8, d, 4 * d, [layers], DEV), EncoderStack(200, d, 4 * d, [layers], DEV)
+    before = many.forward(x).clone()
+    few.forward(x[:8])
+    refill()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    arena.quantize(stream=side)
+    torch.cuda.current_stream().wait_stream(side)
+    fresh = [QuantLinear(l.spec, l.wq.clone(), l.s_w.clone(), None).prepare() for l in layers]
+    want = EncoderStack(200, d, 4 * d, [fresh], DEV).forward(x)
+    got = many.forward(x)
+    assert torch.equal(got, want) and not torch.equal(got, before)
+    assert torch.equal(few.forward(x[:8]), want[:8])
+    # codes written in place by the caller: refresh() behind the writes
+    for l, w in zip(fresh, specs):
+        aqt.aqt_quantize(torch.randn((w.N, w.K), generator=g, device=DEV), w.bits_w, pack=w.bits_w == 4, q_out=l.wq, scale_out=l.s_w)
+        l.refresh()
+    again = EncoderStack(200, d, 4 * d, [fresh], DEV)
+    assert torch.equal(EncoderStack(8, d, 4 * d, [fresh], DEV).forward(x[:8]), again.forward(x)[:8])
+    # a stack is its layers': it outlives no layer whose address another one takes
+    assert all(s.layers[0] is layers[2] for s in many.block._qkv_stacks.values()) and isinstance(layers[2]._stacks[0](), QkvStack)
+
+
 def test_encoder_graph_replays_give_the_same_bits():
     """A captured stack replayed many times: the row maxima cross CTAs through tagged words whose
     tag changes on every execution of a captured launch, so every replay must give the output of
