@@ -112,6 +112,26 @@ def test_backward_partial_outputs_on_split_operands(M):
         assert torch.equal(g.view(torch.int32), h.view(torch.int32))
 
 
+@pytest.mark.parametrize("M,N,K", [(12800, 256, 1024), (40000, 256, 128), (20000, 384, 512)])
+def test_backward_bias_gradient_of_many_rows(M, N, K):
+    """Column sums do not lose bits with the number of rows.  Columns of one constant are the hard case: added one after
+    the other their roundings all go the same way (1e-5 of the sum after 1250 rows).  A value passes at most 5
+    additions in its block of 32, one at the end of the running sum, and 19 + 8 between the parts (at most 148 of them,
+    eight side by side): 33 roundings."""
+    g = torch.Generator(device=DEV).manual_seed(M)
+    dy = torch.randn((M, N), generator=g, device=DEV)
+    dy[:, ::2] = torch.rand((1, N // 2), generator=g, device=DEV) + 0.05
+    dy[7, 5], dy[9, 7], dy[11, 7] = float("inf"), float("inf"), -float("inf")
+    xq = torch.randint(-127, 128, (M, K), generator=g, device=DEV, dtype=torch.int8)
+    wq = torch.randint(-127, 128, (N, K), generator=g, device=DEV, dtype=torch.int8)
+    _, dw, db = aqt.aqt_linear_bwd(dy, xq, torch.ones(M, device=DEV), wq, torch.ones(N, device=DEV), K=K, bits_w=8)
+    want, mags = dy.double().sum(0), dy.double().abs().sum(0)
+    assert torch.isposinf(db[5]) and torch.isnan(db[7])
+    rest = [n for n in range(N) if n not in (5, 7)]
+    assert bool(((db.double() - want).abs() <= 33 * 2.0 ** -24 * mags)[rest].all())
+    assert aqt.aqt_device_status() == 0
+
+
 def test_backward_error_is_of_tf32_size():
     ex, ew = _check(512, 1024, 512, 8, 8, seed=4)
     assert np.median(ex) > 2.0 ** -14 and np.median(ew) > 2.0 ** -14   # the bound is not slack by orders of magnitude
