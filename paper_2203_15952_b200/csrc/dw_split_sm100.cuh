@@ -90,7 +90,7 @@ __device__ __forceinline__ void split_bf16x2(float f0, float f1, uint32_t& hi, u
 }
 // sum += the 32 values, added in a tree; what the running sum rounds away is kept in lost.  (One value after the other, the
 // error of a column sum grows with the rows: 7.5e-7 at 12 800 rows and 1.6e-6 at 15 314, against 2.2e-7 for sums of
-// blocks of 128 rows; this way 1e-7.)
+// blocks of 128 rows; this way 9e-8.)
 __device__ __forceinline__ void colsum_add32(const float (&f)[32], float& sum, float& lost) {
   float t[16];
 #pragma unroll
@@ -106,6 +106,18 @@ __device__ __forceinline__ void colsum_add32(const float (&f)[32], float& sum, f
 __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+
+// A converter's arrival on the leader's barrier, and the leader's side of it.  The arrival of the other CTA is what lets the
+// leader's MMA read that CTA's shared memory, so it releases at the scope of the cluster, but only what is in its own
+// shared memory: a release of everything waits for the warp's load of the next scales as well, half a microsecond an
+// arrival (61 -> 106 us for dw alone at 12 800 x 2048 x 512, this way 62).
+__device__ __forceinline__ void mbar_arrive_shared_release(uint32_t bar, uint32_t rank) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(bar), "r"(rank));
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+}
+__device__ __forceinline__ void fence_shared_acquire() { asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory"); }
 
 __global__ void __launch_bounds__(DwCfg::kThreads, 1)
 dw_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_y,
@@ -197,6 +209,7 @@ dw_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&conv_bar[s]), ph, &abort_flag, t_start)) { ok = false; break; }
+          fence_shared_acquire();
           tc_fence_after();
           const uint32_t stage = smem_ring + s * Cfg::kStageBytes;
           const uint64_t a_desc = smem_desc_k_major_sw128(stage), b_desc = smem_desc_k_major_sw64(stage + Cfg::kABytes);
@@ -266,7 +279,7 @@ dw_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         fence_proxy_async_smem();  // the tensor core reads the rows through the async proxy
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(smem_u32(&conv_bar[s]), 0);
+        if (lane == 0) mbar_arrive_shared_release(smem_u32(&conv_bar[s]), 0);
       }
       it += p.k_blocks;
       if (ok && sums && m < p.M) {

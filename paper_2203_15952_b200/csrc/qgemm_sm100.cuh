@@ -206,9 +206,9 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Arrive on the mbarrier at this shared-memory offset in CTA `rank` of the cluster.
-// Release at the scope of the CTA: what the arrival orders is not global or shared memory that the waiting
-// thread reads, but tensor-memory reads (tcgen05 fences) and operands that the writers have already handed to the
-// async proxy by a fence of their own.  A release at cluster scope drains the thread's memory operations first,
+// Release at the scope of the CTA: for arrivals that say that a warp has read its part of an accumulator, which the
+// tcgen05 fences order and no other thread's memory.  (Data for the other CTA takes a release at cluster scope, see
+// mbar_arrive_shared_release.)  A release of everything at cluster scope drains the thread's memory operations first,
 // 1000 to 1500 clocks an arrival (pair tiles: 265 -> 240 us at 65 536 x 1024 -> 3072, 341 -> 283 us with a residual,
 // 18.1 -> 17.1 us at 12 800 x 2048 -> 512).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank) {

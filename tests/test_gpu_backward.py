@@ -132,6 +132,24 @@ def test_backward_bias_gradient_of_many_rows(M, N, K):
     assert aqt.aqt_device_status() == 0
 
 
+@pytest.mark.parametrize("M,N,K", [(12800, 2048, 512), (4001, 300, 132), (50000, 1024, 1024)])
+def test_backward_weight_gradient_repeats_bit_for_bit(M, N, K):
+    """The two CTAs of a pair hand converted rows to one MMA: one to many tiles and ring rounds per pair, the other
+    product of the backward beside them, the same bits every time."""
+    g = torch.Generator(device=DEV).manual_seed(K)
+    dy = torch.randn((M, N), generator=g, device=DEV)
+    xq = torch.randint(-127, 128, (M, K), generator=g, device=DEV, dtype=torch.int8)
+    wq = torch.randint(-127, 128, (N, K), generator=g, device=DEV, dtype=torch.int8)
+    a = (dy, xq, torch.rand(M, generator=g, device=DEV), wq, torch.rand(N, generator=g, device=DEV))
+    first = aqt.aqt_linear_bwd(*a, K=K, bits_w=8)
+    want = (dy.double() * a[2].double()[:, None]).t() @ xq.double()
+    assert ((first[1].double() - want).norm() / want.norm()).item() < 1e-4  # sixteen bits of dy, sums of M terms
+    for i in range(20):
+        again = aqt.aqt_linear_bwd(*a, K=K, bits_w=8, want_dx=i % 2 == 0)
+        assert torch.equal(again[1], first[1]) and torch.equal(again[2], first[2])
+    assert aqt.aqt_device_status() == 0
+
+
 def test_backward_error_is_of_tf32_size():
     ex, ew = _check(512, 1024, 512, 8, 8, seed=4)
     assert np.median(ex) > 2.0 ** -14 and np.median(ew) > 2.0 ** -14   # the bound is not slack by orders of magnitude
