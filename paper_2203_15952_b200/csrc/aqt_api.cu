@@ -111,7 +111,7 @@ DwLayout dw_layout(int64_t M, int64_t N, int64_t K) {
       L.batches = b;
     }
   }
-  L.chunk = (int64_t)round_up((size_t)ceil_div(M, L.batches), 32);
+  L.chunk = (int64_t)round_up((size_t)ceil_div(M > 0 ? M : 1, L.batches), 32);
   L.batches = ceil_div(M, L.chunk);
   L.wt = 0;
   L.xt = L.wt + round_up((size_t)K * (size_t)N * 4, 256);

@@ -132,3 +132,12 @@ def test_plan_query_and_new_entry_points_reject_bad_arguments():
     assert b.aqt_workspace_bytes(b.OP_FFN_FWD, 256, 2048, 512, 8, 4) > 2 * 4 * 256 * 512 + 256 * 2048
     ops = ctypes.c_int64(0)
     assert L.aqt_selftest_sfu_rate(0, one, ctypes.byref(ops), None) == -1
+
+
+def test_workspace_sizes_of_empty_problems():
+    """No rows, channels or depth: a size for every operation, no fault (an empty batch in training asks for it)."""
+    from paper_2203_15952_b200 import binding as b
+    for op in (b.OP_QMATMUL, b.OP_LINEAR_FWD, b.OP_QMATMUL_REQUANT, b.OP_LINEAR_WEIGHT_ONLY, b.OP_LINEAR_WEIGHT_ONLY_X2, b.OP_LINEAR_BWD,
+               b.OP_FFN_FWD):
+        for M, N, K in ((0, 256, 512), (100, 0, 512), (100, 256, 0), (0, 0, 0)):
+            assert 0 <= b.aqt_workspace_bytes(op, M, N, K, 8, 4) <= b.aqt_workspace_bytes(op, max(M, 1), max(N, 256), max(K, 512), 8, 4)
