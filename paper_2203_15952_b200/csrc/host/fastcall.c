@@ -2,8 +2,8 @@
  *
  * A call of an entry point through ctypes spends 8.6 us of host time turning its twenty arguments
  * into ctypes objects and those into registers, more than the launches behind it (about 2 us each),
- * and small layers are bound by it.  Here an argument is a Python integer (pointers included; None is
- * the null pointer) or float, read by the vector-call convention: 0.5 us.  The interpreter lock is
+ * and small layers are bound by it.  Here an argument is a Python integer (anything int() takes), an
+ * address (None is the null pointer) or a float, read by the vector-call convention: 0.5 us.  The interpreter lock is
  * released around the call, as ctypes does.  The library stays the one file libaqt.so: open() resolves
  * its entry points, nothing is linked. */
 #define PY_SSIZE_T_CLEAN
@@ -24,7 +24,24 @@ typedef union {
 #define F(k) ((float)a[k].f)
 #define Z(k) ((size_t)a[k].i)
 
-/* types: one character per argument, 'i' (integer, pointer, None) or 'f'. */
+/* An integer argument: what int() takes, as the ctypes calls do. */
+static int read_int(PyObject* v, int64_t* out) {
+  if (!PyLong_Check(v)) {
+    PyObject* n = PyNumber_Long(v); /* floats, index types; TypeError for None */
+    if (n == NULL) return 0;
+    const int ok = read_int(n, out);
+    Py_DECREF(n);
+    return ok;
+  }
+  /* addresses are unsigned: the low 64 bits of either reading are the same */
+  int overflow = 0;
+  *out = PyLong_AsLongLongAndOverflow(v, &overflow);
+  if (overflow > 0) *out = (int64_t)PyLong_AsUnsignedLongLong(v);
+  if (overflow < 0) PyErr_SetString(PyExc_OverflowError, "argument out of range");
+  return !((*out == -1 || overflow) && PyErr_Occurred());
+}
+
+/* types: one character per argument, 'p' (address or None), 'i' (integer) or 'f' (float). */
 static int read_args(PyObject* const* args, Py_ssize_t nargs, const char* types, Arg* out) {
   Py_ssize_t n = 0;
   for (; types[n] != 0; ++n) {
@@ -33,15 +50,10 @@ static int read_args(PyObject* const* args, Py_ssize_t nargs, const char* types,
     if (types[n] == 'f') {
       out[n].f = PyFloat_AsDouble(v);
       if (out[n].f == -1.0 && PyErr_Occurred()) return 0;
-    } else if (v == Py_None) {
+    } else if (types[n] == 'p' && v == Py_None) {
       out[n].i = 0;
-    } else {
-      /* pointers are unsigned: the low 64 bits of either reading are the same */
-      int overflow = 0;
-      out[n].i = PyLong_AsLongLongAndOverflow(v, &overflow);
-      if (overflow > 0) out[n].i = (int64_t)PyLong_AsUnsignedLongLong(v);
-      if (overflow < 0) PyErr_SetString(PyExc_OverflowError, "argument out of range");
-      if ((out[n].i == -1 || overflow) && PyErr_Occurred()) return 0;
+    } else if (!read_int(v, &out[n].i)) {
+      return 0;
     }
   }
   if (types[n] != 0 || n != nargs) {
@@ -68,21 +80,21 @@ static int read_args(PyObject* const* args, Py_ssize_t nargs, const char* types,
     Py_END_ALLOW_THREADS return PyLong_FromLong(status);                                          \
   }
 
-ENTRY(quantize, "iiiiiiiiiii", fn(P(0), I(1), I(2), I(3), N(4), N(5), N(6), N(7), P(8), P(9), P(10)))
-ENTRY(qmatmul, "iiiiiiiifiiiiiiiiiiii",
+ENTRY(quantize, "piiiiiiippp", fn(P(0), I(1), I(2), I(3), N(4), N(5), N(6), N(7), P(8), P(9), P(10)))
+ENTRY(qmatmul, "ppippppifiiiiiipippip",
       fn(P(0), P(1), N(2), P(3), P(4), P(5), P(6), I(7), F(8), I(9), I(10), I(11), N(12), N(13), N(14), P(15), I(16), P(17), P(18), Z(19), P(20)))
-ENTRY(qmatmul_with_plan, "iiiiiiiiifiiiiiiiiiiii",
+ENTRY(qmatmul_with_plan, "pppippppifiiiiiipippip",
       fn(P(0), P(1), P(2), N(3), P(4), P(5), P(6), P(7), I(8), F(9), I(10), I(11), I(12), N(13), N(14), N(15), P(16), I(17), P(18), P(19), Z(20), P(21)))
-ENTRY(qmatmul_requant, "iiiiiiiifiiiiiiiiiiiiiiii",
+ENTRY(qmatmul_requant, "ppippppifiiiiiiiiipppipip",
       fn(P(0), P(1), N(2), P(3), P(4), P(5), P(6), I(7), F(8), I(9), I(10), I(11), N(12), N(13), N(14), N(15), N(16), N(17), P(18), P(19),
          P(20), I(21), P(22), Z(23), P(24)))
-ENTRY(linear_fwd, "iiiiiiifiiiiiiiiiiiii",
+ENTRY(linear_fwd, "pippppifiiiiiiiipipip",
       fn(P(0), I(1), P(2), P(3), P(4), P(5), I(6), F(7), I(8), I(9), I(10), N(11), N(12), N(13), N(14), N(15), P(16), I(17), P(18), Z(19), P(20)))
-ENTRY(linear_fwd_weight_only, "iiiiiiifiiiiiiiiiii",
+ENTRY(linear_fwd_weight_only, "pippppifiiiiiipipip",
       fn(P(0), I(1), P(2), P(3), P(4), P(5), I(6), F(7), I(8), I(9), I(10), N(11), N(12), N(13), P(14), I(15), P(16), Z(17), P(18)))
-ENTRY(linear_bwd, "iiiiiiiiiiiiiiiiiiii",
+ENTRY(linear_bwd, "pippiippiiiipipippip",
       fn(P(0), I(1), P(2), P(3), N(4), N(5), P(6), P(7), N(8), I(9), I(10), I(11), P(12), I(13), P(14), I(15), P(16), P(17), Z(18), P(19)))
-ENTRY(ffn_fwd, "iiiiiiiiiiiiiiiiiiiii",
+ENTRY(ffn_fwd, "pipppipppiiiiiiipipip",
       fn(P(0), N(1), P(2), P(3), P(4), N(5), P(6), P(7), P(8), N(9), I(10), I(11), I(12), N(13), N(14), N(15), P(16), N(17), P(18), Z(19), P(20)))
 
 /* ---- chains: the layers' addresses and sizes are read from the QuantLinear objects on every call */
@@ -136,7 +148,7 @@ static PyObject* w_chain_ffn(PyObject* self, PyObject* const* args, Py_ssize_t n
     PyErr_SetString(PyExc_TypeError, "chain_ffn: nine arguments, library open");
     return NULL;
   }
-  if (!read_args(args, 3, "iii", a) || !read_args(args + 5, 4, "iiii", a + 5)) return NULL;
+  if (!read_args(args, 3, "pii", a) || !read_args(args + 5, 4, "piip", a + 5)) return NULL;
   if (!read_layer(args[3], &l[0]) || !read_layer(args[4], &l[1])) return NULL;
   l[1].y = (float*)P(5);
   l[1].ldy = I(6);
@@ -157,7 +169,7 @@ static PyObject* w_chain_encoder(PyObject* self, PyObject* const* args, Py_ssize
     PyErr_SetString(PyExc_TypeError, "chain_encoder: ten arguments, the fourth a list of blocks, library open");
     return NULL;
   }
-  if (!read_args(args, 3, "iii", a) || !read_args(args + 4, 6, "iiiiii", a + 4)) return NULL;
+  if (!read_args(args, 3, "pii", a) || !read_args(args + 4, 6, "pipiip", a + 4)) return NULL;
   const Py_ssize_t n_blocks = PyList_GET_SIZE(args[3]);
   const float* x = (const float*)P(0);
   int64_t ldx = I(1);

@@ -141,3 +141,26 @@ def test_workspace_sizes_of_empty_problems():
                b.OP_FFN_FWD):
         for M, N, K in ((0, 256, 512), (100, 0, 512), (100, 256, 0), (0, 0, 0)):
             assert 0 <= b.aqt_workspace_bytes(op, M, N, K, 8, 4) <= b.aqt_workspace_bytes(op, max(M, 1), max(N, 256), max(K, 512), 8, 4)
+
+
+def test_integer_arguments_are_read_as_int_reads_them():
+    """The extension module takes what int() takes and refuses None where a number belongs; None stays the null pointer."""
+    import numpy as np
+    from paper_2203_15952_b200 import binding as b
+    want = b.aqt_workspace_bytes(b.OP_LINEAR_FWD, 100, 256, 512, 8, 4)
+    assert b.aqt_workspace_bytes(b.OP_LINEAR_FWD, 100.0, np.int64(256), np.float32(512), 8.0, True + 3) == want
+    for bad in (None, "rows", [1]):
+        with pytest.raises((TypeError, ValueError)):
+            b.aqt_workspace_bytes(b.OP_LINEAR_FWD, bad, 256, 512, 8, 4)
+    fast = b._fc()
+    assert fast.quantize(None, 0, 8, 8, 8, 0, 1, 0, None, None, 0) == 0            # empty: no-op
+    assert fast.quantize((1 << 64) - 16, 0, 8, 8, 8.0, 0, 1, False, 1 << 63, None, 0) == 0
+    for i in range(1, 8):                                                         # rows .. pack
+        args = [None, 0, 8, 8, 8, 0, 1, 0, None, None, 0]
+        args[i] = None
+        with pytest.raises(TypeError):
+            fast.quantize(*args)
+    with pytest.raises(TypeError):
+        fast.quantize(None, 0, 8)
+    with pytest.raises(OverflowError):
+        fast.quantize(None, -(1 << 64), 8, 8, 8, 0, 1, 0, None, None, 0)
