@@ -1,5 +1,6 @@
 """Build the CUDA library (libaqt.so) in-tree with nvcc for sm_100a, and the extension module through
-which Python calls its per-layer entry points (_fastcall.so) with the host compiler.
+which Python calls its per-layer entry points (_fastcall, under the suffix of the interpreter it is
+built for) with the host compiler.
 
     python -m paper_2203_15952_b200.build [--force]
 """
@@ -14,7 +15,8 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "libaqt.so")
-FASTCALL_PATH = os.path.join(_HERE, "_fastcall.so")
+# The module's name carries the interpreter's tag: another interpreter does not find it, and builds its own.
+FASTCALL_PATH = os.path.join(_HERE, "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 _FASTCALL_SRC = os.path.join(_CSRC, "host", "fastcall.c")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -44,11 +46,14 @@ def _build_fastcall(force: bool) -> None:
         subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"],
                                _FASTCALL_SRC, "-o", tmp, "-ldl"])
         os.replace(tmp, FASTCALL_PATH)
+    untagged = os.path.join(_HERE, "_fastcall.so")  # of earlier builds: any interpreter would load it
+    if os.path.exists(untagged):
+        os.remove(untagged)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile csrc/aqt_api.cu (one translation unit) into libaqt.so and csrc/host/fastcall.c into
-    _fastcall.so where they are missing or out of date."""
+    _fastcall where they are missing or out of date."""
     _build_fastcall(force)
     if force or is_stale():
         nvcc = os.environ.get("NVCC", "nvcc")

@@ -164,3 +164,17 @@ def test_integer_arguments_are_read_as_int_reads_them():
         fast.quantize(None, 0, 8)
     with pytest.raises(OverflowError):
         fast.quantize(None, -(1 << 64), 8, 8, 8, 0, 1, 0, None, None, 0)
+
+
+def test_extension_module_carries_the_interpreters_tag():
+    """Only the interpreter that it was built for finds it."""
+    import importlib.machinery
+    import sys
+    import sysconfig
+    from paper_2203_15952_b200 import binding as b
+    aqt_build.build()
+    folder = os.path.dirname(aqt_build.FASTCALL_PATH)
+    tag = sysconfig.get_config_var("EXT_SUFFIX")
+    assert "%d%d" % sys.version_info[:2] in tag and tag in importlib.machinery.EXTENSION_SUFFIXES
+    assert "_fastcall" + tag in os.listdir(folder) and "_fastcall.so" not in os.listdir(folder)
+    assert os.path.samefile(b._fc().__file__, aqt_build.FASTCALL_PATH)
