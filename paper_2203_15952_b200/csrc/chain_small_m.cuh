@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       }
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-      const ScaleCtx sc = make_scale_ctx(amax, p.in_qmax);
+      const ScaleCtx sc = make_scale_ctx_zeros(amax, p.in_qmax);
       sx[t] = sc.s;
       for (int c = lane; c < p.K0 / 8; c += 32) {
         const float4 f0 = __ldg(xr + 2 * c), f1 = __ldg(xr + 2 * c + 1);
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       if (r >= rows) continue;
       mbar_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
       const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
-      const ScaleCtx sc = make_scale_ctx(__uint_as_float(m), qmax);
+      const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(m), qmax);
       sx[t] = sc.s;
       uint32_t word[2] = {0u, 0u};
 #pragma unroll

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(LinSmallCfg<NT>::kThreads) linear_small_kernel
     ScaleCtx sc[RW];
 #pragma unroll
     for (int t = 0; t < RW; ++t) {
-      sc[t] = make_scale_ctx(amax[t], p.qmax);
+      sc[t] = make_scale_ctx_zeros(amax[t], p.qmax);
       if (lane == 0) sx_s[warp + W * t] = sc[t].s;
     }
     const bool again = K8 > 32 * U;  // the loads above were more than the registers hold: once more, from L1

@@ -514,7 +514,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       const float amax_row = __uint_as_float(row_amax[set][row_in_tile]);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&ctx_free_bar[set][quad >> 1]));
-      const ScaleCtx sc = make_scale_ctx(amax_row, rp.qmax_out);
+      const ScaleCtx sc = make_scale_ctx_zeros(amax_row, rp.qmax_out);
       if (tn == 0 && m < p.M) rp.s_out[m] = sc.s;
       tmem_st_wait();  // this warp's stores of pass 1
 #pragma unroll 1

@@ -973,7 +973,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         if (!ok) break;
         // ---------------------------------------------------------- pass 2: scale, codes
-        const ScaleCtx sc = make_scale_ctx(__uint_as_float(amax_bits), p.qmax_out);
+        const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(amax_bits), p.qmax_out);
         if (my_part == 0 && row_ok) p.s_out[m] = sc.s;
         tmem_st_wait();  // this warp's stores of pass 1
         for (int c = 0; c < chunks; ++c) {

@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_tensor_vec_kernel(cons
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kQuantThreads / 32; ++w) amax = fmaxf(amax, warp_max[w]);
-    c = make_scale_ctx(amax, qmax);
+    c = make_scale_ctx_zeros(amax, qmax);
     if (blockIdx.x == 0 && threadIdx.x == 0) *scale_out = c.s;
   } else {
     c.s = __ldg(scale_out);  // divided already: rebuild the other constants from it
