@@ -586,9 +586,11 @@ int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w
   // Step 1 (Fig. 2): dynamic quantization of the activations over K; 4-bit codes stay in int8
   // containers between the two kernels, which is what the figure's cast produces.
   const int axis = a_scale_kind == AQT_SCALE_ROW ? AQT_AXIS_ROW : AQT_AXIS_TENSOR;
-  // (one scale: the other M - 1 words of its area are scratch for the quantizer)
+  // (one scale: the other words of its area, at least 63, are scratch for the quantizer; with M - 1 of them two rows had one
+  // block look for their maximum, 285 against 267 us for 2 x 131 072 -> 256)
   const bool one_scale = a_scale_kind == AQT_SCALE_TENSOR;
-  rc = quantize_entry(x, M, K, ldx, bits_a, axis, rounding, 0, codes, s_x, stream, one_scale && M > 1 ? s_x + 1 : nullptr, M - 1);
+  rc = quantize_entry(x, M, K, ldx, bits_a, axis, rounding, 0, codes, s_x, stream, one_scale ? s_x + 1 : nullptr,
+                      (int64_t)(round_up((size_t)M * 4, 256) / 4) - 1);
   if (rc != AQT_OK) return rc;
   // Step 2: integer matmul + de-quantizing epilogue.
   return qmatmul_i8a(codes, s_x, a_scale_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y,

@@ -97,6 +97,21 @@ def test_quantize_tensor_axis_beyond_one_block(rows, cols, ld, std, bits, pack):
         assert np.array_equal(y.cpu().numpy().view(np.uint32), y_ref.view(np.uint32))
 
 
+@pytest.mark.parametrize("M,K", [(1, 20480), (2, 70000), (3, 32768), (65, 16384)])
+def test_linear_with_one_scale_for_a_few_deep_rows(M, K):
+    """The maximum's partial words fit the scale area however few rows there are: the bits of quantizer and matmul one after
+    the other, with a workspace of exactly the stated size between guards."""
+    x, w = gen.normal(13, 1, M, K), gen.weight(13, 2, K, 64)
+    x[M - 1, K - 1] = 9.5  # the maximum is the last element
+    wq, s_w = orc.quantize(w, 8, orc.AXIS_ROW)
+    need = aqt.aqt_workspace_bytes(aqt.OP_LINEAR_FWD, M, 64, K, 8, 8)
+    area = torch.full((256 + need + 256,), 0x5A, dtype=torch.uint8, device=DEV)
+    y = aqt.aqt_linear_fwd(_dev(x), _dev(wq), _dev(s_w), a_scale_kind=aqt.SCALE_TENSOR, workspace=area[256:256 + need])
+    xq, s_x = aqt.aqt_quantize(_dev(x), 8, aqt.AXIS_TENSOR)
+    assert torch.equal(y, aqt.aqt_qmatmul(xq, s_x, _dev(wq), _dev(s_w), K=K, s_x_kind=aqt.SCALE_TENSOR))
+    assert bool((area[:256] == 0x5A).all()) and bool((area[256 + need:] == 0x5A).all())
+
+
 def test_quantize_heavy_tailed_rows():
     x = gen.student_t3(0, 77, 256, 1024)
     q_ref, s_ref = orc.quantize(x, 8, orc.AXIS_ROW)
