@@ -218,9 +218,11 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_with_scales_kernel(
 // Whole-tensor scale for small tensors in one launch: one CTA finds the abs-max, forms the scale
 // and quantizes (the tensor is re-read from L1/L2).  Replaces the four-launch path below where
 // launch latency, not bandwidth, is the cost (e.g. a [64, 256] activation).
-// Beyond what the block keeps in registers the three launches of the vectorized form are shorter (64 x 512: 17.2 us in one
-// block, 4.1 in three launches; 64 x 256: 3.1, 3.9).
-constexpr int kSmallTensorElems = 1 << 14;
+// Beyond what the block can keep in registers the three launches of the vectorized form are shorter (64 x 512: 17.2 us in one
+// block, 4.1 in three launches; 64 x 256: 3.1, 3.9).  A dense tensor up to there stays in registers, others are read
+// twice (64 x 200 with a row pitch: 8.1 us).  Tensors that cannot be read as float4s have the four launches of the
+// element-wise form to compare with: 40 x 511 11.4 us in one block, 12.4 in four launches, 64 x 400 13.7 and 12.3.
+constexpr int kSmallTensorElems = 1 << 14, kSmallTensorElemsScalar = 22 << 10;
 template <int ROUNDING, bool PACK>
 __global__ void __launch_bounds__(1024) quantize_tensor_small_kernel(const float* __restrict__ x, int rows, int cols, int64_t ld,
                                                                       int qmax, void* __restrict__ q_out,
@@ -450,11 +452,12 @@ static int launch_quantize_axis(const float* x, int64_t rows, int64_t cols, int6
                                 float* scale_out, cudaStream_t st, float* partial = nullptr, int64_t max_partials = 0) {
   if (axis == AQT_AXIS_ROW) return launch_quantize_rows<ROUNDING, PACK>(x, rows, cols, ld, qmax, q_out, scale_out, st);
   const bool per_col = axis == AQT_AXIS_COL;
-  if (!per_col && rows * cols <= kSmallTensorElems) {
+  const bool vec = !per_col && tensor_vec_ok(x, cols, ld, q_out);
+  if (!per_col && rows * cols <= (vec ? kSmallTensorElems : kSmallTensorElemsScalar)) {
     quantize_tensor_small_kernel<ROUNDING, PACK><<<1, 1024, 0, st>>>(x, (int)rows, (int)cols, ld, qmax, q_out, scale_out);
     return AQT_LAUNCH_STATUS();
   }
-  if (!per_col && tensor_vec_ok(x, cols, ld, q_out))
+  if (vec)
     return launch_quantize_tensor_vec<ROUNDING, PACK>(x, rows, cols, ld, qmax, q_out, scale_out, partial, max_partials, st);
   const int64_t n_scale = per_col ? cols : 1;
   AQT_RETURN_IF_CUDA(cudaMemsetAsync(scale_out, 0, (size_t)n_scale * sizeof(float), st));

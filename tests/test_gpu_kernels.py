@@ -79,7 +79,7 @@ def test_quantize_col_and_tensor_axes_bit_exact(axis, bits, shape):
                                               (300, 1000, 1004, 1e-30), (70, 1024, 1024, 0.0)])
 @pytest.mark.parametrize("bits,pack", [(8, False), (4, True)])
 def test_quantize_tensor_axis_beyond_one_block(rows, cols, ld, std, bits, pack):
-    """One scale for a tensor of more than 64 K elements read as float4s: dense and with a row pitch, a
+    """One scale for a tensor of more than 16 K elements read as float4s: dense and with a row pitch, a
     remainder in the last block, scales outside the short quotient sequence's range, a tensor of
     zeros.  aqt_linear_fwd finds the same scale through its own scratch words (exact: y is compared
     bit for bit)."""
@@ -95,6 +95,18 @@ def test_quantize_tensor_axis_beyond_one_block(rows, cols, ld, std, bits, pack):
         y = aqt.aqt_linear_fwd(xd, _dev(wq), _dev(s_w), bits_a=bits, a_scale_kind=aqt.SCALE_TENSOR)
         y_ref = orc.linear_fwd(np.ascontiguousarray(x[:, :cols]), wq, s_w, bits_a=bits, a_scale_kind=orc.SCALE_TENSOR)
         assert np.array_equal(y.cpu().numpy().view(np.uint32), y_ref.view(np.uint32))
+
+
+@pytest.mark.parametrize("rows,cols,ld,offset", [(11, 2048, 2048, 1), (11, 2049, 2049, 0), (44, 512, 513, 0), (45, 512, 513, 0), (32, 512, 516, 4),
+                                                 (33, 512, 516, 4), (1, 22529, 22529, 0)])
+def test_quantize_tensor_axis_around_the_one_block_line(rows, cols, ld, offset):
+    """Both sides of the sizes up to which one block takes a tensor: rows that can be read as float4s and rows that cannot."""
+    buf = np.full(offset + rows * ld, 7e9, np.float32)
+    x = np.lib.stride_tricks.as_strided(buf[offset:], (rows, cols), (4 * ld, 4))
+    x[:] = gen.normal(12, 3, rows, cols, std=1.0)
+    q_ref, s_ref = orc.quantize(np.ascontiguousarray(x), 8, orc.AXIS_TENSOR)
+    q, s = aqt.aqt_quantize(torch.as_strided(_dev(buf), (rows, cols), (ld, 1), offset), 8, aqt.AXIS_TENSOR)
+    assert np.array_equal(s.cpu().numpy(), s_ref) and np.array_equal(q.cpu().numpy(), q_ref)
 
 
 @pytest.mark.parametrize("M,K", [(1, 20480), (2, 70000), (3, 32768), (65, 16384)])
