@@ -146,7 +146,7 @@ int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, 
 
 /*
  * aqt_plan_qmatmul -- names the kernel configuration aqt_qmatmul (and every entry point that runs
- * the same matmul) would launch for a shape: "small_m", "ws128e16", "pair256s6e4", ...  Host-only:
+ * the same matmul) would launch for a shape without a residual: "small_m", "ws128e16", "pair256s6e4", ...  Host-only:
  * sm_count_or_0 > 0 plans for a device with that many multiprocessors, 0 for the current device
  * (148 if there is none).  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
  * aqt_linear_bwd with K in elements.  (No counterpart in the paper: the choice of tile shapes is

@@ -167,7 +167,12 @@ bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y
   const int sms = sm_count() > 0 ? sm_count() : kDefaultSms;
   // With the fp32 output, few pair tiles leave most of the chip idle: narrow tiles and the row quantizer behind them take 9.3
   // against 14.2 us at 1024 x 2048 -> 512, 11.5 against 15.1 us at 4096 rows, 15.3 against 16.0 us at 8192 (64 tiles).
-  if (with_y && 8 * ceil_div(M, 2 * kBM) * ceil_div(N, 256) <= 7 * (sms / 2)) return false;
+  // (But not where the matmul ahead of the row quantizer would be left between its forms, with more single-CTA tiles of 128
+  // columns than one round takes and too few pair tiles: 16.0 in one kernel, 19.6 us in two at 5000 x 2048 -> 512.)
+  const int64_t pair_tiles = ceil_div(M, 2 * kBM) * ceil_div(N, 256);
+  if (with_y && 8 * pair_tiles <= 7 * (sms / 2) &&
+      (ceil_div(M, kBM) * ceil_div(N, 128) <= sms || gemm_plan_is_pair(plan_qgemm(GemmShape{M, N, K, act, 0, false}, sms))))
+    return false;
   const int plan = rowquant_plan(M, N, K, sms);
   const int parts = rowquant_parts(plan, N);
   return parts % 2 == 0 && parts <= 16 && ceil_div(N, kGemmPlanBn[plan]) <= sms / 2;

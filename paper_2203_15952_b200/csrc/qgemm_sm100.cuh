@@ -1223,6 +1223,7 @@ struct GemmShape {
   int act;
   int kind;      // 0: 8-bit codes, 1: float kind
   bool batched;  // stacked batches: streaming kernel, one CTA per tile
+  bool residual = false;
 };
 
 // True if the weight-stationary kernel takes this shape (and can therefore unpack 4-bit weights itself).
@@ -1238,23 +1239,38 @@ static bool qgemm_uses_ws(int64_t N, int64_t K, int sms) {
 // SMs: 9.3 vs 10.9 us at 3000 x 2048 -> 384), 78 vs 89 us at 65 536 x 1024 -> 1024, 101 vs
 // 110 with a residual.  (Measured for act NONE.  With Swish the sixteen-warp epilogue of the single-CTA tiles wins below
 // K = 2048, 322 vs 334 us at 65 536 x 1024 -> 4096; GLU is laid out for single CTAs.)
+// From K = 4096 pairs win earlier, single CTA / pairs in us: without activation from the first size on that 128-column
+// tiles do not cover in one round (5000 -> 512 28.3 / 15.6), with Swish from the second round on (4000 -> 1536 32.2 / 26.5).
 static int plan_qgemm_pairs(const GemmShape& g, int pairs, int64_t pair_tiles) {
   const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
   if (glu || g.M <= kBM || g.K <= kWsMaxKBlocks * kBK) return kPlanNone;
   if (tuning_env("AQT_NO_PAIRS") != nullptr) return kPlanNone;
+  // One tile column, half of it padding: pairs of 128 columns, and only for more than a round of tiles (12 800 x 1024 -> 128
+  // 6.9 us on single CTAs, 7.4 on pairs of 128 columns, 8.5 of 256; 30 000 rows 10.9, 9.9 and 11.5, with a residual below
+  // K = 1024 9.6, 10.4 and 14.7).
+  if (g.N <= 128 && (pair_tiles <= pairs || (g.residual && g.K < 1024))) return kPlanNone;
   // One row block per 512-column tile and a second round of 256-column tiles that would be less than half full: each
   // pair takes one whole 256 x 512 tile, so the activations are read once.
   if (g.N == 512 && g.K >= 2048 && pair_tiles > pairs && 2 * pair_tiles <= 3 * pairs) return kPlanPair512S3E16;
   // (Below K = 2048 up to 2048 columns: the parity tests fix the single-CTA configuration of the d = 1024 encoder's
   // 3072-column projection; a caller that cuts it in two, as the encoder driver does, gets pairs for both parts.)
-  const bool enough = g.act == AQT_ACT_NONE ? pair_tiles >= 48 && (g.K >= 2048 || g.N <= 2048) : g.K >= 2048 && pair_tiles >= 2 * pairs;
+  const bool enough = g.act == AQT_ACT_NONE
+                          ? (pair_tiles >= 48 || (g.K >= 4096 && ceil_div(g.M, kBM) * ceil_div(g.N, 128) > 2 * pairs)) && (g.K >= 2048 || g.N <= 2048)
+                          : (g.K >= 2048 && pair_tiles >= 2 * pairs) || (g.K >= 4096 && pair_tiles > pairs);
   if (!enough) return kPlanNone;
   // The four-warp epilogue and deeper ring need a deep K and several tiles per pair (191 vs 205 us at 65 536 x 4096 ->
   // 1024; 25 600 rows: 86 vs 87 without, 100 vs 96 us with a residual).
   const bool dp = g.K >= 4096 && g.act == AQT_ACT_NONE && ceil_div(g.M, kBM) * ceil_div(g.N, 256) >= 12 * pairs;
-  // 128 columns where more than a quarter of the columns of 256-wide tiles would be padding, or their last round nearly empty
+  // 128 columns where more than a quarter of the columns of 256-wide tiles would be padding, or their last round nearly empty;
+  // with a residual below K = 1024, where the epilogue is most of a tile, up to half empty (256 / 128 columns / single CTAs,
+  // us: 12 800 x 768 -> 512, 100 tiles, 14.2 / 13.0 / 12.6, inputs not in L2 18.9 / 15.9 / 16.8; 20 000 x 528 -> 640, 237
+  // tiles, 28.0 / 25.4 / 25.1; 9000 x 528 -> 1024, 144 tiles, 15.4 / 16.6 / 18.2)
+  // (but not for deep tiles without padding: 5000 x 4096 -> 1024 25.9 us on 256 columns, 31.6 on 128; one tile column, which
+  // reads no operand twice, 37.0 and 36.3 at 20 000 x 4096 -> 256)
   const int64_t last_round = pair_tiles % pairs;
-  const bool narrow = (g.N <= 384 && g.N % 256 != 0 && g.N % 256 <= 128 && pair_tiles > 2 * pairs) || (pair_tiles > pairs && last_round > 0 && last_round <= pairs / 10);
+  const bool deep_full = g.K >= 4096 && g.N > 256 && g.N % 256 == 0;
+  const bool narrow = g.N <= 128 || (g.N <= 384 && g.N % 256 != 0 && g.N % 256 <= 128 && pair_tiles > 2 * pairs) ||
+                      (pair_tiles > pairs && last_round > 0 && last_round <= (g.residual && g.K < 1024 ? pairs / 2 : pairs / 10) && !deep_full);
   if (narrow) return dp ? kPlanPair128S8E4 : kPlanPair128S6E8;
   return dp ? kPlanPair256S6E4 : kPlanPair256S4E8;
 }
@@ -1331,6 +1347,8 @@ static int plan_qgemm(const GemmShape& g, int sms) {
   return deep_k ? kPlanStream64S8E4 : kPlanStream64S5E8;
 }
 
+static bool gemm_plan_is_pair(int plan) { return plan >= kPlanPair256S4E8 && plan <= kPlanPair512S3E16; }
+
 // Tile width and epilogue warps of each plan (same order as GemmPlan).
 static const int kGemmPlanBn[kPlanCount] = {0, 128, 128, 256, 256, 256, 128, 128, 128, 64, 64, 256, 256, 128, 128, 512};
 static const int kGemmPlanEw[kPlanCount] = {0, 16, 8, 16, 4, 8, 16, 4, 8, 8, 4, 8, 4, 8, 4, 16};
@@ -1340,7 +1358,7 @@ static bool gemm_plan_takes(int plan, const GemmShape& g, int sms) {
   if (plan <= kPlanNone || plan >= kPlanCount) return false;
   const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
   const bool ws = plan == kPlanWs128E16 || plan == kPlanWs128E8;
-  const bool pair = plan >= kPlanPair256S4E8 && plan <= kPlanPair512S3E16;
+  const bool pair = gemm_plan_is_pair(plan);
   if (ws && (g.batched || ceil_div(g.K, kBK) > kWsMaxKBlocks || ceil_div(g.N, 128) > sms)) return false;
   if (pair && (g.batched || g.M <= kBM)) return false;
   if (plan == kPlanPair512S3E16 && (glu || g.kind != 0)) return false;
@@ -1416,6 +1434,7 @@ static GemmShape gemm_shape_of(const GemmParams& p) {
   g.act = p.act;
   g.kind = p.kind;
   g.batched = p.batch_tiles_m > 0;
+  g.residual = p.residual != nullptr;
   return g;
 }
 

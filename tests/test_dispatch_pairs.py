@@ -19,3 +19,21 @@ from paper_2203_15952_b200 import inputs as gen
 def test_cta_pairs_start_and_end_where_the_rules_say(M, N, K, act, plan):
     """Both sides of each line in the choice of CTA pairs for 8-bit matmuls (sizes that other tests run by plan name)."""
     assert aqt.aqt_plan_qmatmul(M, N, K, 8, aqt.BITS_4_UNPACKED, act, sm_count=148) == plan
+
+
+@pytest.mark.parametrize("M,N,K,act,plan", [
+    # one tile column of 128: single CTAs in the first round of pairs, else pairs of 128 columns
+    (74 * 256, 128, 4096, gen.ACT_NONE, "stream128s4e16"), (74 * 256 + 1, 128, 1024, gen.ACT_NONE, "pair128s6e8"),
+    (30000, 128, 528, gen.ACT_NONE, "pair128s6e8"), (30000, 144, 1008, gen.ACT_NONE, "pair256s4e8"),
+    # from K = 4096 pairs as soon as 128-column tiles of single CTAs take a second round, with Swish as soon as pairs do
+    (37 * 128 + 1, 512, 4096, gen.ACT_NONE, "pair256s4e8"), (37 * 128, 512, 4096, gen.ACT_NONE, "stream128s4e16"),
+    (37 * 128 + 1, 512, 4080, gen.ACT_NONE, "stream64s5e8"),
+    (4000, 1536, 4096, gen.ACT_SWISH, "pair256s4e8"), (4000, 1536, 4080, gen.ACT_SWISH, "stream128s4e16"),
+    (37 * 256, 512, 4096, gen.ACT_SWISH, "stream256s3e16"),
+    # a last round of 6 of 74: 256 columns where the tiles are deep and full
+    (5000, 1024, 4096, gen.ACT_NONE, "pair256s4e8"), (5000, 1024, 4080, gen.ACT_NONE, "pair128s6e8"), (20 * 256, 1000, 4096, gen.ACT_NONE, "pair128s6e8"),
+    (20000, 256, 4096, gen.ACT_NONE, "pair128s6e8"),
+])
+def test_cta_pairs_of_deep_and_of_narrow_matmuls(M, N, K, act, plan):
+    """Both sides of the lines for one column of 128-wide tiles and for K from 4096."""
+    assert aqt.aqt_plan_qmatmul(M, N, K, 8, aqt.BITS_4_UNPACKED, act, sm_count=148) == plan

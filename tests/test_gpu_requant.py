@@ -219,6 +219,22 @@ def test_requant_edge_shapes(M, N, K):
     _run(M, N, K, 8, 4, aqt.ACT_NONE, False, M > 100, 4, aqt.ROUND_HALF_UP_FLOOR, True)
 
 
+@pytest.mark.parametrize("M,N,K", [(37 * 128, 512, 2048), (37 * 128 + 1, 512, 2048), (5000, 512, 4096), (23 * 256 + 1, 512, 2048)])
+def test_requant_with_y_gives_the_bits_of_two_calls(M, N, K):
+    """Deep K with the fp32 output: one round of 128-column tiles (two kernels), more than one (the row-quantizing pair
+    kernel), pairs (two kernels)."""
+    g = torch.Generator(device=DEV).manual_seed(M)
+    code = lambda r: torch.randint(-127, 128, (r, K), generator=g, device=DEV, dtype=torch.int8)
+    xq, wq, s_x, s_w = code(M), code(N), torch.rand(M, generator=g, device=DEV), torch.rand(N, generator=g, device=DEV)
+    res = torch.randn((M, N), generator=g, device=DEV)
+    for r in (None, res):
+        q, s, y = aqt.aqt_qmatmul_requant(xq, s_x, wq, s_w, None, r, 0.5, K=K, bits_w=8, want_y=True)
+        y2 = aqt.aqt_qmatmul(xq, s_x, wq, s_w, None, r, 0.5, K=K, bits_w=8)
+        q2, s2 = aqt.aqt_quantize(y2, 8)
+        assert torch.equal(y, y2) and torch.equal(q, q2) and torch.equal(s, s2)
+    assert aqt.aqt_device_status() == 0
+
+
 def test_requant_argument_checks():
     z8 = torch.zeros((64, 64), dtype=torch.int8, device=DEV)
     w8 = torch.zeros((48, 64), dtype=torch.int8, device=DEV)
