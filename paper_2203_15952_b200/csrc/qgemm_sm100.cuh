@@ -1224,6 +1224,7 @@ struct GemmShape {
   int kind;      // 0: 8-bit codes, 1: float kind
   bool batched;  // stacked batches: streaming kernel, one CTA per tile
   bool residual = false;
+  bool beside = false;  // float kind: the next launch runs beside this one (GemmParams::early_trigger)
 };
 
 // True if the weight-stationary kernel takes this shape (and can therefore unpack 4-bit weights itself).
@@ -1295,25 +1296,34 @@ static int plan_qgemm(const GemmShape& g, int sms) {
     if (!glu) deep_k = atoi(e) != 0;
   }
   if (f32 && !g.batched && g.M > kBM) {
-    // CTA pairs on 256-row tiles, from 32 tiles on (below, too few SMs are left with work: 11.9 vs 10.4 us at 2048 x 512 ->
-    // 512): a pair moves 32 KB per k-block and CTA where a single CTA's tile moves 48 KB.  Pair / single, us, inputs not in
-    // L2: 12 800 x 512 -> 2048 Swish 60 / 73, 12 800 x 2048 -> 2048 144 / 159, 4096 x 1024 -> 4096 Swish 69 / 75, 65 536 x
-    // 4096 -> 1152 862 / 971.  Single tiles keep the sizes whose last round of pairs is nearly empty where theirs is not
-    // (7000 x 2048 -> 2048, four rounds against three: 106 / 91); to K = 512 pairs win there too (40 / 42 at N = 2048).
-    const bool few_rounds = pair_tiles <= 3 * pairs;
+    // CTA pairs on 256-row tiles: a pair moves 32 KB per k-block and CTA where a single CTA's tile moves 48 KB.  Pair /
+    // single, us, inputs not in L2: 12 800 x 512 -> 2048 Swish 60 / 73, 12 800 x 2048 -> 2048 144 / 159, 4096 x 1024 -> 4096
+    // Swish 69 / 75, 65 536 x 4096 -> 1152 862 / 971.  Single tiles keep (k: elements of K)
+    //  - few tiles: fewer than 32, below k = 1024 up to 37, one round of 128-column single tiles (1000 x 256 -> 2048, 32
+    //    tiles, 9.7 / 9.3; 2048 x 512 -> 512 11.9 / 10.4; but 12 800 x 768 -> 256, 50 tiles, 17.4 / 25.9),
+    //  - beyond k = 512 the sizes whose last round of pairs is nearly empty where theirs is not (7000 x 2048 -> 2048, four
+    //    rounds against three: 106 / 91; but 7000 x 512 -> 2048 34.2 / 35.2),
+    //  - below k = 512, where the epilogue is most of a tile, one tile column of 128 in the first round, with an activation in
+    //    the second too (20 000 x 160 -> 128 Swish 12.6 / 11.4), and Swish on one round of tiles with a third of padding
+    //    (7000 x 160 -> 320 11.9 / 9.4).
+    const int64_t k = g.K / 4;
+    const bool few_rounds = pair_tiles <= 3 * pairs, short_k = k < 512;
     const int64_t pair_rounds = ceil_div(pair_tiles, pairs);
     const int64_t single_rounds = ceil_div(ceil_div(g.M, kBM) * ceil_div(g.N, 256), sms);
-    bool pairs_ok = pair_tiles >= 32 && (g.K <= 512 || 8 * single_rounds >= 7 * pair_rounds);
+    bool pairs_ok = (k < 1024 ? 2 * pair_tiles > pairs : pair_tiles >= 32) && (k <= 512 || 8 * single_rounds >= 7 * pair_rounds);
+    if (short_k && g.N <= 128 && pair_rounds <= (g.act == AQT_ACT_NONE ? 1 : 2)) pairs_ok = false;
+    if (short_k && g.act == AQT_ACT_SWISH && pair_rounds == 1 && 2 * 256 * ceil_div(g.N, 256) > 3 * g.N) pairs_ok = false;
     if (tuning_env("AQT_NO_PAIRS") != nullptr) pairs_ok = false;
     if (tuning_env("AQT_FORCE_PAIRS") != nullptr) pairs_ok = true;
     if (pairs_ok) {
-      // Width by the number of rounds: one of 128-column tiles takes 0.7 of one of 256-column tiles, from K = 2048 on 0.8
-      // (256 / 128 wide, us: 65 536 x 4096 -> 1152 862 / 1349, 25 600 x 1024 -> 1024 97 / 120; 9500 x 4096 -> 384, two
-      // rounds either way, 116 / 91; 4096 x 2048 -> 512 38 / 32; 20 000 x 1024 -> 320, three against four, 56 / 52).  The
-      // four-warp epilogue and deeper ring for deep K (801 vs 752 TFLOP/s at 65 536 x 4096 -> 1024; few rounds: 63.7 vs
-      // 60.0 us at 12 800 x 2048 -> 512).
+      // Width by the number of rounds: one of 128-column tiles takes 0.7 of one of 256-column tiles, below k = 512 without a
+      // gate 0.6 (256 / 128 wide, us: 65 536 x 4096 -> 1152 862 / 1349, 25 600 x 1024 -> 1024 97 / 120; 20 000 x 1024 -> 320,
+      // three rounds against four, 46.0 / 42.8; 32 768 x 160 -> 320, four against six, 21.2 / 18.9; 65 536 x
+      // 256 -> 640 gated, eleven against eighteen, 46.6 / 52.9; beside another product, which fills the SMs that a last
+      // round of few wide tiles leaves, 0.7 as well, 35.8 / 39.5 both products of 12 800 x 256 x 512).  The four-warp epilogue and deeper ring for deep K (801 vs
+      // 752 TFLOP/s at 65 536 x 4096 -> 1024; few rounds: 63.7 vs 60.0 us at 12 800 x 2048 -> 512).
       const int64_t narrow_rounds = ceil_div(ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 128), pairs);
-      int bn2 = 10 * pair_rounds <= (g.K >= 2048 ? 8 : 7) * narrow_rounds ? 256 : 128;
+      int bn2 = 10 * pair_rounds <= (short_k && !glu && !g.beside ? 6 : 7) * narrow_rounds ? 256 : 128;
       if (const char* e = tuning_env("AQT_BN")) {
         if (atoi(e) == 128 || atoi(e) == 256) bn2 = atoi(e);
       }
@@ -1435,6 +1445,7 @@ static GemmShape gemm_shape_of(const GemmParams& p) {
   g.kind = p.kind;
   g.batched = p.batch_tiles_m > 0;
   g.residual = p.residual != nullptr;
+  g.beside = p.early_trigger != 0;
   return g;
 }
 

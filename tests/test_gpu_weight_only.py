@@ -218,15 +218,18 @@ def test_weight_only_argument_errors():
     assert aqt.aqt_workspace_bytes(aqt.OP_LINEAR_WEIGHT_ONLY_X2, 128, 256, 128, 0, 4) == 8 * 256 * 128 + 8 * 128 * 128
 
 
-@pytest.mark.parametrize("M,K,N,act", [
-    (12800, 64, 1536, orc.ACT_SWISH),   # 300 pair tiles, more than four rounds
-    (9473, 528, 320, orc.ACT_NONE),     # two rounds of pairs at either width: 128 columns, the last tile half empty
-    (4097, 64, 128, orc.ACT_NONE),      # 17 pair tiles: single CTAs
-    (8000, 64, 128, orc.ACT_NONE),      # 32 pair tiles, one row of tiles 128 wide
-    (9473, 64, 320, orc.ACT_GLU),       # 128 columns of a gated layer
-    (7000, 544, 2048, orc.ACT_NONE),    # four rounds of pairs against three of single CTAs
-    (7000, 512, 2048, orc.ACT_GLU),     # the same, to K = 512 on pairs
+@pytest.mark.parametrize("M,K,N,act,plan", [
+    (12800, 132, 1536, orc.ACT_SWISH, "pair256s4e8"),   # 300 pair tiles, more than four rounds
+    (9473, 528, 320, orc.ACT_NONE, "pair128s6e8"),      # two rounds of pairs at either width: 128 columns, the last tile half empty
+    (4097, 160, 128, orc.ACT_NONE, "stream64s5e8"),     # 17 pair tiles: single CTAs
+    (9700, 512, 128, orc.ACT_NONE, "pair128s6e8"),      # 38 pair tiles, one column of tiles 128 wide
+    (9473, 160, 320, orc.ACT_GLU, "pair128s6e8"),       # 128 columns of a gated layer
+    (9500, 144, 1024, orc.ACT_GLU, "pair256s4e8"),      # 256 columns of a gated layer, two rounds
+    (7000, 544, 2048, orc.ACT_NONE, "stream256s4e8"),   # four rounds of pairs against three of single CTAs
+    (7000, 512, 2048, orc.ACT_GLU, "pair256s4e8"),      # the same, to K = 512 on pairs
+    (7000, 160, 320, orc.ACT_SWISH, "stream64s5e8"),    # a padded Swish layer of one round on single CTAs
 ])
-def test_pairs_and_their_width(M, K, N, act):
+def test_pairs_and_their_width(M, K, N, act, plan):
     """Both sides of the lines between single CTAs, pairs on 128 columns and pairs on 256."""
+    assert aqt.aqt_plan_qmatmul(M, N, K, 0, 8, act, float_kind=True, sm_count=148) == plan
     _check(M, N, K, 8, act, seed=M)
