@@ -88,8 +88,10 @@ BwdLayout bwd_layout(int64_t M, int64_t N, int64_t K) {
 // the scaled transposed weights of the other product.  Its contraction over M is cut into `batches` of `chunk` rows (a
 // multiple of 32): the tiles are few and very deep, and they fill the SM pairs that the other product leaves free, so
 // smaller ones end more evenly (half a tile's time, at 0.39 us a K-block of 32 rows, plus 3 us a tile to start it)
-// against 5 TB/s for adding the partial products.  For the 74 pairs of the one part this library is built for, so that
-// the layout needs no CUDA call.
+// against 5 TB/s for adding the partial products.  Up to 16 batches; more where the batches of that many rows are longer
+// than 1024 and three quarters of the pairs take them all at once (dw alone at 40 000 x 128 x 128: 16 batches 48 us, 36 with
+// more; but at 12 800 rows 74 pairs of short tiles get in the way of the other product, 29 -> 35 us for both).  For the
+// 74 pairs of the one part this library is built for, so that the layout needs no CUDA call.
 struct DwLayout {
   size_t wt, xt, colsum, dwp, total;
   int64_t m_pitch, batches, chunk, n_pad;
@@ -101,7 +103,10 @@ DwLayout dw_layout(int64_t M, int64_t N, int64_t K) {
   L.n_pad = (int64_t)round_up((size_t)N, 256);
   L.batches = 1;
   double best = 1e300;
-  for (int64_t b = 1; b <= 16 && (b == 1 || M / b >= 256); ++b) {
+  int64_t most = 3 * pairs / 4 / (tiles > 0 ? tiles : 1);
+  if (most > M / 1024) most = M / 1024;
+  if (most < 16) most = 16;
+  for (int64_t b = 1; b <= most && (b == 1 || M / b >= 256); ++b) {
     const double tile_us = 0.39 * (double)ceil_div(ceil_div(M, b), 32) + 3.0;
     const double rounds = (double)(tiles * b) / (double)pairs;
     const double main_us = tile_us * (rounds < 1.0 ? 1.0 : rounds + 0.5);
