@@ -279,7 +279,10 @@ dw_split_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         fence_proxy_async_smem();  // the tensor core reads the rows through the async proxy
         __syncwarp();
-        if (lane == 0) mbar_arrive_shared_release(smem_u32(&conv_bar[s]), 0);
+        if (lane == 0) {
+          if (pair_rank == 0) mbar_arrive(smem_u32(&conv_bar[s]));
+          else mbar_arrive_shared_release(smem_u32(&conv_bar[s]), 0);
+        }
       }
       it += p.k_blocks;
       if (ok && sums && m < p.M) {
