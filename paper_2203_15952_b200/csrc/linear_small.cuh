@@ -5,7 +5,7 @@
 // CTA quantizes all rows for itself, which costs the grid x x bytes in reads from L2 and each SM the conversion of all of
 // x, while its share of the weights is on the way from memory, so the form ends where that conversion costs
 // more than the launch it saves (linear_small_applies).
-// A CTA has eight warps and 16, 32 or 64 output channels; the warps cut the channels in tiles of sixteen and K in shares.
+// A CTA has eight warps (sixteen beyond 8 rows) and 16, 32 or 64 output channels; the warps cut the channels in tiles of sixteen and K in shares.
 // The products are mma.sync m16n8k32 (int8) with channels as M and rows as N, as in the chain kernel, whose order of the
 // codes in shared memory and use of packed weights (sixteen times their codes, shifted back) it shares.  For the GLU
 // forms a tile is eight value channels over their eight gates.  Sums are exact and every float operation is that of
@@ -289,7 +289,10 @@ static int lin_small_log_tiles(int N) {
 // us a call, two kernels / this one (8-bit weights, one scale a row): 8 x 1024 -> 4096 8.4 / 5.2, 16 x 2048 -> 512 10.3 / 6.4,
 // 64 x 512 -> 512 8.1 / 6.9, 32 x 1024 -> 1024 8.3 / 6.5; beyond 32 K elements the tensor-core tile of the two-kernel form
 // wins (32 x 2048 -> 512 8.5 / 10.2, 64 x 1024 -> 1024 8.2 / 11.1), but not over its few-row form, which ends at 16
-// rows (16 x 4096 -> 1024 15.4 / 10.5).
+// rows (16 x 4096 -> 1024 15.4 / 10.5).  More than 48 rows on 2 M weights or more beyond K = 256 go to the two kernels too
+// (64 x 512 -> 8192 7.7 / 8.1, with a gate 7.7 / 8.5; 64 x 512 -> 4096 7.4 / 7.5; 48 x 512 -> 8192 7.4 / 7.4).  A call by
+// itself is bound by the host, which is what these figures have in them; replayed from a graph, where launches cost
+// less, two kernels win at 1 to 8 rows from K = 2560 on too (1 x 4096 -> 32 6.6 / 7.8, by itself 8.2 / 7.6).
 static bool linear_small_applies(const LinSmallParams& p, bool packed) {
   if (p.M > kLinSmallMaxRows || p.K % (packed ? 32 : 16) != 0 || !is_aligned(p.x, 16) || p.ldx % 4 != 0) return false;
   if (lin_small_log_tiles(p.N) < 0) return false;
@@ -298,6 +301,7 @@ static bool linear_small_applies(const LinSmallParams& p, bool packed) {
   const uintptr_t x0 = reinterpret_cast<uintptr_t>(p.x), x1 = x0 + ((size_t)(p.M - 1) * p.ldx + p.K) * 4;
   const uintptr_t y0 = reinterpret_cast<uintptr_t>(p.y), y1 = y0 + ((size_t)(p.M - 1) * p.ldy + n_out) * 4;
   if (x0 < y1 && y0 < x1) return false;
+  if (p.M > 48 && p.K > 256 && (int64_t)p.N * p.K >= (2 << 20)) return false;
   const int row_tiles = lin_small_row_tiles(p.M);
   return 8ll * row_tiles * p.K <= (row_tiles <= 2 ? 65536 : 32768);
 }

@@ -41,6 +41,7 @@ def _two_calls(x, wq, s_w, bias, res, rs, bits_a, bits_w, kind, rounding, act):
     (1, 4, 32, aqt.ACT_NONE), (8, 28, 160, aqt.ACT_SWISH), (9, 2368, 1024, aqt.ACT_NONE), (16, 2372, 1056, aqt.ACT_SWISH), (17, 4736, 256, aqt.ACT_NONE),
     (32, 4740, 1024, aqt.ACT_NONE), (33, 9472, 128, aqt.ACT_SWISH), (64, 9476, 128, aqt.ACT_NONE), (64, 512, 512, aqt.ACT_SWISH), (64, 512, 544, aqt.ACT_NONE),
     (65, 512, 64, aqt.ACT_NONE), (8, 512, 8192, aqt.ACT_NONE), (16, 48, 4096, aqt.ACT_NONE), (16, 48, 4128, aqt.ACT_NONE),
+    (48, 8192, 512, aqt.ACT_SWISH), (49, 4092, 512, aqt.ACT_NONE), (49, 4096, 512, aqt.ACT_NONE),  # either side of 48 rows and of 2 M weights
     (5, 8, 64, aqt.ACT_GLU), (16, 2376, 512, aqt.ACT_GLU_SWISH), (40, 4728, 288, aqt.ACT_GLU_SWISH), (3, 4096, 1024, aqt.ACT_GLU)])
 def test_one_launch_gives_the_bits_of_two(M, N, K, act, bits_w, bits_a, kind, rounding):
     x, wq, s_w, bias, res = _case(M, N, K, bits_w, bits_a, act)
