@@ -71,8 +71,9 @@ extern "C" {
 #define AQT_STATIC_WEIGHTS 0x100 /* may be OR-ed into bits_w of the matmul entry points: the weight codes, their scales and
                                     the bias were complete before the work that precedes this call on the stream was enqueued
                                     (weights of a trained model, as opposed to weights re-quantized by the preceding call).
-                                    The kernels then fetch their weights while the preceding kernel is still draining;
-                                    everything else they touch still waits for it. */
+                                    The kernels of aqt_qmatmul_requant that keep their weights in shared memory
+                                    (K <= 1024) then fetch them while the preceding kernel is still draining; everything
+                                    else they touch still waits for it, and so do all other kernels. */
 
 /* operations for aqt_workspace_bytes */
 #define AQT_OP_QMATMUL 1
@@ -334,7 +335,9 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
  * Arithmetic: dx and dw are float matmuls on the tensor cores (tf32 operands: dy and the scaled
  * codes each enter with their upper ten fraction bits; binary32 accumulation), so each is within
  * (2^-9 + depth * 2^-24) of the sum of the absolute values of its terms, depth = N for dx, M for
- * dw.  dbias is summed in binary32 in a fixed order (the same bits on every run).
+ * dw; from 32 rows on (N, K >= 128) dy enters dw with sixteen bits instead, as dy * s_x in two bf16 terms,
+ * within (2^-15 + depth * 2^-24).  That bound holds while no dy * s_x overflows and those that
+ * matter are above 2^-110 (bf16 terms of smaller values are subnormal).  dbias is summed in binary32 in a fixed order (the same bits on every run).
  * dy        fp32 [M, N], row pitch lddy.
  * xq, s_x, s_x_kind, bits_a   the forward's activation codes and scales (as handed to aqt_qmatmul);
  *           only read for dw.

@@ -18,9 +18,9 @@
 //
 // CTA pairs: two CTAs share a 256 x 256 tile; each loads and converts its 128 rows and loads half of the
 // codes into its own shared memory on its own barriers, the leader waits for both CTAs' converters and
-// issues the pair's MMAs.  What bounds it: without any conversion a K-block takes 0.34 us of the pair (the
-// rate cuBLAS reaches in bf16), with it 0.39 to 0.45: a CTA's shared memory then moves 88 KB a K-block
-// (MMA operands 32, TMA 24, conversion 32).  More ring stages (7, 8), more converter warps (12, 16) and
+// issues the pair's MMAs.  What bounds it: at the bf16 rate that cuBLAS reaches a K-block would take 0.38 us of
+// the pair; it takes 0.39 to 0.47.  A CTA's shared memory moves 88 KB a K-block (MMA operands 32, TMA 24, conversion
+// 32): its pipe and the tensor pipe are each active for half of the time (43 and 42 % with 64 of 74 pairs at work).  More ring stages (7, 8), more converter warps (12, 16) and
 // prefetches into L2 were built and change nothing.
 #pragma once
 

@@ -118,7 +118,8 @@ struct GemmParams {
   int rounding = AQT_ROUND_NEAREST_EVEN;
   int has_y = 1;                    // 0: no fp32 output
   // The weights (codes, scales, bias) were complete before the kernel ahead of this one in the stream
-  // was enqueued, so a kernel may read them before that kernel has finished (see grid_dependency_wait).
+  // was enqueued, so a kernel may read them before that kernel has finished (see grid_dependency_wait).  Read by the
+  // requantizing kernel that keeps its weights in shared memory; the kernels of this file wait.
   int static_w = 0;
   // Float kind: the next launch on the stream does not read what this one writes and may start on SMs that fall free (it
   // sees to it that it does not end first, see DwParams::beside_previous).
@@ -1191,13 +1192,13 @@ enum GemmPlan {
   kPlanWs128E16,        // weight stationary (K <= 512), 128-column tiles, sixteen epilogue warps
   kPlanWs128E8,         // the same with eight epilogue warps: the GLU forms (64 output columns per tile)
   kPlanStream256S3E16,  // both operands streamed, 256-column tiles, shallow K
-  kPlanStream256S4E4,   //   deep K: four-warp epilogue, deeper ring
+  kPlanStream256S4E4,   //   four-warp epilogue, deeper ring (by name only: CTA pairs took over the shapes it was for)
   kPlanStream256S4E8,   //   float kind
   kPlanStream128S4E16,
-  kPlanStream128S6E4,
+  kPlanStream128S6E4,   //   float kind, deep K; 8-bit kind by name only
   kPlanStream128S4E8,   //   GLU at width 128
   kPlanStream64S5E8,
-  kPlanStream64S8E4,
+  kPlanStream64S8E4,    //   float kind, deep K; 8-bit kind by name only
   kPlanPair256S4E8,     // CTA pairs on 256-row tiles
   kPlanPair256S6E4,
   kPlanPair128S6E8,
@@ -1341,15 +1342,13 @@ static int plan_qgemm(const GemmShape& g, int sms) {
     const int v = atoi(e);
     if ((v == 64 && !glu) || v == 128 || v == 256) bn = v;
   }
-  // Deep K: operand loads bound the tile, so the ring gets the shared memory and four warps run
-  // the (short) epilogue.  Shallow K: the epilogue bounds the tile and gets more warps.
-  // Float kind: a tile's MMA time is four times that of the 8-bit kind for the same epilogue, so
+  // Deep K (float kind): operand loads bound the tile, so the ring gets the shared memory and four warps
+  // run the (short) epilogue.  Else the epilogue bounds the tile and gets more warps.
+  // Float kind, 256 columns: a tile's MMA time is four times that of the 8-bit kind for the same epilogue, so
   // eight epilogue warps keep up and the shared memory they free buys the fourth ring stage
   // (measured 2-10 % faster than three stages / sixteen warps and than four stages / four warps:
-  // 59.8 vs 62.4 us at 12 800 x 2048 x 512 Swish, 362 vs 398 us at 65 536 x 2048 x 1024 GLU).  The
-  // 8-bit kind loses with it wherever the epilogue evaluates an activation or M is small.
-  if (bn == 256 && f32) return kPlanStream256S4E8;
-  if (bn == 256) return deep_k ? kPlanStream256S4E4 : kPlanStream256S3E16;
+  // 59.8 vs 62.4 us at 12 800 x 2048 x 512 Swish, 362 vs 398 us at 65 536 x 2048 x 1024 GLU).
+  if (bn == 256) return f32 ? kPlanStream256S4E8 : kPlanStream256S3E16;
   // every epilogue warp needs at least one 32-column chunk: a GLU tile of width 128 has only
   // 64 output columns, i.e. two chunks per lane quadrant
   if (bn == 128 && glu) return kPlanStream128S4E8;

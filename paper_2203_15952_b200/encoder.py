@@ -310,7 +310,7 @@ class ConformerBlockLinears:
         self.run = LayerRunner(M, layers_for_sizing, device, **kw)
         f32 = dict(dtype=torch.float32, device=device)
         self.u = torch.empty((M, ff), **f32)
-        # q, k, v come out of one GEMM over the concatenated projection weights (N = 3d)
+        # q and k come out of one matmul over their concatenated weights (N = 2d), v out of its own: one row of the three each
         self.qkv = torch.empty((M, 3 * d), **f32)
         self.q, self.k, self.v = self.qkv[:, 0:d], self.qkv[:, d:2 * d], self.qkv[:, 2 * d:3 * d]
         self._qkv_stacks: Dict[tuple, QkvStack] = {}

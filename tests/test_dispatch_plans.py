@@ -38,12 +38,13 @@ COVERED_BY = {
 
 def _workload_matmul_shapes():
     """(M, N, K, bits_a, bits_w, act) of every matmul the drivers issue for the five configurations,
-    including the one matmul over the concatenated q, k, v projections."""
+    including the matmul over the concatenated q and k projections (and over q, k, v, for callers that keep them together)."""
     shapes = set()
     for cfg, w in gen.WORKLOADS.items():
         for s in gen.workload_layers(w):
             shapes.add((w.M, s.N, s.K, s.bits_a, s.bits_w, s.act))
         if w.kind in ("block", "stack"):
+            shapes.add((w.M, 2 * w.d, w.d, w.bits_a, w.bits_attn_w, gen.ACT_NONE))
             shapes.add((w.M, 3 * w.d, w.d, w.bits_a, w.bits_attn_w, gen.ACT_NONE))
     return sorted(shapes)
 
