@@ -728,7 +728,7 @@ def weight_only_ffn_pair(dev, steps: int = 20):
             bf16, kind = float(json.load(f)["bf16_tflops"]), "measured"
     peak = 0.5 * bf16
     return {"workload": w.name + "_i4w_fp32_activations", "value": tflops, "unit": "TFLOP/s", "ms_per_step": ms,
-            "frames_per_s": M / (ms * 1e-3), "dtype": "tf32", "gpu_launches_per_step": 4, "launch_mode": "cuda graph",
+            "frames_per_s": M / (ms * 1e-3), "dtype": "dx tf32, dw split bf16", "gpu_launches_per_step": 4, "launch_mode": "cuda graph",
             "two_term": {"what": "every activation split exactly into its tf32 part and the rest, both multiplied (operand error 2^-20 "
                                  "instead of 2^-10 of the terms): the fp32-grade form", "ms_per_step": ms_x2,
                          "value": flops / (ms_x2 * 1e-3) / 1e12, "unit": "TFLOP/s of the layer's own 2MNK flops",
@@ -782,7 +782,7 @@ def backward_ffn_layer(dev, steps: int = 20):
     ms = e0.elapsed_time(e1) / (steps * R)
     tflops = 4.0 * M * N * K / (ms * 1e-3) / 1e12
     return {"workload": "ffn_first_layer_M%d_N%d_K%d_w4a8_dx_dw_dbias" % (M, N, K), "value": tflops, "unit": "TFLOP/s", "ms_per_step": ms,
-            "dtype": "tf32", "gpu_launches_per_step": 4, "launch_mode": "cuda graph"}
+            "dtype": "dx tf32, dw split bf16", "gpu_launches_per_step": 4, "launch_mode": "cuda graph"}
 
 
 def run_case(args):
@@ -826,6 +826,22 @@ def run_case(args):
         s_x, s_w = scales(M, 1e-2), scales(N, 1e-3)
         for i in range(it):
             aqt.aqt_linear_bwd(dy, xq, s_x, wq, s_w, K=K, bits_a=8, bits_w=4)
+    elif name in ("linear_few", "weight_only_few"):
+        M, N, K = (8, 4096, 1024) if name == "linear_few" else (64, 2048, 512)
+        x, wq, s_w = torch.randn((M, K), generator=g, device=dev), torch.randint(0, 256, (N, K // 2), generator=g, dtype=torch.uint8, device=dev), scales(N, 1e-3)
+        for i in range(it):
+            if name == "linear_few":
+                aqt.aqt_linear_fwd(x, wq, s_w, bits_w=4, act=aqt.ACT_SWISH)
+            else:
+                aqt.aqt_linear_fwd_weight_only(x, wq, s_w, bits_w=4, act=aqt.ACT_SWISH)
+    elif name == "chain_few":
+        from paper_2203_15952_b200.encoder import EncoderStack, QuantLinear
+        from paper_2203_15952_b200.inputs import block_linears
+        block = [QuantLinear(s, torch.randint(0, 256, (s.N, s.K // 2), generator=g, dtype=torch.uint8, device=dev), scales(s.N, 1e-3), None).prepare()
+                 for s in block_linears(512, 2048, 4, 4, 8)]
+        stack, x = EncoderStack(8, 512, 2048, [block] * 17, dev), torch.randn((8, 512), generator=g, device=dev)
+        for i in range(it):
+            stack.forward(x)
     else:
         raise SystemExit("unknown case " + name)
     torch.cuda.synchronize()
@@ -846,7 +862,7 @@ def main():
     ap.add_argument("--no-sustained", action="store_true", help="skip the half-second sustained run of the headline step")
     ap.add_argument("--no-graph", action="store_true", help="launch every step call by call (no CUDA graph replay)")
     ap.add_argument("--case", default=None, help="run one library call a few times and exit (for profiler captures): quantize_ffn, "
-                    "quantize_large, requant_ffn1, requant_large, gemm_ffn2, gemm_large_ffn2, gemm_large_ffn1, weight_only_ffn1, bwd_ffn1")
+                    "quantize_large, requant_ffn1, requant_large, gemm_ffn2, gemm_large_ffn2, gemm_large_ffn1, weight_only_ffn1, bwd_ffn1, linear_few, weight_only_few, chain_few")
     ap.add_argument("--iters", type=int, default=4, help="--case: number of calls")
     args = ap.parse_args()
     if args.case is not None:
