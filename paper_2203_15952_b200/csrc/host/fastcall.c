@@ -24,21 +24,22 @@ typedef union {
 #define F(k) ((float)a[k].f)
 #define Z(k) ((size_t)a[k].i)
 
-/* An integer argument: what int() takes, as the ctypes calls do. */
-static int read_int(PyObject* v, int64_t* out) {
-  if (!PyLong_Check(v)) {
-    PyObject* n = PyNumber_Long(v); /* floats, index types; TypeError for None */
-    if (n == NULL) return 0;
-    const int ok = read_int(n, out);
-    Py_DECREF(n);
-    return ok;
-  }
-  /* addresses are unsigned: the low 64 bits of either reading are the same */
+/* The value of a Python integer.  Addresses are unsigned: the low 64 bits of either reading are the same. */
+static inline int read_long(PyObject* v, int64_t* out) {
   int overflow = 0;
   *out = PyLong_AsLongLongAndOverflow(v, &overflow);
+  if (__builtin_expect(*out != -1 && overflow == 0, 1)) return 1;
   if (overflow > 0) *out = (int64_t)PyLong_AsUnsignedLongLong(v);
   if (overflow < 0) PyErr_SetString(PyExc_OverflowError, "argument out of range");
-  return !((*out == -1 || overflow) && PyErr_Occurred());
+  return !PyErr_Occurred();
+}
+/* An integer argument that is none yet: what int() takes, as the ctypes calls do (TypeError for None). */
+static int read_number(PyObject* v, int64_t* out) {
+  PyObject* n = PyNumber_Long(v);
+  if (n == NULL) return 0;
+  const int ok = read_long(n, out);
+  Py_DECREF(n);
+  return ok;
 }
 
 /* types: one character per argument, 'p' (address or None), 'i' (integer) or 'f' (float). */
@@ -50,9 +51,11 @@ static int read_args(PyObject* const* args, Py_ssize_t nargs, const char* types,
     if (types[n] == 'f') {
       out[n].f = PyFloat_AsDouble(v);
       if (out[n].f == -1.0 && PyErr_Occurred()) return 0;
+    } else if (PyLong_Check(v)) {
+      if (!read_long(v, &out[n].i)) return 0;
     } else if (types[n] == 'p' && v == Py_None) {
       out[n].i = 0;
-    } else if (!read_int(v, &out[n].i)) {
+    } else if (!read_number(v, &out[n].i)) {
       return 0;
     }
   }
