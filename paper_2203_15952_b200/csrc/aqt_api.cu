@@ -713,7 +713,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
   float* y_dev = y_on_host ? reinterpret_cast<float*>(ws + L.y) : y;
   const bool chain = M <= AQT_CHAIN_MAX_ROWS;
   if (x_on_host && (size_t)M * d * 4 < (chain ? kReadInPlaceBytesChain : kReadInPlaceBytes) && is_aligned(x, 16)) {
-    if (const void* mapped = pinned_on_device(x)) {
+    if (const void* mapped = pinned_on_device(x, (size_t)M * d * 4)) {
       x = reinterpret_cast<const float*>(mapped);
       x_on_host = 0;
     }
@@ -722,7 +722,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
   if (chain) {
     // a few rows: both layers in one launch, which writes the result over the bus itself (us a call, copied or not, d =
     // 512: 16 rows 24 / 23, 64 rows 36 / 26)
-    float* y_out = y_on_host && is_aligned(y, 16) ? reinterpret_cast<float*>(pinned_on_device(y)) : nullptr;
+    float* y_out = y_on_host && is_aligned(y, 16) ? reinterpret_cast<float*>(pinned_on_device(y, (size_t)M * d * 4)) : nullptr;
     const bool y_copied = y_on_host && y_out == nullptr;
     if (y_out == nullptr) y_out = y_dev;
     if (x_on_host) AQT_RETURN_IF_CUDA(cudaMemcpyAsync(x_copy, x, (size_t)M * d * 4, cudaMemcpyHostToDevice, st));

@@ -93,14 +93,18 @@ struct RelaxedCapture {
   ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-// The address at which kernels reach pinned host memory (whose copies run beside the host and beside each other), or null.
-inline void* pinned_on_device(const void* p) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+// The address at which kernels reach these bytes of pinned host memory (whose copies run beside the host and beside each
+// other), or null.  Both ends are looked up: of a buffer that is registered only in part, a kernel must not touch the rest.
+inline void* pinned_on_device(const void* p, size_t bytes) {
+  cudaPointerAttributes a, b;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+      cudaPointerGetAttributes(&b, reinterpret_cast<const uint8_t*>(p) + (bytes > 0 ? bytes - 1 : 0)) != cudaSuccess) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || a.devicePointer == nullptr) return nullptr;
+  const bool whole = reinterpret_cast<uint8_t*>(b.devicePointer) == reinterpret_cast<uint8_t*>(a.devicePointer) + (bytes > 0 ? bytes - 1 : 0);
+  return whole ? a.devicePointer : nullptr;
 }
 
 // Below this many bytes a kernel reads its input over the bus itself: no copy to set up and to wait for.  A quantizer that
@@ -143,7 +147,8 @@ int run_between_host_copies(const float* x_host, float* x_dev, size_t x_row, con
     RelaxedCapture relaxed;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-        (x_host == nullptr || pinned_on_device(x_host) != nullptr) && (y_host == nullptr || pinned_on_device(y_host) != nullptr))
+        (x_host == nullptr || pinned_on_device(x_host, (size_t)rows * x_row) != nullptr) &&
+        (y_host == nullptr || pinned_on_device(y_host, (size_t)rows * y_row) != nullptr))
       lane = take_copy_lane(st, &alone);
     else
       (void)cudaGetLastError();

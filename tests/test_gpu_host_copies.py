@@ -52,6 +52,23 @@ def test_ffn_pieces_give_the_bits_of_one_pass(M, pinned):
     assert torch.equal(yd, ref) and torch.equal(yh, ref.cpu())
 
 
+@pytest.mark.parametrize("M", [3, 40, 300, 2000])
+def test_ffn_on_parts_of_pinned_buffers(M):
+    """Rows from the middle and from the very end of a pinned allocation, read and written in place or copied; the rows around
+    them stay as they are."""
+    w, total = _weights(), 4096  # 8 MB: the end of the tensor is the end of the allocation
+    x, y = torch.randn(total, D).pin_memory(), torch.full((total, D), 7.0).pin_memory()
+    ref = torch.empty(M, D, device="cuda")
+    for r0 in (0, 17, total - M):
+        _ffn(w, x[r0:r0 + M].cuda(), ref, _ws(M))
+        y.fill_(7.0)
+        _ffn(w, x[r0:r0 + M], y[r0:r0 + M], _ws(M))
+        torch.cuda.synchronize()
+        assert torch.equal(y[r0:r0 + M], ref.cpu())
+        assert bool((y[:r0] == 7.0).all()) and bool((y[r0 + M:] == 7.0).all())
+    assert aqt.aqt_device_status() == 0
+
+
 @pytest.mark.parametrize("scale", [aqt.SCALE_ROW, aqt.SCALE_TENSOR])
 def test_linear_host_pieces(scale):
     M, N = 5000, 256
