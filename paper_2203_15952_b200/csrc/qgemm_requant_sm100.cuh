@@ -123,6 +123,13 @@ __device__ __forceinline__ void swish16(float (&a)[16]) {
 // One slot of shared-memory exchange state (final row maxima, hand-over barriers) per accumulator
 // buffer, i.e. per set of epilogue warps: tile i of a CTA uses buffer and slot i mod 4.
 constexpr int kSlots = 4;
+
+// Sets of epilogue warps that share a tile, for a CTA that has n_my of them.  With four tiles or more each set works on one
+// of its own, in another phase than the others; with fewer, whole sets would be idle while one warp a quadrant goes through
+// a tile's four chunks one after the other, with a residual a load of it from memory between any two.  (Two blocks of width
+// 512, graph replay: 256 rows 142.7 -> 133.6 us, 1013 153.0 -> 143.5, 4736 221.0 -> 214.6, 9472 312 -> 306; three tiles or
+// more alike.)
+__device__ __forceinline__ int sets_per_tile(int n_my) { return n_my == 1 ? 4 : (n_my == 2 ? 2 : 1); }
 constexpr int kExchangeBatch = 16;  // n-tiles whose words an exchange warp asks for at once (one 16-byte load each per lane)
 
 // Called between polls of a bounded wait: false once the CTA is aborting or the limit has passed
@@ -140,7 +147,8 @@ __device__ __forceinline__ bool keep_waiting(volatile int* abort_flag, uint64_t 
 // GLU: a tile's 128 weight rows are 64 value channels and their 64 gate channels; it yields 64
 // output columns u = v * sigmoid(g) (then Swish for AQT_ACT_GLU_SWISH), 16 per epilogue warp.
 // The GLU form writes codes and scales only (no fp32 output, no residual, no nibble packing).
-template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
+// SHARED: CTAs with one or two tiles have several sets of warps work on each (sets_per_tile).
+template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
 __global__ void __launch_bounds__(32 * 20, 1)
 qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                      const __grid_constant__ CUtensorMap tm_y,
@@ -163,6 +171,8 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   __shared__ __align__(16) uint32_t row_amax[kSlots][kBM];  // final row maxima (bit patterns) of a tile awaiting pass 2
   __shared__ uint64_t ctx_ready_bar[kSlots][2];  // an exchange warp has filled its half of row_amax[.]
   __shared__ uint64_t ctx_free_bar[kSlots][2];   // the set's two warps on that half of the rows have read theirs
+  __shared__ float part_amax[kSlots][kBM];       // tile shared by several sets: a set's maxima of its columns
+  __shared__ uint64_t part_bar[kSlots][4];       // ... of lane quadrant q are there, by first set of the tile
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
@@ -181,6 +191,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   const int group = blockIdx.x / p.tiles_n;
   const int groups = gridDim.x / p.tiles_n;
   const int n_my = group < p.tiles_m ? (p.tiles_m - group + groups - 1) / groups : 0;
+  const int split = SHARED ? sets_per_tile(n_my) : 1;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -194,7 +205,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     }
     for (int b = 0; b < 4; ++b) {
       mbar_init(smem_u32(&tmem_full_bar[b]), 1);
-      mbar_init(smem_u32(&tmem_empty_bar[b]), 4);  // the four warps of the set that owns the buffer
+      mbar_init(smem_u32(&tmem_empty_bar[b]), 4 * split);  // the warps of the sets that share the buffer's tile
     }
     for (int w = 0; w < EW; ++w) mbar_init(smem_u32(&res_bar[w]), 1);
     mbar_init(smem_u32(&b_loaded_bar), 1);
@@ -202,8 +213,9 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     for (int b = 0; b < kSlots; ++b) {
       for (int h = 0; h < 2; ++h) {
         mbar_init(smem_u32(&ctx_ready_bar[b][h]), 1);
-        mbar_init(smem_u32(&ctx_free_bar[b][h]), 2);
+        mbar_init(smem_u32(&ctx_free_bar[b][h]), 2 * split);
       }
+      for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&part_bar[b][q]), split > 1 ? split - 1 : 1);
     }
     fence_barrier_init();
     fence_proxy_async_smem();
@@ -355,7 +367,11 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     // (pass 2), wait for the exchange, or wait for the tensor core.
     const int ew = warp - 2;
     const int quad = warp & 3;  // TMEM lane quadrant this warp may access
-    const int set = ew >> 2;    // accumulator buffer and tile residue (mod 4) of this warp
+    const int set = ew >> 2;
+    // The tile's sets are consecutive; this one takes chunks c_begin .. c_end - 1 of it.
+    const int part = SHARED ? set % split : 0;
+    const int c_begin = part * (4 / split), c_end = c_begin + 4 / split;
+    const int i_first = SHARED ? set / split : set, i_step = 4 / split;  // this warp's tiles of the CTA
     constexpr int CW = GLU ? 16 : 32;  // output columns per chunk; four chunks per tile
     const int row_in_tile = quad * 32 + lane;
     const uint32_t y_buf = smem_epi + ew * kStageBufBytes;
@@ -397,15 +413,15 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     if (early_w) grid_dependency_wait();  // scales of the activations, residual, outputs: everything but the weights
     const uint32_t tag = mix_tag(rp.tag, __ldcg(rp.generation + group));  // see the exchange warps
     uint32_t res_count = 0;  // residual boxes this warp has consumed (phase of its barrier)
-    if (ok && has_res && lane == 0 && set < n_my) {
-      const int r0 = (group + set * groups) * kBM + quad * 32;
+    if (ok && has_res && lane == 0 && i_first < n_my) {
+      const int r0 = (group + i_first * groups) * kBM + quad * 32, c0 = oc0 + c_begin * CW;
       mbar_arrive_expect_tx(smem_u32(&res_bar[ew]), kStageBufBytes);
-      tma_load_2d(y_buf, &tm_r, oc0 < n_out ? oc0 : 0, r0 < p.M ? r0 : 0, smem_u32(&res_bar[ew]));
+      tma_load_2d(y_buf, &tm_r, c0 < n_out ? c0 : 0, r0 < p.M ? r0 : 0, smem_u32(&res_bar[ew]));
     }
 
-    const uint32_t buf = (uint32_t)set;
+    const uint32_t buf = (uint32_t)i_first;  // accumulator buffer and exchange slot of this warp's tiles (i mod 4)
     const uint32_t tbase = tmem_base + buf * BN + ((uint32_t)(quad * 32) << 16);
-    for (int i = set; ok && i < n_my; i += 4) {
+    for (int i = i_first; ok && i < n_my; i += i_step) {
       const int tm = group + i * groups;
       const uint32_t aph = (uint32_t)(i >> 2) & 1u;
       const int row0_warp = tm * kBM + quad * 32;
@@ -417,7 +433,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       // -------------------------------------------------------------- pass 1: u, row maxima; u back to TMEM
       float amax = 0.0f;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = c_begin; c < c_end; ++c) {
         const int col = c * CW;
         const bool cols_ok = oc0 + col < n_out;  // columns beyond N contribute nothing
         const uint32_t c_sw = smem_scale + (uint32_t)col * 4, c_bias = c_sw + BN * 4;
@@ -490,35 +506,47 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             if (lane == 0) {
               if (cols_ok && row0_warp < p.M) tma_store_2d(&tm_y, y_buf, oc0 + col, row0_warp);
               tma_store_commit();
-              if (has_res) {
+              const bool more_here = c + 1 < c_end;
+              if (has_res && (more_here || i + i_step < n_my)) {
                 // the next chunk's residual goes into the same buffer once this store has read it out
                 tma_store_wait_read<0>();
-                const bool more_here = c + 1 < 4;
-                if (more_here || i + 4 < n_my) {
-                  const int ncol = oc0 + (more_here ? col + CW : 0);
-                  const int nr = (more_here ? tm : tm + 4 * groups) * kBM + quad * 32;
-                  mbar_arrive_expect_tx(smem_u32(&res_bar[ew]), kStageBufBytes);
-                  tma_load_2d(y_buf, &tm_r, ncol < n_out ? ncol : 0, nr < p.M ? nr : 0, smem_u32(&res_bar[ew]));
-                }
+                const int ncol = oc0 + (more_here ? col + CW : c_begin * CW);
+                const int nr = (more_here ? tm : tm + i_step * groups) * kBM + quad * 32;
+                mbar_arrive_expect_tx(smem_u32(&res_bar[ew]), kStageBufBytes);
+                tma_load_2d(y_buf, &tm_r, ncol < n_out ? ncol : 0, nr < p.M ? nr : 0, smem_u32(&res_bar[ew]));
               }
             }
           }
         }
       }
       if (!ok) break;
-      // this CTA's maxima of the tile's rows, each tagged valid: one word per row, straight from the registers
-      st_relaxed_gpu_64(rp.exchange + ((size_t)tm * p.tiles_n + tn) * kBM + row_in_tile, ((uint64_t)tag << 32) | __float_as_uint(amax));
+      // This CTA's maxima of the tile's rows, each tagged valid: one word per row.  Of a tile that several sets share, the
+      // first set's warp publishes the maximum of all parts (a CTA that shares tiles has one for every group of sets, so
+      // the barrier is waited on once).
+      if (SHARED && split > 1) {
+        part_amax[set][row_in_tile] = amax;
+        __syncwarp();
+        const uint32_t bar = smem_u32(&part_bar[set - part][quad]);
+        if (part != 0) {
+          if (lane == 0) mbar_arrive(bar);
+        } else {
+          if (!mbar_wait(bar, 0, &abort_flag, t_start)) { ok = false; break; }
+          for (int s = 1; s < split; ++s) amax = fmaxf(amax, part_amax[set + s][row_in_tile]);
+        }
+      }
+      if (part == 0)
+        st_relaxed_gpu_64(rp.exchange + ((size_t)tm * p.tiles_n + tn) * kBM + row_in_tile, ((uint64_t)tag << 32) | __float_as_uint(amax));
 
       // -------------------------------------------------------------- pass 2: scale, codes
-      if (!mbar_wait(smem_u32(&ctx_ready_bar[set][quad >> 1]), aph, &abort_flag, t_start)) { ok = false; break; }
-      const float amax_row = __uint_as_float(row_amax[set][row_in_tile]);
+      if (!mbar_wait(smem_u32(&ctx_ready_bar[buf][quad >> 1]), aph, &abort_flag, t_start)) { ok = false; break; }
+      const float amax_row = __uint_as_float(row_amax[buf][row_in_tile]);
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&ctx_free_bar[set][quad >> 1]));
+      if (lane == 0) mbar_arrive(smem_u32(&ctx_free_bar[buf][quad >> 1]));
       const ScaleCtx sc = make_scale_ctx_zeros(amax_row, rp.qmax_out);
-      if (tn == 0 && m < p.M) rp.s_out[m] = sc.s;
+      if (tn == 0 && part == 0 && m < p.M) rp.s_out[m] = sc.s;
       tmem_st_wait();  // this warp's stores of pass 1
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = c_begin; c < c_end; ++c) {
         const int col = c * CW;
         const int oc = oc0 + col;
         const bool cols_ok = oc < n_out;
@@ -526,7 +554,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           uint32_t u[16], w[4];
           tmem_ld_32x16(tbase + col, u);
           tmem_ld_wait();
-          if (c == 3) {
+          if (c + 1 == c_end) {
             // the tile has been read out by this warp: the accumulator buffer goes back to the MMA
             tc_fence_before();
             __syncwarp();
@@ -539,7 +567,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           uint32_t u[32], w[8];
           tmem_ld_32x32(tbase + col, u);
           tmem_ld_wait();
-          if (c == 3) {
+          if (c + 1 == c_end) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tmem_empty_bar[buf]));
@@ -602,8 +630,8 @@ static bool requant_applies(int64_t M, int64_t N, int64_t K, int act, bool with_
   return ceil_div(K, kBK) <= kRequantDeepKBlocks && !with_y && (!glu || !pack_out);
 }
 
-template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
-static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, RequantParams rp,
+template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
+static int launch_requant_form(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, RequantParams rp,
                                void* exchange, cudaStream_t st) {
   using Cfg = RequantCfg<WITH_Y, DEEP>;
   GemmParams& p = rp.g;
@@ -635,7 +663,7 @@ static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, floa
       if (rc != AQT_OK) return rc;
     }
   }
-  auto kernel = qgemm_requant_kernel<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP>;
+  auto kernel = qgemm_requant_kernel<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, SHARED>;
   static std::atomic<uint64_t> smem_opted_in{0};
   rc = ensure_dynamic_smem(kernel, Cfg::kSmemBytes, smem_opted_in);
   if (rc != AQT_OK) return rc;
@@ -647,6 +675,17 @@ static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, floa
   // SMs occupied for seconds, the bounded waits give up and report AQT_ERR_TIMEOUT.
   return launch_pdl(kernel, dim3((unsigned)(groups * p.tiles_n), 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 1, tm_a, tm_b,
                     tm_y, tm_r, rp);
+}
+
+template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
+static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, const RequantParams& rp,
+                               void* exchange, cudaStream_t st) {
+  const int sms = sm_count();
+  if (sms <= 0) return AQT_ERR_CUDA;
+  const int64_t groups = sms / ceil_div(rp.g.N, 128);
+  if (ceil_div(rp.g.M, kBM) <= 2 * groups)
+    return launch_requant_form<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, true>(a, b, q_out, y, ldy, rp, exchange, st);
+  return launch_requant_form<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, false>(a, b, q_out, y, ldy, rp, exchange, st);
 }
 
 // a: int8 [M, K]; b: int8 [N, K] or (b_packed) nibbles [N, K/2]; y may be null (then no fp32 output

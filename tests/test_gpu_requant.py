@@ -116,6 +116,14 @@ def test_requant_with_residual_stream_many_tiles_per_cta():
     _run(5000, 512, 256, 8, 8, aqt.ACT_NONE, False, True, 4, aqt.ROUND_HALF_UP_FLOOR, True)
 
 
+@pytest.mark.parametrize("M,N,K", [(36 * 128 + 5, 512, 512), (37 * 128 + 1, 512, 128), (74 * 128, 512, 256), (74 * 128 + 1, 512, 64),
+                                   (9 * 128 + 7, 2048, 64), (18 * 128 + 1, 2048, 64)])
+@pytest.mark.parametrize("with_res", [True, False])
+def test_requant_sets_that_share_a_tile(M, N, K, with_res):
+    # one, two and three tiles per CTA, and CTAs with one and two in the same launch (148 SMs: 37 or 9 groups of CTAs)
+    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False)
+
+
 def test_requant_many_tiles_per_cta():
     """More m-tiles than groups of CTAs: every TMEM buffer and both exchange slots are reused."""
     _run(12800, 2048, 512, 8, 4, aqt.ACT_SWISH, False, False, 8, aqt.ROUND_NEAREST_EVEN, False)
