@@ -72,8 +72,9 @@ extern "C" {
                                     the bias were complete before the work that precedes this call on the stream was enqueued
                                     (weights of a trained model, as opposed to weights re-quantized by the preceding call).
                                     The kernels of aqt_qmatmul_requant that keep their weights in shared memory
-                                    (K <= 1024) then fetch them while the preceding kernel is still draining; everything
-                                    else they touch still waits for it, and so do all other kernels. */
+                                    (K <= 1024), and those for outputs of a few tiles, then fetch them while the preceding
+                                    kernel is still draining; everything else they touch still waits for it, and so do
+                                    all other kernels. */
 
 /* operations for aqt_workspace_bytes */
 #define AQT_OP_QMATMUL 1
@@ -151,7 +152,9 @@ int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, 
  * sm_count_or_0 > 0 plans for a device with that many multiprocessors, 0 for the current device
  * (148 if there is none).  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
  * aqt_linear_bwd with K in elements.  (No counterpart in the paper: the choice of tile shapes is
- * this library's.)  name_out receives a NUL-terminated string of at most name_bytes bytes.
+ * this library's.)  Outputs of a few tiles run in a kernel of their own ahead of this choice
+ * (K <= 512, and deeper gate forms); the name is then that of the configuration behind it, which
+ * acc_debug and aqt_qmatmul_with_plan reach.  name_out receives a NUL-terminated string of at most name_bytes bytes.
  */
 int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int float_kind,
                      int sm_count_or_0, char* name_out, size_t name_bytes);
@@ -198,6 +201,20 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
                         int64_t N, int64_t K, int bits_a, int bits_w, int act, int bits_out, int rounding,
                         int pack_out, void* q_out, float* s_out, float* y, int64_t ldy, void* workspace,
                         size_t workspace_bytes, void* stream);
+
+/*
+ * aqt_qmatmul_requant_from -- one matmul over N stacked output channels of which the last ones, from
+ * column `first` on, are quantized for the next layer (query, key and value projections: only the value
+ * is the input of a quantized layer):
+ *   y            = aqt_qmatmul(act NONE, no residual), fp32 [M, N] with row pitch ldy
+ *   q_out, s_out = aqt_quantize(y[:, first:], axis = AQT_AXIS_ROW, bits_out, rounding), int8 [M, N - first] dense, fp32 [M]
+ * workspace as for aqt_qmatmul_requant of N channels.  first and N are multiples of 16.  One launch where the
+ * output has few tiles, else aqt_qmatmul over the first channels and aqt_qmatmul_requant over the others.
+ */
+int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w,
+                             const float* bias, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int bits_out,
+                             int rounding, void* q_out, float* s_out, float* y, int64_t ldy, void* workspace,
+                             size_t workspace_bytes, void* stream);
 
 /*
  * aqt_linear_fwd -- the whole layer for fp32 activations: aqt_quantize(x, axis = K) with a

@@ -31,7 +31,7 @@ STATIC_WEIGHTS = 0x100  # OR into bits_w: the weights were complete before the p
 
 EXPORTS = ("aqt_version", "aqt_status_string", "aqt_quantize", "aqt_pack_int4", "aqt_unpack_int4", "aqt_qmatmul",
            "aqt_linear_fwd", "aqt_linear_fwd_host", "aqt_workspace_bytes", "aqt_device_status", "aqt_qmatmul_w4_noalloc",
-           "aqt_selftest_bounded_wait", "aqt_qmatmul_requant", "aqt_linear_fwd_weight_only", "aqt_linear_bwd",
+           "aqt_selftest_bounded_wait", "aqt_qmatmul_requant", "aqt_qmatmul_requant_from", "aqt_linear_fwd_weight_only", "aqt_linear_bwd",
            "aqt_plan_qmatmul", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_chain_fwd", "aqt_selftest_sfu_rate")
 NOALLOC_MAX_WEIGHT_BYTES = 4 << 20
 CHAIN_MAX_ROWS = 112
@@ -326,6 +326,20 @@ def aqt_qmatmul_requant(xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s
                                q_out.data_ptr(), s_out.data_ptr(), _addr(y), _pitch(y), ws, ws_bytes, _raw_stream(stream))
     if st != AQT_OK:
         raise AqtError("aqt_qmatmul_requant", st)
+    return q_out, s_out, y
+
+
+def aqt_qmatmul_requant_from(first: int, xq: torch.Tensor, s_x: torch.Tensor, wq: torch.Tensor, s_w: torch.Tensor,
+                             bias: Optional[torch.Tensor] = None, *, K: int, bits_a: int = 8, bits_w: int = 8, s_x_kind: int = SCALE_ROW,
+                             bits_out: int = 8, rounding: int = ROUND_NEAREST_EVEN, q_out: torch.Tensor, s_out: torch.Tensor, y: torch.Tensor,
+                             workspace: torch.Tensor, stream=None):
+    """One matmul over stacked output channels, those from `first` on also quantized for the next layer: y fp32 [M, N],
+    q_out int8 [M, N - first], s_out [M]."""
+    st = _fc().qmatmul_requant_from(first, xq.data_ptr(), s_x.data_ptr(), s_x_kind, wq.data_ptr(), s_w.data_ptr(), _addr(bias), xq.shape[0],
+                                    wq.shape[0], K, bits_a, bits_w, bits_out, rounding, q_out.data_ptr(), s_out.data_ptr(), y.data_ptr(),
+                                    y.stride(0), workspace.data_ptr(), workspace.numel(), _raw_stream(stream))
+    if st != AQT_OK:
+        raise AqtError("aqt_qmatmul_requant_from", st)
     return q_out, s_out, y
 
 

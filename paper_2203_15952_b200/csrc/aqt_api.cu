@@ -6,6 +6,7 @@
 #include "qgemm_sm100.cuh"
 #include "dw_split_sm100.cuh"
 #include "qgemm_requant_sm100.cuh"
+#include "qgemm_few_tiles_sm100.cuh"
 #include "qgemv_small_m.cuh"
 #include "quantize.cuh"
 #include "chain_small_m.cuh"
@@ -217,14 +218,68 @@ int run_small_m(const void* xq, bool a_packed, const float* s_x, int s_x_kind, c
   return launch_small_m(sp, st);
 }
 
+// The matmul for outputs of a few tiles, the columns from rq_first on quantized (rq_first = the output's columns: none).
+// Arguments are checked, packed activations expanded; scratch: where packed weights that the kernel does not expand go.
+int run_few_tiles(int bn, const int8_t* a_codes, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
+                  const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_w, bool static_w,
+                  int act, int64_t rq_first, int bits_out, int rounding, void* q_out, float* s_out, float* y, int64_t ldy, uint8_t* scratch,
+                  void* exchange, cudaStream_t st) {
+  const void* b_codes = wq;
+  bool b_packed = false;
+  if (is_packed(bits_w)) {
+    if (K % 32 == 0 && ceil_div(K, kBK) <= kWsMaxKBlocks) {
+      b_packed = true;
+    } else {
+      const int rc = launch_unpack_int4(reinterpret_cast<const uint8_t*>(wq), N * K / 2, reinterpret_cast<int8_t*>(scratch), st);
+      if (rc != AQT_OK) return rc;
+      b_codes = scratch;
+    }
+  }
+  FewTilesParams fp;
+  GemmParams& p = fp.rp.g;
+  p.s_x = s_x;
+  p.s_w = s_w;
+  p.bias = bias;
+  p.residual = residual;
+  p.acc_debug = nullptr;
+  p.ldr = ldr;
+  p.residual_scale = residual_scale;
+  p.s_x_kind = s_x_kind;
+  p.act = act;
+  p.M = (int)M;
+  p.N = (int)N;
+  p.K = (int)K;
+  p.n_out = is_glu(act) ? (int)(N / 2) : (int)N;
+  p.small_acc = 0;
+  p.static_w = (static_w && (!is_packed(bits_w) || b_packed)) ? 1 : 0;  // not for weights unpacked into the workspace just now
+  fp.rp.q_out = reinterpret_cast<uint8_t*>(q_out);
+  fp.rp.s_out = s_out;
+  fp.rp.exchange = reinterpret_cast<uint64_t*>(exchange);
+  fp.rp.generation = nullptr;
+  fp.rp.tag = 0;
+  fp.rp.qmax_out = qmax_of(bits_out);
+  fp.rp.rounding = rounding;
+  fp.rp.pack_out = 0;
+  fp.rq_first = (int)rq_first;
+  fp.b_packed = b_packed ? 1 : 0;
+  return launch_few_tiles(bn, a_codes, b_codes, y, ldy, fp, st);
+}
+
 // Codes already in int8 containers for A; B possibly packed.  ws holds B's unpacked copy.
 int qmatmul_i8a(const int8_t* a_codes, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
                 const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w,
-                int act, float* y, int64_t ldy, int32_t* acc_debug, uint8_t* ws, cudaStream_t st, int forced_plan = kPlanNone) {
+                int act, float* y, int64_t ldy, int32_t* acc_debug, uint8_t* ws, cudaStream_t st, int forced_plan = kPlanNone,
+                bool static_w = false) {
   if (forced_plan == kPlanNone && small_m_applies(M, K)) {
     // a few rows: weight-bandwidth-bound kernel, packed weights read as they are
     return run_small_m(a_codes, false, s_x, s_x_kind, wq, is_packed(bits_w), s_w, bias, residual, ldr, residual_scale, M, N, K, act, y, ldy,
                        acc_debug, st);
+  }
+  if (forced_plan == kPlanNone && acc_debug == nullptr && sm_count() > 0) {
+    const int bn = few_tiles_bn(M, N, K, act, -1, sm_count());
+    if (bn != 0)
+      return run_few_tiles(bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w, act,
+                           is_glu(act) ? N / 2 : N, 8, AQT_ROUND_NEAREST_EVEN, nullptr, nullptr, y, ldy, ws, nullptr, st);
   }
   // 4-bit weights: the weight-stationary kernel (K <= 512) sign-extends them itself in shared
   // memory after TMA staging; deeper K takes a one-off sign-extended copy in the workspace.
@@ -363,6 +418,7 @@ static int qmatmul_entry(const void* xq, const float* s_x, int s_x_kind, const v
                          const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_a,
                          int bits_w, int act, float* y, int64_t ldy, int32_t* acc_debug, void* workspace, size_t workspace_bytes,
                          void* stream, int forced_plan) {
+  const bool static_w = (bits_w & AQT_STATIC_WEIGHTS) != 0;
   bits_w &= ~AQT_STATIC_WEIGHTS;
   int rc = validate_matmul_shape(M, N, K, bits_a, bits_w, act, s_x_kind);
   if (rc != AQT_OK) return rc;
@@ -394,7 +450,7 @@ static int qmatmul_entry(const void* xq, const float* s_x, int s_x_kind, const v
     ws += round_up((size_t)M * (size_t)K, 256);
   }
   return qmatmul_i8a(a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y,
-                     ldy, acc_debug, ws, st, forced_plan);
+                     ldy, acc_debug, ws, st, forced_plan, static_w);
 }
 
 int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
@@ -463,7 +519,21 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
 
-  if (!requant_applies(M, N, K, act, y != nullptr, pack_out != 0) && rowquant_pair_applies(M, N, K, act, y != nullptr, pack_out != 0)) {
+  const bool ws_form = requant_applies(M, N, K, act, y != nullptr, pack_out != 0);
+  const bool pair_form = !ws_form && rowquant_pair_applies(M, N, K, act, y != nullptr, pack_out != 0);
+  const int few_bn = pack_out || (!ws_form && !pair_form && y == nullptr) || sm_count() <= 0 ? 0 : few_tiles_bn(M, N, K, act, 0, sm_count());
+  if (few_bn != 0 && few_tiles_exchange_bytes(M, N, few_bn) <= workspace_bytes - mm_bytes) {
+    const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
+    if (is_packed(bits_a)) {
+      rc = launch_unpack_int4(reinterpret_cast<const uint8_t*>(xq), M * K / 2, reinterpret_cast<int8_t*>(ws), st);
+      if (rc != AQT_OK) return rc;
+      a_codes = reinterpret_cast<const int8_t*>(ws);
+      ws += round_up((size_t)M * (size_t)K, 256);
+    }
+    return run_few_tiles(few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w != 0, act, 0,
+                             bits_out, rounding, q_out, s_out, y, ldy, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);
+  }
+  if (pair_form) {
     // Deep K (the second feed-forward layers): the CTA-pair kernel with the row-quantizing epilogue
     const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
     if (is_packed(bits_a)) {
@@ -506,7 +576,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
     if (sms <= 0) return AQT_ERR_CUDA;
     return launch_qgemm_rowquant(rowquant_plan(M, N, K, sms), a_codes, b_codes, y, ldy, p, st);
   }
-  if (!requant_applies(M, N, K, act, y != nullptr, pack_out != 0)) {
+  if (!ws_form) {
     // Shapes the fused kernels do not take: the two steps one after the other, through y.
     if (y == nullptr) return AQT_ERR_UNSUPPORTED;
     rc = aqt_qmatmul(xq, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y, ldy, nullptr,
@@ -560,6 +630,43 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   return launch_requant(a_codes, b_codes, b_packed, q_out, y, ldy, rp, reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);
 }
 
+int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
+                             int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int bits_out, int rounding, void* q_out, float* s_out,
+                             float* y, int64_t ldy, void* workspace, size_t workspace_bytes, void* stream) {
+  const int static_w = (bits_w & AQT_STATIC_WEIGHTS) ? 1 : 0, width = bits_w & ~AQT_STATIC_WEIGHTS;
+  int rc = validate_matmul_shape(M, N, K, bits_a, width, AQT_ACT_NONE, s_x_kind);
+  if (rc != AQT_OK) return rc;
+  if (first < 0 || first >= N || first % 16 != 0 || N % 16 != 0 || !quant_bits_ok(bits_out)) return AQT_ERR_BADARG;
+  if (rounding != AQT_ROUND_HALF_UP_FLOOR && rounding != AQT_ROUND_NEAREST_EVEN) return AQT_ERR_BADARG;
+  if (M == 0) return AQT_OK;
+  if (xq == nullptr || s_x == nullptr || wq == nullptr || s_w == nullptr || q_out == nullptr || s_out == nullptr || y == nullptr) return AQT_ERR_BADARG;
+  if (ldy < N || ldy % 4 != 0) return AQT_ERR_BADARG;
+  if (!is_aligned(xq, 16) || !is_aligned(wq, 16) || !is_aligned(q_out, 16) || !is_aligned(s_w, 16) || !is_aligned(s_x, 4) || !is_aligned(s_out, 4) ||
+      !is_aligned(y, 16) || (bias != nullptr && !is_aligned(bias, 16)))
+    return AQT_ERR_ALIGN;
+  const size_t mm_bytes = round_up(ws_qmatmul(M, N, K, bits_a, width), 256);
+  if (workspace == nullptr || workspace_bytes < mm_bytes + requant_exchange_bytes(M, N)) return AQT_ERR_WORKSPACE;
+  if (!is_aligned(workspace, 256)) return AQT_ERR_ALIGN;
+  rc = check_device();
+  if (rc != AQT_OK) return rc;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const int sms = sm_count();
+  const int bn = sms > 0 && !is_packed(bits_a) ? few_tiles_bn(M, N, K, AQT_ACT_NONE, first, sms) : 0;
+  if (bn != 0)
+    return run_few_tiles(bn, reinterpret_cast<const int8_t*>(xq), s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, width, static_w != 0,
+                             AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, reinterpret_cast<uint8_t*>(workspace),
+                             reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);
+  // the two parts one after the other (row `first` of the weights keeps the 16-byte alignment: `first` and K are multiples of 16)
+  if (first > 0) {
+    rc = aqt_qmatmul(xq, s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, first, K, bits_a, width, AQT_ACT_NONE, y, ldy, nullptr, workspace,
+                     workspace_bytes, stream);
+    if (rc != AQT_OK) return rc;
+  }
+  const uint8_t* w_rest = reinterpret_cast<const uint8_t*>(wq) + first * (is_packed(width) ? K / 2 : K);
+  return aqt_qmatmul_requant(xq, s_x, s_x_kind, w_rest, s_w + first, bias == nullptr ? nullptr : bias + first, nullptr, 0, 0.0f, M, N - first, K,
+                             bits_a, bits_w, AQT_ACT_NONE, bits_out, rounding, 0, q_out, s_out, y + first, ldy, workspace, workspace_bytes, stream);
+}
+
 int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w, const float* bias, const float* residual,
                    int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w,
                    int a_scale_kind, int rounding, int act, float* y, int64_t ldy, void* workspace, size_t workspace_bytes,
@@ -602,9 +709,9 @@ int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w
   rc = quantize_entry(x, M, K, ldx, bits_a, axis, rounding, 0, codes, s_x, stream, one_scale ? s_x + 1 : nullptr,
                       (int64_t)(round_up((size_t)M * 4, 256) / 4) - 1);
   if (rc != AQT_OK) return rc;
-  // Step 2: integer matmul + de-quantizing epilogue.
+  // Step 2: integer matmul + de-quantizing epilogue.  (The weights were complete before the quantizer was enqueued.)
   return qmatmul_i8a(codes, s_x, a_scale_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y,
-                     ldy, nullptr, ws_mm, st);
+                     ldy, nullptr, ws_mm, st, kPlanNone, true);
 }
 
 int aqt_linear_fwd_host(const float* x, int x_on_host, const void* wq, const float* s_w, const float* bias, int64_t M,
@@ -755,7 +862,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
     // The codes of u are still in L2: narrower tiles that read them twice, and start and drain sooner, then beat the tile
     // over all 512 columns (12 800 x 512: 62.3 -> 59.0 us the pair)
     const bool wide = !small_m_applies(rows, ff) && plan_qgemm(GemmShape{rows, d, ff, AQT_ACT_NONE, 0, false}, sms) == kPlanPair512S3E16;
-    return qmatmul_entry(q2, s2, AQT_SCALE_ROW, w2q, s_w2, bias2, nullptr, 0, 0.0f, rows, d, ff, bits_mm, bits_w2, AQT_ACT_NONE, yr, d, nullptr,
+    return qmatmul_entry(q2, s2, AQT_SCALE_ROW, w2q, s_w2, bias2, nullptr, 0, 0.0f, rows, d, ff, bits_mm, bits_w2 | AQT_STATIC_WEIGHTS, AQT_ACT_NONE, yr, d, nullptr,
                          ws + L.mm, mm_bytes, stream, wide ? kPlanPair256S4E8 : kPlanNone);
   });
 }

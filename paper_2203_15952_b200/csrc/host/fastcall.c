@@ -91,6 +91,8 @@ ENTRY(qmatmul_with_plan, "pppippppifiiiiiipippip",
 ENTRY(qmatmul_requant, "ppippppifiiiiiiiiipppipip",
       fn(P(0), P(1), N(2), P(3), P(4), P(5), P(6), I(7), F(8), I(9), I(10), I(11), N(12), N(13), N(14), N(15), N(16), N(17), P(18), P(19),
          P(20), I(21), P(22), Z(23), P(24)))
+ENTRY(qmatmul_requant_from, "ippippp" "iiiiiii" "ppp" "ipip",
+      fn(I(0), P(1), P(2), N(3), P(4), P(5), P(6), I(7), I(8), I(9), N(10), N(11), N(12), N(13), P(14), P(15), P(16), I(17), P(18), Z(19), P(20)))
 ENTRY(linear_fwd, "pippppifiiiiiiiipipip",
       fn(P(0), I(1), P(2), P(3), P(4), P(5), I(6), F(7), I(8), I(9), I(10), N(11), N(12), N(13), N(14), N(15), P(16), I(17), P(18), Z(19), P(20)))
 ENTRY(linear_fwd_weight_only, "pippppifiiiiiipipip",
@@ -236,6 +238,7 @@ static PyObject* w_open(PyObject* self, PyObject* path) {
   RESOLVE(quantize)
   RESOLVE(qmatmul)
   RESOLVE(qmatmul_requant)
+  RESOLVE(qmatmul_requant_from)
   RESOLVE(linear_fwd)
   RESOLVE(linear_fwd_weight_only)
   RESOLVE(linear_bwd)
@@ -251,6 +254,7 @@ static PyMethodDef methods[] = {{"open", w_open, METH_O, "Resolve the entry poin
                                 METHOD(quantize),
                                 METHOD(qmatmul),
                                 METHOD(qmatmul_requant),
+                                METHOD(qmatmul_requant_from),
                                 METHOD(linear_fwd),
                                 METHOD(linear_fwd_weight_only),
                                 METHOD(linear_bwd),

@@ -210,24 +210,26 @@ class LayerRunner:
 
     def matmul(self, layer: QuantLinear, xq: torch.Tensor, s_x: torch.Tensor, y: torch.Tensor,
                residual: Optional[torch.Tensor] = None, residual_scale: float = 1.0, plan: Optional[str] = None) -> torch.Tensor:
-        """Integer matmul + epilogue of `layer` on already-quantized activations (int8 containers); plan: see aqt_qmatmul."""
+        """Integer matmul + epilogue of `layer` on already-quantized activations (int8 containers), behind a kernel that the caller
+        enqueued after the weights were complete; plan: see aqt_qmatmul."""
         s = layer.spec
         return aqt.aqt_qmatmul(xq, s_x, layer.mm_weight, layer.s_w, layer.bias, residual, residual_scale, K=s.K, bits_a=_container_bits(s.bits_a),
-                               bits_w=layer.mm_bits, act=s.act, s_x_kind=self.a_scale_kind, y=y, workspace=self.workspace, plan=plan)
+                               bits_w=layer.mm_bits | aqt.STATIC_WEIGHTS, act=s.act, s_x_kind=self.a_scale_kind, y=y, workspace=self.workspace,
+                               plan=plan)
 
     def fuses_requant(self, layer: QuantLinear, with_y: bool = True) -> bool:
-        """True if `layer`'s matmul can quantize its own output rows in its epilogue (the GLU
-        forms and 512 < K <= 1024 only when the fp32 output is not wanted as well; 1024 < K < 2048
-        not at all)."""
+        """True if `layer`'s matmul and the quantizer of its output rows go into one call: with the fp32 output any but the GLU
+        forms (the library runs the two steps one after the other where no kernel does both), without it what such a kernel
+        exists for (not 1024 < K < 2048)."""
         s = layer.spec
         ok = self.a_scale_kind == aqt.SCALE_ROW and s.K % 16 == 0 and s.n_out % 32 == 0 and s.N <= 128 * 148
         glu = s.act in (aqt.ACT_GLU, aqt.ACT_GLU_SWISH)
+        if with_y:
+            return ok and not glu
         if s.K >= 2048:
             # deep K: the CTA-pair kernel quantizes its rows (no GLU; at most 16 column parts per row)
             return ok and not glu and self.M > 128 and s.N <= 2048
-        if glu or s.K > 512:
-            return ok and not with_y and s.K <= 1024
-        return ok
+        return ok and s.K <= 1024
 
     def code_buffers(self, role: str, cols: int):
         """Codes (int8 containers) and row scales of an activation tensor, one pair of buffers per role."""
@@ -334,28 +336,27 @@ class ConformerBlockLinears:
                 keep[name] = t.clone()
 
         parity = keep is not None  # then every fp32 intermediate is written as well
+        wq, s_w, bias = self._fused_qkv(L)  # (the first time this writes them: ahead of kernels that wait for it)
         hq, hs = self._ffn(L[0], L[1], h_in, self.h_a, 0.5, parity, note, xq=in_codes[0] if in_codes else None,
                            xs=in_codes[1] if in_codes else None, out_role="ha", out_bits=L[2].spec.bits_a, static=not first or in_codes is None)
         note(L[1].spec.name, self.h_a)
         # q, k, v read the same h: its codes come out of the second feed-forward matmul's epilogue
-        # (or one quantizer pass; the codes do not depend on the consumer).  q and k run as one matmul over
-        # their concatenated output channels; v is also needed as codes, which its own matmul's epilogue
-        # produces where it can.
+        # (or one quantizer pass; the codes do not depend on the consumer).  They run as one matmul over their
+        # concatenated output channels; v is also needed as codes, which its columns' epilogue produces where it
+        # can (batches of many rows: two launches, q and k, then v).
         if hq is None:
             hq, hs = run.quantize_input(self.h_a, L[2].spec.bits_a)
-        wq, s_w, bias = self._fused_qkv(L)
         d = self.d
-        args = dict(K=d, bits_a=_container_bits(L[2].spec.bits_a), bits_w=L[2].mm_bits, act=aqt.ACT_NONE, s_x_kind=run.a_scale_kind,
-                    workspace=run.workspace)
-        aqt.aqt_qmatmul(hq, hs, wq[:2 * d], s_w[:2 * d], None if bias is None else bias[:2 * d], None, 1.0, y=self.qkv[:, :2 * d], **args)
-        bias_v = None if bias is None else bias[2 * d:]
+        args = dict(K=d, bits_a=_container_bits(L[2].spec.bits_a), s_x_kind=run.a_scale_kind, workspace=run.workspace)
         bq = bs = cq = cs = vq = vs = None
         if run.fuses_requant(L[4]):
             vq, vs = run.code_buffers("v", d)
-            aqt.aqt_qmatmul_requant(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, bits_out=L[5].spec.bits_a, rounding=run.rounding, q_out=vq,
-                                    s_out=vs, y=self.v, **dict(args, bits_w=L[4].mm_bits | aqt.STATIC_WEIGHTS))
+            aqt.aqt_qmatmul_requant_from(2 * d, hq, hs, wq, s_w, bias, bits_w=L[4].mm_bits | aqt.STATIC_WEIGHTS, bits_out=L[5].spec.bits_a,
+                                         rounding=run.rounding, q_out=vq, s_out=vs, y=self.qkv, **args)
         else:
-            aqt.aqt_qmatmul(hq, hs, wq[2 * d:], s_w[2 * d:], bias_v, None, 1.0, y=self.v, **args)
+            args.update(bits_w=L[2].mm_bits, act=aqt.ACT_NONE)
+            aqt.aqt_qmatmul(hq, hs, wq[:2 * d], s_w[:2 * d], None if bias is None else bias[:2 * d], None, 1.0, y=self.qkv[:, :2 * d], **args)
+            aqt.aqt_qmatmul(hq, hs, wq[2 * d:], s_w[2 * d:], None if bias is None else bias[2 * d:], None, 1.0, y=self.v, **args)
         note(L[2].spec.name, self.q); note(L[3].spec.name, self.k); note(L[4].spec.name, self.v)
         # h_b = h_a + W_o v is needed both as fp32 (residual stream) and as codes (pointwise 1)
         if run.fuses_requant(L[5]):
