@@ -105,6 +105,7 @@ struct GemmParams {
   int64_t b_rows = 0;
   int n_out;    // N, or N / 2 for the GLU forms
   int tiles_m, tiles_n, k_blocks;
+  int whole_tiles = 0;  // 256-column CTA-pair tiles from this one on are taken as two halves (see unit_at)
   int small_acc;  // every |accumulator| < 2^22: the int -> float conversion can use the exponent trick
   // Row-quantizing epilogue (template argument RQ of the CTA-pair kernel): the output rows leave the
   // kernel as codes and scales as well (or only), see the kernel.
@@ -470,6 +471,24 @@ __device__ __forceinline__ bool tile_at(const GemmParams& p, int i, int& tm, int
   return tile < p.tiles_m * p.tiles_n;
 }
 
+// i-th unit of work of this CTA: a tile (part 0) or, of the last tiles of a launch of 256-column CTA-pair tiles, the first
+// (part 1) or second (part 2) half of its columns.  Where the last round of whole tiles would occupy less than half of the
+// pairs, every pair takes half a tile there instead, which ends the launch half a tile's time earlier.
+template <bool WS, bool CTA2, bool HALVES>
+__device__ __forceinline__ bool unit_at(const GemmParams& p, int i, int& tm, int& tn, int& part) {
+  part = 0;
+  if (!HALVES) return tile_at<WS, CTA2>(p, i, tm, tn);
+  int tile = (blockIdx.x >> 1) + i * (gridDim.x >> 1);
+  if (tile >= p.whole_tiles) {
+    const int h = tile - p.whole_tiles;
+    tile = p.whole_tiles + (h >> 1);
+    part = 1 + (h & 1);
+  }
+  tm = tile / p.tiles_n;
+  tn = tile - tm * p.tiles_n;
+  return tile < p.tiles_m * p.tiles_n;
+}
+
 // RQ (CTA pairs, no GLU): the epilogue also quantizes the output rows for the next layer (Fig. 2 of
 // the paper on u = what the plain epilogue writes): pass 1 is the plain epilogue, which also keeps
 // the row maxima and writes u back over its accumulators; every thread then publishes the maximum
@@ -478,7 +497,7 @@ __device__ __forceinline__ bool tile_at(const GemmParams& p, int i, int& tm, int
 // rows at the same time), and pass 2 turns u into codes.  The next tile's MMAs run meanwhile in
 // the other accumulator buffer.  The pairs of a group (tiles_n consecutive pairs) always share
 // their rows, so the grid is a multiple of tiles_n pairs.
-template <int BN, int STAGES, int EW, bool WS, bool BPACK, int ACCK, bool DEBUG, bool CTA2 = false, bool RQ = false>
+template <int BN, int STAGES, int EW, bool WS, bool BPACK, int ACCK, bool DEBUG, bool CTA2 = false, bool RQ = false, bool HALVES = false>
 __global__ void __launch_bounds__(32 * (2 + EW), 1)
 qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                 const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_r, const GemmParams p) {
@@ -486,6 +505,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
   constexpr int HALF = BN / 2;
   constexpr int SBUFS = Cfg::kStageBufs;
   constexpr int TILE_M = CTA2 ? 2 * kBM : kBM;  // rows of a tile (of the pair's tile)
+  static_assert(!HALVES || (CTA2 && BN == 256 && !RQ), "halves are taken of 256-column CTA-pair tiles");
   static_assert(!BPACK || WS, "packed weights are unpacked into the resident slab");
   constexpr bool TF32 = (ACCK == kAccFloat);  // float operands: no activation scale, accumulators are binary32
   static_assert(!(TF32 && (BPACK || DEBUG)), "the float kind reads expanded weights and has no integer accumulators to dump");
@@ -606,11 +626,12 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           }
         }
       }
-      int tm, tn;
-      for (int i = 0; ok && tile_at<WS, CTA2>(p, i, tm, tn); ++i) {
+      int tm, tn, part;
+      for (int i = 0; ok && unit_at<WS, CTA2, HALVES>(p, i, tm, tn, part); ++i) {
         // B rows of the two half-tiles: adjacent output channels, or (value, gate) halves for GLU
-        const int row0 = glu ? tn * HALF : tn * BN;
-        const int row1 = glu ? p.N / 2 + tn * HALF : tn * BN + HALF;
+        const int half_cols = part == 0 ? HALF : HALF / 2;
+        const int row0 = (glu ? tn * HALF : tn * BN) + (part == 2 ? (glu ? HALF / 2 : HALF) : 0);
+        const int row1 = glu ? p.N / 2 + row0 : row0 + half_cols;
         for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1, &abort_flag, t_start)) { ok = false; break; }
@@ -619,7 +640,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           if (CTA2) {
             // The leader's barrier counts both CTAs' bytes; each CTA loads its 128 rows of A and
             // its half of the weight rows (leader: first half / values, peer: second half / gates).
-            if (pair_rank == 0) mbar_arrive_expect_tx(bar, 2 * Cfg::kStageBytes);
+            if (pair_rank == 0) mbar_arrive_expect_tx(bar, HALVES && part != 0 ? 2 * (Cfg::kABytes + Cfg::kBBytes / 2) : 2 * Cfg::kStageBytes);
             tma_load_2d_pair(stage, &tm_a, kb * kBK, tm * TILE_M + row_in_tile, bar);
             if (BN == 512) {
               // two MMAs of 256 columns per k-step: this CTA supplies 128 weight rows to each
@@ -627,7 +648,10 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
               tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
               tma_load_2d_pair(stage + Cfg::kABytes + 128 * kBK, &tm_b, kb * kBK, r + 256, bar);
             } else {
-              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, pair_rank == 0 ? row0 : row1, bar);
+              const int r = pair_rank == 0 ? row0 : row1;
+              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
+              // (boxes of half a CTA's rows, so that half a tile is one of them)
+              if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, &tm_b, kb * kBK, r + HALF / 2, bar);
             }
             continue;
           }
@@ -645,12 +669,14 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0 && pair_rank == 0) {
-      constexpr uint32_t idesc = TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M);
+      constexpr uint32_t idesc_whole = TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M);
+      constexpr uint32_t idesc_half = TF32 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_i8(Cfg::kMmaN / 2, TILE_M);
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       if (WS) ok = mbar_wait(smem_u32(BPACK ? &b_ready_bar : &b_loaded_bar), 0, &abort_flag, t_start);
-      int tm, tn;
-      for (int i = 0; ok && tile_at<WS, CTA2>(p, i, tm, tn); ++i, ++tcount) {
+      int tm, tn, part;
+      for (int i = 0; ok && unit_at<WS, CTA2, HALVES>(p, i, tm, tn, part); ++i, ++tcount) {
+        const uint32_t idesc = HALVES && part != 0 ? idesc_half : idesc_whole;
         const uint32_t buf = tcount % Cfg::kAccBufs, aph = (tcount / Cfg::kAccBufs) & 1;
         if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
         tc_fence_after();
@@ -692,12 +718,12 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     const int quad = warp & 3;  // TMEM lane quadrant this warp may read
     const int chalf = ew >> 2;  // which share of the tile's output columns (0 .. EW/4 - 1)
     const uint32_t my_stage = smem_epi + ew * SBUFS * kStageBufBytes;
-    const int out_cols_tile = glu ? HALF : BN;         // output columns per tile
-    const int chunks = out_cols_tile / 32 / (EW / 4);  // 32-column chunks per epilogue warp and tile
+    const int out_cols_tile = glu ? HALF : BN;               // output columns per tile
+    const int chunks_whole = out_cols_tile / 32 / (EW / 4);  // 32-column chunks per epilogue warp and tile
     const bool has_res = p.residual != nullptr;
     const int n_value_limit = glu ? p.N / 2 : p.N;
     // where the scales of this warp's chunk c start: per-CTA slab (WS) or per-warp slab
-    const uint32_t slab_sw = WS ? smem_scale + (uint32_t)(chalf * chunks * 32) * 4 : smem_scale + ew * 2 * Cfg::kSlabFloats * 4;
+    const uint32_t slab_sw = WS ? smem_scale + (uint32_t)(chalf * chunks_whole * 32) * 4 : smem_scale + ew * 2 * Cfg::kSlabFloats * 4;
     const uint32_t slab_bias = WS ? slab_sw + BN * 4 : slab_sw + Cfg::kSlabFloats * 4;
     const uint32_t slab_chunk_stride = (WS || !glu) ? 128 : 256;  // bytes between consecutive chunks of this warp
     const uint32_t slab_gate_off = WS ? HALF * 4 : 128;           // gate columns relative to the value columns
@@ -739,18 +765,19 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
       }
     }
 
-    int tm, tn;
+    int tm, tn, part;
     // residual prefetch for the very first chunk of this warp
-    if (ok && has_res && lane == 0 && tile_at<WS, CTA2>(p, 0, tm, tn)) {
-      const int oc0 = tn * out_cols_tile + chalf * chunks * 32, r0 = tm * TILE_M + row_in_tile + quad * 32;
+    if (ok && has_res && lane == 0 && unit_at<WS, CTA2, HALVES>(p, 0, tm, tn, part)) {
+      const int oc0 = tn * out_cols_tile + (part == 2 ? out_cols_tile / 2 : 0) + chalf * (part == 0 ? chunks_whole : chunks_whole / 2) * 32, r0 = tm * TILE_M + row_in_tile + quad * 32;
       const uint32_t bar = smem_u32(&res_bar[ew][0]);
       mbar_arrive_expect_tx(bar, kStageBufBytes);
       tma_load_2d(my_stage, &tm_r, oc0 < p.n_out ? oc0 : 0, r0 < p.M ? r0 : 0, bar);
     }
 
-    for (int i = 0; ok && tile_at<WS, CTA2>(p, i, tm, tn); ++i) {
+    for (int i = 0; ok && unit_at<WS, CTA2, HALVES>(p, i, tm, tn, part); ++i) {
       const uint32_t buf = i % Cfg::kAccBufs, aph = (i / Cfg::kAccBufs) & 1;
-      const int out0 = tn * out_cols_tile;  // first output column of the tile
+      const int out0 = tn * out_cols_tile + (part == 2 ? out_cols_tile / 2 : 0);  // first output column of the tile, or of the half taken
+      const int chunks = part == 0 ? chunks_whole : chunks_whole / 2;
       const int row0_warp = tm * TILE_M + row_in_tile + quad * 32;  // first output row of this warp
       const int m = row0_warp + lane;
       const bool row_ok = m < p.M;
@@ -760,7 +787,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         __syncwarp();
         for (int c = 0; c < chunks; ++c) {
           const int col = (chalf * chunks + c) * 32;
-          const int nv = (glu ? out0 : tn * BN) + col + lane;  // value channel of this lane
+          const int nv = out0 + col + lane;  // value channel of this lane
           const uint32_t off = c * slab_chunk_stride + lane * 4;
           float wv = 0.0f, bv = 0.0f;
           if (nv < n_value_limit) {
@@ -812,19 +839,19 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           }
           if (DEBUG) {
             if (p.acc_debug != nullptr && row_ok) {
-              const int n0 = tn * BN + col;
+              const int n0 = out0 + col;
 #pragma unroll
               for (int j = 0; j < 32; ++j)
                 if (n0 + j < p.N) p.acc_debug[(int64_t)m * p.N + n0 + j] = (int32_t)acc[j];
             }
           }
           if (Cfg::kScaleSlab) dequant32<ACCK>(acc, sx, c_sw, c_bias, a);
-          else dequant32_gmem<ACCK>(acc, sx, p.s_w, p.bias, tn * BN + col, p.N, a);
+          else dequant32_gmem<ACCK>(acc, sx, p.s_w, p.bias, out0 + col, p.N, a);
           if (p.act == AQT_ACT_SWISH) swish32(a);
         } else {
           // gates first: g = sigmoid(z_gate); then the values are scaled by it
           float g[32];
-          tmem_ld_32x32(lane_addr + HALF + col, acc);
+          tmem_ld_32x32(lane_addr + (part == 0 ? HALF : HALF / 2) + col, acc);
           tmem_ld_wait();
           if (DEBUG) {
             if (p.acc_debug != nullptr && row_ok) {
@@ -863,13 +890,13 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
 
         // the chunk this warp handles after this one (for the residual prefetch)
-        int ntm = tm, ntn = tn, nc = c + 1;
+        int ntm = tm, ntn = tn, npart = part, nc = c + 1;
         bool have_next = true;
         if (nc == chunks) {
           nc = 0;
-          have_next = tile_at<WS, CTA2>(p, i + 1, ntm, ntn);
+          have_next = unit_at<WS, CTA2, HALVES>(p, i + 1, ntm, ntn, npart);
         }
-        const int noc = ntn * out_cols_tile + (chalf * chunks + nc) * 32, nr = ntm * TILE_M + row_in_tile + quad * 32;
+        const int noc = ntn * out_cols_tile + (npart == 2 ? out_cols_tile / 2 : 0) + (chalf * (npart == 0 ? chunks_whole : chunks_whole / 2) + nc) * 32, nr = ntm * TILE_M + row_in_tile + quad * 32;
 
         if (has_res) {
           if (SBUFS == 2) {
@@ -1105,8 +1132,19 @@ static int pick_bn(int64_t M, int64_t N, bool glu, int sms) {
   return best_bn;
 }
 
+// 256-column CTA-pair tiles that are taken whole; the last round is taken in halves where it would keep less than half of the
+// pairs busy: -11 % at 20 000 x 512 -> 512 in the float kind, -4 % at 12 800 x 512 -> 2048, -5 % at 14 080 x 1024 -> 512 with a
+// residual (int8).  Beside another product, which fills the pairs that such a round leaves, only of the second round
+// (both products of 12 800 x 512 x 2048 and what goes with them -2.4 %; 20 000 x 640 x 2560, fourth round, +1.5 %; 12 800 x
+// 2048 x 512, sixth, +1.2 %).
+static int64_t whole_pair_tiles(int64_t tiles, int64_t pairs, bool beside) {
+  const int64_t last_round = tiles % pairs;
+  const bool halves = tiles > pairs && last_round > 0 && 2 * last_round <= pairs && !(beside && tiles > 2 * pairs);
+  return halves ? tiles - last_round : tiles;
+}
+
 // b: weight codes as the kernel reads them -- int8 [N, K], or (BPACK) packed nibbles [N, K/2].
-template <int BN, int STAGES, int EW, bool WS, bool BPACK, int ACCK, bool DEBUG, bool CTA2 = false, bool RQ = false>
+template <int BN, int STAGES, int EW, bool WS, bool BPACK, int ACCK, bool DEBUG, bool CTA2 = false, bool RQ = false, bool HALVES = false>
 static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t ldy, const GemmParams& p0, cudaStream_t st) {
   using Cfg = GemmCfg<BN, STAGES, EW, WS, CTA2>;
   GemmParams p = p0;
@@ -1115,6 +1153,11 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
   p.k_blocks = (int)ceil_div(p.K, kBK);
   const int sms = sm_count();
   if (sms <= 0) return AQT_ERR_CUDA;
+  if constexpr (CTA2 && BN == 256 && !RQ && !HALVES) {
+    const int64_t tiles = (int64_t)p.tiles_m * p.tiles_n;
+    if (whole_pair_tiles(tiles, sms / 2, p.early_trigger != 0) < tiles)
+      return launch_qgemm_inst<BN, STAGES, EW, WS, BPACK, ACCK, DEBUG, CTA2, RQ, true>(a, b, y, ldy, p0, st);
+  }
   {
     const bool glu = (p.act == AQT_ACT_GLU) || (p.act == AQT_ACT_GLU_SWISH);
     if ((glu ? BN / 2 : BN) / 32 / (EW / 4) < 1) return AQT_ERR_UNSUPPORTED;  // a warp without columns would never release TMEM
@@ -1130,7 +1173,7 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
     rc = make_map_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_UINT8, b, (uint64_t)p.N, (uint64_t)p.K / 2, (uint64_t)p.K / 2, BN / 2, 64, 0);
   } else {
     rc = make_map_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_UINT8, b, (uint64_t)(p.b_rows != 0 ? p.b_rows : p.N), (uint64_t)p.K, (uint64_t)p.K,
-                     BN == 512 ? 128 : BN / 2, kBK);
+                     BN == 512 ? 128 : (HALVES ? BN / 4 : BN / 2), kBK);
   }
   if (rc != AQT_OK) return rc;
   if (p.batch_tiles_m > 0 && (WS || CTA2)) return AQT_ERR_UNSUPPORTED;
@@ -1148,7 +1191,7 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
   } else {
     tm_r = tm_y;  // never dereferenced
   }
-  auto kernel = qgemm_i8_kernel<BN, STAGES, EW, WS, BPACK, ACCK, DEBUG, CTA2, RQ>;
+  auto kernel = qgemm_i8_kernel<BN, STAGES, EW, WS, BPACK, ACCK, DEBUG, CTA2, RQ, HALVES>;
   static std::atomic<uint64_t> smem_opted_in{0};
   rc = ensure_dynamic_smem(kernel, Cfg::kSmemBytes, smem_opted_in);
   if (rc != AQT_OK) return rc;
@@ -1164,6 +1207,7 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
       if (p.tiles_n > pairs || p.exchange_parts != p.tiles_n * (EW / 4) || p.exchange_parts % 2 != 0) return AQT_ERR_UNSUPPORTED;
       pairs = pairs / p.tiles_n * p.tiles_n;
     }
+    if (HALVES) p.whole_tiles = (int)whole_pair_tiles(tiles, pairs, p.early_trigger != 0);
     grid = 2u * (unsigned)(tiles < pairs ? tiles : pairs);
     return launch_pdl(kernel, dim3(grid, 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 2, tm_a, tm_b, tm_y, tm_r, p);
   }
