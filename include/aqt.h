@@ -66,7 +66,7 @@ extern "C" {
  * 8-bit container; the packed form is this library's storage layout. */
 #define AQT_BITS_4_UNPACKED 48 /* 4-bit codes, one per int8 container: what aqt_quantize(bits 4, pack 0) and
                                   aqt_unpack_int4 produce.  Same layout as 8-bit codes; the smaller range lets the
-                                  epilogue convert accumulators on the plain ALUs up to a deeper K. */
+                                  epilogue of CTA pairs convert accumulators on the plain ALUs up to a deeper K. */
 
 #define AQT_STATIC_WEIGHTS 0x100 /* may be OR-ed into bits_w of the matmul entry points: the weight codes, their scales and
                                     the bias were complete before the work that precedes this call on the stream was enqueued

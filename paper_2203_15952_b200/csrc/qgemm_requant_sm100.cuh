@@ -148,7 +148,7 @@ __device__ __forceinline__ bool keep_waiting(volatile int* abort_flag, uint64_t 
 // output columns u = v * sigmoid(g) (then Swish for AQT_ACT_GLU_SWISH), 16 per epilogue warp.
 // The GLU form writes codes and scales only (no fp32 output, no residual, no nibble packing).
 // SHARED: CTAs with one or two tiles have several sets of warps work on each (sets_per_tile).
-template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
+template <bool BPACK, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
 __global__ void __launch_bounds__(32 * 20, 1)
 qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                      const __grid_constant__ CUtensorMap tm_y,
@@ -444,10 +444,10 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           tmem_ld_32x16(tbase + HALF + col, accg);
           tmem_ld_32x16(tbase + col, accv);
           tmem_ld_wait();
-          dequant16<SMALL>(accg, sx, c_sw + HALF * 4, c_bias + HALF * 4, g);
+          dequant16<kAccInt32>(accg, sx, c_sw + HALF * 4, c_bias + HALF * 4, g);
 #pragma unroll
           for (int j = 0; j < 16; ++j) g[j] = sigmoid_f(g[j]);
-          dequant16<SMALL>(accv, sx, c_sw, c_bias, av);
+          dequant16<kAccInt32>(accv, sx, c_sw, c_bias, av);
 #pragma unroll
           for (int j = 0; j < 16; ++j) av[j] = av[j] * g[j];
           if (p.act == AQT_ACT_GLU_SWISH) swish16(av);
@@ -464,7 +464,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           float a[32];
           tmem_ld_32x32(tbase + col, acc);
           tmem_ld_wait();
-          dequant32<SMALL>(acc, sx, c_sw, c_bias, a);
+          dequant32<kAccInt32>(acc, sx, c_sw, c_bias, a);
           if (p.act == AQT_ACT_SWISH) swish32(a);
           if (has_res) {
             if (!mbar_wait(smem_u32(&res_bar[ew]), res_count & 1u, &abort_flag, t_start)) { ok = false; break; }
@@ -635,7 +635,7 @@ static bool requant_applies(int64_t M, int64_t N, int64_t K, int act, bool with_
   return ceil_div(K, kBK) <= kRequantDeepKBlocks && !with_y && (!glu || !pack_out);
 }
 
-template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
+template <bool BPACK, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
 static int launch_requant_form(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, RequantParams rp,
                                void* exchange, cudaStream_t st) {
   using Cfg = RequantCfg<WITH_Y, DEEP>;
@@ -668,7 +668,7 @@ static int launch_requant_form(const int8_t* a, const void* b, void* q_out, floa
       if (rc != AQT_OK) return rc;
     }
   }
-  auto kernel = qgemm_requant_kernel<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, SHARED>;
+  auto kernel = qgemm_requant_kernel<BPACK, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, SHARED>;
   static std::atomic<uint64_t> smem_opted_in{0};
   rc = ensure_dynamic_smem(kernel, Cfg::kSmemBytes, smem_opted_in);
   if (rc != AQT_OK) return rc;
@@ -682,56 +682,49 @@ static int launch_requant_form(const int8_t* a, const void* b, void* q_out, floa
                     tm_y, tm_r, rp);
 }
 
-template <bool BPACK, bool SMALL, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
+template <bool BPACK, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
 static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, const RequantParams& rp,
                                void* exchange, cudaStream_t st) {
   const int sms = sm_count();
   if (sms <= 0) return AQT_ERR_CUDA;
   const int64_t groups = sms / ceil_div(rp.g.N, 128);
   if (ceil_div(rp.g.M, kBM) <= 2 * groups)
-    return launch_requant_form<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, true>(a, b, q_out, y, ldy, rp, exchange, st);
-  return launch_requant_form<BPACK, SMALL, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, false>(a, b, q_out, y, ldy, rp, exchange, st);
+    return launch_requant_form<BPACK, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, true>(a, b, q_out, y, ldy, rp, exchange, st);
+  return launch_requant_form<BPACK, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, false>(a, b, q_out, y, ldy, rp, exchange, st);
 }
 
 // a: int8 [M, K]; b: int8 [N, K] or (b_packed) nibbles [N, K/2]; y may be null (then no fp32 output
 // and no residual).  exchange: requant_exchange_bytes(M, N) bytes.
 static int launch_requant(const int8_t* a, const void* b, bool b_packed, void* q_out, float* y, int64_t ldy, const RequantParams& rp,
                           void* exchange, cudaStream_t st) {
-  const bool small = rp.g.small_acc != 0;
   const bool glu = rp.g.act == AQT_ACT_GLU || rp.g.act == AQT_ACT_GLU_SWISH;
   if (ceil_div(rp.g.K, kBK) > kWsMaxKBlocks) {
     // deep-K form: int8 weights, codes and scales only
     if (y != nullptr || b_packed || (glu && rp.pack_out)) return AQT_ERR_UNSUPPORTED;
-#define AQT_RQ_DEEP(SM, PK, GL)                                                                                                   \
-  (rp.rounding == AQT_ROUND_HALF_UP_FLOOR ? launch_requant_inst<false, SM, false, AQT_ROUND_HALF_UP_FLOOR, PK, GL, true>(a, b, q_out, y, ldy, rp, exchange, st) \
-                                          : launch_requant_inst<false, SM, false, AQT_ROUND_NEAREST_EVEN, PK, GL, true>(a, b, q_out, y, ldy, rp, exchange, st))
-    if (glu) return small ? AQT_RQ_DEEP(true, false, true) : AQT_RQ_DEEP(false, false, true);
-    if (rp.pack_out) return small ? AQT_RQ_DEEP(true, true, false) : AQT_RQ_DEEP(false, true, false);
-    return small ? AQT_RQ_DEEP(true, false, false) : AQT_RQ_DEEP(false, false, false);
+#define AQT_RQ_DEEP(PK, GL)                                                                                                       \
+  (rp.rounding == AQT_ROUND_HALF_UP_FLOOR ? launch_requant_inst<false, false, AQT_ROUND_HALF_UP_FLOOR, PK, GL, true>(a, b, q_out, y, ldy, rp, exchange, st) \
+                                          : launch_requant_inst<false, false, AQT_ROUND_NEAREST_EVEN, PK, GL, true>(a, b, q_out, y, ldy, rp, exchange, st))
+    if (glu) return AQT_RQ_DEEP(false, true);
+    return rp.pack_out ? AQT_RQ_DEEP(true, false) : AQT_RQ_DEEP(false, false);
 #undef AQT_RQ_DEEP
   }
   if (glu) {
     if (y != nullptr || rp.pack_out) return AQT_ERR_UNSUPPORTED;
-#define AQT_RQ_GLU(BP, SM)                                                                                                        \
-  (rp.rounding == AQT_ROUND_HALF_UP_FLOOR ? launch_requant_inst<BP, SM, false, AQT_ROUND_HALF_UP_FLOOR, false, true>(a, b, q_out, y, ldy, rp, exchange, st) \
-                                          : launch_requant_inst<BP, SM, false, AQT_ROUND_NEAREST_EVEN, false, true>(a, b, q_out, y, ldy, rp, exchange, st))
-    if (b_packed) return small ? AQT_RQ_GLU(true, true) : AQT_RQ_GLU(true, false);
-    return small ? AQT_RQ_GLU(false, true) : AQT_RQ_GLU(false, false);
+#define AQT_RQ_GLU(BP)                                                                                                            \
+  (rp.rounding == AQT_ROUND_HALF_UP_FLOOR ? launch_requant_inst<BP, false, AQT_ROUND_HALF_UP_FLOOR, false, true>(a, b, q_out, y, ldy, rp, exchange, st) \
+                                          : launch_requant_inst<BP, false, AQT_ROUND_NEAREST_EVEN, false, true>(a, b, q_out, y, ldy, rp, exchange, st))
+    return b_packed ? AQT_RQ_GLU(true) : AQT_RQ_GLU(false);
 #undef AQT_RQ_GLU
   }
-#define AQT_RQ(BP, SM, WY)                                                                                                 \
+#define AQT_RQ(BP, WY)                                                                                                     \
   (rp.pack_out ? (rp.rounding == AQT_ROUND_HALF_UP_FLOOR                                                                     \
-                      ? launch_requant_inst<BP, SM, WY, AQT_ROUND_HALF_UP_FLOOR, true>(a, b, q_out, y, ldy, rp, exchange, st) \
-                      : launch_requant_inst<BP, SM, WY, AQT_ROUND_NEAREST_EVEN, true>(a, b, q_out, y, ldy, rp, exchange, st)) \
+                      ? launch_requant_inst<BP, WY, AQT_ROUND_HALF_UP_FLOOR, true>(a, b, q_out, y, ldy, rp, exchange, st) \
+                      : launch_requant_inst<BP, WY, AQT_ROUND_NEAREST_EVEN, true>(a, b, q_out, y, ldy, rp, exchange, st)) \
                : (rp.rounding == AQT_ROUND_HALF_UP_FLOOR                                                                     \
-                      ? launch_requant_inst<BP, SM, WY, AQT_ROUND_HALF_UP_FLOOR, false>(a, b, q_out, y, ldy, rp, exchange, st) \
-                      : launch_requant_inst<BP, SM, WY, AQT_ROUND_NEAREST_EVEN, false>(a, b, q_out, y, ldy, rp, exchange, st)))
-  if (y != nullptr) {
-    if (b_packed) return small ? AQT_RQ(true, true, true) : AQT_RQ(true, false, true);
-    return small ? AQT_RQ(false, true, true) : AQT_RQ(false, false, true);
-  }
-  if (b_packed) return small ? AQT_RQ(true, true, false) : AQT_RQ(true, false, false);
-  return small ? AQT_RQ(false, true, false) : AQT_RQ(false, false, false);
+                      ? launch_requant_inst<BP, WY, AQT_ROUND_HALF_UP_FLOOR, false>(a, b, q_out, y, ldy, rp, exchange, st) \
+                      : launch_requant_inst<BP, WY, AQT_ROUND_NEAREST_EVEN, false>(a, b, q_out, y, ldy, rp, exchange, st)))
+  if (y != nullptr) return b_packed ? AQT_RQ(true, true) : AQT_RQ(false, true);
+  return b_packed ? AQT_RQ(true, false) : AQT_RQ(false, false);
 #undef AQT_RQ
 }
 

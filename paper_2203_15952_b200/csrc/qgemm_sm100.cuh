@@ -363,6 +363,9 @@ __device__ __forceinline__ float sigmoid_f(float z) {
 //   kAccInt32Small int32 with |acc| < 2^22 guaranteed by the caller: adding the integer to the bit
 //                  pattern of 1.5 * 2^23 and subtracting that constant is exact and stays off the
 //                  conversion unit
+//                  conversion unit.  For CTA pairs only, whose eight warps convert a tile twice as wide (30 000 x 2048
+//                  -> 512 Swish 89.3 us, 91.2 with conversions); sixteen warps on 128 columns are shorter of issue slots
+//                  than of conversions (feed-forward pair on 12 800 rows 56.4 / 55.5, 12 800 x 512 -> 2048 gated 39.0 / 37.9)
 //   kAccFloat      binary32 already (the float matmul of the weight-only layer)
 constexpr int kAccInt32 = 0, kAccInt32Small = 1, kAccFloat = 2;
 template <int ACCK>
@@ -1223,7 +1226,9 @@ static int launch_qgemm_cfg(const int8_t* a, const void* b, float* y, int64_t ld
     return AQT_ERR_UNSUPPORTED;
   }
   if (p.acc_debug != nullptr) return launch_qgemm_inst<BN, STAGES, EW, WS, BPACK, kAccInt32, true, CTA2>(a, b, y, ldy, p, st);
-  if (p.small_acc) return launch_qgemm_inst<BN, STAGES, EW, WS, BPACK, kAccInt32Small, false, CTA2>(a, b, y, ldy, p, st);
+  if constexpr (CTA2) {
+    if (p.small_acc) return launch_qgemm_inst<BN, STAGES, EW, WS, BPACK, kAccInt32Small, false, CTA2>(a, b, y, ldy, p, st);
+  }
   return launch_qgemm_inst<BN, STAGES, EW, WS, BPACK, kAccInt32, false, CTA2>(a, b, y, ldy, p, st);
 }
 
