@@ -209,12 +209,13 @@ class LayerRunner:
         return self._shared_q, self._shared_s
 
     def matmul(self, layer: QuantLinear, xq: torch.Tensor, s_x: torch.Tensor, y: torch.Tensor,
-               residual: Optional[torch.Tensor] = None, residual_scale: float = 1.0, plan: Optional[str] = None) -> torch.Tensor:
-        """Integer matmul + epilogue of `layer` on already-quantized activations (int8 containers), behind a kernel that the caller
-        enqueued after the weights were complete; plan: see aqt_qmatmul."""
+               residual: Optional[torch.Tensor] = None, residual_scale: float = 1.0, plan: Optional[str] = None,
+               static: bool = False) -> torch.Tensor:
+        """Integer matmul + epilogue of `layer` on already-quantized activations (int8 containers); plan: see aqt_qmatmul, static:
+        see matmul_requant."""
         s = layer.spec
         return aqt.aqt_qmatmul(xq, s_x, layer.mm_weight, layer.s_w, layer.bias, residual, residual_scale, K=s.K, bits_a=_container_bits(s.bits_a),
-                               bits_w=layer.mm_bits | aqt.STATIC_WEIGHTS, act=s.act, s_x_kind=self.a_scale_kind, y=y, workspace=self.workspace,
+                               bits_w=layer.mm_bits | (aqt.STATIC_WEIGHTS if static else 0), act=s.act, s_x_kind=self.a_scale_kind, y=y, workspace=self.workspace,
                                plan=plan)
 
     def fuses_requant(self, layer: QuantLinear, with_y: bool = True) -> bool:
@@ -286,7 +287,7 @@ class FfnPair:
         l0, l1 = self.layers
         xq, xs = self.run.quantize_input(x, l0.spec.bits_a)
         uq, us = self.run.matmul_requant(l0, xq, xs, l1.spec.bits_a, "u", y=self.u, static=True)
-        return self.run.matmul(l1, uq, us, y, plan=self._plan)
+        return self.run.matmul(l1, uq, us, y, plan=self._plan, static=True)
 
     def _chains(self) -> bool:
         """True if a step is small enough for both layers to run in one launch (shape permitting)."""
@@ -364,7 +365,7 @@ class ConformerBlockLinears:
                 vq, vs = run.quantize_input(self.v, L[5].spec.bits_a)
             bq, bs = run.matmul_requant(L[5], vq, vs, L[6].spec.bits_a, "h", y=self.h_b, residual=self.h_a, residual_scale=1.0, static=True)
         elif vq is not None:
-            run.matmul(L[5], vq, vs, self.h_b, residual=self.h_a, residual_scale=1.0)
+            run.matmul(L[5], vq, vs, self.h_b, residual=self.h_a, residual_scale=1.0, static=True)
         else:
             run(L[5], self.v, self.h_b, residual=self.h_a, residual_scale=1.0)
         note(L[5].spec.name, self.h_b)
@@ -374,7 +375,7 @@ class ConformerBlockLinears:
                 bq, bs = run.quantize_input(self.h_b, L[6].spec.bits_a)
             cq, cs = run.matmul_requant(L[6], bq, bs, L[7].spec.bits_a, "c", static=True)
         elif bq is not None:
-            run.matmul(L[6], bq, bs, self.c)
+            run.matmul(L[6], bq, bs, self.c, static=True)
         else:
             run(L[6], self.h_b, self.c)
         if cq is None:
@@ -388,7 +389,7 @@ class ConformerBlockLinears:
             out_codes = self._ffn(L[8], L[9], self.h_a, h_out, 0.5, parity, note, xq=aq, xs=as_, out_role="hb", out_bits=next_bits)
         else:
             if cq is not None:
-                run.matmul(L[7], cq, cs, self.h_a, residual=self.h_b, residual_scale=1.0)
+                run.matmul(L[7], cq, cs, self.h_a, residual=self.h_b, residual_scale=1.0, static=True)
             else:
                 run(L[7], self.c, self.h_a, residual=self.h_b, residual_scale=1.0)
             note(L[7].spec.name, self.h_a)
@@ -421,7 +422,7 @@ class ConformerBlockLinears:
             aqt.aqt_quantize(self.u, l1.spec.bits_a, aqt.AXIS_ROW, run.rounding, q_out=uq, scale_out=us)
         if fuse_out:
             return run.matmul_requant(l1, uq, us, out_bits, out_role, y=out, residual=h, residual_scale=rs, static=True)
-        run.matmul(l1, uq, us, out, residual=h, residual_scale=rs)
+        run.matmul(l1, uq, us, out, residual=h, residual_scale=rs, static=True)
         return None, None
 
     def _fused_qkv(self, L: List[QuantLinear]):
