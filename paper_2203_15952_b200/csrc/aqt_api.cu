@@ -364,7 +364,7 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY_X2) return ws_weight_only(M, N, K, AQT_FLOAT_TF32X2);
   if (op == AQT_OP_LINEAR_BWD) return bwd_workspace(M, N, K);
   if (op == AQT_OP_FFN_FWD) return ffn_layout(M, K, N, bits_w, bits_w).total;
-  if (op == AQT_OP_QMATMUL_REQUANT) return round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256) + requant_exchange_bytes(M, N);
+  if (op == AQT_OP_QMATMUL_REQUANT) return round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256) + requant_exchange_bytes_few(M, N);
   return 0;
 }
 
@@ -652,7 +652,7 @@ int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, in
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int sms = sm_count();
   const int bn = sms > 0 && !is_packed(bits_a) ? few_tiles_bn(M, N, K, AQT_ACT_NONE, first, sms) : 0;
-  if (bn != 0)
+  if (bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= workspace_bytes - mm_bytes)
     return run_few_tiles(bn, reinterpret_cast<const int8_t*>(xq), s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, width, static_w != 0,
                              AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, reinterpret_cast<uint8_t*>(workspace),
                              reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);

@@ -608,20 +608,22 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   if (tn == 0 && threadIdx.x == 0) rp.generation[group] = __ldcg(rp.generation + group) + 1u;
 }
 
-// Bytes of the exchange area: one 64-bit word per m-tile, n-tile and row for this kernel and the one of
-// qgemm_few_tiles_sm100.cuh, or per row (padded to the 256 rows of a pair tile) and column part for the CTA-pair kernel with
-// the row-quantizing epilogue (at most one part per 64 columns, at least two), then the generation counters.
+// Bytes of the exchange area: one 64-bit word per m-tile, n-tile and row for this kernel, or per
+// row (padded to the 256 rows of a pair tile) and column part for the CTA-pair kernel with the
+// row-quantizing epilogue (at most one part per 64 columns, at least two), then the generation counters.
 static size_t requant_exchange_bytes(int64_t M, int64_t N) {
   const size_t tiles_m = (size_t)ceil_div(M, kBM);
   const size_t ws_form = tiles_m * (size_t)ceil_div(N, 128) * kBM * 8;
   const size_t parts = (size_t)ceil_div(N, 64) < 2 ? 2 : (size_t)ceil_div(N, 64);
   const size_t pair_form = (size_t)ceil_div(M, 2 * kBM) * 2 * kBM * parts * 8;
-  // (narrow tiles, one per CTA: as many tiles of 32 columns as there are SMs)
-  const size_t tiles32 = tiles_m * (size_t)ceil_div(N, 32), sms = (size_t)(sm_count() > 0 ? sm_count() : kDefaultSms);
-  const size_t few_form = (tiles32 < sms ? tiles32 : sms) * kBM * 8;
-  size_t most = ws_form > pair_form ? ws_form : pair_form;
-  if (few_form > most) most = few_form;
-  return round_up(most + (size_t)kMaxGroups * 4, 256);
+  return round_up((ws_form > pair_form ? ws_form : pair_form) + (size_t)kMaxGroups * 4, 256);
+}
+// With room for the narrow tiles of qgemm_few_tiles_sm100.cuh (as many of 32 columns as there are SMs), which a call whose
+// area is smaller does without.
+static size_t requant_exchange_bytes_few(int64_t M, int64_t N) {
+  const size_t tiles32 = (size_t)ceil_div(M, kBM) * (size_t)ceil_div(N, 32), sms = (size_t)(sm_count() > 0 ? sm_count() : kDefaultSms);
+  const size_t few_form = round_up((tiles32 < sms ? tiles32 : sms) * kBM * 8 + (size_t)kMaxGroups * 4, 256), others = requant_exchange_bytes(M, N);
+  return few_form > others ? few_form : others;
 }
 
 // True if this kernel takes the call: K <= 512; NONE / Swish in every form, the GLU forms when

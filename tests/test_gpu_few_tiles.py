@@ -73,3 +73,18 @@ def test_few_tiles_replayed():
         assert torch.equal(q, q_ref) and torch.equal(s, s_ref)
         s_x.div_(scale)
     assert aqt.aqt_device_status() == 0
+
+
+def test_few_tiles_do_without_room_for_their_exchange():
+    # the area that the wider tiles need, one row short of it, and the bits of either form
+    M, N, K = 300, 512, 512
+    rng = np.random.default_rng(5)
+    args = (_dev(_codes(rng, M, K, 8)), _dev(rng.uniform(1e-3, 5e-2, M).astype(np.float32)), _dev(_codes(rng, N, K, 8)),
+            _dev(rng.uniform(1e-4, 5e-3, N).astype(np.float32)))
+    need = -(-M // 256) * 256 * (N // 64) * 8 + 256 * 4
+    assert aqt.aqt_workspace_bytes(aqt.OP_QMATMUL_REQUANT, M, N, K, 8, 8) > need
+    q0, s0, _ = aqt.aqt_qmatmul_requant(*args, K=K)
+    q1, s1, _ = aqt.aqt_qmatmul_requant(*args, K=K, workspace=torch.empty(need, dtype=torch.uint8, device="cuda"))
+    assert torch.equal(q0, q1) and torch.equal(s0, s1) and aqt.aqt_device_status() == 0
+    with pytest.raises(aqt.AqtError):
+        aqt.aqt_qmatmul_requant(*args, K=K, workspace=torch.empty(need - 256, dtype=torch.uint8, device="cuda"))
