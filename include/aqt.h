@@ -186,7 +186,9 @@ int aqt_qmatmul_with_plan(const char* plan, const void* xq, const float* s_x, in
  * y         NULL, or fp32 [M, N_out] with row pitch ldy: also receives u (a residual stream, or
  *           a parity check).  residual != NULL requires y != NULL.
  * workspace at least aqt_workspace_bytes(AQT_OP_QMATMUL_REQUANT, ...) bytes, 256-byte aligned:
- *           what aqt_qmatmul needs plus the area through which CTAs exchange row maxima.
+ *           what aqt_qmatmul needs plus the area through which CTAs exchange row maxima.  Its last KB counts
+ *           executions, by which a replayed CUDA graph tells its row maxima from those of the replay before:
+ *           calls of one graph that share a workspace are given the same size of it.
  * Limits: those of aqt_qmatmul, and N_out % 16 == 0 (N_out % 32 == 0 if pack_out).  One kernel
  * does both steps for: K <= 512 with act NONE or SWISH; the GLU forms when only int8 codes and
  * scales are asked for (y == NULL, pack_out == 0); 512 < K <= 1024 when y == NULL; and K >= 2048

@@ -223,7 +223,7 @@ int run_small_m(const void* xq, bool a_packed, const float* s_x, int s_x_kind, c
 int run_few_tiles(int bn, const int8_t* a_codes, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
                   const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_w, bool static_w,
                   int act, int64_t rq_first, int bits_out, int rounding, void* q_out, float* s_out, float* y, int64_t ldy, uint8_t* scratch,
-                  void* exchange, cudaStream_t st) {
+                  void* exchange, uint32_t* generation, cudaStream_t st) {
   const void* b_codes = wq;
   bool b_packed = false;
   if (is_packed(bits_w)) {
@@ -255,7 +255,7 @@ int run_few_tiles(int bn, const int8_t* a_codes, const float* s_x, int s_x_kind,
   fp.rp.q_out = reinterpret_cast<uint8_t*>(q_out);
   fp.rp.s_out = s_out;
   fp.rp.exchange = reinterpret_cast<uint64_t*>(exchange);
-  fp.rp.generation = nullptr;
+  fp.rp.generation = generation;
   fp.rp.tag = 0;
   fp.rp.qmax_out = qmax_of(bits_out);
   fp.rp.rounding = rounding;
@@ -279,7 +279,7 @@ int qmatmul_i8a(const int8_t* a_codes, const float* s_x, int s_x_kind, const voi
     const int bn = few_tiles_bn(M, N, K, act, -1, sm_count());
     if (bn != 0)
       return run_few_tiles(bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w, act,
-                           is_glu(act) ? N / 2 : N, 8, AQT_ROUND_NEAREST_EVEN, nullptr, nullptr, y, ldy, ws, nullptr, st);
+                           is_glu(act) ? N / 2 : N, 8, AQT_ROUND_NEAREST_EVEN, nullptr, nullptr, y, ldy, ws, nullptr, nullptr, st);
   }
   // 4-bit weights: the weight-stationary kernel (K <= 512) sign-extends them itself in shared
   // memory after TMA staging; deeper K takes a one-off sign-extended copy in the workspace.
@@ -531,7 +531,8 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
       ws += round_up((size_t)M * (size_t)K, 256);
     }
     return run_few_tiles(few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w != 0, act, 0,
-                             bits_out, rounding, q_out, s_out, y, ldy, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);
+                             bits_out, rounding, q_out, s_out, y, ldy, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes,
+                             generation_counters(workspace, workspace_bytes), st);
   }
   if (pair_form) {
     // Deep K (the second feed-forward layers): the CTA-pair kernel with the row-quantizing epilogue
@@ -567,7 +568,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
     p.q_out = reinterpret_cast<uint8_t*>(q_out);
     p.s_out = s_out;
     p.exchange = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(workspace) + mm_bytes);
-    p.generation = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(workspace) + mm_bytes + requant_exchange_bytes(M, N) - (size_t)kMaxGroups * 4);
+    p.generation = generation_counters(workspace, workspace_bytes);
     p.tag = next_launch_tag();
     p.qmax_out = qmax_of(bits_out);
     p.rounding = rounding;
@@ -624,6 +625,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   rp.q_out = nullptr;
   rp.s_out = s_out;
   rp.exchange = nullptr;
+  rp.generation = generation_counters(workspace, workspace_bytes);
   rp.qmax_out = qmax_of(bits_out);
   rp.rounding = rounding;
   rp.pack_out = pack_out;
@@ -655,7 +657,7 @@ int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, in
   if (bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= workspace_bytes - mm_bytes)
     return run_few_tiles(bn, reinterpret_cast<const int8_t*>(xq), s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, width, static_w != 0,
                              AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, reinterpret_cast<uint8_t*>(workspace),
-                             reinterpret_cast<uint8_t*>(workspace) + mm_bytes, st);
+                             reinterpret_cast<uint8_t*>(workspace) + mm_bytes, generation_counters(workspace, workspace_bytes), st);
   // the two parts one after the other (row `first` of the weights keeps the 16-byte alignment: `first` and K are multiples of 16)
   if (first > 0) {
     rc = aqt_qmatmul(xq, s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, first, K, bits_a, width, AQT_ACT_NONE, y, ldy, nullptr, workspace,

@@ -480,7 +480,6 @@ static int launch_few_tiles_inst(const int8_t* a, const void* b, float* y, int64
   if (fp.b_packed && p.k_blocks > kWsMaxKBlocks) return AQT_ERR_UNSUPPORTED;
   if (fp.rq_first < p.n_out) {
     if (fp.rq_first % Cfg::kOutCols != 0) return AQT_ERR_UNSUPPORTED;
-    fp.rp.generation = reinterpret_cast<uint32_t*>(fp.rp.exchange + (size_t)p.tiles_m * p.tiles_n * kBM);
     fp.rp.tag = next_launch_tag();
   } else {
     fp.rq_first = p.tiles_n * Cfg::kOutCols;  // no tile

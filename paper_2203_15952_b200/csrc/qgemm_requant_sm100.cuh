@@ -40,7 +40,7 @@ struct RequantParams {
   uint8_t* q_out;       // codes of the output: int8 [M, N] or packed nibbles [M, N/2], dense
   float* s_out;         // [M] scales of the output rows
   uint64_t* exchange;   // [tiles_m][tiles_n][128] words: (launch tag << 32) | bit pattern of a CTA's row maximum
-  uint32_t* generation; // [groups] counters behind the words: each group of CTAs bumps its own when it has finished
+  uint32_t* generation; // [groups] counters (generation_counters): each group of CTAs bumps its own when it has finished
   uint32_t tag;         // tag of this call (no other call of the process uses it); a word counts once its upper half
                         // equals this tag mixed with the group's generation, which differs on every execution of the call
   int qmax_out;         // 127 or 7
@@ -610,7 +610,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
 
 // Bytes of the exchange area: one 64-bit word per m-tile, n-tile and row for this kernel, or per
 // row (padded to the 256 rows of a pair tile) and column part for the CTA-pair kernel with the
-// row-quantizing epilogue (at most one part per 64 columns, at least two), then the generation counters.
+// row-quantizing epilogue (at most one part per 64 columns, at least two), and the generation counters.
 static size_t requant_exchange_bytes(int64_t M, int64_t N) {
   const size_t tiles_m = (size_t)ceil_div(M, kBM);
   const size_t ws_form = tiles_m * (size_t)ceil_div(N, 128) * kBM * 8;
@@ -649,7 +649,6 @@ static int launch_requant_form(const int8_t* a, const void* b, void* q_out, floa
   if (sms <= 0) return AQT_ERR_CUDA;
   if (p.k_blocks > Cfg::kKBlocks || p.tiles_n > sms) return AQT_ERR_UNSUPPORTED;
   rp.exchange = reinterpret_cast<uint64_t*>(exchange);
-  rp.generation = reinterpret_cast<uint32_t*>(rp.exchange + (size_t)p.tiles_m * p.tiles_n * kBM);
   rp.tag = next_launch_tag();
 
   CUtensorMap tm_a, tm_b, tm_y, tm_r;
@@ -696,7 +695,7 @@ static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, floa
 }
 
 // a: int8 [M, K]; b: int8 [N, K] or (b_packed) nibbles [N, K/2]; y may be null (then no fp32 output
-// and no residual).  exchange: requant_exchange_bytes(M, N) bytes.
+// and no residual).  exchange: the words of requant_exchange_bytes(M, N); rp carries the counters.
 static int launch_requant(const int8_t* a, const void* b, bool b_packed, void* q_out, float* y, int64_t ldy, const RequantParams& rp,
                           void* exchange, cudaStream_t st) {
   const bool glu = rp.g.act == AQT_ACT_GLU || rp.g.act == AQT_ACT_GLU_SWISH;

@@ -115,5 +115,13 @@ static uint32_t next_launch_tag() {
 
 constexpr int kMaxGroups = 256;  // at most one group per SM
 
+// The generation counters of a workspace: its last kMaxGroups words.  Behind the exchange words of the call they would lie
+// where those of another call on the same workspace (another shape, another base) can fall: a replayed graph then finds its
+// counter back at the value of the replay before, and with it takes that replay's maxima for its own.  Every call whose rows
+// exchange maxima requires its words and this area, so no word of any of them reaches it.
+static uint32_t* generation_counters(void* workspace, size_t workspace_bytes) {
+  return reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(workspace) + workspace_bytes / 256 * 256 - (size_t)kMaxGroups * 4);
+}
+
 
 }  // namespace aqt

@@ -194,7 +194,8 @@ class LayerRunner:
         self.M, self.device, self.a_scale_kind, self.rounding = M, device, a_scale_kind, rounding
         need = max(max(aqt.aqt_workspace_bytes(op, M, 3 * l.spec.N, l.spec.K, l.spec.bits_a, l.spec.bits_w)
                        for op in (aqt.OP_LINEAR_FWD, aqt.OP_QMATMUL_REQUANT)) for l in layers)
-        self.workspace = torch.empty(need, dtype=torch.uint8, device=device)
+        # (and a KB at its end, for the counters of the calls that exchange row maxima, beyond the reach of every other call)
+        self.workspace = torch.empty(need + 1024, dtype=torch.uint8, device=device)
         self._codes: Dict[str, tuple] = {}
 
     def quantize_input(self, x: torch.Tensor, bits_a: int):

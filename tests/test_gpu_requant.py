@@ -243,6 +243,38 @@ def test_requant_with_y_gives_the_bits_of_two_calls(M, N, K):
     assert aqt.aqt_device_status() == 0
 
 
+def test_replayed_calls_that_share_a_workspace_keep_their_maxima_apart():
+    """A replayed graph of two calls on one workspace.  The second call's packed weights put its exchange words right behind
+    the first call's, and its inputs stay as they are, so what it leaves there is the same in every replay; the first call's
+    inputs change from replay to replay, and its codes and scales with them."""
+    M = 300
+    rng = np.random.default_rng(8)
+    f = lambda lo, hi, n: _dev(rng.uniform(lo, hi, n).astype(np.float32))
+    a = (_dev(_codes(rng, M, 512, 8)), f(1e-3, 5e-2, M), _dev(_codes(rng, 512, 512, 8)), f(1e-4, 5e-3, 512))
+    # 3 x 16 tiles of 128 rows and 32 columns, a word of 8 bytes a row: as many bytes as the other call's expanded weights
+    b = (_dev(_codes(rng, M, 384, 8)), f(1e-3, 5e-2, M), _dev(orc.pack_int4(_codes(rng, 128, 384, 4))), f(1e-4, 5e-3, 128))
+    ws = torch.empty(max(aqt.aqt_workspace_bytes(aqt.OP_QMATMUL_REQUANT, M, 512, 512, 8, 8),
+                         aqt.aqt_workspace_bytes(aqt.OP_QMATMUL_REQUANT, M, 128, 384, 8, 4)), dtype=torch.uint8, device=DEV)
+    q, s = torch.empty(M, 512, dtype=torch.int8, device=DEV), torch.empty(M, device=DEV)
+    qb, sb = torch.empty(M, 128, dtype=torch.int8, device=DEV), torch.empty(M, device=DEV)
+
+    def both():
+        aqt.aqt_qmatmul_requant(*a, K=512, q_out=q, s_out=s, workspace=ws)
+        aqt.aqt_qmatmul_requant(*b, K=384, bits_w=4, q_out=qb, s_out=sb, workspace=ws)
+    both()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        both()
+    s_x = a[1].clone()
+    for scale in (1.0, 0.25, 3.0, 0.5):
+        torch.mul(s_x, scale, out=a[1])
+        g.replay()
+        q_ref, s_ref = aqt.aqt_quantize(aqt.aqt_qmatmul(*a, K=512), 8)
+        assert torch.equal(s, s_ref) and torch.equal(q, q_ref), scale
+    assert aqt.aqt_device_status() == 0
+
+
 def test_requant_argument_checks():
     z8 = torch.zeros((64, 64), dtype=torch.int8, device=DEV)
     w8 = torch.zeros((48, 64), dtype=torch.int8, device=DEV)
