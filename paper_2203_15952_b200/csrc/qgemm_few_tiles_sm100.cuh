@@ -108,6 +108,8 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   __shared__ uint64_t res_bar[EW];   // a warp's residual box has landed
   __shared__ uint64_t part_bar[4];   // sets 1 .. 3 have left their maxima of this lane quadrant's rows
   __shared__ uint64_t ctx_bar[2];    // an exchange warp has the final maxima of its half of the rows
+  __shared__ uint64_t tag_bar;       // tag_slot is there
+  __shared__ uint32_t tag_slot;
   __shared__ float part_amax[4][kBM];
   __shared__ __align__(16) uint32_t row_amax[kBM];
   __shared__ uint32_t tmem_base_slot;
@@ -144,6 +146,7 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     for (int w = 0; w < EW; ++w) mbar_init(smem_u32(&res_bar[w]), 1);
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&part_bar[q]), 3);
     for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&ctx_bar[h]), 1);
+    mbar_init(smem_u32(&tag_bar), 1);
     fence_barrier_init();
     fence_proxy_async_smem();
     // the weights' loads are on their way before the CTA's set-up is complete
@@ -221,9 +224,11 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     if (rq) {
       const int xh = warp - (2 + EW);
       grid_dependency_wait();
-      const uint32_t tag = mix_tag(rp.tag, __ldcg(rp.generation + tm));  // of this execution, see qgemm_requant_sm100.cuh
+      if (xh == 0 && lane == 0) hand_out_tag(rp, tm, &tag_slot, &tag_bar);
+      bool ok = mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start);
+      ok = __all_sync(0xffffffffu, ok) != 0;
+      const uint32_t tag = *(volatile uint32_t*)&tag_slot;
       const uint64_t* xt = rp.exchange + (size_t)tm * parts * kBM + 64 * xh + 2 * lane;
-      bool ok = true;
       uint2 m2 = make_uint2(0u, 0u);
       for (int t0 = 0; ok && t0 < parts; t0 += kExchangeBatch) {
         for (uint32_t spin = 1;; ++spin) {
@@ -320,9 +325,10 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       // (a box that would start outside the tensor is redirected to its origin and never used)
       tma_load_2d(box, &tm_r, cols_ok ? oc : 0, row0_warp < p.M ? row0_warp : 0, smem_u32(&res_bar[ew]));
     }
-    const uint32_t tag = rq ? mix_tag(rp.tag, __ldcg(rp.generation + tm)) : 0u;
     const float sx = p.s_x_kind == AQT_SCALE_ROW ? (m < p.M ? __ldg(p.s_x + m) : 0.0f) : __ldg(p.s_x);
 
+    if (ok && rq && set == 0) ok = wait(tag_bar);  // (long before the accumulators are complete)
+    const uint32_t tag = *(volatile uint32_t*)&tag_slot;
     float a[C];
     if (ok) ok = wait(acc_bar);
     if (ok) {
@@ -432,7 +438,7 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     tc_fence_after();
     tmem_dealloc(tmem_base, Cfg::kTmemCols);
   }
-  // every CTA of the m-tile has read the counter: this one could not finish without their maxima
+  // every CTA of the m-tile has read the counter (hand_out_tag): this one could not finish without their maxima
   if (rq && tn == tn_first && threadIdx.x == 0) rp.generation[tm] = __ldcg(rp.generation + tm) + 1u;
 }
 

@@ -130,6 +130,15 @@ constexpr int kSlots = 4;
 // 512, graph replay: 256 rows 142.7 -> 133.6 us, 1013 153.0 -> 143.5, 4736 221.0 -> 214.6, 9472 312 -> 306; three tiles or
 // more alike.)
 __device__ __forceinline__ int sets_per_tile(int n_my) { return n_my == 1 ? 4 : (n_my == 2 ? 2 : 1); }
+
+// Tag of this execution's exchange words, from one thread to all of the CTA.  A replayed CUDA graph repeats the call's own
+// tag, so the group's generation counter goes into it.  It is read once per CTA and every word that the CTA publishes
+// carries what was read; the group's first CTA bumps it at its end, which it does not reach without words of all of them.
+// (Warps that each read the counter for themselves would not all have done so by then.)
+__device__ __forceinline__ void hand_out_tag(const RequantParams& rp, int group, uint32_t* slot, uint64_t* bar) {
+  *(volatile uint32_t*)slot = mix_tag(rp.tag, __ldcg(rp.generation + group));
+  mbar_arrive(smem_u32(bar));
+}
 constexpr int kExchangeBatch = 16;  // n-tiles whose words an exchange warp asks for at once (one 16-byte load each per lane)
 
 // Called between polls of a bounded wait: false once the CTA is aborting or the limit has passed
@@ -173,6 +182,8 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   __shared__ uint64_t ctx_free_bar[kSlots][2];   // the set's two warps on that half of the rows have read theirs
   __shared__ float part_amax[kSlots][kBM];       // tile shared by several sets: a set's maxima of its columns
   __shared__ uint64_t part_bar[kSlots][4];       // ... of lane quadrant q are there, by first set of the tile
+  __shared__ uint64_t tag_bar;                   // tag_slot is there
+  __shared__ uint32_t tag_slot;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
@@ -210,6 +221,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     for (int w = 0; w < EW; ++w) mbar_init(smem_u32(&res_bar[w]), 1);
     mbar_init(smem_u32(&b_loaded_bar), 1);
     mbar_init(smem_u32(&b_ready_bar), EW);
+    mbar_init(smem_u32(&tag_bar), 1);
     for (int b = 0; b < kSlots; ++b) {
       for (int h = 0; h < 2; ++h) {
         mbar_init(smem_u32(&ctx_ready_bar[b][h]), 1);
@@ -312,12 +324,10 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     // Two warps, each for one half of the tile's rows: lane l of warp h owns rows 64h + 2l and
     // 64h + 2l + 1, i.e. one 16-byte load (two words) per n-tile, kExchangeBatch of them in flight.
     const int xh = warp - (2 + EW);
-    bool ok = true;
     if (early_w) grid_dependency_wait();
-    // Tag of this execution's exchange words.  A replayed CUDA graph repeats the call's own tag, so the
-    // group's generation counter goes into it: every CTA of the group reads it at its start, and the
-    // group's first CTA bumps it after its last tile, which it cannot finish before all of them have started.
-    const uint32_t tag = mix_tag(rp.tag, __ldcg(rp.generation + group));
+    if (xh == 0 && lane == 0) hand_out_tag(rp, group, &tag_slot, &tag_bar);
+    bool ok = mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start);
+    const uint32_t tag = *(volatile uint32_t*)&tag_slot;
     for (int i = 0; ok && i < n_my; ++i) {
       const int tm = group + i * groups;
       const uint32_t par = i % kSlots, ph = (i / kSlots) & 1;
@@ -411,13 +421,14 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     }
 
     if (early_w) grid_dependency_wait();  // scales of the activations, residual, outputs: everything but the weights
-    const uint32_t tag = mix_tag(rp.tag, __ldcg(rp.generation + group));  // see the exchange warps
     uint32_t res_count = 0;  // residual boxes this warp has consumed (phase of its barrier)
     if (ok && has_res && lane == 0 && i_first < n_my) {
       const int r0 = (group + i_first * groups) * kBM + quad * 32, c0 = oc0 + c_begin * CW;
       mbar_arrive_expect_tx(smem_u32(&res_bar[ew]), kStageBufBytes);
       tma_load_2d(y_buf, &tm_r, c0 < n_out ? c0 : 0, r0 < p.M ? r0 : 0, smem_u32(&res_bar[ew]));
     }
+    if (ok) ok = mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start);
+    const uint32_t tag = *(volatile uint32_t*)&tag_slot;
 
     const uint32_t buf = (uint32_t)i_first;  // accumulator buffer and exchange slot of this warp's tiles (i mod 4)
     const uint32_t tbase = tmem_base + buf * BN + ((uint32_t)(quad * 32) << 16);

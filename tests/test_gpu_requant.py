@@ -275,6 +275,31 @@ def test_replayed_calls_that_share_a_workspace_keep_their_maxima_apart():
     assert aqt.aqt_device_status() == 0
 
 
+@pytest.mark.parametrize("M,N,K", [(1013, 512, 512), (300, 2048, 2048), (20000, 1024, 256), (3000, 512, 1024)])
+def test_many_replays_in_a_row(M, N, K):
+    """Replays with nothing between them: every CTA of each one has to find the count of its own (tiles of 32 columns, of
+    many k-blocks; weight-stationary tiles, several per CTA; the eight-k-block form)."""
+    rng = np.random.default_rng(M)
+    f = lambda lo, hi, n: _dev(rng.uniform(lo, hi, n).astype(np.float32))
+    args = (_dev(_codes(rng, M, K, 8)), f(1e-3, 5e-2, M), _dev(_codes(rng, N, K, 8)), f(1e-4, 5e-3, N))
+    with_y = K > 1024
+    ws = torch.empty(aqt.aqt_workspace_bytes(aqt.OP_QMATMUL_REQUANT, M, N, K, 8, 8), dtype=torch.uint8, device=DEV)
+    q, s, y = torch.empty(M, N, dtype=torch.int8, device=DEV), torch.empty(M, device=DEV), torch.empty(M, N, device=DEV)
+
+    def call():
+        aqt.aqt_qmatmul_requant(*args, K=K, q_out=q, s_out=s, y=y if with_y else None, workspace=ws)
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(4):
+            call()
+    for _ in range(100):
+        g.replay()
+    q_ref, s_ref = aqt.aqt_quantize(aqt.aqt_qmatmul(*args, K=K), 8)
+    assert torch.equal(s, s_ref) and torch.equal(q, q_ref) and aqt.aqt_device_status() == 0
+
+
 def test_requant_argument_checks():
     z8 = torch.zeros((64, 64), dtype=torch.int8, device=DEV)
     w8 = torch.zeros((48, 64), dtype=torch.int8, device=DEV)
