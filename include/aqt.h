@@ -76,6 +76,9 @@ extern "C" {
                                     kernel is still draining; everything else they touch still waits for it, and so do
                                     all other kernels. */
 
+#define AQT_MAY_WAIT 0x200 /* may be OR-ed into bits_w of aqt_qmatmul_requant: whatever the shape, the call may run in a kernel
+                              whose CTAs wait on one another (see there), and q_out and s_out are not xq and s_x. */
+
 /* operations for aqt_workspace_bytes */
 #define AQT_OP_QMATMUL 1
 #define AQT_OP_LINEAR_FWD 2
@@ -192,11 +195,16 @@ int aqt_qmatmul_with_plan(const char* plan, const void* xq, const float* s_x, in
  * Limits: those of aqt_qmatmul, and N_out % 16 == 0 (N_out % 32 == 0 if pack_out).  One kernel
  * does both steps for: K <= 512 with act NONE or SWISH; the GLU forms when only int8 codes and
  * scales are asked for (y == NULL, pack_out == 0); 512 < K <= 1024 when y == NULL; and K >= 2048
- * with act NONE or SWISH, M > 128, N <= 2048 and pack_out == 0 (with or without y).  The CTAs of
- * such a kernel wait on one another (row maxima cross CTAs), with the same bounded waits as
- * everything else, so it runs on at most one CTA per SM and reports AQT_ERR_TIMEOUT through the
- * device status word if other work keeps SMs from it for seconds.  Other calls run the two
- * steps one after the other through y and return AQT_ERR_UNSUPPORTED if y is NULL.
+ * with act NONE or SWISH, M > 128, N <= 2048 and pack_out == 0 (with or without y; one or two
+ * kernels by the size).  With AQT_MAY_WAIT, one kernel also for the other calls with y and
+ * pack_out == 0 whose output has few tiles.  The CTAs of such a kernel wait on one another (row
+ * maxima cross CTAs), with the same bounded waits as everything else.  All of them have to be on
+ * the device at once, one per SM and up to as many as there are SMs; the kernel reports
+ * AQT_ERR_TIMEOUT through the device status word if other work keeps SMs from it for seconds.
+ * Such other work is also a second call of this kind, on another stream, when each has got a
+ * part of the SMs that it needs; such calls are best on one stream, or ordered by events.  The
+ * remaining calls run the two steps one after the other through y, wait on nobody, and return
+ * AQT_ERR_UNSUPPORTED if y is NULL; q_out and s_out may then be xq and s_x.
  */
 int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w,
                         const float* bias, const float* residual, int64_t ldr, float residual_scale, int64_t M,
@@ -211,7 +219,8 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
  *   y            = aqt_qmatmul(act NONE, no residual), fp32 [M, N] with row pitch ldy
  *   q_out, s_out = aqt_quantize(y[:, first:], axis = AQT_AXIS_ROW, bits_out, rounding), int8 [M, N - first] dense, fp32 [M]
  * workspace as for aqt_qmatmul_requant of N channels.  first and N are multiples of 16.  One launch where the
- * output has few tiles, else aqt_qmatmul over the first channels and aqt_qmatmul_requant over the others.
+ * output has few tiles, else aqt_qmatmul over the first channels and aqt_qmatmul_requant over the others; the CTAs
+ * may wait on one another in every case, as there with AQT_MAY_WAIT.
  */
 int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w,
                              const float* bias, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int bits_out,

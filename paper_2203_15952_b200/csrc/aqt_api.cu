@@ -184,6 +184,13 @@ bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y
   return parts % 2 == 0 && parts <= 16 && ceil_div(N, kGemmPlanBn[plan]) <= sms / 2;
 }
 
+// The calls of aqt_qmatmul_requant that the header says may wait across CTAs.  The others are two kernels of which neither
+// does, unless the caller allows it: other work that holds SMs until it sees their result is then no deadlock, and the codes
+// may be written over those that were read.
+bool waits_across_ctas(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out) {
+  return requant_applies(M, N, K, act, with_y, pack_out) || (K >= 2048 && M > kBM && N <= 2048 && !is_glu(act) && !pack_out);
+}
+
 int validate_matmul_shape(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int s_x_kind) {
   if (M < 0 || N < 0 || K <= 0) return AQT_ERR_BADARG;
   if (!bits_ok(bits_a) || !bits_ok(bits_w) || !act_ok(act)) return AQT_ERR_BADARG;
@@ -358,6 +365,7 @@ const char* aqt_status_string(int status) {
 
 size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w) {
   if (M < 0 || N < 0 || K < 0) return 0;
+  bits_w &= ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
   if (op == AQT_OP_QMATMUL) return ws_qmatmul(M, N, K, bits_a, bits_w);
   if (op == AQT_OP_LINEAR_FWD) return ws_linear(M, N, K, bits_w);
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return ws_weight_only(0, N, K, AQT_FLOAT_TF32);
@@ -494,7 +502,8 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
                         int bits_w, int act, int bits_out, int rounding, int pack_out, void* q_out, float* s_out, float* y,
                         int64_t ldy, void* workspace, size_t workspace_bytes, void* stream) {
   const int static_w = (bits_w & AQT_STATIC_WEIGHTS) ? 1 : 0;
-  bits_w &= ~AQT_STATIC_WEIGHTS;
+  const bool may_wait = (bits_w & AQT_MAY_WAIT) != 0;
+  bits_w &= ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
   int rc = validate_matmul_shape(M, N, K, bits_a, bits_w, act, s_x_kind);
   if (rc != AQT_OK) return rc;
   if (!quant_bits_ok(bits_out) || (pack_out != 0 && pack_out != 1) || (pack_out == 1 && bits_out != 4)) return AQT_ERR_BADARG;
@@ -521,7 +530,8 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
 
   const bool ws_form = requant_applies(M, N, K, act, y != nullptr, pack_out != 0);
   const bool pair_form = !ws_form && rowquant_pair_applies(M, N, K, act, y != nullptr, pack_out != 0);
-  const int few_bn = pack_out || (!ws_form && !pair_form && y == nullptr) || sm_count() <= 0 ? 0 : few_tiles_bn(M, N, K, act, 0, sm_count());
+  const bool few_form = may_wait || waits_across_ctas(M, N, K, act, y != nullptr, pack_out != 0);
+  const int few_bn = pack_out || !few_form || (!ws_form && !pair_form && y == nullptr) || sm_count() <= 0 ? 0 : few_tiles_bn(M, N, K, act, 0, sm_count());
   if (few_bn != 0 && few_tiles_exchange_bytes(M, N, few_bn) <= workspace_bytes - mm_bytes) {
     const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
     if (is_packed(bits_a)) {
@@ -635,7 +645,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
 int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
                              int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int bits_out, int rounding, void* q_out, float* s_out,
                              float* y, int64_t ldy, void* workspace, size_t workspace_bytes, void* stream) {
-  const int static_w = (bits_w & AQT_STATIC_WEIGHTS) ? 1 : 0, width = bits_w & ~AQT_STATIC_WEIGHTS;
+  const int static_w = (bits_w & AQT_STATIC_WEIGHTS) ? 1 : 0, width = bits_w & ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
   int rc = validate_matmul_shape(M, N, K, bits_a, width, AQT_ACT_NONE, s_x_kind);
   if (rc != AQT_OK) return rc;
   if (first < 0 || first >= N || first % 16 != 0 || N % 16 != 0 || !quant_bits_ok(bits_out)) return AQT_ERR_BADARG;
@@ -666,7 +676,7 @@ int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, in
   }
   const uint8_t* w_rest = reinterpret_cast<const uint8_t*>(wq) + first * (is_packed(width) ? K / 2 : K);
   return aqt_qmatmul_requant(xq, s_x, s_x_kind, w_rest, s_w + first, bias == nullptr ? nullptr : bias + first, nullptr, 0, 0.0f, M, N - first, K,
-                             bits_a, bits_w, AQT_ACT_NONE, bits_out, rounding, 0, q_out, s_out, y + first, ldy, workspace, workspace_bytes, stream);
+                             bits_a, bits_w | AQT_MAY_WAIT, AQT_ACT_NONE, bits_out, rounding, 0, q_out, s_out, y + first, ldy, workspace, workspace_bytes, stream);
 }
 
 int aqt_linear_fwd(const float* x, int64_t ldx, const void* wq, const float* s_w, const float* bias, const float* residual,

@@ -249,7 +249,7 @@ class LayerRunner:
         s = layer.spec
         q, sc = self.code_buffers(role, s.n_out)
         aqt.aqt_qmatmul_requant(xq, s_x, layer.mm_weight, layer.s_w, layer.bias, residual, residual_scale, K=s.K, bits_a=_container_bits(s.bits_a),
-                                bits_w=layer.mm_bits | (aqt.STATIC_WEIGHTS if static else 0), act=s.act, s_x_kind=self.a_scale_kind, bits_out=bits_out,
+                                bits_w=layer.mm_bits | aqt.MAY_WAIT | (aqt.STATIC_WEIGHTS if static else 0), act=s.act, s_x_kind=self.a_scale_kind, bits_out=bits_out,
                                 rounding=self.rounding, pack_out=False, q_out=q, s_out=sc, y=y, workspace=self.workspace)
         return q, sc
 

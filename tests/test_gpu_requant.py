@@ -300,6 +300,24 @@ def test_many_replays_in_a_row(M, N, K):
     assert torch.equal(s, s_ref) and torch.equal(q, q_ref) and aqt.aqt_device_status() == 0
 
 
+@pytest.mark.parametrize("M,N,K,act", [(1013, 1024, 1024, aqt.ACT_NONE), (100, 2048, 2048, aqt.ACT_SWISH), (256, 1024, 512, aqt.ACT_GLU_SWISH),
+                                       (600, 1040, 1040, aqt.ACT_NONE)])
+def test_requant_calls_that_wait_on_nobody_write_over_their_input(M, N, K, act):
+    """With y and outside what the header lists, the codes are written behind the whole matmul, so they may replace the ones
+    that it read; with AQT_MAY_WAIT the same bits, in other buffers."""
+    rng = np.random.default_rng(M)
+    f = lambda lo, hi, n: _dev(rng.uniform(lo, hi, n).astype(np.float32))
+    n_out = N // 2 if act == aqt.ACT_GLU_SWISH else N
+    xq, s_x, wq, s_w = _dev(_codes(rng, M, K, 8)), f(1e-3, 5e-2, M), _dev(_codes(rng, N, K, 8)), f(1e-4, 5e-3, N)
+    assert n_out == K
+    y_ref = aqt.aqt_qmatmul(xq, s_x, wq, s_w, K=K, act=act)
+    q_ref, s_ref = aqt.aqt_quantize(y_ref, 8)
+    q, s, y = aqt.aqt_qmatmul_requant(xq, s_x, wq, s_w, K=K, act=act, bits_w=8 | aqt.MAY_WAIT, want_y=True)
+    assert torch.equal(y, y_ref) and torch.equal(q, q_ref) and torch.equal(s, s_ref)
+    aqt.aqt_qmatmul_requant(xq, s_x, wq, s_w, K=K, act=act, q_out=xq, s_out=s_x, y=y)
+    assert torch.equal(y, y_ref) and torch.equal(xq, q_ref) and torch.equal(s_x, s_ref) and aqt.aqt_device_status() == 0
+
+
 def test_requant_argument_checks():
     z8 = torch.zeros((64, 64), dtype=torch.int8, device=DEV)
     w8 = torch.zeros((48, 64), dtype=torch.int8, device=DEV)
