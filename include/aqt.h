@@ -151,13 +151,11 @@ int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, 
 
 /*
  * aqt_plan_qmatmul -- names the kernel configuration aqt_qmatmul (and every entry point that runs
- * the same matmul) would launch for a shape without a residual: "small_m", "ws128e16", "pair256s6e4", ...  Host-only:
+ * the same matmul) would launch for a shape without a residual: "small_m", "few64", "ws128e16", "pair256s6e4", ...  Host-only:
  * sm_count_or_0 > 0 plans for a device with that many multiprocessors, 0 for the current device
  * (148 if there is none).  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
  * aqt_linear_bwd with K in elements.  (No counterpart in the paper: the choice of tile shapes is
- * this library's.)  Outputs of a few tiles run in a kernel of their own ahead of this choice
- * (K <= 512, and deeper gate forms); the name is then that of the configuration behind it, which
- * acc_debug and aqt_qmatmul_with_plan reach.  name_out receives a NUL-terminated string of at most name_bytes bytes.
+ * this library's.)  name_out receives a NUL-terminated string of at most name_bytes bytes.
  */
 int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int float_kind,
                      int sm_count_or_0, char* name_out, size_t name_bytes);

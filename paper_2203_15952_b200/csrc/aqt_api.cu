@@ -229,8 +229,8 @@ int run_small_m(const void* xq, bool a_packed, const float* s_x, int s_x_kind, c
 // Arguments are checked, packed activations expanded; scratch: where packed weights that the kernel does not expand go.
 int run_few_tiles(int bn, const int8_t* a_codes, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
                   const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_w, bool static_w,
-                  int act, int64_t rq_first, int bits_out, int rounding, void* q_out, float* s_out, float* y, int64_t ldy, uint8_t* scratch,
-                  void* exchange, uint32_t* generation, cudaStream_t st) {
+                  int act, int64_t rq_first, int bits_out, int rounding, void* q_out, float* s_out, float* y, int64_t ldy,
+                  int32_t* acc_debug, uint8_t* scratch, void* exchange, uint32_t* generation, cudaStream_t st) {
   const void* b_codes = wq;
   bool b_packed = false;
   if (is_packed(bits_w)) {
@@ -248,7 +248,7 @@ int run_few_tiles(int bn, const int8_t* a_codes, const float* s_x, int s_x_kind,
   p.s_w = s_w;
   p.bias = bias;
   p.residual = residual;
-  p.acc_debug = nullptr;
+  p.acc_debug = acc_debug;
   p.ldr = ldr;
   p.residual_scale = residual_scale;
   p.s_x_kind = s_x_kind;
@@ -282,12 +282,12 @@ int qmatmul_i8a(const int8_t* a_codes, const float* s_x, int s_x_kind, const voi
     return run_small_m(a_codes, false, s_x, s_x_kind, wq, is_packed(bits_w), s_w, bias, residual, ldr, residual_scale, M, N, K, act, y, ldy,
                        acc_debug, st);
   }
-  if (forced_plan == kPlanNone && acc_debug == nullptr && sm_count() > 0) {
-    const int bn = few_tiles_bn(M, N, K, act, -1, sm_count());
-    if (bn != 0)
-      return run_few_tiles(bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w, act,
-                           is_glu(act) ? N / 2 : N, 8, AQT_ROUND_NEAREST_EVEN, nullptr, nullptr, y, ldy, ws, nullptr, nullptr, st);
-  }
+  const int few_bn = gemm_plan_is_few(forced_plan)                     ? kGemmPlanBn[forced_plan]
+                     : forced_plan == kPlanNone && sm_count() > 0 ? few_tiles_bn(M, N, K, act, -1, sm_count())
+                                                                  : 0;
+  if (few_bn != 0)
+    return run_few_tiles(few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w, act,
+                         is_glu(act) ? N / 2 : N, 8, AQT_ROUND_NEAREST_EVEN, nullptr, nullptr, y, ldy, acc_debug, ws, nullptr, nullptr, st);
   // 4-bit weights: the weight-stationary kernel (K <= 512) sign-extends them itself in shared
   // memory after TMA staging; deeper K takes a one-off sign-extended copy in the workspace.
   const void* b_codes = wq;
@@ -489,6 +489,8 @@ int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, in
   const char* name;
   if (!float_kind && small_m_applies(M, K)) {
     name = "small_m";
+  } else if (const int bn = float_kind ? 0 : few_tiles_bn(M, N, K, act, -1, sms)) {
+    name = gemm_plan_name(bn == 32 ? kPlanFew32 : (bn == 64 ? kPlanFew64 : kPlanFew128));
   } else {
     name = gemm_plan_name(plan_qgemm(GemmShape{M, N, float_kind ? 4 * K : K, act, float_kind ? 1 : 0, false}, sms));
   }
@@ -541,7 +543,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
       ws += round_up((size_t)M * (size_t)K, 256);
     }
     return run_few_tiles(few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w != 0, act, 0,
-                             bits_out, rounding, q_out, s_out, y, ldy, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes,
+                             bits_out, rounding, q_out, s_out, y, ldy, nullptr, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes,
                              generation_counters(workspace, workspace_bytes), st);
   }
   if (pair_form) {
@@ -666,7 +668,7 @@ int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, in
   const int bn = sms > 0 && !is_packed(bits_a) ? few_tiles_bn(M, N, K, AQT_ACT_NONE, first, sms) : 0;
   if (bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= workspace_bytes - mm_bytes)
     return run_few_tiles(bn, reinterpret_cast<const int8_t*>(xq), s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, width, static_w != 0,
-                             AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, reinterpret_cast<uint8_t*>(workspace),
+                             AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, nullptr, reinterpret_cast<uint8_t*>(workspace),
                              reinterpret_cast<uint8_t*>(workspace) + mm_bytes, generation_counters(workspace, workspace_bytes), st);
   // the two parts one after the other (row `first` of the weights keeps the 16-byte alignment: `first` and K are multiples of 16)
   if (first > 0) {

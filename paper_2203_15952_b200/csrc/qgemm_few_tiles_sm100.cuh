@@ -81,6 +81,15 @@ __device__ __forceinline__ void swish_cols(float (&a)[C]) {
   for (int j = 0; j < C; ++j) a[j] = __fmul_rn(a[j], sigmoid_f(a[j]));
 }
 
+// Accumulators of row m from column n on, those below `limit`, as the matrix product that they are (DEBUG).
+template <int C>
+__device__ __forceinline__ void dump_acc(const GemmParams& p, int m, int n, int limit, const uint32_t (&acc)[C]) {
+  if (m >= p.M) return;
+#pragma unroll
+  for (int j = 0; j < C; ++j)
+    if (n + j < limit) p.acc_debug[(int64_t)m * p.N + n + j] = (int32_t)acc[j];
+}
+
 // Byte offset of 16-byte chunk j of row r in a box of 32 rows x C floats as the copy engine lays it out under the
 // swizzle of its row length (32, 64 or 128 bytes).
 template <int C>
@@ -90,7 +99,7 @@ __device__ __forceinline__ uint32_t box_offset(int r, int j) {
   return (uint32_t)(r * 32 + ((j ^ ((r >> 2) & 1)) << 4));
 }
 
-template <int BN, bool GLU>
+template <int BN, bool GLU, bool DEBUG>
 __global__ void __launch_bounds__(32 * 20, 1)
 qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                        const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_r, const FewTilesParams fp) {
@@ -341,6 +350,8 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         tmem_ld_cols(t_addr + HALF, accg);
         tmem_ld_cols(t_addr, acc);
         tmem_ld_wait();
+        if (DEBUG) dump_acc<C>(p, m, p.N / 2 + oc, p.N, accg);
+        if (DEBUG) dump_acc<C>(p, m, oc, p.N / 2, acc);
         dequant_cols<C>(accg, sx, slab + C * 4, slab_bias + C * 4, g);
         dequant_cols<C>(acc, sx, slab, slab_bias, a);
 #pragma unroll
@@ -349,6 +360,7 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       } else {
         tmem_ld_cols(t_addr, acc);
         tmem_ld_wait();
+        if (DEBUG) dump_acc<C>(p, m, oc, p.N, acc);
         dequant_cols<C>(acc, sx, slab, slab_bias, a);
         if (p.act == AQT_ACT_SWISH) swish_cols<C>(a);
       }
@@ -471,8 +483,8 @@ static size_t few_tiles_exchange_bytes(int64_t M, int64_t N, int bn) {
   return round_up((size_t)ceil_div(M, kBM) * (size_t)ceil_div(N, bn) * kBM * 8 + (size_t)kMaxGroups * 4, 256);
 }
 
-template <int BN, bool GLU>
-static int launch_few_tiles_inst(const int8_t* a, const void* b, float* y, int64_t ldy, FewTilesParams fp, cudaStream_t st) {
+template <int BN, bool GLU, bool DEBUG>
+static int launch_few_tiles_form(const int8_t* a, const void* b, float* y, int64_t ldy, FewTilesParams fp, cudaStream_t st) {
   using Cfg = FewTilesCfg<BN, GLU>;
   GemmParams& p = fp.rp.g;
   p.tiles_m = (int)ceil_div(p.M, kBM);
@@ -506,12 +518,18 @@ static int launch_few_tiles_inst(const int8_t* a, const void* b, float* y, int64
     rc = make_map_2d(&tm_r, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, p.residual, (uint64_t)p.M, (uint64_t)p.n_out, (uint64_t)p.ldr * 4, 32, Cfg::C, 4 * Cfg::C);
     if (rc != AQT_OK) return rc;
   }
-  auto kernel = qgemm_few_tiles_kernel<BN, GLU>;
+  auto kernel = qgemm_few_tiles_kernel<BN, GLU, DEBUG>;
   static std::atomic<uint64_t> smem_opted_in{0};
   rc = ensure_dynamic_smem(kernel, Cfg::kSmemBytes, smem_opted_in);
   if (rc != AQT_OK) return rc;
   return launch_pdl(kernel, dim3((unsigned)(p.tiles_m * p.tiles_n), 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 1, tm_a, tm_b, tm_y,
                     tm_r, fp);
+}
+
+template <int BN, bool GLU>
+static int launch_few_tiles_inst(const int8_t* a, const void* b, float* y, int64_t ldy, const FewTilesParams& fp, cudaStream_t st) {
+  return fp.rp.g.acc_debug != nullptr ? launch_few_tiles_form<BN, GLU, true>(a, b, y, ldy, fp, st)
+                                      : launch_few_tiles_form<BN, GLU, false>(a, b, y, ldy, fp, st);
 }
 
 // a: int8 [M, K]; b: int8 [N, K], or (fp.b_packed) nibbles [N, K/2]; y may be null if every column is quantized.

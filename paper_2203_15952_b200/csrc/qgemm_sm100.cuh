@@ -1253,12 +1253,15 @@ enum GemmPlan {
   kPlanPair128S6E8,
   kPlanPair128S8E4,
   kPlanPair512S3E16,    // CTA pairs on 256 x 512 tiles, one accumulator buffer (few, deep tiles)
+  kPlanFew32,           // outputs of a few tiles, one per CTA (qgemm_few_tiles_sm100.cuh): a kernel of its own, chosen and
+  kPlanFew64,           //   launched ahead of plan_qgemm and launch_qgemm (few_tiles_bn)
+  kPlanFew128,
   kPlanCount
 };
 static const char* const kGemmPlanNames[kPlanCount] = {
     "none",          "ws128e16",      "ws128e8",       "stream256s3e16", "stream256s4e4", "stream256s4e8",
     "stream128s4e16", "stream128s6e4", "stream128s4e8", "stream64s5e8",   "stream64s8e4",  "pair256s4e8",
-    "pair256s6e4",   "pair128s6e8",   "pair128s8e4",   "pair512s3e16"};
+    "pair256s6e4",   "pair128s6e8",   "pair128s8e4",   "pair512s3e16",   "few32",         "few64",         "few128"};
 static const char* gemm_plan_name(int plan) { return plan > 0 && plan < kPlanCount ? kGemmPlanNames[plan] : kGemmPlanNames[0]; }
 static int gemm_plan_by_name(const char* name) {
   if (name == nullptr) return kPlanNone;
@@ -1405,15 +1408,16 @@ static int plan_qgemm(const GemmShape& g, int sms) {
   return deep_k ? kPlanStream64S8E4 : kPlanStream64S5E8;
 }
 
+static bool gemm_plan_is_few(int plan) { return plan >= kPlanFew32 && plan <= kPlanFew128; }
 static bool gemm_plan_is_pair(int plan) { return plan >= kPlanPair256S4E8 && plan <= kPlanPair512S3E16; }
 
 // Tile width and epilogue warps of each plan (same order as GemmPlan).
-static const int kGemmPlanBn[kPlanCount] = {0, 128, 128, 256, 256, 256, 128, 128, 128, 64, 64, 256, 256, 128, 128, 512};
-static const int kGemmPlanEw[kPlanCount] = {0, 16, 8, 16, 4, 8, 16, 4, 8, 8, 4, 8, 4, 8, 4, 16};
+static const int kGemmPlanBn[kPlanCount] = {0, 128, 128, 256, 256, 256, 128, 128, 128, 64, 64, 256, 256, 128, 128, 512, 32, 64, 128};
+static const int kGemmPlanEw[kPlanCount] = {0, 16, 8, 16, 4, 8, 16, 4, 8, 8, 4, 8, 4, 8, 4, 16, 16, 16, 16};
 
 // True if `plan` can run this shape at all (used when a caller names the plan itself).
 static bool gemm_plan_takes(int plan, const GemmShape& g, int sms) {
-  if (plan <= kPlanNone || plan >= kPlanCount) return false;
+  if (plan <= kPlanNone || plan >= kPlanCount || gemm_plan_is_few(plan)) return false;
   const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
   const bool ws = plan == kPlanWs128E16 || plan == kPlanWs128E8;
   const bool pair = gemm_plan_is_pair(plan);

@@ -112,7 +112,8 @@ def test_plan_query_and_new_entry_points_reject_bad_arguments():
     i64, vp = ctypes.c_int64, ctypes.c_void_p
     one = vp(256)
     buf = ctypes.create_string_buffer(64)
-    assert L.aqt_plan_qmatmul(i64(1000), i64(512), i64(512), 8, 4, 0, 0, 148, buf, ctypes.c_size_t(64)) == 0 and buf.value == b"ws128e16"
+    assert L.aqt_plan_qmatmul(i64(1000), i64(512), i64(512), 8, 4, 0, 0, 148, buf, ctypes.c_size_t(64)) == 0 and buf.value == b"few32"
+    assert L.aqt_plan_qmatmul(i64(12800), i64(512), i64(512), 8, 4, 0, 0, 148, buf, ctypes.c_size_t(64)) == 0 and buf.value == b"ws128e16"
     assert L.aqt_plan_qmatmul(i64(1000), i64(512), i64(512), 8, 4, 0, 0, 148, buf, ctypes.c_size_t(4)) == -1      # name does not fit
     assert L.aqt_plan_qmatmul(i64(0), i64(512), i64(512), 8, 4, 0, 0, 148, buf, ctypes.c_size_t(64)) == -1
     assert L.aqt_plan_qmatmul(i64(8), i64(512), i64(512), 8, 5, 0, 0, 148, buf, ctypes.c_size_t(64)) == -1         # unknown width

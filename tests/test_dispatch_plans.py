@@ -21,6 +21,9 @@ COVERED_BY = {
     "small_m": ("test_gpu_kernels.py", "test_qmatmul_small_batch"),
     "ws128e16": ("test_gpu_kernels.py", "test_qmatmul_single_cta_plans_named"),
     "ws128e8": ("test_gpu_kernels.py", "test_qmatmul_activations"),
+    "few32": ("test_gpu_few_tiles.py", "test_few_tiles_plans_named"),
+    "few64": ("test_gpu_few_tiles.py", "test_few_tiles_plans_named"),
+    "few128": ("test_gpu_few_tiles.py", "test_few_tiles_plans_named"),
     "stream256s3e16": ("test_gpu_kernels.py", "test_qmatmul_single_cta_plans_named"),
     "stream256s4e4": ("test_gpu_kernels.py", "test_qmatmul_single_cta_plans_named"),
     "stream128s4e16": ("test_gpu_kernels.py", "test_qmatmul_single_cta_plans_named"),
@@ -77,7 +80,8 @@ def test_plans_of_the_headline_shapes():
     assert p(65536, 1024, 4096, 8, 4) == "pair256s6e4"
     assert p(65536, 4096, 1024, 8, 4, gen.ACT_SWISH) == "stream256s3e16"
     assert p(8, 512, 2048, 8, 4) == "small_m"
-    assert p(64, 256, 256, 8, 8) == "ws128e16"
+    assert p(64, 256, 256, 8, 8) == "few32" and p(1013, 1024, 512, 8, 4) == "few64" and p(4736, 512, 512, 8, 4) == "few128"
+    assert p(4737, 512, 512, 8, 4) == "ws128e16" and p(300, 1024, 1024, 8, 4, gen.ACT_GLU_SWISH) == "few64"
     # the float kind (weight-only layer, backward) plans with K in elements
     assert p(65536, 1024, 4096, 0, 4, float_kind=True) == "pair256s6e4"
     # a device with other SM counts changes the choice only through the number of rounds

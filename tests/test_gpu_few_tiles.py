@@ -6,6 +6,7 @@ import torch
 
 import oracle as orc
 from paper_2203_15952_b200 import binding as aqt
+from test_gpu_kernels import _run_qmatmul
 from test_gpu_requant import _codes, _dev, _run
 
 pytestmark = pytest.mark.gpu
@@ -26,6 +27,25 @@ def test_few_tiles_requant(M, N, K, with_res):
 @pytest.mark.parametrize("rounding", [aqt.ROUND_NEAREST_EVEN, aqt.ROUND_HALF_UP_FLOOR])
 def test_few_tiles_packed_weights_swish(M, N, K, rounding):
     _run(M, N, K, 4, 4, aqt.ACT_SWISH, False, False, 4, rounding, False)
+
+
+@pytest.mark.parametrize("plan", ["few32", "few64", "few128"])
+def test_few_tiles_plans_named(plan):
+    # accumulators and output of every width, whether or not the library would choose it: one row, edges of tiles in both
+    # directions, one k-block up to several turns of the ring, packed weights expanded in the kernel and ahead of it
+    _run_qmatmul(1, 4, 32, 8, 8, aqt.ACT_NONE, True, True, plan=plan, extremes=True)
+    _run_qmatmul(129, 36, 512, 8, 4, aqt.ACT_SWISH, True, True, plan=plan)
+    _run_qmatmul(333, 1000, 400, 4, 4, aqt.ACT_NONE, False, False, plan=plan, s_x_kind=aqt.SCALE_TENSOR)
+    _run_qmatmul(700, 260, 1296, 8, 8, aqt.ACT_NONE, True, True, plan=plan)
+    if plan != "few32":
+        _run_qmatmul(200, 520, 512, 8, 4, aqt.ACT_GLU, True, True, plan=plan)
+        _run_qmatmul(129, 72, 1040, 8, 8, aqt.ACT_GLU_SWISH, False, False, plan=plan)
+    with pytest.raises(aqt.AqtError) as e:  # a tile per SM, and no more
+        _run_qmatmul(149 * 128, 32, 32, 8, 8, aqt.ACT_NONE, False, False, plan=plan)
+    assert e.value.status == -3
+    with pytest.raises(aqt.AqtError) as e:
+        _run_qmatmul(130, 64, 64, 8, 8, aqt.ACT_GLU, False, False, plan="few32")
+    assert e.value.status == -3
 
 
 @pytest.mark.parametrize("M,N,K,first", [(200, 768, 256, 512), (1013, 1536, 512, 1024), (1537, 1536, 512, 1024), (140, 96, 64, 32), (300, 480, 128, 16)])

@@ -225,9 +225,10 @@ def test_qmatmul_int4_operands(bits_a, bits_w, M, N, K):
 @pytest.mark.parametrize("act", [aqt.ACT_SWISH, aqt.ACT_GLU, aqt.ACT_GLU_SWISH])
 @pytest.mark.parametrize("M,N,K", [(256, 512, 256), (300, 1024, 512), (100, 136, 64)])
 def test_qmatmul_activations(act, M, N, K):
-    if act != aqt.ACT_SWISH and M > 128:
-        assert aqt.aqt_plan_qmatmul(M, N, K, 8, 4, act) == "ws128e8"      # the GLU forms of the weight-stationary kernel
+    assert aqt.aqt_plan_qmatmul(M, N, K, 8, 4, act) == ("few32" if act == aqt.ACT_SWISH else "few64")
     _run_qmatmul(M, N, K, 8, 4, act, True, True)
+    # the forms of the weight-stationary kernel, which more rows take
+    _run_qmatmul(M, N, K, 8, 4, act, True, True, plan="ws128e16" if act == aqt.ACT_SWISH else "ws128e8")
 
 
 @pytest.mark.parametrize("plan", ["stream128s4e8", "stream256s3e16"])
