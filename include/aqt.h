@@ -211,6 +211,18 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
                         size_t workspace_bytes, void* stream);
 
 /*
+ * aqt_plan_qmatmul_requant -- names how aqt_qmatmul_requant (first == 0) or aqt_qmatmul_requant_from runs
+ * a call: "few32", "few64", "few128" (outputs of a few tiles), "ws128" (weights kept in shared memory),
+ * "pair256s4e8" (CTA pairs), all of them one kernel, or "two_kernels"; with first > 0, where one kernel
+ * does not take all columns, how the quantized ones run.  Host-only.  AQT_ERR_UNSUPPORTED for a call that
+ * would be refused so.  bits_w with AQT_MAY_WAIT or without; workspace_bytes of the call, 0 for what
+ * aqt_workspace_bytes says; the other arguments as aqt_plan_qmatmul.
+ */
+int aqt_plan_qmatmul_requant(int64_t first, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act,
+                             int with_y, int pack_out, size_t workspace_bytes, int sm_count_or_0, char* name_out,
+                             size_t name_bytes);
+
+/*
  * aqt_qmatmul_requant_from -- one matmul over N stacked output channels of which the last ones, from
  * column `first` on, are quantized for the next layer (query, key and value projections: only the value
  * is the input of a quantized layer):

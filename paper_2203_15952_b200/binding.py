@@ -33,7 +33,7 @@ STATIC_WEIGHTS = 0x100  # OR into bits_w: the weights were complete before the p
 EXPORTS = ("aqt_version", "aqt_status_string", "aqt_quantize", "aqt_pack_int4", "aqt_unpack_int4", "aqt_qmatmul",
            "aqt_linear_fwd", "aqt_linear_fwd_host", "aqt_workspace_bytes", "aqt_device_status", "aqt_qmatmul_w4_noalloc",
            "aqt_selftest_bounded_wait", "aqt_qmatmul_requant", "aqt_qmatmul_requant_from", "aqt_linear_fwd_weight_only", "aqt_linear_bwd",
-           "aqt_plan_qmatmul", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_chain_fwd", "aqt_selftest_sfu_rate")
+           "aqt_plan_qmatmul", "aqt_plan_qmatmul_requant", "aqt_qmatmul_with_plan", "aqt_ffn_fwd", "aqt_chain_fwd", "aqt_selftest_sfu_rate")
 NOALLOC_MAX_WEIGHT_BYTES = 4 << 20
 CHAIN_MAX_ROWS = 112
 
@@ -183,6 +183,16 @@ def aqt_plan_qmatmul(M: int, N: int, K: int, bits_a: int = 8, bits_w: int = 8, a
     buf = ctypes.create_string_buffer(64)
     _check("aqt_plan_qmatmul", lib().aqt_plan_qmatmul(_i64(M), _i64(N), _i64(K), int(bits_a), int(bits_w), int(act),
                                                       int(bool(float_kind)), int(sm_count), buf, ctypes.c_size_t(64)))
+    return buf.value.decode()
+
+
+def aqt_plan_qmatmul_requant(M: int, N: int, K: int, bits_a: int = 8, bits_w: int = 8, act: int = ACT_NONE, with_y: bool = False,
+                             pack_out: bool = False, first: int = 0, workspace_bytes: int = 0, sm_count: int = 0) -> str:
+    """How aqt_qmatmul_requant, or with `first` aqt_qmatmul_requant_from, runs a call (host-only)."""
+    buf = ctypes.create_string_buffer(64)
+    _check("aqt_plan_qmatmul_requant",
+           lib().aqt_plan_qmatmul_requant(_i64(first), _i64(M), _i64(N), _i64(K), int(bits_a), int(bits_w), int(act), int(bool(with_y)),
+                                          int(bool(pack_out)), ctypes.c_size_t(workspace_bytes), int(sm_count), buf, ctypes.c_size_t(64)))
     return buf.value.decode()
 
 

@@ -165,12 +165,11 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
 
 // True if the CTA-pair kernel with the row-quantizing epilogue takes the call: deep K, no GLU, int8
 // codes out (4-bit codes stay in their containers), at most 16 column parts per row.
-bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out) {
+bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out, int sms) {
   // (from K = 2048: at K = 1024 a tile's MMAs are shorter than its two epilogue passes, and the
   // two kernels are faster: 162 vs 209 us at 65 536 x 1024 -> 1024 with the fp32 output)
   if (pack_out || M <= kBM || K < 2048) return false;
   if (act != AQT_ACT_NONE && act != AQT_ACT_SWISH) return false;
-  const int sms = sm_count() > 0 ? sm_count() : kDefaultSms;
   // With the fp32 output, few pair tiles leave most of the chip idle: narrow tiles and the row quantizer behind them take 9.3
   // against 14.2 us at 1024 x 2048 -> 512, 11.5 against 15.1 us at 4096 rows, 15.3 against 16.0 us at 8192 (64 tiles).
   // (But not where the matmul ahead of the row quantizer would be left between its forms, with more single-CTA tiles of 128
@@ -187,8 +186,31 @@ bool rowquant_pair_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y
 // The calls of aqt_qmatmul_requant that the header says may wait across CTAs.  The others are two kernels of which neither
 // does, unless the caller allows it: other work that holds SMs until it sees their result is then no deadlock, and the codes
 // may be written over those that were read.
-bool waits_across_ctas(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out) {
-  return requant_applies(M, N, K, act, with_y, pack_out) || (K >= 2048 && M > kBM && N <= 2048 && !is_glu(act) && !pack_out);
+bool waits_across_ctas(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out, int sms) {
+  return requant_applies(M, N, K, act, with_y, pack_out, sms) || (K >= 2048 && M > kBM && N <= 2048 && !is_glu(act) && !pack_out);
+}
+
+// How aqt_qmatmul_requant runs a call: one kernel (tiles of few_bn columns, weight-stationary tiles, CTA pairs), the two steps
+// through y, or not at all.  exchange_room: workspace beyond what the matmul needs, at least requant_exchange_bytes.
+enum RequantForm { kRequantRefused, kRequantFew, kRequantWs, kRequantPair, kRequantTwoKernels };
+struct RequantRoute {
+  RequantForm form;
+  int few_bn;
+};
+RequantRoute requant_route(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out, bool may_wait, size_t exchange_room, int sms) {
+  const bool ws_form = requant_applies(M, N, K, act, with_y, pack_out, sms);
+  const bool pair_form = !ws_form && rowquant_pair_applies(M, N, K, act, with_y, pack_out, sms);
+  if (!ws_form && !pair_form && !with_y) return {kRequantRefused, 0};
+  if (!pack_out && (may_wait || waits_across_ctas(M, N, K, act, with_y, pack_out, sms))) {
+    const int bn = few_tiles_bn(M, N, K, act, 0, sms);
+    if (bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= exchange_room) return {kRequantFew, bn};
+  }
+  return {ws_form ? kRequantWs : (pair_form ? kRequantPair : kRequantTwoKernels), 0};
+}
+// The same for aqt_qmatmul_requant_from: 0, or the width of the tiles that take all columns in one launch.
+int requant_from_bn(int64_t first, int64_t M, int64_t N, int64_t K, int bits_a, size_t exchange_room, int sms) {
+  const int bn = is_packed(bits_a) ? 0 : few_tiles_bn(M, N, K, AQT_ACT_NONE, first, sms);
+  return bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= exchange_room ? bn : 0;
 }
 
 int validate_matmul_shape(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int s_x_kind) {
@@ -372,7 +394,7 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY_X2) return ws_weight_only(M, N, K, AQT_FLOAT_TF32X2);
   if (op == AQT_OP_LINEAR_BWD) return bwd_workspace(M, N, K);
   if (op == AQT_OP_FFN_FWD) return ffn_layout(M, K, N, bits_w, bits_w).total;
-  if (op == AQT_OP_QMATMUL_REQUANT) return round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256) + requant_exchange_bytes_few(M, N);
+  if (op == AQT_OP_QMATMUL_REQUANT) return round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256) + requant_exchange_bytes_few(M, N, sm_count() > 0 ? sm_count() : kDefaultSms);
   return 0;
 }
 
@@ -499,6 +521,38 @@ int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, in
   return AQT_OK;
 }
 
+int aqt_plan_qmatmul_requant(int64_t first, int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int with_y, int pack_out,
+                             size_t workspace_bytes, int sm_count_or_0, char* name_out, size_t name_bytes) {
+  const bool may_wait = (bits_w & AQT_MAY_WAIT) != 0;
+  bits_w &= ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
+  if (name_out == nullptr || name_bytes == 0 || M <= 0 || N <= 0 || first < 0 || first >= N || first % 16 != 0) return AQT_ERR_BADARG;
+  const int rc = validate_matmul_shape(M, N, K, bits_a, bits_w, act, AQT_SCALE_ROW);
+  if (rc != AQT_OK) return rc;
+  if ((is_glu(act) ? N / 2 : N) % (pack_out ? 32 : 16) != 0 || (first > 0 && (act != AQT_ACT_NONE || pack_out || !with_y))) return AQT_ERR_BADARG;
+  int sms = sm_count_or_0;
+  if (sms <= 0) sms = sm_count();
+  if (sms <= 0) sms = kDefaultSms;
+  const size_t mm_bytes = round_up(ws_qmatmul(M, N, K, bits_a, bits_w), 256);
+  if (workspace_bytes == 0) workspace_bytes = mm_bytes + requant_exchange_bytes_few(M, N, sms);
+  if (workspace_bytes < mm_bytes + requant_exchange_bytes(M, N)) return AQT_ERR_WORKSPACE;
+  RequantRoute r = {kRequantFew, first > 0 ? requant_from_bn(first, M, N, K, bits_a, workspace_bytes - mm_bytes, sms) : 0};
+  if (r.few_bn == 0) {
+    const size_t room = workspace_bytes - round_up(ws_qmatmul(M, N - first, K, bits_a, bits_w), 256);
+    r = requant_route(M, N - first, K, act, with_y != 0, pack_out != 0, may_wait || first > 0, room, sms);
+  }
+  const char* name = nullptr;
+  switch (r.form) {
+    case kRequantRefused: return AQT_ERR_UNSUPPORTED;
+    case kRequantFew: name = gemm_plan_name(r.few_bn == 32 ? kPlanFew32 : (r.few_bn == 64 ? kPlanFew64 : kPlanFew128)); break;
+    case kRequantWs: name = "ws128"; break;
+    case kRequantPair: name = gemm_plan_name(rowquant_plan(M, N - first, K, sms)); break;
+    case kRequantTwoKernels: name = "two_kernels"; break;
+  }
+  if (strlen(name) + 1 > name_bytes) return AQT_ERR_BADARG;
+  memcpy(name_out, name, strlen(name) + 1);
+  return AQT_OK;
+}
+
 int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const void* wq, const float* s_w, const float* bias,
                         const float* residual, int64_t ldr, float residual_scale, int64_t M, int64_t N, int64_t K, int bits_a,
                         int bits_w, int act, int bits_out, int rounding, int pack_out, void* q_out, float* s_out, float* y,
@@ -530,11 +584,11 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
 
-  const bool ws_form = requant_applies(M, N, K, act, y != nullptr, pack_out != 0);
-  const bool pair_form = !ws_form && rowquant_pair_applies(M, N, K, act, y != nullptr, pack_out != 0);
-  const bool few_form = may_wait || waits_across_ctas(M, N, K, act, y != nullptr, pack_out != 0);
-  const int few_bn = pack_out || !few_form || (!ws_form && !pair_form && y == nullptr) || sm_count() <= 0 ? 0 : few_tiles_bn(M, N, K, act, 0, sm_count());
-  if (few_bn != 0 && few_tiles_exchange_bytes(M, N, few_bn) <= workspace_bytes - mm_bytes) {
+  const int sms = sm_count();
+  if (sms <= 0) return AQT_ERR_CUDA;
+  const RequantRoute route = requant_route(M, N, K, act, y != nullptr, pack_out != 0, may_wait, workspace_bytes - mm_bytes, sms);
+  if (route.form == kRequantRefused) return AQT_ERR_UNSUPPORTED;
+  if (route.form == kRequantFew) {
     const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
     if (is_packed(bits_a)) {
       rc = launch_unpack_int4(reinterpret_cast<const uint8_t*>(xq), M * K / 2, reinterpret_cast<int8_t*>(ws), st);
@@ -542,11 +596,11 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
       a_codes = reinterpret_cast<const int8_t*>(ws);
       ws += round_up((size_t)M * (size_t)K, 256);
     }
-    return run_few_tiles(few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w != 0, act, 0,
+    return run_few_tiles(route.few_bn, a_codes, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_w, static_w != 0, act, 0,
                              bits_out, rounding, q_out, s_out, y, ldy, nullptr, ws, reinterpret_cast<uint8_t*>(workspace) + mm_bytes,
                              generation_counters(workspace, workspace_bytes), st);
   }
-  if (pair_form) {
+  if (route.form == kRequantPair) {
     // Deep K (the second feed-forward layers): the CTA-pair kernel with the row-quantizing epilogue
     const int8_t* a_codes = reinterpret_cast<const int8_t*>(xq);
     if (is_packed(bits_a)) {
@@ -585,13 +639,9 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
     p.qmax_out = qmax_of(bits_out);
     p.rounding = rounding;
     p.has_y = y != nullptr ? 1 : 0;
-    const int sms = sm_count();
-    if (sms <= 0) return AQT_ERR_CUDA;
     return launch_qgemm_rowquant(rowquant_plan(M, N, K, sms), a_codes, b_codes, y, ldy, p, st);
   }
-  if (!ws_form) {
-    // Shapes the fused kernels do not take: the two steps one after the other, through y.
-    if (y == nullptr) return AQT_ERR_UNSUPPORTED;
+  if (route.form == kRequantTwoKernels) {
     rc = aqt_qmatmul(xq, s_x, s_x_kind, wq, s_w, bias, residual, ldr, residual_scale, M, N, K, bits_a, bits_w, act, y, ldy, nullptr,
                      workspace, mm_bytes, stream);
     if (rc != AQT_OK) return rc;
@@ -665,8 +715,9 @@ int aqt_qmatmul_requant_from(int64_t first, const void* xq, const float* s_x, in
   if (rc != AQT_OK) return rc;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int sms = sm_count();
-  const int bn = sms > 0 && !is_packed(bits_a) ? few_tiles_bn(M, N, K, AQT_ACT_NONE, first, sms) : 0;
-  if (bn != 0 && few_tiles_exchange_bytes(M, N, bn) <= workspace_bytes - mm_bytes)
+  if (sms <= 0) return AQT_ERR_CUDA;
+  const int bn = requant_from_bn(first, M, N, K, bits_a, workspace_bytes - mm_bytes, sms);
+  if (bn != 0)
     return run_few_tiles(bn, reinterpret_cast<const int8_t*>(xq), s_x, s_x_kind, wq, s_w, bias, nullptr, 0, 0.0f, M, N, K, width, static_w != 0,
                              AQT_ACT_NONE, first, bits_out, rounding, q_out, s_out, y, ldy, nullptr, reinterpret_cast<uint8_t*>(workspace),
                              reinterpret_cast<uint8_t*>(workspace) + mm_bytes, generation_counters(workspace, workspace_bytes), st);
@@ -827,7 +878,7 @@ int aqt_ffn_fwd(const float* x, int x_on_host, const void* w1q, const float* s_w
   if (!is_aligned(workspace, 256)) return AQT_ERR_ALIGN;
   int rc = check_device();
   if (rc != AQT_OK) return rc;
-  if (!requant_applies(M, ff, d, act, false, false)) return AQT_ERR_UNSUPPORTED;
+  if (!requant_applies(M, ff, d, act, false, false, sm_count() > 0 ? sm_count() : kDefaultSms)) return AQT_ERR_UNSUPPORTED;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   float* x_copy = reinterpret_cast<float*>(ws + L.x);

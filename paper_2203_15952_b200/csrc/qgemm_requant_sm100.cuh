@@ -631,16 +631,15 @@ static size_t requant_exchange_bytes(int64_t M, int64_t N) {
 }
 // With room for the narrow tiles of qgemm_few_tiles_sm100.cuh (as many of 32 columns as there are SMs), which a call whose
 // area is smaller does without.
-static size_t requant_exchange_bytes_few(int64_t M, int64_t N) {
-  const size_t tiles32 = (size_t)ceil_div(M, kBM) * (size_t)ceil_div(N, 32), sms = (size_t)(sm_count() > 0 ? sm_count() : kDefaultSms);
-  const size_t few_form = round_up((tiles32 < sms ? tiles32 : sms) * kBM * 8 + (size_t)kMaxGroups * 4, 256), others = requant_exchange_bytes(M, N);
+static size_t requant_exchange_bytes_few(int64_t M, int64_t N, int sms) {
+  const size_t tiles32 = (size_t)ceil_div(M, kBM) * (size_t)ceil_div(N, 32);
+  const size_t few_form = round_up((tiles32 < (size_t)sms ? tiles32 : (size_t)sms) * kBM * 8 + (size_t)kMaxGroups * 4, 256), others = requant_exchange_bytes(M, N);
   return few_form > others ? few_form : others;
 }
 
 // True if this kernel takes the call: K <= 512; NONE / Swish in every form, the GLU forms when
 // only int8 codes and scales are asked for (no fp32 output, hence no residual, no nibble packing).
-static bool requant_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out) {
-  const int sms = sm_count() > 0 ? sm_count() : kDefaultSms;
+static bool requant_applies(int64_t M, int64_t N, int64_t K, int act, bool with_y, bool pack_out, int sms) {
   if (!(M > 0 && ceil_div(N, 128) <= sms)) return false;
   const bool glu = !(act == AQT_ACT_NONE || act == AQT_ACT_SWISH);
   if (ceil_div(K, kBK) <= kWsMaxKBlocks) return !glu || (!with_y && !pack_out);

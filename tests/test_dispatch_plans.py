@@ -11,6 +11,8 @@ tests assert the plan name themselves, so the table cannot drift from what they 
 import os
 import re
 
+import pytest
+
 from paper_2203_15952_b200 import binding as aqt
 from paper_2203_15952_b200 import inputs as gen
 
@@ -86,3 +88,33 @@ def test_plans_of_the_headline_shapes():
     assert p(65536, 1024, 4096, 0, 4, float_kind=True) == "pair256s6e4"
     # a device with other SM counts changes the choice only through the number of rounds
     assert aqt.aqt_plan_qmatmul(12800, 2048, 512, 8, 4, gen.ACT_SWISH, sm_count=8) == "stream256s3e16"
+
+
+def test_how_row_quantizing_calls_run():
+    p = lambda *a, **k: aqt.aqt_plan_qmatmul_requant(*a, sm_count=148, **k)
+    w8, may = aqt.BITS_4_UNPACKED, aqt.MAY_WAIT
+    # one tile per SM, in the narrowest width that leaves one; at most sixteen parts of a row below 128 columns
+    assert p(1013, 512, 512) == "few32" and p(1013, 1024, 512) == "few64" and p(4736, 512, 512, with_y=True) == "few128"
+    assert p(300, 1024, 896) == "few64" and p(300, 1040, 896) == "ws128" and p(4737, 512, 512) == "ws128"
+    # packed codes out, and a workspace with no room for the narrow tiles' words
+    assert p(1013, 512, 512, bits_w=4, pack_out=True) == "ws128"
+    need = -(-300 // 256) * 256 * 8 * 8 + 1024
+    assert p(300, 512, 512, workspace_bytes=need) == "ws128" and p(300, 512, 512, workspace_bytes=need + 65536) == "few32"
+    # what the header lists waits across CTAs, the others only if they may
+    for shape, kw, wide in (((1013, 1024, 1024), {}, "two_kernels"), ((100, 512, 2048), {}, "two_kernels"),
+                            ((300, 1024, 512), dict(act=gen.ACT_GLU_SWISH), "two_kernels"), ((200, 512, 2048), {}, "few32")):
+        assert p(*shape, with_y=True, **kw) == wide, shape
+        assert p(*shape, with_y=True, bits_w=8 | may, **kw).startswith("few")
+    assert p(25600, 512, 2048, bits_w=w8, with_y=True) == "pair256s4e8" and p(65536, 1024, 1024, bits_w=w8 | may, with_y=True) == "two_kernels"
+    # refused: nothing quantizes the rows and there is no y to go through
+    for shape in ((64, 256, 2048), (300, 512, 1536)):
+        with pytest.raises(aqt.AqtError) as e:
+            p(*shape, bits_w=8 | may)
+        assert e.value.status == -3
+    # the last columns only: one launch, or how they run by themselves
+    assert p(1013, 1536, 512, first=1024, with_y=True) == "few128" and p(12800, 1536, 512, first=1024, with_y=True) == "ws128"
+    assert p(300, 480, 128, first=16, with_y=True) == "few32"
+    for bad in (dict(first=8, with_y=True), dict(first=512, with_y=True), dict(first=16), dict(pack_out=True, bits_w=5)):
+        with pytest.raises(aqt.AqtError) as e:
+            p(300, 512, 512, **bad)
+        assert e.value.status == -1

@@ -13,20 +13,23 @@ pytestmark = pytest.mark.gpu
 
 # (148 SMs) one CTA per tile: 32, 64 and 128 columns, the last size that each covers, rows and columns that end inside a tile,
 # one k-block, a ragged one, as many as the ring has stages, one more, and several turns of the ring
-SHAPES = [(1, 512, 512), (113, 1056, 144), (128, 4736, 64), (129, 512, 9 * 128), (1013, 512, 9 * 128 + 16), (1153, 512, 512),
-          (2304, 512, 2048), (2305, 512, 512), (300, 1040, 7 * 128), (700, 800, 8 * 128), (1013, 2048, 512), (37 * 128, 512, 512)]
+SHAPES = [(1, 512, 512, "few32"), (113, 1056, 144, "few128"), (128, 4736, 64, "few128"), (129, 512, 9 * 128, "few32"),
+          (1013, 512, 9 * 128 + 16, "few32"), (1153, 512, 512, "few64"), (2304, 512, 2048, "few64"), (2305, 512, 512, "few128"),
+          (300, 1024, 7 * 128, "few64"), (700, 800, 8 * 128, "few64"), (1013, 2048, 512, "few128"), (37 * 128, 512, 512, "few128")]
 
 
-@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("M,N,K,plan", SHAPES)
 @pytest.mark.parametrize("with_res", [False, True])
-def test_few_tiles_requant(M, N, K, with_res):
-    _run(M, N, K, 8, 8, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, special_rows=not with_res, may_refuse_without_y=True)
+def test_few_tiles_requant(M, N, K, plan, with_res):
+    refused = 1024 < K < 2048  # without y
+    _run(M, N, K, 8, 8, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, special_rows=not with_res, may_refuse_without_y=refused,
+         plan=plan, plan_without_y=None if refused else plan, may_wait=True)
 
 
-@pytest.mark.parametrize("M,N,K", [(200, 512, 512), (1013, 2048, 256), (1000, 1024, 96)])
+@pytest.mark.parametrize("M,N,K,plan", [(200, 512, 512, "few32"), (1013, 2048, 256, "few128"), (1000, 1024, 96, "few64")])
 @pytest.mark.parametrize("rounding", [aqt.ROUND_NEAREST_EVEN, aqt.ROUND_HALF_UP_FLOOR])
-def test_few_tiles_packed_weights_swish(M, N, K, rounding):
-    _run(M, N, K, 4, 4, aqt.ACT_SWISH, False, False, 4, rounding, False)
+def test_few_tiles_packed_weights_swish(M, N, K, plan, rounding):
+    _run(M, N, K, 4, 4, aqt.ACT_SWISH, False, False, 4, rounding, False, plan=plan, plan_without_y=plan)
 
 
 @pytest.mark.parametrize("plan", ["few32", "few64", "few128"])
@@ -48,10 +51,12 @@ def test_few_tiles_plans_named(plan):
     assert e.value.status == -3
 
 
-@pytest.mark.parametrize("M,N,K,first", [(200, 768, 256, 512), (1013, 1536, 512, 1024), (1537, 1536, 512, 1024), (140, 96, 64, 32), (300, 480, 128, 16)])
+@pytest.mark.parametrize("M,N,K,first,plan", [(200, 768, 256, 512, "few32"), (1013, 1536, 512, 1024, "few128"), (1537, 1536, 512, 1024, "few64"),
+                                              (140, 96, 64, 32, "few32"), (300, 480, 128, 16, "few32"), (4800, 640, 64, 128, "ws128")])
 @pytest.mark.parametrize("bits_w", [4, 8])
-def test_last_columns_quantized(M, N, K, first, bits_w):
-    # one launch or two by the size; first = 16 is no multiple of a tile's columns
+def test_last_columns_quantized(M, N, K, first, plan, bits_w):
+    # one launch or (1537 rows: 156 tiles of 128 columns) two by the size; first = 16 is no multiple of a tile's columns
+    assert aqt.aqt_plan_qmatmul_requant(M, N, K, 8, bits_w, with_y=True, first=first) == plan
     rng = np.random.default_rng(M + N + first)
     xq, wq = _codes(rng, M, K, 8), _codes(rng, N, K, bits_w)
     s_x, s_w = rng.uniform(1e-3, 5e-2, M).astype(np.float32), rng.uniform(1e-4, 5e-3, N).astype(np.float32)
@@ -103,6 +108,7 @@ def test_few_tiles_do_without_room_for_their_exchange():
             _dev(rng.uniform(1e-4, 5e-3, N).astype(np.float32)))
     need = -(-M // 256) * 256 * (N // 64) * 8 + 256 * 4
     assert aqt.aqt_workspace_bytes(aqt.OP_QMATMUL_REQUANT, M, N, K, 8, 8) > need
+    assert aqt.aqt_plan_qmatmul_requant(M, N, K) == "few32" and aqt.aqt_plan_qmatmul_requant(M, N, K, workspace_bytes=need) == "ws128"
     q0, s0, _ = aqt.aqt_qmatmul_requant(*args, K=K)
     q1, s1, _ = aqt.aqt_qmatmul_requant(*args, K=K, workspace=torch.empty(need, dtype=torch.uint8, device="cuda"))
     assert torch.equal(q0, q1) and torch.equal(s0, s1) and aqt.aqt_device_status() == 0

@@ -208,18 +208,24 @@ def _run_qmatmul(M, N, K, bits_a, bits_w, act, with_bias, with_res, s_x_kind=aqt
 
 @pytest.mark.parametrize("M,N,K", [(128, 64, 128), (128, 128, 128), (128, 256, 128), (128, 256, 512), (256, 512, 256)])
 def test_qmatmul_single_tiles_int8(M, N, K):
-    _run_qmatmul(M, N, K, 8, 8, aqt.ACT_NONE, False, False, extremes=True)
+    for plan in (None, "ws128e16"):
+        _run_qmatmul(M, N, K, 8, 8, aqt.ACT_NONE, False, False, extremes=True, plan=plan)
 
 
 @pytest.mark.parametrize("M,N,K", [(64, 256, 256), (200, 192, 96), (1000, 520, 160), (129, 36, 32), (1, 4, 32), (333, 1536, 512)])
 def test_qmatmul_ragged_shapes(M, N, K):
     _run_qmatmul(M, N, K, 8, 8, aqt.ACT_NONE, True, True)
+    if M > 16:
+        # sizes that the kernel for outputs of a few tiles took over: the weight-stationary kernel on its ragged edges
+        assert aqt.aqt_plan_qmatmul(M, N, K).startswith("few")
+        _run_qmatmul(M, N, K, 8, 8, aqt.ACT_NONE, True, True, plan="ws128e16")
 
 
 @pytest.mark.parametrize("bits_a,bits_w", [(8, 4), (4, 4), (4, 8)])
 @pytest.mark.parametrize("M,N,K", [(384, 512, 512), (130, 200, 2048)])
 def test_qmatmul_int4_operands(bits_a, bits_w, M, N, K):
-    _run_qmatmul(M, N, K, bits_a, bits_w, aqt.ACT_NONE, True, False, extremes=True)
+    for plan in (None, "ws128e16") if K <= 512 else (None,):
+        _run_qmatmul(M, N, K, bits_a, bits_w, aqt.ACT_NONE, True, False, extremes=True, plan=plan)
 
 
 @pytest.mark.parametrize("act", [aqt.ACT_SWISH, aqt.ACT_GLU, aqt.ACT_GLU_SWISH])

@@ -21,7 +21,12 @@ def _codes(rng, rows, K, bits):
 
 
 def _run(M, N, K, bits_a, bits_w, act, with_bias, with_res, bits_out, rounding, pack_out, special_rows=False,
-         may_refuse_without_y=False):
+         may_refuse_without_y=False, plan=None, plan_without_y=None, may_wait=False):
+    """plan, plan_without_y: how the call is to run with the fp32 output and without it (aqt_plan_qmatmul_requant)."""
+    flags = aqt.MAY_WAIT if may_wait else 0
+    for name, with_y in ((plan, True), (plan_without_y, False)):
+        if name is not None:
+            assert aqt.aqt_plan_qmatmul_requant(M, N, K, bits_a, bits_w | flags, act, with_y=with_y, pack_out=pack_out) == name
     rng = np.random.default_rng(7 + 1000 * M + N + K + bits_out)
     xq = _codes(rng, M, K, bits_a)
     wq = _codes(rng, N, K, bits_w)
@@ -41,7 +46,7 @@ def _run(M, N, K, bits_a, bits_w, act, with_bias, with_res, bits_out, rounding, 
     xq_d = _dev(orc.pack_int4(xq)) if bits_a == 4 else _dev(xq)
     wq_d = _dev(orc.pack_int4(wq)) if bits_w == 4 else _dev(wq)
     args = (xq_d, _dev(s_x), wq_d, _dev(s_w), None if bias is None else _dev(bias), None if res is None else _dev(res), 0.5)
-    kw = dict(K=K, bits_a=bits_a, bits_w=bits_w, act=act, bits_out=bits_out, rounding=rounding, pack_out=pack_out)
+    kw = dict(K=K, bits_a=bits_a, bits_w=bits_w | flags, act=act, bits_out=bits_out, rounding=rounding, pack_out=pack_out)
     q_shape = (M, N // 2) if pack_out else (M, N)
     q_d = torch.full(q_shape, 0x55, dtype=torch.uint8 if pack_out else torch.int8, device=DEV)
     s_d = torch.full((M,), float("nan"), dtype=torch.float32, device=DEV)
@@ -103,10 +108,11 @@ def test_requant_bit_widths_and_rounding(bits_a, bits_w, bits_out, pack_out, rou
     _run(333, 512, 256, bits_a, bits_w, aqt.ACT_NONE, False, False, bits_out, rounding, pack_out, special_rows=True)
 
 
-@pytest.mark.parametrize("M,N,K", [(256, 512, 512), (1300, 512, 128), (77, 1024, 512)])
+@pytest.mark.parametrize("M,N,K,plan", [(256, 512, 512, "few32"), (1300, 512, 128, "few64"), (77, 1024, 512, "few64"), (4800, 512, 512, "ws128"),
+                                        (1500, 1680, 128, "ws128")])
 @pytest.mark.parametrize("act", [aqt.ACT_NONE, aqt.ACT_SWISH])
-def test_requant_with_residual_stream(M, N, K, act):
-    _run(M, N, K, 8, 4, act, True, True, 8, aqt.ROUND_NEAREST_EVEN, False)
+def test_requant_with_residual_stream(M, N, K, plan, act):
+    _run(M, N, K, 8, 4, act, True, True, 8, aqt.ROUND_NEAREST_EVEN, False, plan=plan)
 
 
 def test_requant_with_residual_stream_many_tiles_per_cta():
@@ -116,12 +122,19 @@ def test_requant_with_residual_stream_many_tiles_per_cta():
     _run(5000, 512, 256, 8, 8, aqt.ACT_NONE, False, True, 4, aqt.ROUND_HALF_UP_FLOOR, True)
 
 
-@pytest.mark.parametrize("M,N,K", [(36 * 128 + 5, 512, 512), (37 * 128 + 1, 512, 128), (74 * 128, 512, 256), (74 * 128 + 1, 512, 64),
+@pytest.mark.parametrize("M,N,K", [(50 * 128 + 5, 512, 512), (37 * 128 + 1, 512, 128), (74 * 128, 512, 256), (74 * 128 + 1, 512, 64),
                                    (9 * 128 + 7, 2048, 64), (18 * 128 + 1, 2048, 64)])
 @pytest.mark.parametrize("with_res", [True, False])
 def test_requant_sets_that_share_a_tile(M, N, K, with_res):
     # one, two and three tiles per CTA, and CTAs with one and two in the same launch (148 SMs: 37 or 9 groups of CTAs)
-    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False)
+    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, plan="ws128", plan_without_y="ws128")
+
+
+@pytest.mark.parametrize("M,N,K", [(200, 512, 512), (1013, 512, 256), (700, 1056, 64)])
+@pytest.mark.parametrize("with_res", [True, False])
+def test_requant_packed_codes_of_few_tiles(M, N, K, with_res):
+    # one tile per CTA, all four sets on it: packed codes leave only the weight-stationary kernel
+    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 4, aqt.ROUND_NEAREST_EVEN, True, plan="ws128", plan_without_y="ws128")
 
 
 def test_requant_many_tiles_per_cta():
@@ -143,11 +156,15 @@ def test_requant_deep_k_form(M, N, K, bits_w, act):
 
 @pytest.mark.parametrize("act", [aqt.ACT_GLU, aqt.ACT_GLU_SWISH])
 @pytest.mark.parametrize("M,N,K,bits_w", [(128, 128, 128, 8), (300, 1024, 512, 4), (1000, 2048, 256, 4), (77, 288, 144, 8),
-                                           (2600, 1024, 512, 8), (129, 4224, 64, 4), (300, 2048, 1024, 4), (129, 512, 640, 8)])
+                                           (2600, 1024, 512, 8), (129, 4224, 64, 4), (300, 2048, 1024, 4), (129, 512, 640, 8),
+                                           (2500, 1024, 512, 4), (1300, 2080, 96, 4), (1500, 2048, 640, 4)])
 def test_requant_glu_forms(act, M, N, K, bits_w):
     """The GLU forms (a tile = 64 value + 64 gate channels -> 64 output columns).  With y the call
     runs matmul + quantizer through y, which is checked against the oracle like every other form;
     without y the fused kernel must give the very same codes and scales."""
+    few = -(-M // 128) * -(-N // 128) <= 148
+    assert aqt.aqt_plan_qmatmul_requant(M, N, K, 8, bits_w, act, with_y=True) == "two_kernels"
+    assert aqt.aqt_plan_qmatmul_requant(M, N, K, 8, bits_w, act)[:3] == ("few" if few and (K <= 512 or (M, N) == (129, 512)) else "ws1")
     for rounding, bits_out in ((aqt.ROUND_NEAREST_EVEN, 8), (aqt.ROUND_HALF_UP_FLOOR, 4)):
         rng = np.random.default_rng(11 + M + N + K + bits_out)
         xq, wq = _codes(rng, M, K, 8), _codes(rng, N, K, bits_w)
@@ -209,9 +226,11 @@ def test_requant_random_shapes(seed):
 
 
 def test_requant_unfused_shapes_go_through_y():
-    """K > 1024 (and K > 512 or the GLU forms with an fp32 output) are not taken by the fused
-    kernel: the call runs the two steps through y."""
-    _run(200, 512, 2048, 8, 4, aqt.ACT_NONE, True, True, 8, aqt.ROUND_NEAREST_EVEN, False)
+    """K > 512 and the GLU forms with an fp32 output, up to K = 2048 or 128 rows, are not taken by a fused
+    kernel unless the caller allows it: the call runs the two steps through y."""
+    _run(100, 512, 2048, 8, 4, aqt.ACT_NONE, True, True, 8, aqt.ROUND_NEAREST_EVEN, False, plan="two_kernels")
+    _run(200, 512, 1536, 8, 4, aqt.ACT_NONE, True, True, 8, aqt.ROUND_NEAREST_EVEN, False, plan="two_kernels")
+    _run(200, 512, 2048, 8, 4, aqt.ACT_NONE, True, True, 8, aqt.ROUND_NEAREST_EVEN, False, plan="few32")
     rng = np.random.default_rng(3)
     xq, wq = _codes(rng, 64, 2048, 8), _codes(rng, 256, 2048, 8)
     with pytest.raises(aqt.AqtError) as e:
@@ -345,6 +364,13 @@ def test_requant_second_ffn_layers_small(M, N, K, act, with_res):
     come from several warps and, beyond 512 columns, several CTA pairs."""
     _run(M, N, K, 8, 4, act, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, special_rows=True)
     _run(M, N, K, 8, 8 if K <= 2048 else 4, act, False, with_res, 4, aqt.ROUND_HALF_UP_FLOOR, False)
+
+
+@pytest.mark.parametrize("M,N,act,with_res,plan", [(2500, 512, aqt.ACT_NONE, False, "two_kernels"), (2433, 784, aqt.ACT_SWISH, False, "two_kernels"),
+                                                   (5000, 480, aqt.ACT_NONE, True, "pair256s4e8")])
+def test_requant_pairs_of_ragged_outputs(M, N, act, with_res, plan):
+    # outputs of more than a few tiles whose last tiles are partly beyond the last row and column
+    _run(M, N, 2048, 8, 4, act, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, special_rows=True, plan=plan, plan_without_y="pair256s4e8")
 
 
 @pytest.mark.parametrize("M,N,K,plan", [(25600, 512, 2048, "pair256s4e8"), (12800, 512, 2048, "pair512s3e16"),
