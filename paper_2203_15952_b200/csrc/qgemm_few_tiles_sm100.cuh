@@ -155,7 +155,7 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     for (int w = 0; w < EW; ++w) mbar_init(smem_u32(&res_bar[w]), 1);
     for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&part_bar[q]), 3);
     for (int h = 0; h < 2; ++h) mbar_init(smem_u32(&ctx_bar[h]), 1);
-    mbar_init(smem_u32(&tag_bar), 1);
+    mbar_init(smem_u32(&tag_bar), 2);
     fence_barrier_init();
     fence_proxy_async_smem();
     // the weights' loads are on their way before the CTA's set-up is complete
@@ -233,10 +233,8 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     if (rq) {
       const int xh = warp - (2 + EW);
       grid_dependency_wait();
-      if (xh == 0 && lane == 0) hand_out_tag(rp, tm, &tag_slot, &tag_bar);
-      bool ok = mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start);
-      ok = __all_sync(0xffffffffu, ok) != 0;
-      const uint32_t tag = *(volatile uint32_t*)&tag_slot;
+      bool ok = true;
+      const uint32_t tag = hand_out_tag(rp, tm, &tag_slot, &tag_bar);
       const uint64_t* xt = rp.exchange + (size_t)tm * parts * kBM + 64 * xh + 2 * lane;
       uint2 m2 = make_uint2(0u, 0u);
       for (int t0 = 0; ok && t0 < parts; t0 += kExchangeBatch) {

@@ -131,13 +131,18 @@ constexpr int kSlots = 4;
 // more alike.)
 __device__ __forceinline__ int sets_per_tile(int n_my) { return n_my == 1 ? 4 : (n_my == 2 ? 2 : 1); }
 
-// Tag of this execution's exchange words, from one thread to all of the CTA.  A replayed CUDA graph repeats the call's own
-// tag, so the group's generation counter goes into it.  It is read once per CTA and every word that the CTA publishes
-// carries what was read; the group's first CTA bumps it at its end, which it does not reach without words of all of them.
-// (Warps that each read the counter for themselves would not all have done so by then.)
-__device__ __forceinline__ void hand_out_tag(const RequantParams& rp, int group, uint32_t* slot, uint64_t* bar) {
-  *(volatile uint32_t*)slot = mix_tag(rp.tag, __ldcg(rp.generation + group));
-  mbar_arrive(smem_u32(bar));
+// Tag of this execution's exchange words.  A replayed CUDA graph repeats the call's own tag, so the group's generation
+// counter goes into it.  Whoever reads the counter hands the tag out (an arrival each on `bar`), and a CTA publishes nothing
+// before that; the group's first CTA bumps the counter at its end, which it does not reach without words of all of them.
+// (Warps that each read it for themselves alone would not all have done so by then.)  Readers are exchange warps: one here,
+// both where a CTA has one tile (pair of 12 800 rows 57.7 us with one, 57.95 with two; block of 1013 rows 65.7 and 65.45).
+__device__ __forceinline__ uint32_t hand_out_tag(const RequantParams& rp, int group, uint32_t* slot, uint64_t* bar) {
+  const uint32_t tag = __shfl_sync(0xffffffffu, mix_tag(rp.tag, __ldcg(rp.generation + group)), 0);
+  if ((threadIdx.x & 31) == 0) {
+    *(volatile uint32_t*)slot = tag;
+    mbar_arrive(smem_u32(bar));
+  }
+  return tag;
 }
 constexpr int kExchangeBatch = 16;  // n-tiles whose words an exchange warp asks for at once (one 16-byte load each per lane)
 
@@ -325,8 +330,10 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     // 64h + 2l + 1, i.e. one 16-byte load (two words) per n-tile, kExchangeBatch of them in flight.
     const int xh = warp - (2 + EW);
     if (early_w) grid_dependency_wait();
-    if (xh == 0 && lane == 0) hand_out_tag(rp, group, &tag_slot, &tag_bar);
-    bool ok = mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start);
+    bool ok = true;
+    if (xh == 0) hand_out_tag(rp, group, &tag_slot, &tag_bar);
+    else ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&tag_bar), 0, &abort_flag, t_start)) != 0;
+    __syncwarp();
     const uint32_t tag = *(volatile uint32_t*)&tag_slot;
     for (int i = 0; ok && i < n_my; ++i) {
       const int tm = group + i * groups;
