@@ -14,9 +14,10 @@ and are replaced by the identity:
     h <- h + 1/2 * W_b2 . Swish(W_b1 . h)          feed-forward module b
 
 Residual adds are fp32 and are fused into the epilogue of the producing linear.  Where a linear
-with K <= 512 feeds another quantized linear, its epilogue also quantizes its output rows
-(aqt_qmatmul_requant): the fp32 tensor between the two is then written only if it is needed as
-well (the residual stream, or a parity check; the GLU layer only fuses when it is not).
+feeds another quantized linear, its epilogue also quantizes its output rows where a kernel does
+both (aqt_qmatmul_requant; else a second kernel behind it does): the fp32 tensor between the two is
+written only if it is needed as well (the residual stream, or a parity check; the GLU layer only
+hands codes over when it is not).
 """
 from __future__ import annotations
 
@@ -263,8 +264,8 @@ class LayerRunner:
 
 class FfnPair:
     """y = W_2 . Swish(W_1 . x).  The second layer consumes the first layer's output as codes and
-    row scales; the first matmul produces them in its epilogue when it can (`fused`), and the fp32
-    hidden tensor u is then written only with keep_u (parity checks)."""
+    row scales; the first matmul's call produces them when it can (`fused`), in its epilogue but for
+    some shapes with keep_u, and the fp32 hidden tensor u is then written only with keep_u (parity checks)."""
 
     def __init__(self, M: int, layers: List[QuantLinear], device, fused: bool = True, keep_u: bool = False, **kw):
         assert len(layers) == 2
@@ -297,8 +298,13 @@ class FfnPair:
     @property
     def launches_per_step(self) -> int:
         """Kernels of the library launched by one forward() of a batch (a few rows take one)."""
-        l0, l1 = self.layers
-        return 3 if self.fused else 4
+        if not self.fused or self.run.M == 0:
+            return 4
+        l0 = self.layers[0]
+        s = l0.spec
+        how = aqt.aqt_plan_qmatmul_requant(self.run.M, s.N, s.K, _container_bits(s.bits_a), l0.mm_bits | aqt.MAY_WAIT, s.act, with_y=self.keep_u,
+                                           workspace_bytes=self.run.workspace.numel())
+        return 4 if how == "two_kernels" else 3
 
     @property
     def ops(self) -> int:

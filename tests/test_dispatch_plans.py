@@ -118,3 +118,17 @@ def test_how_row_quantizing_calls_run():
         with pytest.raises(aqt.AqtError) as e:
             p(300, 512, 512, **bad)
         assert e.value.status == -1
+
+
+def test_launches_of_a_feed_forward_pair():
+    """The pair counts the row quantizer that runs behind the first matmul where no kernel does both."""
+    import torch
+    from paper_2203_15952_b200.encoder import FfnPair, QuantLinear
+    from paper_2203_15952_b200.inputs import LinearSpec
+
+    def pair(M, d, **kw):
+        specs = [LinearSpec("a", d, 4 * d, gen.ACT_SWISH, 8), LinearSpec("b", 4 * d, d, gen.ACT_NONE, 8)]
+        return FfnPair(M, [QuantLinear(s, torch.empty(s.N, s.K, dtype=torch.int8), torch.empty(s.N), None) for s in specs], "cpu", **kw)
+    assert pair(5000, 512).launches_per_step == 3 and pair(5000, 512, keep_u=True).launches_per_step == 3
+    assert pair(5000, 1024).launches_per_step == 3 and pair(5000, 1024, keep_u=True).launches_per_step == 4
+    assert pair(5000, 512, fused=False).launches_per_step == 4
