@@ -61,26 +61,6 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[8]) {
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[16]) { tmem_ld_32x16(taddr, r); }
 __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[32]) { tmem_ld_32x32(taddr, r); }
 
-// dequant32 / swish32 of qgemm_sm100.cuh on C columns.
-template <int C>
-__device__ __forceinline__ void dequant_cols(const uint32_t (&acc)[C], float sx, uint32_t sw_smem, uint32_t b_smem, float (&z)[C]) {
-#pragma unroll
-  for (int j = 0; j < C / 4; ++j) {
-    float w0, w1, w2, w3, b0, b1, b2, b3;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3) : "r"(sw_smem + 16 * j));
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b0), "=f"(b1), "=f"(b2), "=f"(b3) : "r"(b_smem + 16 * j));
-    z[4 * j + 0] = __fmaf_rn(__fmul_rn(acc_to_float<kAccInt32>(acc[4 * j + 0]), sx), w0, b0);
-    z[4 * j + 1] = __fmaf_rn(__fmul_rn(acc_to_float<kAccInt32>(acc[4 * j + 1]), sx), w1, b1);
-    z[4 * j + 2] = __fmaf_rn(__fmul_rn(acc_to_float<kAccInt32>(acc[4 * j + 2]), sx), w2, b2);
-    z[4 * j + 3] = __fmaf_rn(__fmul_rn(acc_to_float<kAccInt32>(acc[4 * j + 3]), sx), w3, b3);
-  }
-}
-template <int C>
-__device__ __forceinline__ void swish_cols(float (&a)[C]) {
-#pragma unroll
-  for (int j = 0; j < C; ++j) a[j] = __fmul_rn(a[j], sigmoid_f(a[j]));
-}
-
 // Accumulators of row m from column n on, those below `limit`, as the matrix product that they are (DEBUG).
 template <int C>
 __device__ __forceinline__ void dump_acc(const GemmParams& p, int m, int n, int limit, const uint32_t (&acc)[C]) {
@@ -233,35 +213,10 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     if (rq) {
       const int xh = warp - (2 + EW);
       grid_dependency_wait();
-      bool ok = true;
       const uint32_t tag = hand_out_tag(rp, tm, &tag_slot, &tag_bar);
       const uint64_t* xt = rp.exchange + (size_t)tm * parts * kBM + 64 * xh + 2 * lane;
-      uint2 m2 = make_uint2(0u, 0u);
-      for (int t0 = 0; ok && t0 < parts; t0 += kExchangeBatch) {
-        for (uint32_t spin = 1;; ++spin) {
-          ulonglong2 w[kExchangeBatch];
-#pragma unroll
-          for (int t = 0; t < kExchangeBatch; ++t) {
-            const uint64_t none = (uint64_t)tag << 32;  // a maximum of zero
-            w[t] = t0 + t < parts ? ld_relaxed_gpu_2x64(xt + (size_t)(t0 + t) * kBM) : make_ulonglong2(none, none);
-          }
-          bool all = true;
-          uint2 b2 = make_uint2(0u, 0u);
-#pragma unroll
-          for (int t = 0; t < kExchangeBatch; ++t) {
-            all = all && (uint32_t)(w[t].x >> 32) == tag && (uint32_t)(w[t].y >> 32) == tag;
-            b2.x = max(b2.x, (uint32_t)w[t].x);
-            b2.y = max(b2.y, (uint32_t)w[t].y);
-          }
-          if (__all_sync(0xffffffffu, all)) {
-            m2.x = max(m2.x, b2.x);
-            m2.y = max(m2.y, b2.y);
-            break;
-          }
-          if ((spin & 0xF) == 0 && !__all_sync(0xffffffffu, keep_waiting(&abort_flag, t_start))) { ok = false; break; }  // warp-uniform
-        }
-      }
-      if (ok) {
+      uint2 m2;
+      if (collect_maxima(xt, parts, tag, &abort_flag, t_start, m2)) {
         *reinterpret_cast<uint2*>(&row_amax[64 * xh + 2 * lane]) = m2;
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctx_bar[xh]));
@@ -300,26 +255,7 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       // sign-extend the packed weights into the stages (layout of a swizzled load of int8 codes)
       ok = wait(b_loaded_bar);
       if (ok) {
-        const int pieces = p.k_blocks * BN * 4;  // 16 packed bytes -> 32 codes each
-        for (int q = ew * 32 + lane; q < pieces; q += EW * 32) {
-          const int kb = q / (BN * 4), rem = q - kb * (BN * 4);
-          const int r = rem >> 2, piece = rem & 3;
-          uint32_t w0, w1, w2, w3;
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3)
-                       : "r"(smem_epi + kb * BN * 64 + r * 64 + piece * 16)
-                       : "memory");
-          uint32_t o[8];
-          unpack_word(w0, o[0], o[1]);
-          unpack_word(w1, o[2], o[3]);
-          unpack_word(w2, o[4], o[5]);
-          unpack_word(w3, o[6], o[7]);
-          const uint32_t row_base = smem_ring + kb * Cfg::kStageBytes + kBM * kBK + r * 128;
-          const uint32_t d0 = row_base + (((2 * piece) ^ (r & 7)) << 4);
-          const uint32_t d1 = row_base + (((2 * piece + 1) ^ (r & 7)) << 4);
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d0), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d1), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
-        }
+        expand_packed_slab<BN, EW * 32>(smem_epi, smem_ring + kBM * kBK, Cfg::kStageBytes, p.k_blocks, ew * 32 + lane);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&b_ready_bar));
@@ -350,17 +286,17 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         tmem_ld_wait();
         if (DEBUG) dump_acc<C>(p, m, p.N / 2 + oc, p.N, accg);
         if (DEBUG) dump_acc<C>(p, m, oc, p.N / 2, acc);
-        dequant_cols<C>(accg, sx, slab + C * 4, slab_bias + C * 4, g);
-        dequant_cols<C>(acc, sx, slab, slab_bias, a);
+        dequant_smem<kAccInt32>(accg, sx, slab + C * 4, slab_bias + C * 4, g);
+        dequant_smem<kAccInt32>(acc, sx, slab, slab_bias, a);
 #pragma unroll
         for (int j = 0; j < C; ++j) a[j] = __fmul_rn(a[j], sigmoid_f(g[j]));
-        if (p.act == AQT_ACT_GLU_SWISH) swish_cols<C>(a);
+        if (p.act == AQT_ACT_GLU_SWISH) swish(a);
       } else {
         tmem_ld_cols(t_addr, acc);
         tmem_ld_wait();
         if (DEBUG) dump_acc<C>(p, m, oc, p.N, acc);
-        dequant_cols<C>(acc, sx, slab, slab_bias, a);
-        if (p.act == AQT_ACT_SWISH) swish_cols<C>(a);
+        dequant_smem<kAccInt32>(acc, sx, slab, slab_bias, a);
+        if (p.act == AQT_ACT_SWISH) swish(a);
       }
       if (has_res) {
         ok = wait(res_bar[ew]);

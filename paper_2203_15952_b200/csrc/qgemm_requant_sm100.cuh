@@ -91,35 +91,6 @@ __device__ __forceinline__ void tmem_st_32x16(uint32_t taddr, const uint32_t (&r
       "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
 }
-// dequant32 / swish32 of qgemm_sm100.cuh on 16 columns.
-template <int ACCK>
-__device__ __forceinline__ void dequant16(const uint32_t (&acc)[16], float sx, uint32_t sw_smem, uint32_t b_smem, float (&z)[16]) {
-  const float2 sx2 = make_float2(sx, sx);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    float w0, w1, w2, w3, b0, b1, b2, b3;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3) : "r"(sw_smem + 16 * j));
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b0), "=f"(b1), "=f"(b2), "=f"(b3) : "r"(b_smem + 16 * j));
-    const float2 z01 = __ffma2_rn(__fmul2_rn(acc_to_float2<ACCK>(acc[4 * j + 0], acc[4 * j + 1]), sx2), make_float2(w0, w1), make_float2(b0, b1));
-    const float2 z23 = __ffma2_rn(__fmul2_rn(acc_to_float2<ACCK>(acc[4 * j + 2], acc[4 * j + 3]), sx2), make_float2(w2, w3), make_float2(b2, b3));
-    z[4 * j + 0] = z01.x;
-    z[4 * j + 1] = z01.y;
-    z[4 * j + 2] = z23.x;
-    z[4 * j + 3] = z23.y;
-  }
-}
-__device__ __forceinline__ void swish16(float (&a)[16]) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float2 z = make_float2(a[2 * j], a[2 * j + 1]);
-    const float2 t = __fmul2_rn(z, make_float2(-1.4426950408889634f, -1.4426950408889634f));
-    const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(ex2_approx(t.x), ex2_approx(t.y)));
-    const float2 y = __fmul2_rn(z, make_float2(rcp_approx(d.x), rcp_approx(d.y)));
-    a[2 * j] = y.x;
-    a[2 * j + 1] = y.y;
-  }
-}
-
 // One slot of shared-memory exchange state (final row maxima, hand-over barriers) per accumulator
 // buffer, i.e. per set of epilogue warps: tile i of a CTA uses buffer and slot i mod 4.
 constexpr int kSlots = 4;
@@ -154,6 +125,38 @@ __device__ __forceinline__ bool keep_waiting(volatile int* abort_flag, uint64_t 
     *abort_flag = 1;
     atomicExch(&g_device_status, AQT_ERR_TIMEOUT);
     return false;
+  }
+  return true;
+}
+
+// Final maxima of two rows (this lane's), the largest of what `parts` CTAs publish: one 16-byte load (two words) per part,
+// kExchangeBatch of them in flight, and the whole batch again until every word carries this execution's tag.  The same
+// answer in every lane of the warp: false once the CTA is aborting.
+__device__ __forceinline__ bool collect_maxima(const uint64_t* xt, int parts, uint32_t tag, volatile int* abort_flag, uint64_t t_start, uint2& m2) {
+  m2 = make_uint2(0u, 0u);
+  for (int t0 = 0; t0 < parts; t0 += kExchangeBatch) {
+    for (uint32_t spin = 1;; ++spin) {
+      ulonglong2 w[kExchangeBatch];
+#pragma unroll
+      for (int t = 0; t < kExchangeBatch; ++t) {
+        const uint64_t none = (uint64_t)tag << 32;  // a maximum of zero
+        w[t] = t0 + t < parts ? ld_relaxed_gpu_2x64(xt + (size_t)(t0 + t) * kBM) : make_ulonglong2(none, none);
+      }
+      bool all = true;
+      uint2 b2 = make_uint2(0u, 0u);
+#pragma unroll
+      for (int t = 0; t < kExchangeBatch; ++t) {
+        all = all && (uint32_t)(w[t].x >> 32) == tag && (uint32_t)(w[t].y >> 32) == tag;
+        b2.x = max(b2.x, (uint32_t)w[t].x);
+        b2.y = max(b2.y, (uint32_t)w[t].y);
+      }
+      if (__all_sync(0xffffffffu, all)) {
+        m2.x = max(m2.x, b2.x);
+        m2.y = max(m2.y, b2.y);
+        break;
+      }
+      if ((spin & 0xF) == 0 && !__all_sync(0xffffffffu, keep_waiting(abort_flag, t_start))) return false;
+    }
   }
   return true;
 }
@@ -338,35 +341,10 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
     for (int i = 0; ok && i < n_my; ++i) {
       const int tm = group + i * groups;
       const uint32_t par = i % kSlots, ph = (i / kSlots) & 1;
-      if (!mbar_wait(smem_u32(&ctx_free_bar[par][xh]), ph ^ 1, &abort_flag, t_start)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctx_free_bar[par][xh]), ph ^ 1, &abort_flag, t_start))) break;
       const uint64_t* xt = rp.exchange + (size_t)tm * p.tiles_n * kBM + 64 * xh + 2 * lane;
-      uint2 m2 = make_uint2(0u, 0u);
-      for (int t0 = 0; ok && t0 < p.tiles_n; t0 += kExchangeBatch) {
-        // all loads of the batch in flight at once; the whole batch is asked for again until every word carries this launch's tag
-        for (uint32_t spin = 1;; ++spin) {
-          ulonglong2 w[kExchangeBatch];
-#pragma unroll
-          for (int t = 0; t < kExchangeBatch; ++t) {
-            const uint64_t none = (uint64_t)tag << 32;  // a maximum of zero
-            w[t] = t0 + t < p.tiles_n ? ld_relaxed_gpu_2x64(xt + (size_t)(t0 + t) * kBM) : make_ulonglong2(none, none);
-          }
-          bool all = true;
-          uint2 b2 = make_uint2(0u, 0u);
-#pragma unroll
-          for (int t = 0; t < kExchangeBatch; ++t) {
-            all = all && (uint32_t)(w[t].x >> 32) == tag && (uint32_t)(w[t].y >> 32) == tag;
-            b2.x = max(b2.x, (uint32_t)w[t].x);
-            b2.y = max(b2.y, (uint32_t)w[t].y);
-          }
-          if (__all_sync(0xffffffffu, all)) {
-            m2.x = max(m2.x, b2.x);
-            m2.y = max(m2.y, b2.y);
-            break;
-          }
-          if ((spin & 0xF) == 0 && !__all_sync(0xffffffffu, keep_waiting(&abort_flag, t_start))) { ok = false; break; }  // warp-uniform
-        }
-      }
-      if (!__all_sync(0xffffffffu, ok)) break;
+      uint2 m2;
+      if (!collect_maxima(xt, p.tiles_n, tag, &abort_flag, t_start, m2)) break;
       // final maxima of this warp's rows for the epilogue warps
       *reinterpret_cast<uint2*>(&row_amax[par][64 * xh + 2 * lane]) = m2;
       __syncwarp();
@@ -400,26 +378,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       // sign-extend the packed weights into the resident slab (layout of a swizzled int8 load)
       ok = mbar_wait(smem_u32(&b_loaded_bar), 0, &abort_flag, t_start);
       if (ok) {
-        const int pieces = p.k_blocks * BN * 4;
-        for (int q = (ew * 32 + lane); q < pieces; q += EW * 32) {
-          const int kb = q / (BN * 4), rem = q - kb * (BN * 4);
-          const int r = rem >> 2, piece = rem & 3;
-          uint32_t w0, w1, w2, w3;
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3)
-                       : "r"(smem_epi + kb * BN * 64 + r * 64 + piece * 16)
-                       : "memory");
-          uint32_t o[8];
-          unpack_word(w0, o[0], o[1]);
-          unpack_word(w1, o[2], o[3]);
-          unpack_word(w2, o[4], o[5]);
-          unpack_word(w3, o[6], o[7]);
-          const uint32_t row_base = smem_res_b + kb * Cfg::kBBytes + r * 128;
-          const uint32_t d0 = row_base + (((2 * piece) ^ (r & 7)) << 4);
-          const uint32_t d1 = row_base + (((2 * piece + 1) ^ (r & 7)) << 4);
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d0), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d1), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
-        }
+        expand_packed_slab<BN, EW * 32>(smem_epi, smem_res_b, Cfg::kBBytes, p.k_blocks, ew * 32 + lane);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&b_ready_bar));
@@ -462,13 +421,13 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           tmem_ld_32x16(tbase + HALF + col, accg);
           tmem_ld_32x16(tbase + col, accv);
           tmem_ld_wait();
-          dequant16<kAccInt32>(accg, sx, c_sw + HALF * 4, c_bias + HALF * 4, g);
+          dequant_smem<kAccInt32>(accg, sx, c_sw + HALF * 4, c_bias + HALF * 4, g);
 #pragma unroll
           for (int j = 0; j < 16; ++j) g[j] = sigmoid_f(g[j]);
-          dequant16<kAccInt32>(accv, sx, c_sw, c_bias, av);
+          dequant_smem<kAccInt32>(accv, sx, c_sw, c_bias, av);
 #pragma unroll
           for (int j = 0; j < 16; ++j) av[j] = av[j] * g[j];
-          if (p.act == AQT_ACT_GLU_SWISH) swish16(av);
+          if (p.act == AQT_ACT_GLU_SWISH) swish(av);
           float cmax = 0.0f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -482,8 +441,8 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           float a[32];
           tmem_ld_32x32(tbase + col, acc);
           tmem_ld_wait();
-          dequant32<kAccInt32>(acc, sx, c_sw, c_bias, a);
-          if (p.act == AQT_ACT_SWISH) swish32(a);
+          dequant_smem<kAccInt32>(acc, sx, c_sw, c_bias, a);
+          if (p.act == AQT_ACT_SWISH) swish(a);
           if (has_res) {
             if (!mbar_wait(smem_u32(&res_bar[ew]), res_count & 1u, &abort_flag, t_start)) { ok = false; break; }
             ++res_count;

@@ -362,7 +362,6 @@ __device__ __forceinline__ float sigmoid_f(float z) {
 //   kAccInt32      int32, converted round-to-nearest-even (exact below 2^24)
 //   kAccInt32Small int32 with |acc| < 2^22 guaranteed by the caller: adding the integer to the bit
 //                  pattern of 1.5 * 2^23 and subtracting that constant is exact and stays off the
-//                  conversion unit
 //                  conversion unit.  For CTA pairs only, whose eight warps convert a tile twice as wide (30 000 x 2048
 //                  -> 512 Swish 89.3 us, 91.2 with conversions); sixteen warps on 128 columns are shorter of issue slots
 //                  than of conversions (feed-forward pair on 12 800 rows 56.4 / 55.5, 12 800 x 512 -> 2048 gated 39.0 / 37.9)
@@ -385,15 +384,15 @@ __device__ __forceinline__ float2 acc_to_float2(uint32_t a0, uint32_t a1) {
   return make_float2(__int2float_rn((int)a0), __int2float_rn((int)a1));
 }
 
-// z[i] = fma(float(acc[i]) * sx, s_w[i], bias[i]) for 32 consecutive columns whose scales and
+// z[i] = fma(float(acc[i]) * sx, s_w[i], bias[i]) for NV consecutive columns whose scales and
 // biases sit at `sw_smem` / `b_smem` (shared-memory byte addresses, 16-byte aligned).  The
 // arithmetic runs on the packed two-lane fp32 instructions of this architecture (each lane an
 // ordinary round-to-nearest IEEE operation), which halves the issue slots it takes.
-template <int ACCK>
-__device__ __forceinline__ void dequant32(const uint32_t (&acc)[32], float sx, uint32_t sw_smem, uint32_t b_smem, float (&z)[32]) {
+template <int ACCK, int NV>
+__device__ __forceinline__ void dequant_smem(const uint32_t (&acc)[NV], float sx, uint32_t sw_smem, uint32_t b_smem, float (&z)[NV]) {
   const float2 sx2 = make_float2(sx, sx);
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < NV / 4; ++j) {
     float w0, w1, w2, w3, b0, b1, b2, b3;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3) : "r"(sw_smem + 16 * j));
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b0), "=f"(b1), "=f"(b2), "=f"(b3) : "r"(b_smem + 16 * j));
@@ -406,11 +405,12 @@ __device__ __forceinline__ void dequant32(const uint32_t (&acc)[32], float sx, u
   }
 }
 
-// a[i] = a[i] * sigmoid(a[i]) (see sigmoid_f) for 32 values, two per instruction where the
+// a[i] = a[i] * sigmoid(a[i]) (see sigmoid_f) for NV values, two per instruction where the
 // operation is an IEEE multiply or add.
-__device__ __forceinline__ void swish32(float (&a)[32]) {
+template <int NV>
+__device__ __forceinline__ void swish(float (&a)[NV]) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
+  for (int j = 0; j < NV / 2; ++j) {
     const float2 z = make_float2(a[2 * j], a[2 * j + 1]);
     const float2 t = __fmul2_rn(z, make_float2(-1.4426950408889634f, -1.4426950408889634f));
     const float2 d = __fadd2_rn(make_float2(1.0f, 1.0f), make_float2(ex2_approx(t.x), ex2_approx(t.y)));
@@ -431,7 +431,7 @@ __device__ __forceinline__ float4 ld4_guard(const float* base, int n, int limit,
   return r;
 }
 
-// The same with scales and biases read from global memory (warp-uniform addresses, served by L1).
+// dequant_smem with scales and biases read from global memory (warp-uniform addresses, served by L1).
 template <int ACCK>
 __device__ __forceinline__ void dequant32_gmem(const uint32_t (&acc)[32], float sx, const float* s_w, const float* bias, int n0,
                                                int limit, float (&z)[32]) {
@@ -443,6 +443,34 @@ __device__ __forceinline__ void dequant32_gmem(const uint32_t (&acc)[32], float 
     z[4 * j + 1] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 1]), sx), w.y, b.y);
     z[4 * j + 2] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 2]), sx), w.z, b.z);
     z[4 * j + 3] = __fmaf_rn(__fmul_rn(acc_to_float<ACCK>(acc[4 * j + 3]), sx), w.w, b.w);
+  }
+}
+
+// Sign-extends packed weights that a bulk copy has left in shared memory ([k_blocks][BN rows] of 64 bytes at `packed`) into
+// operand slabs, one per k-block, `dst_stride` bytes apart, in the layout a swizzled TMA load of int8 codes would have
+// produced: row r of a k-block is 128 bytes, its 16-byte chunk j sits at position j ^ (r & 7).  Exact (integers).  Thread
+// `t` of THREADS; the caller makes the stores visible to the tensor core.
+template <int BN, int THREADS>
+__device__ __forceinline__ void expand_packed_slab(uint32_t packed, uint32_t dst, uint32_t dst_stride, int k_blocks, int t) {
+  const int pieces = k_blocks * BN * 4;  // 16 packed bytes -> 32 codes each
+  for (int q = t; q < pieces; q += THREADS) {
+    const int kb = q / (BN * 4), rem = q - kb * (BN * 4);
+    const int r = rem >> 2, piece = rem & 3;
+    uint32_t w0, w1, w2, w3;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3)
+                 : "r"(packed + kb * BN * 64 + r * 64 + piece * 16)
+                 : "memory");
+    uint32_t o[8];
+    unpack_word(w0, o[0], o[1]);
+    unpack_word(w1, o[2], o[3]);
+    unpack_word(w2, o[4], o[5]);
+    unpack_word(w3, o[6], o[7]);
+    const uint32_t row_base = dst + kb * dst_stride + r * 128;
+    const uint32_t d0 = row_base + (((2 * piece) ^ (r & 7)) << 4);
+    const uint32_t d1 = row_base + (((2 * piece + 1) ^ (r & 7)) << 4);
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d0), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d1), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
   }
 }
 
@@ -735,31 +763,10 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     const bool do_store = !RQ || p.has_y != 0;  // the fp32 output is written (always, without RQ)
 
     if (WS && BPACK) {
-      // Sign-extend the CTA's packed weights into the resident slab, in the layout a swizzled
-      // TMA load of int8 codes would have produced: row r of a k-block is 128 bytes, its 16-byte
-      // chunk j sits at position j ^ (r & 7).  Exact (integers), done once per CTA.
+      // the CTA's packed weights into the resident slab, once
       ok = mbar_wait(smem_u32(&b_loaded_bar), 0, &abort_flag, t_start);
       if (ok) {
-        const int pieces = p.k_blocks * BN * 4;  // 16 packed bytes -> 32 codes each
-        for (int q = (ew * 32 + lane); q < pieces; q += EW * 32) {
-          const int kb = q / (BN * 4), rem = q - kb * (BN * 4);
-          const int r = rem >> 2, piece = rem & 3;
-          uint32_t w0, w1, w2, w3;
-          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3)
-                       : "r"(smem_epi + kb * BN * 64 + r * 64 + piece * 16)
-                       : "memory");
-          uint32_t o[8];
-          unpack_word(w0, o[0], o[1]);
-          unpack_word(w1, o[2], o[3]);
-          unpack_word(w2, o[4], o[5]);
-          unpack_word(w3, o[6], o[7]);
-          const uint32_t row_base = smem_res_b + kb * Cfg::kBBytes + r * 128;
-          const uint32_t d0 = row_base + (((2 * piece) ^ (r & 7)) << 4);
-          const uint32_t d1 = row_base + (((2 * piece + 1) ^ (r & 7)) << 4);
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d0), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]) : "memory");
-          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d1), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
-        }
+        expand_packed_slab<BN, EW * 32>(smem_epi, smem_res_b, Cfg::kBBytes, p.k_blocks, ew * 32 + lane);
         fence_proxy_async_smem();  // the tensor core reads the slab through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&b_ready_bar));
@@ -848,9 +855,9 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 if (n0 + j < p.N) p.acc_debug[(int64_t)m * p.N + n0 + j] = (int32_t)acc[j];
             }
           }
-          if (Cfg::kScaleSlab) dequant32<ACCK>(acc, sx, c_sw, c_bias, a);
+          if (Cfg::kScaleSlab) dequant_smem<ACCK>(acc, sx, c_sw, c_bias, a);
           else dequant32_gmem<ACCK>(acc, sx, p.s_w, p.bias, out0 + col, p.N, a);
-          if (p.act == AQT_ACT_SWISH) swish32(a);
+          if (p.act == AQT_ACT_SWISH) swish(a);
         } else {
           // gates first: g = sigmoid(z_gate); then the values are scaled by it
           float g[32];
@@ -864,7 +871,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 if (ng + j < p.N) p.acc_debug[(int64_t)m * p.N + ng + j] = (int32_t)acc[j];
             }
           }
-          if (Cfg::kScaleSlab) dequant32<ACCK>(acc, sx, c_sw + slab_gate_off, c_bias + slab_gate_off, g);
+          if (Cfg::kScaleSlab) dequant_smem<ACCK>(acc, sx, c_sw + slab_gate_off, c_bias + slab_gate_off, g);
           else dequant32_gmem<ACCK>(acc, sx, p.s_w, p.bias, p.N / 2 + oc, p.N, g);
 #pragma unroll
           for (int j = 0; j < 32; ++j) g[j] = sigmoid_f(g[j]);
@@ -885,11 +892,11 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                 if (oc + j < p.N / 2) p.acc_debug[(int64_t)m * p.N + oc + j] = (int32_t)acc[j];
             }
           }
-          if (Cfg::kScaleSlab) dequant32<ACCK>(acc, sx, c_sw, c_bias, a);
+          if (Cfg::kScaleSlab) dequant_smem<ACCK>(acc, sx, c_sw, c_bias, a);
           else dequant32_gmem<ACCK>(acc, sx, p.s_w, p.bias, oc, p.N / 2, a);
 #pragma unroll
           for (int j = 0; j < 32; ++j) a[j] = a[j] * g[j];
-          if (p.act == AQT_ACT_GLU_SWISH) swish32(a);
+          if (p.act == AQT_ACT_GLU_SWISH) swish(a);
         }
 
         // the chunk this warp handles after this one (for the residual prefetch)
