@@ -46,6 +46,7 @@ struct RequantParams {
   int qmax_out;         // 127 or 7
   int rounding;
   int pack_out;         // 1: two 4-bit codes per byte
+  int one_tile_sets;    // sets of epilogue warps on the tile of a CTA that has one (sets_per_tile)
 };
 
 // DEEP: the resident weight slab holds eight k-blocks (K <= 1024, the d = 1024 encoder's first
@@ -97,10 +98,9 @@ constexpr int kSlots = 4;
 
 // Sets of epilogue warps that share a tile, for a CTA that has n_my of them.  With four tiles or more each set works on one
 // of its own, in another phase than the others; with fewer, whole sets would be idle while one warp a quadrant goes through
-// a tile's four chunks one after the other, with a residual a load of it from memory between any two.  (Two blocks of width
-// 512, graph replay: 256 rows 142.7 -> 133.6 us, 1013 153.0 -> 143.5, 4736 221.0 -> 214.6, 9472 312 -> 306; three tiles or
-// more alike.)
-__device__ __forceinline__ int sets_per_tile(int n_my) { return n_my == 1 ? 4 : (n_my == 2 ? 2 : 1); }
+// a tile's four chunks one after the other, with a residual a load of it from memory between any two.  Which launches:
+// see launch_requant_inst.
+__device__ __forceinline__ int sets_per_tile(int n_my, int one_tile_sets) { return n_my == 1 ? one_tile_sets : (n_my == 2 ? 2 : 1); }
 
 // Tag of this execution's exchange words.  A replayed CUDA graph repeats the call's own tag, so the group's generation
 // counter goes into it.  Whoever reads the counter hands the tag out (an arrival each on `bar`), and a CTA publishes nothing
@@ -164,7 +164,7 @@ __device__ __forceinline__ bool collect_maxima(const uint64_t* xt, int parts, ui
 // GLU: a tile's 128 weight rows are 64 value channels and their 64 gate channels; it yields 64
 // output columns u = v * sigmoid(g) (then Swish for AQT_ACT_GLU_SWISH), 16 per epilogue warp.
 // The GLU form writes codes and scales only (no fp32 output, no residual, no nibble packing).
-// SHARED: CTAs with one or two tiles have several sets of warps work on each (sets_per_tile).
+// SHARED: CTAs with one or two tiles may have several sets of warps work on each (sets_per_tile).
 template <bool BPACK, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU, bool DEEP, bool SHARED>
 __global__ void __launch_bounds__(32 * 20, 1)
 qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
@@ -210,7 +210,7 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   const int group = blockIdx.x / p.tiles_n;
   const int groups = gridDim.x / p.tiles_n;
   const int n_my = group < p.tiles_m ? (p.tiles_m - group + groups - 1) / groups : 0;
-  const int split = SHARED ? sets_per_tile(n_my) : 1;
+  const int split = SHARED ? sets_per_tile(n_my, rp.one_tile_sets) : 1;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -659,14 +659,25 @@ static int launch_requant_form(const int8_t* a, const void* b, void* q_out, floa
                     tm_y, tm_r, rp);
 }
 
+// Sets of warps share tiles where no CTA has more than two, by what the epilogue does (us a call in a replayed graph, for one /
+// two / four sets on the tile of a CTA that has one, while CTAs that have two put two on each; most outputs of a tile per CTA
+// do not come here but to qgemm_few_tiles_sm100.cuh):
+//   codes only, no activation  not at all: 4864 x 512 -> 512 7.79 / 8.22 / 8.21, 3840 x 512 -> 1024 8.48 / 8.68 / 8.86
+//   codes only, Swish          two: 1863 x 512 -> 2048 10.32 / 10.03 / 10.09, 1152 x 1024 -> 2048 9.96 / 9.56 / 9.75
+//   gate forms, fp32 output    four if no CTA has two tiles, else two: residual, 4864 x 512 -> 512 11.20 / 10.55 / 10.83, packed
+//                              codes, 1013 x 512 -> 512 9.23 / 8.28 / 7.82; gates, 512 x 1024 -> 2048 8.82 / 8.71 / 8.40
+// (Three tiles a CTA gain nothing in any form.)
 template <bool BPACK, bool WITH_Y, int ROUNDING, bool PACK_OUT, bool GLU = false, bool DEEP = false>
-static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, const RequantParams& rp,
-                               void* exchange, cudaStream_t st) {
+static int launch_requant_inst(const int8_t* a, const void* b, void* q_out, float* y, int64_t ldy, RequantParams rp, void* exchange,
+                               cudaStream_t st) {
   const int sms = sm_count();
   if (sms <= 0) return AQT_ERR_CUDA;
-  const int64_t groups = sms / ceil_div(rp.g.N, 128);
-  if (ceil_div(rp.g.M, kBM) <= 2 * groups)
+  const int64_t groups = sms / ceil_div(rp.g.N, 128), tiles_m = ceil_div(rp.g.M, kBM);
+  if (tiles_m <= 2 * groups && (WITH_Y || GLU || rp.g.act != AQT_ACT_NONE)) {
+    rp.one_tile_sets = tiles_m <= groups && (WITH_Y || GLU) ? 4 : 2;
     return launch_requant_form<BPACK, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, true>(a, b, q_out, y, ldy, rp, exchange, st);
+  }
+  rp.one_tile_sets = 1;
   return launch_requant_form<BPACK, WITH_Y, ROUNDING, PACK_OUT, GLU, DEEP, false>(a, b, q_out, y, ldy, rp, exchange, st);
 }
 

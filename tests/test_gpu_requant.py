@@ -127,14 +127,16 @@ def test_requant_with_residual_stream_many_tiles_per_cta():
 @pytest.mark.parametrize("with_res", [True, False])
 def test_requant_sets_that_share_a_tile(M, N, K, with_res):
     # one, two and three tiles per CTA, and CTAs with one and two in the same launch (148 SMs: 37 or 9 groups of CTAs)
-    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, plan="ws128", plan_without_y="ws128")
+    for act in (aqt.ACT_NONE, aqt.ACT_SWISH):
+        _run(M, N, K, 8, 4, act, True, with_res, 8, aqt.ROUND_NEAREST_EVEN, False, plan="ws128", plan_without_y="ws128")
 
 
 @pytest.mark.parametrize("M,N,K", [(200, 512, 512), (1013, 512, 256), (700, 1056, 64)])
 @pytest.mark.parametrize("with_res", [True, False])
 def test_requant_packed_codes_of_few_tiles(M, N, K, with_res):
     # one tile per CTA, all four sets on it: packed codes leave only the weight-stationary kernel
-    _run(M, N, K, 8, 4, aqt.ACT_NONE, True, with_res, 4, aqt.ROUND_NEAREST_EVEN, True, plan="ws128", plan_without_y="ws128")
+    for act in (aqt.ACT_NONE, aqt.ACT_SWISH):
+        _run(M, N, K, 8, 4, act, True, with_res, 4, aqt.ROUND_NEAREST_EVEN, True, plan="ws128", plan_without_y="ws128")
 
 
 def test_requant_many_tiles_per_cta():
