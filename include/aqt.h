@@ -32,7 +32,7 @@
 extern "C" {
 #endif
 
-#define AQT_VERSION 201
+#define AQT_VERSION 202
 
 /* status codes */
 #define AQT_OK 0

@@ -682,7 +682,7 @@ int aqt_qmatmul_requant(const void* xq, const float* s_x, int s_x_kind, const vo
   p.K = (int)K;
   p.n_out = (int)n_out;
   p.tiles_m = p.tiles_n = p.k_blocks = 0;
-  p.small_acc = (K * (int64_t)(qmax_of(code_bits(bits_a)) + 1) * (qmax_of(code_bits(bits_w)) + 1) <= (1ll << 22)) ? 1 : 0;
+  p.small_acc = 0;
   p.static_w = (static_w && (!is_packed(bits_w) || b_packed)) ? 1 : 0;  // not for weights unpacked into the workspace just now
   rp.q_out = nullptr;
   rp.s_out = s_out;

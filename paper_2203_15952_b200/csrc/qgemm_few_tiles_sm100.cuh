@@ -16,7 +16,8 @@
 //   - weights that were complete before the kernel ahead fill their part of the ring while that kernel drains.
 // Measured (graph replay, us): see few_tiles_bn.
 //
-// The exchange of row maxima, the tags of its words and the bounded waits are those of qgemm_requant_sm100.cuh.
+// The exchange of row maxima (collect_maxima), the tags of its words (hand_out_tag) and the bounded waits are those of
+// qgemm_requant_sm100.cuh.
 #pragma once
 
 #include "qgemm_requant_sm100.cuh"
@@ -395,7 +396,10 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
 //   - K <= 512: matmul 0.62-0.78 / 0.82 on 32 and 64 columns, 0.88-0.93 / 0.95 on 128; the whole layer on floats 0.71-0.83 / 0.93
 //     and 0.90-0.94 / 0.97; with the row quantizer 0.74-0.90 / 0.96 and 0.86-0.96 / 1.00 (against the weight-stationary tiles
 //     of 128 columns).  At most sixteen parts of a row, which an exchange warp reads in one go, unless the tile is 128 wide
-//     (64 parts 1.05 / 1.25, 128 parts 1.34 / 1.71).
+//     (64 parts 1.05 / 1.25, 128 parts 1.34 / 1.71).  Without the row quantizer at most 64 n-tiles below 128 columns: beyond,
+//     a few rows lose with the narrower tiles (us at the wider and the narrower: 20 x 512 -> 4096 4.21 / 4.52, -> 9472 4.53 /
+//     5.27, 64 x 512 -> 9472 4.72 / 4.95), while full tiles and short contractions would gain (128 x 512 -> 4736 5.14 / 4.31,
+//     20 x 128 -> 4736 3.35 / 3.08): against the kernels before this one either is faster.
 //   - deeper: with the row quantizer 0.72-0.97 / 1.02 (two kernels, or pairs); without one only the gate forms, from 65
 //     rows on, 0.90-0.92 / 1.00: for the others the streaming kernel's tiles of 64 columns have the same latency
 //     (0.98-1.04 / 1.13).  Four stages of 128 columns are too few.

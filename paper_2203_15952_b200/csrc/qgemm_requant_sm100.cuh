@@ -13,15 +13,17 @@
 // through global memory, one 64-bit word per (m-tile, n-tile, row): the maximum's bit pattern below a
 // tag that identifies this execution, so a word is its own validity and nothing is cleared,
 // counted or fenced.
-//   epilogue warps    four sets of four warps (one warp per TMEM lane quadrant); set s owns
-//                     accumulator buffer s and every fourth tile, all 128 columns of it:
+//   epilogue warps    four sets of four warps (one warp per TMEM lane quadrant).  In a CTA with
+//                     many tiles set s owns accumulator buffer s and every fourth tile, all 128
+//                     columns of it; a CTA with one or two may put several sets on each
+//                     (sets_per_tile), which then take chunks of its columns and merge their maxima:
 //                       pass 1  accumulators -> u (registers) -> row maxima; u goes back into the
 //                               TMEM columns it came from; the maxima are published
 //                       wait    for the group's other CTAs (the exchange warps do the polling)
 //                       pass 2  scale from the final maximum, u from TMEM, codes, stores; the TMEM
 //                               buffer goes back to the MMA
-//                     The four warps on a scheduler thus sit in four different phases of four
-//                     different tiles, which is what keeps the special-function unit (pass 1 of a
+//                     With many tiles the four warps on a scheduler thus sit in four different
+//                     phases of four different tiles, which is what keeps the special-function unit (pass 1 of a
 //                     Swish tile) and the other pipes (pass 2) busy at the same time.
 //   exchange warps    two, one per half of the rows: for each tile in turn read the words of all
 //                     n-tiles (all requests in flight together), again until every one is valid,
@@ -353,8 +355,8 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
   } else {
     // ------------------------------------------------------------------ epilogue warps
     // Four sets of four warps, one warp of a set per TMEM lane quadrant (hence one per scheduler).
-    // Set s owns accumulator buffer s and with it every fourth tile of this CTA, all of its
-    // columns: pass 1 chunk by chunk, publication of the rows' maxima straight from registers
+    // Unless sets share tiles (see below), set s owns accumulator buffer s and with it every fourth
+    // tile of this CTA, all of its columns: pass 1 chunk by chunk, publication of the rows' maxima straight from registers
     // (a thread has seen its whole row of the tile, so nothing is merged across warps), the wait
     // for the other n-tiles' maxima, pass 2.  The four warps that share a scheduler therefore work
     // on four different tiles in four different phases: while one is on the special-function unit

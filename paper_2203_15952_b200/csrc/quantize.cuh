@@ -422,8 +422,9 @@ static int launch_quantize_tensor_vec(const float* x, int64_t rows, int64_t cols
   // in registers (graph replay of the layer: 300 x 128 9.2 -> 7.2 us, 641 x 288 10.8 -> 8.7, 3000 x 256 10.8 -> 9.7; the line is
   // where the blocks that wait would keep others of either pass from the SMs: 7411 x 512, 927 blocks, 17.2 -> 17.5; 65 536 x
   // 512 100 -> 113).
-  const int64_t grid = want < 148 * 8 ? want : 148 * 8;
-  const bool beside = want <= 148 * 4;
+  const int64_t sms = sm_count() > 0 ? sm_count() : kDefaultSms;
+  const int64_t grid = want < sms * 8 ? want : sms * 8;
+  const bool beside = want <= sms * 4;
   int rc;
   if (partial == nullptr) {
     rc = launch_pdl(clear_scale_kernel, dim3(1, 1, 1), dim3(1, 1, 1), 0, st, 1, scale_out);
