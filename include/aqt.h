@@ -106,6 +106,7 @@ const char* aqt_status_string(int status);
  *           figure's cast does).  pack == 1 (bits == 4 only, cols even): uint8 [rows, cols/2].
  * scale_out fp32, extent given by `axis` (see AQT_AXIS_*).  For AQT_AXIS_COL and
  *           AQT_AXIS_TENSOR it also serves as the abs-max accumulator while the call runs.
+ * NaN is left out of the maximum and has code 0.
  * Alignment: none required; 16-byte aligned x with ld % 4 == 0 and cols % 4 == 0 takes the
  * vectorised path.  rows or cols == 0 is a no-op.
  */

@@ -345,9 +345,11 @@ qgemm_few_tiles_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         tma_store_commit();
       }
     }
+    const float any_nan = chunk_max(0.0f, a);  // (this warp has nothing to do until the other CTAs have published)
     if (ok && rq) ok = wait(ctx_bar[quad >> 1]);
     if (ok && rq) {
-      const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(row_amax[row_in_tile]), rp.qmax_out);
+      ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(row_amax[row_in_tile]), rp.qmax_out);
+      sc.fast = sc.fast && any_nan == any_nan;  // see chunk_max
       if (tn == tn_first && set == 0 && m < p.M) rp.s_out[m] = sc.s;
       uint32_t u[C], w[C / 4];
 #pragma unroll

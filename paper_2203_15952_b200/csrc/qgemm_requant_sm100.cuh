@@ -430,13 +430,9 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
 #pragma unroll
           for (int j = 0; j < 16; ++j) av[j] = av[j] * g[j];
           if (p.act == AQT_ACT_GLU_SWISH) swish(av);
-          float cmax = 0.0f;
+          if (cols_ok) amax = chunk_max(amax, av);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            cmax = fmaxf(cmax, fabsf(av[j]));
-            accv[j] = __float_as_uint(av[j]);
-          }
-          if (cols_ok) amax = fmaxf(amax, cmax);
+          for (int j = 0; j < 16; ++j) accv[j] = __float_as_uint(av[j]);
           tmem_st_32x16(tbase + col, accv);  // u replaces the value accumulators
         } else {
           uint32_t acc[32];
@@ -460,13 +456,9 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
             }
             __syncwarp();  // every lane has read its residual row before the buffer is overwritten
           }
-          float cmax = 0.0f;
+          if (cols_ok) amax = chunk_max(amax, a);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            cmax = fmaxf(cmax, fabsf(a[j]));
-            acc[j] = __float_as_uint(a[j]);
-          }
-          if (cols_ok) amax = fmaxf(amax, cmax);
+          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(a[j]);
           tmem_st_32x32(tbase + col, acc);  // u replaces the accumulators it was made from
           if (WITH_Y) {
             if (!has_res) {
@@ -499,6 +491,20 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
         }
       }
       if (!ok) break;
+      const bool has_nan = __any_sync(0xffffffffu, amax != amax) != 0;
+      if (has_nan) {
+        // the maxima of the warp's rows once more, from what pass 1 has left in tensor memory
+        tmem_st_wait();
+        amax = 0.0f;
+#pragma unroll 1
+        for (int c = c_begin; c < c_end && oc0 + c * CW < n_out; ++c) {
+          uint32_t u[CW];
+          if constexpr (GLU) tmem_ld_32x16(tbase + c * CW, u);
+          else tmem_ld_32x32(tbase + c * CW, u);
+          tmem_ld_wait();
+          amax = numbers_max(amax, u);
+        }
+      }
       // This CTA's maxima of the tile's rows, each tagged valid: one word per row.  Of a tile that several sets share, the
       // first set's warp publishes the maximum of all parts (a CTA that shares tiles has one for every group of sets, so
       // the barrier is waited on once).
@@ -521,7 +527,8 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
       const float amax_row = __uint_as_float(row_amax[buf][row_in_tile]);
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&ctx_free_bar[buf][quad >> 1]));
-      const ScaleCtx sc = make_scale_ctx_zeros(amax_row, rp.qmax_out);
+      ScaleCtx sc = make_scale_ctx_zeros(amax_row, rp.qmax_out);
+      sc.fast = sc.fast && !has_nan;
       if (tn == 0 && part == 0 && m < p.M) rp.s_out[m] = sc.s;
       tmem_st_wait();  // this warp's stores of pass 1
 #pragma unroll 1

@@ -944,13 +944,9 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         if constexpr (RQ) {
           // u stays in tensor memory, over the accumulators it was made from, until the row's scale is known
-          float cmax = 0.0f;
+          if (oc < p.n_out) rq_amax = chunk_max(rq_amax, a);  // columns beyond N contribute nothing
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            cmax = fmaxf(cmax, fabsf(a[j]));
-            acc[j] = __float_as_uint(a[j]);
-          }
-          if (oc < p.n_out) rq_amax = fmaxf(rq_amax, cmax);  // columns beyond N contribute nothing
+          for (int j = 0; j < 32; ++j) acc[j] = __float_as_uint(a[j]);
           tmem_st_32x32(lane_addr + col, acc);
         }
         // row `lane` of the 32 x 32 box; 16-byte chunk j sits at (j ^ (row & 7)) under the 128-byte swizzle
@@ -987,6 +983,18 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         // ---------------------------------------------------------- the row's maximum over all of N
         const int parts = p.exchange_parts;
         const int my_part = tn * (EW / 4) + chalf;
+        const bool rq_nan = __any_sync(0xffffffffu, rq_amax != rq_amax) != 0;
+        if (rq_nan) {
+          // the maxima of the warp's rows once more, from what pass 1 has left in tensor memory
+          tmem_st_wait();
+          rq_amax = 0.0f;
+          for (int c = 0; c < chunks && out0 + (chalf * chunks + c) * 32 < p.n_out; ++c) {
+            uint32_t u[32];
+            tmem_ld_32x32(lane_addr + (chalf * chunks + c) * 32, u);
+            tmem_ld_wait();
+            rq_amax = numbers_max(rq_amax, u);
+          }
+        }
         uint64_t* xrow = p.exchange + (size_t)m * parts;  // rows up to the padded tile height are allocated
         st_relaxed_gpu_64(xrow + my_part, ((uint64_t)rq_tag << 32) | __float_as_uint(rq_amax));
         uint32_t amax_bits = 0u;
@@ -1011,7 +1019,8 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
         if (!ok) break;
         // ---------------------------------------------------------- pass 2: scale, codes
-        const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(amax_bits), p.qmax_out);
+        ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(amax_bits), p.qmax_out);
+        sc.fast = sc.fast && !rq_nan;
         if (my_part == 0 && row_ok) p.s_out[m] = sc.s;
         tmem_st_wait();  // this warp's stores of pass 1
         for (int c = 0; c < chunks; ++c) {

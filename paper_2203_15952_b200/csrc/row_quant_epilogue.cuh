@@ -70,6 +70,33 @@ __device__ __forceinline__ uint32_t nibbles_of(uint32_t w0, uint32_t w1) {
   return __byte_perm(y0, y1, 0x6420);
 }
 
+// Values that are not numbers are left out of a row's maximum, as the quantizers leave them out, and their code is 0, which
+// the additions of code_bits2 do not give: rows that have some take the general sequence (ScaleCtx::fast off).  So that rows
+// of numbers pay nothing, their maxima let NaN through (chunk_max), which costs no more than to drop it, and whoever finds
+// one at the end takes the maximum again (numbers_max).
+__device__ __forceinline__ float max3_through_nan(float a, float b, float c) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+  return m;
+}
+// max(m, |a[.]|), NaN if one of them is.
+template <int NV>
+__device__ __forceinline__ float chunk_max(float m, const float (&a)[NV]) {
+  float m1 = 0.0f;
+#pragma unroll
+  for (int j = 0; j < NV; j += 4) {
+    m = max3_through_nan(m, fabsf(a[j]), fabsf(a[j + 1]));
+    m1 = max3_through_nan(m1, fabsf(a[j + 2]), fabsf(a[j + 3]));
+  }
+  return max3_through_nan(m, m1, 0.0f);
+}
+template <int NV>
+__device__ __forceinline__ float numbers_max(float m, const uint32_t (&u)[NV]) {
+#pragma unroll
+  for (int j = 0; j < NV; ++j) m = fmaxf(m, fabsf(__uint_as_float(u[j])));
+  return m;
+}
+
 // NV (32 or 16) values of one row -> NV / 4 words of int8 codes (PACK: NV / 8 words of nibbles).
 template <int ROUNDING, bool PACK, int NV>
 __device__ __forceinline__ void codes_of(const uint32_t (&u)[NV], const ScaleCtx& c, int qmax, uint32_t (&w)[NV / 4]) {

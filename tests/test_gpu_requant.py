@@ -339,6 +339,45 @@ def test_requant_calls_that_wait_on_nobody_write_over_their_input(M, N, K, act):
     assert torch.equal(y, y_ref) and torch.equal(xq, q_ref) and torch.equal(s_x, s_ref) and aqt.aqt_device_status() == 0
 
 
+@pytest.mark.parametrize("M,N,K,act,res,pack_out,plan", [
+    (200, 512, 512, aqt.ACT_NONE, True, False, "few32"), (1013, 1024, 1024, aqt.ACT_NONE, True, False, "few64"),
+    (1013, 2048, 256, aqt.ACT_SWISH, False, False, "few128"), (300, 1024, 512, aqt.ACT_GLU_SWISH, False, False, "few64"),
+    (5000, 512, 256, aqt.ACT_NONE, True, False, "ws128"), (5000, 512, 256, aqt.ACT_SWISH, False, False, "ws128"),
+    (13000, 1024, 128, aqt.ACT_NONE, False, False, "ws128"), (2600, 1024, 512, aqt.ACT_GLU, False, False, "ws128"),
+    (700, 1024, 512, aqt.ACT_NONE, True, True, "ws128"), (1500, 4096, 1024, aqt.ACT_SWISH, False, False, "ws128"),
+    (5000, 480, 2048, aqt.ACT_NONE, True, False, "pair256s4e8"), (2500, 512, 2048, aqt.ACT_NONE, False, False, "pair256s4e8")])
+def test_requant_values_that_are_not_numbers(M, N, K, act, res, pack_out, plan):
+    """NaN (from a bias or the residual), rows of nothing else and rows with an infinity: the codes and scales of aqt_quantize
+    on the output rows, which leaves NaN out of the maximum and gives it code 0."""
+    rng = np.random.default_rng(M)
+    n_out = N // 2 if act in (aqt.ACT_GLU, aqt.ACT_GLU_SWISH) else N
+    s_x, bias = rng.uniform(1e-3, 5e-2, M).astype(np.float32), (rng.standard_normal(N) * 0.1).astype(np.float32)
+    bias[[3, N - 1]] = np.nan
+    s_x[[5, M - 1]] = np.inf
+    s_x[6] = np.nan
+    r = None
+    if res:
+        r = rng.standard_normal((M, n_out)).astype(np.float32)
+        r[::7, ::11] = np.nan
+        r[9, 2] = -np.inf
+    xq = _codes(rng, M, K, 8)
+    xq[4] = 0
+    args = (_dev(xq), _dev(s_x), _dev(_codes(rng, N, K, 8)), _dev(rng.uniform(1e-4, 5e-3, N).astype(np.float32)), _dev(bias),
+            None if r is None else _dev(r), 0.5)
+    bits_out = 4 if pack_out else 8
+    y_ref = aqt.aqt_qmatmul(*args, K=K, act=act)
+    assert bool(y_ref.isnan().any(dim=1).all()) and bool(y_ref[6].isnan().all())
+    q_ref, s_ref = aqt.aqt_quantize(y_ref, bits_out, pack=pack_out)
+    for with_y in ((True,) if res else (False, True)):
+        if with_y == res:
+            assert aqt.aqt_plan_qmatmul_requant(M, N, K, 8, 8 | aqt.MAY_WAIT, act, with_y=with_y, pack_out=pack_out) == plan
+        q, s, y = aqt.aqt_qmatmul_requant(*args, K=K, bits_w=8 | aqt.MAY_WAIT, act=act, bits_out=bits_out, pack_out=pack_out, want_y=with_y)
+        assert torch.equal(s.view(torch.int32), s_ref.view(torch.int32))
+        assert torch.equal(q, q_ref), (with_y, int((q != q_ref).sum()))
+        assert y is None or torch.equal(y.nan_to_num(7.5), y_ref.nan_to_num(7.5))
+    assert aqt.aqt_device_status() == 0
+
+
 def test_requant_argument_checks():
     z8 = torch.zeros((64, 64), dtype=torch.int8, device=DEV)
     w8 = torch.zeros((48, 64), dtype=torch.int8, device=DEV)
