@@ -149,7 +149,7 @@ def test_requant_many_tiles_per_cta():
                                                (260, 1024, 768, 4, aqt.ACT_NONE)])
 def test_requant_deep_k_form(M, N, K, bits_w, act):
     """512 < K <= 1024 (the d = 1024 encoder): the fused kernel with an eight-k-block weight slab
-    takes the call when only codes and scales are wanted.  _run checks the two-step path (with y)
+    takes the call when only codes and scales are wanted (the kernel for few tiles where it applies).  _run checks the two-step path (with y)
     against the oracle and then the fused path (without y) against it, bit for bit."""
     _run(M, N, K, 8, bits_w, act, True, False, 8, aqt.ROUND_NEAREST_EVEN, False)
     # (the huge-scale special row stays finite only with 4-bit weights at this depth)
