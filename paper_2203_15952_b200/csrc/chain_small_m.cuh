@@ -23,16 +23,23 @@
 // cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
 // scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
 // wait of the library.
-// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 425 vs 1250 us, 32 rows
-// 427 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 626 vs 1340; beyond, a
+// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 337 vs 1250 us, 32 rows
+// 346 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 507 vs 1340; beyond, a
 // second wave of clusters or 32 rows per cluster lose to the per-layer kernels at d = 1024 (860 vs 700
 // us for 8 blocks at 113 rows), which is where AQT_CHAIN_MAX_ROWS lies.
-// What a layer then costs is a chain of latencies and of instructions that every warp issues once: no
-// integer division and no dependent parameter load in the loops (the step table sits in shared memory
-// with everything derived from the sizes), the next layer's weights, scales and prefetches are asked
-// for while the row maxima are under way, eight warps instead of sixteen, and packed weights are used as sixteen times their codes
-// (a nibble in the upper half of a byte; the sums are shifted back, exact), two instructions per four
-// codes instead of eleven per eight, against activation codes stored in the same even / odd order.
+// What a layer then costs (2000 to 2600 ns; clock stamps in a copy) is a chain of latencies and of instructions that every warp
+// issues once, at the pace at which their lines are fetched:
+//   * eight warps form the products and eight take the rows from there, so that the next weights are asked for while the rows
+//     are de-quantized and exchanged (asking takes 1000 clocks of a layer's 5000), and the products of q and k do not wait
+//     for the rows of the layer before (445 -> 383 us);
+//   * what is not always run stands aside: the general code sequence in a function, the wide form's second words behind a
+//     branch, the loop over pieces left at the last one (383 -> 344 us); stores of a layer's outputs wait until its maxima are on their way;
+//   * no integer division and no dependent parameter load in the loops (the step table sits in shared memory with everything
+//     derived from the sizes), and packed weights are used as sixteen times their codes (a nibble in the upper half of a
+//     byte; the sums are shifted back, exact), two instructions per four codes instead of eleven per eight, against
+//     activation codes stored in the same even / odd order.
+// (One exchange of whole fp32 rows, quantized by every CTA for itself, instead of maxima and then codes: 446 -> 463 us.  Scales and
+// residuals in registers ahead of the sums, with a path for unaligned ones: 383 -> 385, sixteen rows 571 -> 612.)
 // The arithmetic is that of the per-layer kernels operation by operation (exact int32 sums, the same
 // de-quantization, activation and quantizer), so the results are the same bits.
 #pragma once
@@ -45,11 +52,12 @@
 namespace aqt {
 
 constexpr int kChainCtas = 16;     // CTAs of a cluster (beyond the portable eight: allowed per function)
-constexpr int kChainWarps = 8;
-constexpr int kChainThreads = 32 * kChainWarps;
+constexpr int kChainWarps = 8;     // warps that form products, and as many that take the rows from there
+constexpr int kChainRowThreads = 32 * kChainWarps;
+constexpr int kChainThreads = 2 * kChainRowThreads;
 constexpr int kChainChunk = 8;     // pieces (two 16-byte weight loads per lane) in flight
 constexpr int kChainMaxSteps = 256;
-constexpr int kChainMaxN = kChainCtas * kChainThreads;  // one scale per thread
+constexpr int kChainMaxN = kChainCtas * kChainRowThreads;  // one scale per thread
 constexpr int kChainMaxCols = 256;              // output columns per CTA: eight floats per lane and row
 
 struct ChainStep {
@@ -116,6 +124,10 @@ __device__ __forceinline__ void chain_st_async_v2(uint32_t addr, uint32_t v0, ui
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v0), "r"(v1), "r"(bar)
                : "memory");
 }
+// Named barriers between the two halves of a block: one side arrives, the other waits.  Barrier 1 + slot: partial sums are
+// there; 3 + slot: they have been read.
+__device__ __forceinline__ void chain_bar_arrive(int id) { asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "n"(kChainThreads) : "memory"); }
+__device__ __forceinline__ void chain_bar_sync(int id) { asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "n"(kChainThreads) : "memory"); }
 __device__ __forceinline__ void chain_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -129,18 +141,26 @@ __device__ __forceinline__ void chain_order8(bool packed, uint32_t& w0, uint32_t
   w1 = packed ? odd : w1;
 }
 
-// Four codes of a row as one word.
-template <int ROUNDING>
-__device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax) {
-  if (c.fast)
-    return pack4_i8(quantize_fast<ROUNDING>(v[0], c.s, c.r), quantize_fast<ROUNDING>(v[1], c.s, c.r), quantize_fast<ROUNDING>(v[2], c.s, c.r),
-                    quantize_fast<ROUNDING>(v[3], c.s, c.r));
-  return pack4_i8(quantize_elem<ROUNDING>(v[0], c, qmax), quantize_elem<ROUNDING>(v[1], c, qmax), quantize_elem<ROUNDING>(v[2], c, qmax),
-                  quantize_elem<ROUNDING>(v[3], c, qmax));
+// Four codes of a row as one word.  The general sequence stands apart: every warp runs through the code of a step once, and
+// pays for each instruction line that it fetches.
+__device__ __noinline__ uint32_t chain_codes4_general(float v0, float v1, float v2, float v3, float s, int qmax, int rounding) {
+  const ScaleCtx c = {s, 0.0f, false};
+  if (rounding == AQT_ROUND_HALF_UP_FLOOR)
+    return pack4_i8(quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v0, c, qmax), quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v1, c, qmax),
+                    quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v2, c, qmax), quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v3, c, qmax));
+  return pack4_i8(quantize_elem<AQT_ROUND_NEAREST_EVEN>(v0, c, qmax), quantize_elem<AQT_ROUND_NEAREST_EVEN>(v1, c, qmax),
+                  quantize_elem<AQT_ROUND_NEAREST_EVEN>(v2, c, qmax), quantize_elem<AQT_ROUND_NEAREST_EVEN>(v3, c, qmax));
 }
 __device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax, int rounding) {
-  return rounding == AQT_ROUND_HALF_UP_FLOOR ? chain_codes4<AQT_ROUND_HALF_UP_FLOOR>(v, c, qmax)
-                                             : chain_codes4<AQT_ROUND_NEAREST_EVEN>(v, c, qmax);
+  if (__builtin_expect(!c.fast, 0)) return chain_codes4_general(v[0], v[1], v[2], v[3], c.s, qmax, rounding);
+  const bool half_up = rounding == AQT_ROUND_HALF_UP_FLOOR;
+  int q[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float q0 = __fmul_rn(v[e], c.r), t = __fmaf_rn(__fmaf_rn(-q0, c.s, v[e]), c.r, q0);  // as quantize_fast
+    q[e] = half_up ? __float2int_rd(__fadd_rn(t, 0.5f)) : __float2int_rn(t);
+  }
+  return pack4_i8(q[0], q[1], q[2], q[3]);
 }
 __device__ __forceinline__ float chain_max4(float m, const float (&v)[4]) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
@@ -153,7 +173,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   constexpr int SETS = NT == 1 ? 2 : 1;  // independent accumulators per row tile (the products of one set depend on one another)
   extern __shared__ __align__(128) uint8_t chain_smem[];
   __shared__ __align__(16) ChainStep steps[MAXS];
-  __shared__ __align__(16) float sw_s[2][kChainThreads], bias_s[2][kChainThreads];
+  __shared__ __align__(16) float sw_s[2][kChainRowThreads], bias_s[2][kChainRowThreads];
   __shared__ uint32_t amax_s[R][kChainCtas];  // bit patterns of the row maxima of every CTA's columns
   __shared__ uint64_t amax_bar[R];            // a row's sixteen maxima have arrived
   __shared__ uint64_t codes_bar;              // all codes of the next input have arrived
@@ -161,7 +181,9 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   uint8_t* codes = chain_smem;
   float* h = reinterpret_cast<float*>(chain_smem + p.code_bytes + 2 * p.part_bytes);  // [R][h_cols]
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const bool rows_half = threadIdx.x < kChainRowThreads;    // this warp works on rows, else on products
+  const int warp = (threadIdx.x >> 5) & (kChainWarps - 1);  // of its half
   const int g = lane >> 2, kq = lane & 3;
   const int rank = (int)cluster_ctarank();
   const int row0 = (int)(blockIdx.x / kChainCtas) * R;
@@ -180,344 +202,376 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
   __syncthreads();
   grid_dependency_wait();
 
-  // ---- This warp's products in program order: units (sixteen channels and a share of K), each in items of up to
-  // kChainChunk pieces (16 bytes of two channels' weights per lane: 128 of K packed, 64 of K int8).  The next
-  // item's pieces are in nxt (zeros beyond its end).
-  int it_step = 0, it_u = warp;  // unit of the item
-  int u_left = 0;                // pieces from the item to the end of the unit
-  int u_a = 0, u_part = 0;       // this lane's first activation code (byte offset), first partial sum (index)
-  bool u_first = true, u_both = true;  // the unit's first item; its upper eight channels exist
-  const uint8_t *u_src0 = nullptr, *u_src1 = nullptr;
-  uint4 nxt[kChainChunk][2];
-  auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
-    while (it_step < n_steps && it_u >= steps[it_step].units) {
-      ++it_step;
-      it_u = warp;
-    }
-    u_left = 0;
-    if (it_step >= n_steps) return;
-    const ChainStep& st = steps[it_step];
-    const int k128 = st.K >> 7, per_cta = st.N >> 4;
-    const int shift = (st.flags & kChainPacked) ? 1 : 0;
-    int tile = it_u, kb0 = 0, kb1 = k128, ks = 0;  // tiles fastest, then shares of K
-    if (st.ks_n > 1) {
-      ks = (int)((uint32_t)it_u * st.inv_tiles >> 16);
-      tile = it_u - ks * st.tiles;
-      kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks_lo >> 16);
-      kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks_lo >> 16);
-    }
-    const int c0 = tile * 16 + g;  // this lane's channels among the CTA's: c0 and c0 + 8
-    u_both = tile * 16 + 8 < per_cta;
-    const int c1 = u_both ? c0 + 8 : c0;
-    int n0 = rank * per_cta + c0, n1 = rank * per_cta + c1;
-    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value channels, then the gate channels of the same output columns
-      const int cols = per_cta >> 1, gate_off = (st.N >> 1) - cols;
-      n0 = rank * cols + c0 + (c0 >= cols ? gate_off : 0);
-      n1 = rank * cols + c1 + (c1 >= cols ? gate_off : 0);
-    }
-    u_left = (kb1 - kb0) << (1 - shift);
-    const uint8_t* w = st.w + (kb0 << (7 - shift)) + kq * 16;
-    u_src0 = w + (int64_t)n0 * (st.K >> shift);
-    u_src1 = w + (int64_t)n1 * (st.K >> shift);
-    u_a = g * chain_pitch(st.K, shift != 0) + kb0 * 128 + kq * (16 << shift);
-    u_part = (ks * R + 2 * kq) * (per_cta + 4) + c0;
-    u_first = true;
-  };
-  auto load_piece = [&](int j) {
-    nxt[j][0] = nxt[j][1] = make_uint4(0u, 0u, 0u, 0u);
-    if (j < u_left) {
-      nxt[j][0] = __ldg(reinterpret_cast<const uint4*>(u_src0 + j * 64));
-      nxt[j][1] = __ldg(reinterpret_cast<const uint4*>(u_src1 + j * 64));
-    }
-  };
-  auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
-    wv = bv = 0.0f;
-    if (s >= n_steps) return;
-    const ChainStep& st = steps[s];
-    const int per_cta = st.N >> 4, c = threadIdx.x;
-    if (c - lane >= per_cta || c >= per_cta) return;
-    int n = rank * per_cta + c;
-    if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
-      const int cols = per_cta >> 1, gate = c >= cols ? 1 : 0;
-      n = gate * (st.N >> 1) + rank * cols + c - gate * cols;
-    }
-    wv = __ldg(st.s_w + n);
-    if (st.bias != nullptr) bv = __ldg(st.bias + n);
-  };
-  auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2 (the last thread: it has no row of a single row tile)
-    if (threadIdx.x != kChainThreads - 1 || s >= n_steps || blockIdx.x >= kChainCtas) return;
-    const ChainStep& st = steps[s];
-    const bool glu = (st.flags & kChainActMask) >= AQT_ACT_GLU;
-    const int row_bytes = (st.flags & kChainPacked) ? st.K >> 1 : st.K, rows_here = st.N >> (glu ? 5 : 4);
-    const uint8_t* src = st.w + (int64_t)rank * rows_here * row_bytes;
-    for (int gate = 0; gate <= (glu ? 1 : 0); ++gate, src += (int64_t)(st.N >> 1) * row_bytes)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(rows_here * row_bytes)) : "memory");
-  };
-
-  open_unit();
-#pragma unroll
-  for (int j = 0; j < kChainChunk; ++j) load_piece(j);
-  prefetch_slice(1);
-  float wv, bv;  // scale and bias of this thread's channel of the next step, on their way to sw_s / bias_s
-  load_scales(0, wv, bv);
-
-  // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
-  float sx[NT];  // input scales of this warp's rows (warp, warp + 8, ...)
-  {
-    const int pitch = chain_pitch(p.K0, (steps[0].flags & kChainPacked) != 0);
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int r = warp + 8 * t;
-      sx[t] = 0.0f;
-      if (r >= rows) continue;
-      const float4* xr = reinterpret_cast<const float4*>(p.x + (int64_t)(row0 + r) * p.ldx);
-      float amax = 0.0f;
-      for (int c = lane; c < p.K0 / 4; c += 32) {
-        const float4 f = __ldg(xr + c);
-        const float v[4] = {f.x, f.y, f.z, f.w};
-        amax = chain_max4(amax, v);
+  if (!rows_half) {
+    // ---- This warp's products in program order: units (sixteen channels and a share of K), each in items of up to
+    // kChainChunk pieces (16 bytes of two channels' weights per lane: 128 of K packed, 64 of K int8).  The next
+    // item's pieces are in nxt (zeros beyond its end).
+    int it_step = 0, it_u = warp;  // unit of the item
+    int u_left = 0;                // pieces from the item to the end of the unit
+    int u_a = 0, u_part = 0;       // this lane's first activation code (byte offset), first partial sum (index)
+    bool u_first = true, u_both = true;  // the unit's first item; its upper eight channels exist
+    const uint8_t *u_src0 = nullptr, *u_src1 = nullptr;
+    uint4 nxt[kChainChunk][2];
+    auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
+      while (it_step < n_steps && it_u >= steps[it_step].units) {
+        ++it_step;
+        it_u = warp;
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-      const ScaleCtx sc = make_scale_ctx_zeros(amax, p.in_qmax);
-      sx[t] = sc.s;
-      for (int c = lane; c < p.K0 / 8; c += 32) {
-        const float4 f0 = __ldg(xr + 2 * c), f1 = __ldg(xr + 2 * c + 1);
-        const float v0[4] = {f0.x, f0.y, f0.z, f0.w}, v1[4] = {f1.x, f1.y, f1.z, f1.w};
-        uint32_t w0 = chain_codes4(v0, sc, p.in_qmax, rounding), w1 = chain_codes4(v1, sc, p.in_qmax, rounding);
-        chain_order8((steps[0].flags & kChainPacked) != 0, w0, w1);
-        *reinterpret_cast<uint2*>(codes + r * pitch + 8 * c) = make_uint2(w0, w1);
+      u_left = 0;
+      if (it_step >= n_steps) return;
+      const ChainStep& st = steps[it_step];
+      const int k128 = st.K >> 7, per_cta = st.N >> 4;
+      const int shift = (st.flags & kChainPacked) ? 1 : 0;
+      int tile = it_u, kb0 = 0, kb1 = k128, ks = 0;  // tiles fastest, then shares of K
+      if (st.ks_n > 1) {
+        ks = (int)((uint32_t)it_u * st.inv_tiles >> 16);
+        tile = it_u - ks * st.tiles;
+        kb0 = (int)((uint32_t)(ks * k128) * st.inv_ks_lo >> 16);
+        kb1 = (int)((uint32_t)((ks + 1) * k128) * st.inv_ks_lo >> 16);
       }
-      for (int c = lane; c < h_cols / 4; c += 32)
-        *reinterpret_cast<float4*>(h + r * h_cols + 4 * c) = __ldg(xr + rank * (h_cols / 4) + c);
-    }
-  }
-  chain_cluster_sync();  // own codes ready; every CTA's barriers exist
+      const int c0 = tile * 16 + g;  // this lane's channels among the CTA's: c0 and c0 + 8
+      u_both = tile * 16 + 8 < per_cta;
+      const int c1 = u_both ? c0 + 8 : c0;
+      int n0 = rank * per_cta + c0, n1 = rank * per_cta + c1;
+      if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value channels, then the gate channels of the same output columns
+        const int cols = per_cta >> 1, gate_off = (st.N >> 1) - cols;
+        n0 = rank * cols + c0 + (c0 >= cols ? gate_off : 0);
+        n1 = rank * cols + c1 + (c1 >= cols ? gate_off : 0);
+      }
+      u_left = (kb1 - kb0) << (1 - shift);
+      const uint8_t* w = st.w + (kb0 << (7 - shift)) + kq * 16;
+      u_src0 = w + (int64_t)n0 * (st.K >> shift);
+      u_src1 = w + (int64_t)n1 * (st.K >> shift);
+      u_a = g * chain_pitch(st.K, shift != 0) + kb0 * 128 + kq * (16 << shift);
+      u_part = (ks * R + 2 * kq) * (per_cta + 4) + c0;
+      u_first = true;
+    };
+    auto load_piece = [&](int j) {
+      nxt[j][0] = nxt[j][1] = make_uint4(0u, 0u, 0u, 0u);
+      if (j < u_left) {
+        nxt[j][0] = __ldg(reinterpret_cast<const uint4*>(u_src0 + j * 64));
+        nxt[j][1] = __ldg(reinterpret_cast<const uint4*>(u_src1 + j * 64));
+      }
+    };
+    auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2 
+      if (threadIdx.x != kChainThreads - 1 || s >= n_steps || blockIdx.x >= kChainCtas) return;
+      const ChainStep& st = steps[s];
+      const bool glu = (st.flags & kChainActMask) >= AQT_ACT_GLU;
+      const int row_bytes = (st.flags & kChainPacked) ? st.K >> 1 : st.K, rows_here = st.N >> (glu ? 5 : 4);
+      const uint8_t* src = st.w + (int64_t)rank * rows_here * row_bytes;
+      for (int gate = 0; gate <= (glu ? 1 : 0); ++gate, src += (int64_t)(st.N >> 1) * row_bytes)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(rows_here * row_bytes)) : "memory");
+    };
 
-  // lane l sends its warp's row maxima to CTA l of the cluster
-  const uint32_t to_amax = chain_mapa(smem_u32(&amax_s[0][rank]), lane & 15), to_amax_bar = chain_mapa(smem_u32(&amax_bar[0]), lane & 15);
-  uint32_t exchange_parity = 0;  // of the exchange in progress (steps that are no side steps)
-  bool fresh = false;            // the codes of this step's input come from the exchange before it
-  for (int s = 0; s < n_steps; ++s) {
-    const ChainStep st = steps[s];
-    const bool packed = (st.flags & kChainPacked) != 0;
-    const uint32_t act = st.flags & kChainActMask;
-    const bool glu = act >= AQT_ACT_GLU;
-    const int per_cta = st.N >> 4, units = st.units, ks_n = st.ks_n;
-    const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
-    const int n_out = glu ? st.N >> 1 : st.N;
-    const int pitch = chain_pitch(st.K, packed), part_pitch = per_cta + 4;
-    const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
-    // two buffers of partial sums: after a side step the next products are written while these are read
-    int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
-    const int slot = s & 1;  // of sw_s / bias_s
-    if (fresh) mbar_wait(smem_u32(&codes_bar), exchange_parity ^ 1u, &abort_flag, t_start);
+    open_unit();
+#pragma unroll
+    for (int j = 0; j < kChainChunk; ++j) load_piece(j);
+    prefetch_slice(1);
+    chain_cluster_sync();  // the input's codes are ready; every CTA's barriers exist
 
-    // ---- integer products
-    bool used = false;
-    int acc[NT][SETS][4];
-    while (it_step == s) {
-      const int n = u_left, part0 = u_part;
-      const bool both = u_both;
-      const uint8_t* a0 = codes + u_a;
-      if (u_first) {
-#pragma unroll
-        for (int t = 0; t < NT; ++t)
-#pragma unroll
-          for (int j = 0; j < 4 * SETS; ++j) acc[t][j >> 2][j & 3] = 0;
+    uint32_t codes_parity = 0;  // of the codes that the next step with a new input reads
+    bool fresh = false;         // the codes of this step's input come from the exchange before it
+    for (int s = 0; s < n_steps; ++s) {
+      const ChainStep& st = steps[s];
+      const bool packed = (st.flags & kChainPacked) != 0;
+      const int units = st.units, pitch = chain_pitch(st.K, packed), part_pitch = (st.N >> 4) + 4;
+      int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
+      if (fresh) {
+        mbar_wait(smem_u32(&codes_bar), codes_parity, &abort_flag, t_start);
+        codes_parity ^= 1u;
       }
-      // the next item: loaded piece by piece below if it belongs to this step, else while the maxima are under way
-      bool more = true;
-      if (n > kChainChunk) {
-        u_left -= kChainChunk;
-        u_src0 += kChainChunk * 64;
-        u_src1 += kChainChunk * 64;
-        u_a += kChainChunk * (packed ? 128 : 64);
-        u_first = false;
-      } else {
-        it_u += kChainWarps;
-        more = it_u < units;
-        if (more) open_unit();
-        else used = true;
-      }
+      if (s >= 2) chain_bar_sync(3 + (s & 1));  // the sums of two steps ago have been read
+      bool used = false;
+      int acc[NT][SETS][4];
+      while (it_step == s) {
+        const int n = u_left, part0 = u_part;
+        const bool both = u_both;
+        const uint8_t* a0 = codes + u_a;
+        if (u_first) {
 #pragma unroll
-      for (int jj = 0; jj < kChainChunk; jj += 2) {
-        if (jj < n) {
+          for (int t = 0; t < NT; ++t)
 #pragma unroll
-          for (int j = jj; j < jj + 2; ++j) {
-            const uint4 w0 = nxt[j][0], w1 = nxt[j][1];
-            if (packed) {
-              // sixteen times the codes: the even ones' nibbles moved up, the odd ones' in place
-              constexpr uint32_t kHigh = 0xF0F0F0F0u;
-              const uint32_t e[8] = {(w0.x << 4) & kHigh, (w1.x << 4) & kHigh, (w0.y << 4) & kHigh, (w1.y << 4) & kHigh,
-                                     (w0.z << 4) & kHigh, (w1.z << 4) & kHigh, (w0.w << 4) & kHigh, (w1.w << 4) & kHigh};
-              const uint32_t o[8] = {w0.x & kHigh, w1.x & kHigh, w0.y & kHigh, w1.y & kHigh, w0.z & kHigh, w1.z & kHigh, w0.w & kHigh, w1.w & kHigh};
+            for (int j = 0; j < 4 * SETS; ++j) acc[t][j >> 2][j & 3] = 0;
+        }
+        // the next item: loaded piece by piece below if it belongs to this step, else while the maxima are under way
+        bool more = true;
+        if (n > kChainChunk) {
+          u_left -= kChainChunk;
+          u_src0 += kChainChunk * 64;
+          u_src1 += kChainChunk * 64;
+          u_a += kChainChunk * (packed ? 128 : 64);
+          u_first = false;
+        } else {
+          it_u += kChainWarps;
+          more = it_u < units;
+          if (more) open_unit();
+          else used = true;
+        }
 #pragma unroll
-              for (int t = 0; t < NT; ++t) {
-                const uint8_t* a = a0 + t * 8 * pitch + j * 128;
-                const uint4 x0 = *reinterpret_cast<const uint4*>(a), x1 = *reinterpret_cast<const uint4*>(a + 16);
-                mma_s8_16x8x32(acc[t][0], e[0], e[1], o[0], o[1], x0.x, x0.y);
-                mma_s8_16x8x32(acc[t][SETS - 1], e[2], e[3], o[2], o[3], x0.z, x0.w);
-                mma_s8_16x8x32(acc[t][0], e[4], e[5], o[4], o[5], x1.x, x1.y);
-                mma_s8_16x8x32(acc[t][SETS - 1], e[6], e[7], o[6], o[7], x1.z, x1.w);
-              }
-            } else {
+        for (int jj = 0; jj < kChainChunk; jj += 2) {
+          if (jj >= n && !more) break;
+          if (jj < n) {
 #pragma unroll
-              for (int t = 0; t < NT; ++t) {
-                const uint4 x0 = *reinterpret_cast<const uint4*>(a0 + t * 8 * pitch + j * 64);
-                mma_s8_16x8x32(acc[t][0], w0.x, w1.x, w0.y, w1.y, x0.x, x0.y);
-                mma_s8_16x8x32(acc[t][SETS - 1], w0.z, w1.z, w0.w, w1.w, x0.z, x0.w);
+            for (int j = jj; j < jj + 2; ++j) {
+              const uint4 w0 = nxt[j][0], w1 = nxt[j][1];
+              if (packed) {
+                // sixteen times the codes: the even ones' nibbles moved up, the odd ones' in place
+                constexpr uint32_t kHigh = 0xF0F0F0F0u;
+                const uint32_t e[8] = {(w0.x << 4) & kHigh, (w1.x << 4) & kHigh, (w0.y << 4) & kHigh, (w1.y << 4) & kHigh,
+                                       (w0.z << 4) & kHigh, (w1.z << 4) & kHigh, (w0.w << 4) & kHigh, (w1.w << 4) & kHigh};
+                const uint32_t o[8] = {w0.x & kHigh, w1.x & kHigh, w0.y & kHigh, w1.y & kHigh, w0.z & kHigh, w1.z & kHigh, w0.w & kHigh, w1.w & kHigh};
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                  const uint8_t* a = a0 + t * 8 * pitch + j * 128;
+                  const uint4 x0 = *reinterpret_cast<const uint4*>(a), x1 = *reinterpret_cast<const uint4*>(a + 16);
+                  mma_s8_16x8x32(acc[t][0], e[0], e[1], o[0], o[1], x0.x, x0.y);
+                  mma_s8_16x8x32(acc[t][SETS - 1], e[2], e[3], o[2], o[3], x0.z, x0.w);
+                  mma_s8_16x8x32(acc[t][0], e[4], e[5], o[4], o[5], x1.x, x1.y);
+                  mma_s8_16x8x32(acc[t][SETS - 1], e[6], e[7], o[6], o[7], x1.z, x1.w);
+                }
+              } else {
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                  const uint4 x0 = *reinterpret_cast<const uint4*>(a0 + t * 8 * pitch + j * 64);
+                  mma_s8_16x8x32(acc[t][0], w0.x, w1.x, w0.y, w1.y, x0.x, x0.y);
+                  mma_s8_16x8x32(acc[t][SETS - 1], w0.z, w1.z, w0.w, w1.w, x0.z, x0.w);
+                }
               }
             }
           }
-        }
-        if (more) {
-          load_piece(jj);
-          load_piece(jj + 1);
-        }
-      }
-      if (n <= kChainChunk) {  // the unit's last item
-        const int shift = packed ? 4 : 0;
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          int* dst = part + part0 + 8 * t * part_pitch;
-          if (SETS == 2) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[t][0][j] += acc[t][SETS - 1][j];
-          }
-          dst[0] = acc[t][0][0] >> shift;
-          dst[part_pitch] = acc[t][0][1] >> shift;
-          if (both) {
-            dst[8] = acc[t][0][2] >> shift;
-            dst[part_pitch + 8] = acc[t][0][3] >> shift;
+          if (more) {
+            load_piece(jj);
+            load_piece(jj + 1);
           }
         }
-      }
-      if (!more) break;
-    }
-    sw_s[slot][threadIdx.x] = wv;
-    bias_s[slot][threadIdx.x] = bv;
-    __syncthreads();
-    if (*(volatile int*)&abort_flag) break;  // a wait gave up: every thread leaves here
-
-    // ---- epilogue: warp w owns rows w, w + 8, ..., a lane four consecutive columns at a time
-    float v[NT][2][4];
-    if (threadIdx.x == 0 && !side && !last) mbar_arrive_expect_tx(smem_u32(&codes_bar), (uint32_t)(rows * n_out));
+        if (n <= kChainChunk) {  // the unit's last item
+          const int shift = packed ? 4 : 0;
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      float amax = 0.0f;
-      const int r = warp + 8 * t;
-      if (r >= rows) continue;
+          for (int t = 0; t < NT; ++t) {
+            int* dst = part + part0 + 8 * t * part_pitch;
+            if (SETS == 2) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int c = 4 * lane + 128 * j;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[t][j][e] = 0.0f;
-        if (c >= cols) continue;
-        auto dequant = [&](int cc, float (&z)[4]) {
-          const int* src = part + r * part_pitch + cc;
-          int4 a = *reinterpret_cast<const int4*>(src);
-          for (int ks = 1; ks < ks_n; ++ks) {
-            src += R * part_pitch;
-            const int4 q = *reinterpret_cast<const int4*>(src);
-            a.x += q.x; a.y += q.y; a.z += q.z; a.w += q.w;
+              for (int j = 0; j < 4; ++j) acc[t][0][j] += acc[t][SETS - 1][j];
+            }
+            dst[0] = acc[t][0][0] >> shift;
+            dst[part_pitch] = acc[t][0][1] >> shift;
+            if (both) {
+              dst[8] = acc[t][0][2] >> shift;
+              dst[part_pitch + 8] = acc[t][0][3] >> shift;
+            }
           }
-          const float4 w4 = *reinterpret_cast<const float4*>(&sw_s[slot][cc]);
-          const float4 b4 = *reinterpret_cast<const float4*>(&bias_s[slot][cc]);
-          z[0] = __fmaf_rn(__fmul_rn(__int2float_rn(a.x), sx[t]), w4.x, b4.x);
-          z[1] = __fmaf_rn(__fmul_rn(__int2float_rn(a.y), sx[t]), w4.y, b4.y);
-          z[2] = __fmaf_rn(__fmul_rn(__int2float_rn(a.z), sx[t]), w4.z, b4.z);
-          z[3] = __fmaf_rn(__fmul_rn(__int2float_rn(a.w), sx[t]), w4.w, b4.w);
-        };
-        float (&o)[4] = v[t][j];
-        dequant(c, o);
-        if (glu) {
-          float zg[4];
-          dequant(cols + c, zg);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(zg[e]));
         }
-        if (act == AQT_ACT_SWISH || act == AQT_ACT_GLU_SWISH) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(o[e]));
-        }
-        if (st.flags & kChainAdd) {
-          float4* hr = reinterpret_cast<float4*>(h + r * h_cols + c);
-          const float4 r4 = *hr;
-          o[0] = __fmaf_rn(st.rs, o[0], r4.x);
-          o[1] = __fmaf_rn(st.rs, o[1], r4.y);
-          o[2] = __fmaf_rn(st.rs, o[2], r4.z);
-          o[3] = __fmaf_rn(st.rs, o[3], r4.w);
-          *hr = make_float4(o[0], o[1], o[2], o[3]);
-        }
-        if (st.y != nullptr)
-          *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + rank * cols + c) = make_float4(o[0], o[1], o[2], o[3]);
-        amax = chain_max4(amax, o);
+        if (!more) break;
       }
-      if (side || last) continue;
-      const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative floats order like their bit patterns
-      if (lane == 0) mbar_arrive_expect_tx(smem_u32(&amax_bar[r]), kChainCtas * 4);
-      if (lane < kChainCtas) chain_st_async(to_amax + r * (kChainCtas * 4), m, to_amax_bar + r * 8);
-    }
-    if (last) break;
-
-    // ---- what the next step needs from memory, asked for while the maxima are under way
-    if (used) {
-      open_unit();
+      chain_bar_arrive(1 + (s & 1));
+      // the next step's weights are asked for while the rows of this one are worked on
+      if (used) {
+        open_unit();
 #pragma unroll
-      for (int j = 0; j < kChainChunk; ++j) load_piece(j);
-    }
-    fresh = !side;
-    if (side) {
-      load_scales(s + 1, wv, bv);
+        for (int j = 0; j < kChainChunk; ++j) load_piece(j);
+      }
       prefetch_slice(s + 2);
-      continue;
+      fresh = (st.flags & kChainSide) == 0;
     }
+  } else {
+    auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
+      wv = bv = 0.0f;
+      if (s >= n_steps) return;
+      const ChainStep& st = steps[s];
+      const int per_cta = st.N >> 4, c = threadIdx.x;
+      if (c - lane >= per_cta || c >= per_cta) return;
+      int n = rank * per_cta + c;
+      if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
+        const int cols = per_cta >> 1, gate = c >= cols ? 1 : 0;
+        n = gate * (st.N >> 1) + rank * cols + c - gate * cols;
+      }
+      wv = __ldg(st.s_w + n);
+      if (st.bias != nullptr) bv = __ldg(st.bias + n);
+    };
+    float wv, bv;  // scale and bias of this thread's channel of the next step, on their way to sw_s / bias_s
+    load_scales(0, wv, bv);
 
-    // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
-    // CTA has finished its products, so nobody reads the old codes any more.
-    const int qmax = (st.flags & kChainOut4) ? 7 : 127;
-    const bool next_packed = (steps[s + 1].flags & kChainPacked) != 0;
-    const int out_pitch = chain_pitch(n_out, next_packed);
+    // ---- the input: every CTA quantizes all rows for itself and keeps its columns of the residual stream
+    float sx[NT];  // input scales of this warp's rows (warp, warp + 8, ...)
+    {
+      const int pitch = chain_pitch(p.K0, (steps[0].flags & kChainPacked) != 0);
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int r = warp + 8 * t;
-      if (r >= rows) continue;
-      mbar_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
-      const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
-      const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(m), qmax);
-      sx[t] = sc.s;
-      uint32_t word[2] = {0u, 0u};
+      for (int t = 0; t < NT; ++t) {
+        const int r = warp + 8 * t;
+        sx[t] = 0.0f;
+        if (r >= rows) continue;
+        const float4* xr = reinterpret_cast<const float4*>(p.x + (int64_t)(row0 + r) * p.ldx);
+        float amax = 0.0f;
+        for (int c = lane; c < p.K0 / 4; c += 32) {
+          const float4 f = __ldg(xr + c);
+          const float v[4] = {f.x, f.y, f.z, f.w};
+          amax = chain_max4(amax, v);
+        }
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (4 * lane + 128 * j >= cols) continue;
-        word[j] = chain_codes4(v[t][j], sc, qmax, rounding);
-      }
-      // to all sixteen CTAs, eight codes per lane and store: `span` lanes (a power of two) cover the row's share,
-      // so a store instruction is 32 / span runs of consecutive bytes (the interconnect is paid per run: 250 clocks
-      // for a store scattered over sixteen CTAs)
-      const int span_bits = cols <= 16 ? 1 : 32 - __clz((cols >> 3) - 1), span = 1 << span_bits, i = lane & (span - 1);
-      uint32_t w0, w1;
-      if (cols <= 128) {
-        w0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31);
-        w1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
-      } else {  // columns from 128 on sit in the lanes' second word
-        const uint32_t x0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31), x1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
-        const uint32_t y0 = __shfl_sync(0xffffffffu, word[1], (2 * i) & 31), y1 = __shfl_sync(0xffffffffu, word[1], (2 * i + 1) & 31);
-        w0 = i < 16 ? x0 : y0;
-        w1 = i < 16 ? x1 : y1;
-      }
-      chain_order8(next_packed, w0, w1);
-      const uint32_t dst = smem_u32(codes) + (uint32_t)(r * out_pitch + rank * cols + 8 * i);
-      const uint32_t bar_off = smem_u32(&codes_bar) - dst;  // the same distance in every CTA's window
-      for (int to = lane >> span_bits; to < kChainCtas; to += 32 >> span_bits) {
-        const uint32_t remote = chain_mapa(dst, (uint32_t)(rank + to) & (kChainCtas - 1));
-        if (8 * i < cols) chain_st_async_v2(remote, w0, w1, remote + bar_off);
+        for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
+        const ScaleCtx sc = make_scale_ctx_zeros(amax, p.in_qmax);
+        sx[t] = sc.s;
+        for (int c = lane; c < p.K0 / 8; c += 32) {
+          const float4 f0 = __ldg(xr + 2 * c), f1 = __ldg(xr + 2 * c + 1);
+          const float v0[4] = {f0.x, f0.y, f0.z, f0.w}, v1[4] = {f1.x, f1.y, f1.z, f1.w};
+          uint32_t w0 = chain_codes4(v0, sc, p.in_qmax, rounding), w1 = chain_codes4(v1, sc, p.in_qmax, rounding);
+          chain_order8((steps[0].flags & kChainPacked) != 0, w0, w1);
+          *reinterpret_cast<uint2*>(codes + r * pitch + 8 * c) = make_uint2(w0, w1);
+        }
+        for (int c = lane; c < h_cols / 4; c += 32)
+          *reinterpret_cast<float4*>(h + r * h_cols + 4 * c) = __ldg(xr + rank * (h_cols / 4) + c);
       }
     }
-    load_scales(s + 1, wv, bv);
-    prefetch_slice(s + 2);
-    exchange_parity ^= 1u;
+    chain_cluster_sync();  // own codes ready; every CTA's barriers exist
+
+    // lane l sends its warp's row maxima to CTA l of the cluster
+    const uint32_t to_amax = chain_mapa(smem_u32(&amax_s[0][rank]), lane & 15), to_amax_bar = chain_mapa(smem_u32(&amax_bar[0]), lane & 15);
+    // the CTAs' windows of the cluster's shared memory lie at equal distances
+    const uint32_t codes_first = chain_mapa(smem_u32(codes), 0), codes_bar_first = chain_mapa(smem_u32(&codes_bar), 0);
+    const uint32_t window = chain_mapa(smem_u32(codes), 1) - codes_first;
+    uint32_t exchange_parity = 0;  // of the exchange in progress (steps that are no side steps)
+    for (int s = 0; s < n_steps; ++s) {
+      const ChainStep st = steps[s];
+      const uint32_t act = st.flags & kChainActMask;
+      const bool glu = act >= AQT_ACT_GLU;
+      const int per_cta = st.N >> 4, ks_n = st.ks_n;
+      const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
+      const int n_out = glu ? st.N >> 1 : st.N;
+      const int part_pitch = per_cta + 4;
+      const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
+      const int slot = s & 1;  // of the partial sums and of sw_s / bias_s
+      const int* part = reinterpret_cast<const int*>(chain_smem + p.code_bytes + slot * p.part_bytes);
+      sw_s[slot][threadIdx.x] = wv;
+      bias_s[slot][threadIdx.x] = bv;
+      chain_bar_sync(1 + slot);
+
+      // ---- epilogue: warp w owns rows w, w + 8, ..., a lane four consecutive columns at a time
+      float v[NT][2][4];
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        float amax = 0.0f;
+        const int r = warp + 8 * t;
+        if (r >= rows) continue;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int c = 4 * lane + 128 * j;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[t][j][e] = 0.0f;
+          if (j > 0 && __builtin_expect(cols <= 128, 1)) break;
+          if (c >= cols) continue;
+          auto dequant = [&](int cc, float (&z)[4]) {
+            const int* src = part + r * part_pitch + cc;
+            int4 a = *reinterpret_cast<const int4*>(src);
+#pragma unroll 1
+            for (int ks = 1; ks < ks_n; ks += 3) {  // three loads at a time, not one behind the other
+              int4 q[3];
+#pragma unroll
+              for (int i = 0; i < 3; ++i) {
+                q[i] = make_int4(0, 0, 0, 0);
+                src += R * part_pitch;
+                if (ks + i < ks_n) q[i] = *reinterpret_cast<const int4*>(src);
+              }
+              a.x += q[0].x + q[1].x + q[2].x;
+              a.y += q[0].y + q[1].y + q[2].y;
+              a.z += q[0].z + q[1].z + q[2].z;
+              a.w += q[0].w + q[1].w + q[2].w;
+            }
+            const float4 w4 = *reinterpret_cast<const float4*>(&sw_s[slot][cc]);
+            const float4 b4 = *reinterpret_cast<const float4*>(&bias_s[slot][cc]);
+            z[0] = __fmaf_rn(__fmul_rn(__int2float_rn(a.x), sx[t]), w4.x, b4.x);
+            z[1] = __fmaf_rn(__fmul_rn(__int2float_rn(a.y), sx[t]), w4.y, b4.y);
+            z[2] = __fmaf_rn(__fmul_rn(__int2float_rn(a.z), sx[t]), w4.z, b4.z);
+            z[3] = __fmaf_rn(__fmul_rn(__int2float_rn(a.w), sx[t]), w4.w, b4.w);
+          };
+          float (&o)[4] = v[t][j];
+          dequant(c, o);
+          if (glu) {
+            float zg[4];
+            dequant(cols + c, zg);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(zg[e]));
+          }
+          if (act == AQT_ACT_SWISH || act == AQT_ACT_GLU_SWISH) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = __fmul_rn(o[e], small_sigmoid(o[e]));
+          }
+          if (st.flags & kChainAdd) {
+            const float4 r4 = *reinterpret_cast<const float4*>(h + r * h_cols + c);
+            o[0] = __fmaf_rn(st.rs, o[0], r4.x);
+            o[1] = __fmaf_rn(st.rs, o[1], r4.y);
+            o[2] = __fmaf_rn(st.rs, o[2], r4.z);
+            o[3] = __fmaf_rn(st.rs, o[3], r4.w);
+          }
+          amax = chain_max4(amax, o);
+        }
+        if (side || last) continue;
+        const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative floats order like their bit patterns
+        if (lane < kChainCtas) chain_st_async(to_amax + r * (kChainCtas * 4), m, to_amax_bar + r * 8);
+        if (lane == 0) mbar_arrive_expect_tx(smem_u32(&amax_bar[r]), kChainCtas * 4);
+      }
+      // what else is to be done, while the maxima are under way
+      if (threadIdx.x == 0 && !side && !last) mbar_arrive_expect_tx(smem_u32(&codes_bar), (uint32_t)(rows * n_out));
+      if ((st.flags & kChainAdd) || st.y != nullptr) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int r = warp + 8 * t, c = 4 * lane + 128 * j;
+            if (r >= rows || c >= cols) continue;
+            const float4 o = make_float4(v[t][j][0], v[t][j][1], v[t][j][2], v[t][j][3]);
+            if (st.flags & kChainAdd) *reinterpret_cast<float4*>(h + r * h_cols + c) = o;
+            if (st.y != nullptr) *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + rank * cols + c) = o;
+          }
+      }
+      if (s + 2 < n_steps) chain_bar_arrive(3 + slot);
+      if (last) break;
+
+      load_scales(s + 1, wv, bv);  // while the maxima are under way
+      if (side) continue;
+
+      // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
+      // CTA has finished its products, so nobody reads the old codes any more.
+      const int qmax = (st.flags & kChainOut4) ? 7 : 127;
+      const bool next_packed = (steps[s + 1].flags & kChainPacked) != 0;
+      const int out_pitch = chain_pitch(n_out, next_packed);
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const int r = warp + 8 * t;
+        if (r >= rows) continue;
+        mbar_wait(smem_u32(&amax_bar[r]), exchange_parity, &abort_flag, t_start);
+        const uint32_t m = __reduce_max_sync(0xffffffffu, amax_s[r][lane & (kChainCtas - 1)]);
+        const ScaleCtx sc = make_scale_ctx_zeros(__uint_as_float(m), qmax);
+        sx[t] = sc.s;
+        uint32_t word[2] = {0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if (j > 0 && __builtin_expect(cols <= 128, 1)) break;
+          if (4 * lane + 128 * j >= cols) continue;
+          word[j] = chain_codes4(v[t][j], sc, qmax, rounding);
+        }
+        // to all sixteen CTAs, eight codes per lane and store: `span` lanes (a power of two) cover the row's share,
+        // so a store instruction is 32 / span runs of consecutive bytes (the interconnect is paid per run: 250 clocks
+        // for a store scattered over sixteen CTAs)
+        const int span_bits = cols <= 16 ? 1 : 32 - __clz((cols >> 3) - 1), span = 1 << span_bits, i = lane & (span - 1);
+        uint32_t w0, w1;
+        if (__builtin_expect(cols <= 128, 1)) {
+          w0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31);
+          w1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
+        } else {  // columns from 128 on sit in the lanes' second word
+          const uint32_t x0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31), x1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
+          const uint32_t y0 = __shfl_sync(0xffffffffu, word[1], (2 * i) & 31), y1 = __shfl_sync(0xffffffffu, word[1], (2 * i + 1) & 31);
+          w0 = i < 16 ? x0 : y0;
+          w1 = i < 16 ? x1 : y1;
+        }
+        chain_order8(next_packed, w0, w1);
+        const uint32_t dst = codes_first + (uint32_t)(r * out_pitch + rank * cols + 8 * i);
+        for (int to = lane >> span_bits; to < kChainCtas; to += 32 >> span_bits) {
+          const uint32_t at = ((uint32_t)(rank + to) & (kChainCtas - 1)) * window;
+          if (8 * i < cols) chain_st_async_v2(dst + at, w0, w1, codes_bar_first + at);
+        }
+      }
+      exchange_parity ^= 1u;
+    }
   }
   grid_dependents_launch();
   chain_cluster_sync();  // no CTA leaves while its shared memory may still be written
