@@ -141,18 +141,9 @@ __device__ __forceinline__ void chain_order8(bool packed, uint32_t& w0, uint32_t
   w1 = packed ? odd : w1;
 }
 
-// Four codes of a row as one word.  The general sequence stands apart: every warp runs through the code of a step once, and
-// pays for each instruction line that it fetches.
-__device__ __noinline__ uint32_t chain_codes4_general(float v0, float v1, float v2, float v3, float s, int qmax, int rounding) {
-  const ScaleCtx c = {s, 0.0f, false};
-  if (rounding == AQT_ROUND_HALF_UP_FLOOR)
-    return pack4_i8(quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v0, c, qmax), quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v1, c, qmax),
-                    quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v2, c, qmax), quantize_elem<AQT_ROUND_HALF_UP_FLOOR>(v3, c, qmax));
-  return pack4_i8(quantize_elem<AQT_ROUND_NEAREST_EVEN>(v0, c, qmax), quantize_elem<AQT_ROUND_NEAREST_EVEN>(v1, c, qmax),
-                  quantize_elem<AQT_ROUND_NEAREST_EVEN>(v2, c, qmax), quantize_elem<AQT_ROUND_NEAREST_EVEN>(v3, c, qmax));
-}
+// Four codes of a row as one word.
 __device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax, int rounding) {
-  if (__builtin_expect(!c.fast, 0)) return chain_codes4_general(v[0], v[1], v[2], v[3], c.s, qmax, rounding);
+  if (__builtin_expect(!c.fast, 0)) return codes4_general(v[0], v[1], v[2], v[3], c.s, qmax, rounding);
   const bool half_up = rounding == AQT_ROUND_HALF_UP_FLOOR;
   int q[4];
 #pragma unroll

@@ -17,11 +17,13 @@ __device__ __forceinline__ uint32_t pack4_i8(int a, int b, int c, int d) {
   const uint32_t hi = __byte_perm((uint32_t)c, (uint32_t)d, 0x0040);  // c.b0, d.b0
   return __byte_perm(lo, hi, 0x5410);
 }
-__device__ __forceinline__ uint32_t pack4_i4(int a, int b, int c, int d) {
-  const uint32_t x = pack4_i8(a, b, c, d) & 0x0F0F0F0Fu;
+// Four codes in a word as nibbles.
+__device__ __forceinline__ uint32_t nibbles4(uint32_t w) {
+  const uint32_t x = w & 0x0F0F0F0Fu;
   const uint32_t y = x | (x >> 4);         // byte 0 = n0 | n1 << 4, byte 2 = n2 | n3 << 4
   return __byte_perm(y, 0u, 0x4420) & 0xFFFFu;
 }
+__device__ __forceinline__ uint32_t pack4_i4(int a, int b, int c, int d) { return nibbles4(pack4_i8(a, b, c, d)); }
 
 // Four elements of a row whose scale constants are known, fast path of quantize_elem: the
 // correctly rounded quotient by one multiply and two FMAs, then one conversion.  No clip: with
@@ -85,24 +87,15 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_rows_reg_kernel(
   for (int i = 0; i < kQuantMaxVec; ++i) {
     const int idx = t + i * G;
     if (idx < nvec) {
-      int a, b, cc, d;
-      if (c.fast) {  // uniform over the row
-        a = quantize_fast<ROUNDING>(v[i].x, c.s, c.r);
-        b = quantize_fast<ROUNDING>(v[i].y, c.s, c.r);
-        cc = quantize_fast<ROUNDING>(v[i].z, c.s, c.r);
-        d = quantize_fast<ROUNDING>(v[i].w, c.s, c.r);
-      } else {
-        a = quantize_elem<ROUNDING>(v[i].x, c, qmax);
-        b = quantize_elem<ROUNDING>(v[i].y, c, qmax);
-        cc = quantize_elem<ROUNDING>(v[i].z, c, qmax);
-        d = quantize_elem<ROUNDING>(v[i].w, c, qmax);
-      }
+      uint32_t w;  // four codes
+      if (__builtin_expect(c.fast, 1))  // uniform over the row
+        w = pack4_i8(quantize_fast<ROUNDING>(v[i].x, c.s, c.r), quantize_fast<ROUNDING>(v[i].y, c.s, c.r), quantize_fast<ROUNDING>(v[i].z, c.s, c.r),
+                     quantize_fast<ROUNDING>(v[i].w, c.s, c.r));
+      else
+        w = codes4_general(v[i].x, v[i].y, v[i].z, v[i].w, c.s, qmax, ROUNDING);
       // one output word per float4: 2 bytes of nibbles or 4 bytes of int8 codes
-      if (PACK) {
-        reinterpret_cast<uint16_t*>(q_out)[row * (int64_t)nvec + idx] = (uint16_t)pack4_i4(a, b, cc, d);
-      } else {
-        reinterpret_cast<uint32_t*>(q_out)[row * (int64_t)nvec + idx] = pack4_i8(a, b, cc, d);
-      }
+      if (PACK) reinterpret_cast<uint16_t*>(q_out)[row * (int64_t)nvec + idx] = (uint16_t)nibbles4(w);
+      else reinterpret_cast<uint32_t*>(q_out)[row * (int64_t)nvec + idx] = w;
     }
   }
 }
@@ -345,24 +338,25 @@ __global__ void __launch_bounds__(kQuantThreads) absmax_tensor_vec_kernel(const 
 }
 
 // BESIDE: every block has one share of the tensor, and may start while pass 1 runs.
-template <int ROUNDING, bool PACK, bool BESIDE>
+template <int ROUNDING, bool PACK, bool BESIDE, int VEC>
 __global__ void __launch_bounds__(kQuantThreads) quantize_tensor_vec_kernel(const float* __restrict__ x, int64_t n4, int64_t nvec, int64_t ld4,
                                                                             int qmax, const float* __restrict__ partial, int partials,
                                                                             float* __restrict__ scale_out, void* __restrict__ q_out) {
   __shared__ float warp_max[kQuantThreads / 32];
   // The kernel ahead is pass 1 of the same call: it writes none of x, and this one can only have started when whatever
   // wrote x was complete.  So its loads need not wait for pass 1.
-  float4 v[kTensorVec];
+  float4 v[VEC];
   const auto load = [&](int64_t i0) {
 #pragma unroll
-    for (int j = 0; j < kTensorVec; ++j) {
+    for (int j = 0; j < VEC; ++j) {
       const int64_t i = i0 + j * kQuantThreads;
       if (i < n4) v[j] = __ldg(tensor_vec(x, i, nvec, ld4));
     }
   };
-  const int64_t first = (int64_t)blockIdx.x * kQuantThreads * kTensorVec + threadIdx.x;
+  const int64_t first = (int64_t)blockIdx.x * kQuantThreads * VEC + threadIdx.x;
   if (BESIDE) load(first);
   grid_dependency_wait();
+  grid_dependents_launch();  // (the next kernel waits for the end of this one; what it can do ahead of that it may begin)
   ScaleCtx c;
   if (partial != nullptr) {
     float amax = 0.0f;
@@ -381,30 +375,23 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_tensor_vec_kernel(cons
     c.fast = normal || c.s == 0.0f;
     c.r = normal ? __frcp_rn(c.s) : 0.0f;
   }
-  const int64_t step = (int64_t)gridDim.x * kQuantThreads * kTensorVec;
+  const int64_t step = (int64_t)gridDim.x * kQuantThreads * VEC;
   for (int64_t i0 = first; i0 < n4; i0 += step) {
     if (!BESIDE) load(i0);
 #pragma unroll
-    for (int j = 0; j < kTensorVec; ++j) {
+    for (int j = 0; j < VEC; ++j) {
       const int64_t i = i0 + j * kQuantThreads;
       if (i >= n4) break;
-      int a, b, cc, d;
-      if (c.fast) {
-        a = quantize_fast<ROUNDING>(v[j].x, c.s, c.r);
-        b = quantize_fast<ROUNDING>(v[j].y, c.s, c.r);
-        cc = quantize_fast<ROUNDING>(v[j].z, c.s, c.r);
-        d = quantize_fast<ROUNDING>(v[j].w, c.s, c.r);
-      } else {
-        a = quantize_elem<ROUNDING>(v[j].x, c, qmax);
-        b = quantize_elem<ROUNDING>(v[j].y, c, qmax);
-        cc = quantize_elem<ROUNDING>(v[j].z, c, qmax);
-        d = quantize_elem<ROUNDING>(v[j].w, c, qmax);
-      }
-      if (PACK) reinterpret_cast<uint16_t*>(q_out)[i] = (uint16_t)pack4_i4(a, b, cc, d);
-      else reinterpret_cast<uint32_t*>(q_out)[i] = pack4_i8(a, b, cc, d);
+      uint32_t w;
+      if (__builtin_expect(c.fast, 1))
+        w = pack4_i8(quantize_fast<ROUNDING>(v[j].x, c.s, c.r), quantize_fast<ROUNDING>(v[j].y, c.s, c.r), quantize_fast<ROUNDING>(v[j].z, c.s, c.r),
+                     quantize_fast<ROUNDING>(v[j].w, c.s, c.r));
+      else
+        w = codes4_general(v[j].x, v[j].y, v[j].z, v[j].w, c.s, qmax, ROUNDING);
+      if (PACK) reinterpret_cast<uint16_t*>(q_out)[i] = (uint16_t)nibbles4(w);
+      else reinterpret_cast<uint32_t*>(q_out)[i] = w;
     }
   }
-  grid_dependents_launch();
 }
 
 static bool tensor_vec_ok(const float* x, int64_t cols, int64_t ld, const void* q_out) {
@@ -419,21 +406,23 @@ static int launch_quantize_tensor_vec(const float* x, int64_t rows, int64_t cols
   int64_t blocks = want < kAbsmaxBlocks ? want : kAbsmaxBlocks;
   if (partial != nullptr && blocks > max_partials) blocks = max_partials;
   // Where pass 2's blocks fit beside those of pass 1, each with one share of the tensor, they wait for the scale with that share
-  // in registers (graph replay of the layer: 300 x 128 9.2 -> 7.2 us, 641 x 288 10.8 -> 8.7, 3000 x 256 10.8 -> 9.7; the line is
-  // where the blocks that wait would keep others of either pass from the SMs: 7411 x 512, 927 blocks, 17.2 -> 17.5; 65 536 x
-  // 512 100 -> 113).
+  // in registers: four float4s a thread, or eight (graph replay of the layer: 300 x 128 9.2 -> 7.2 us, 641 x 288 10.8 -> 8.7,
+  // 3000 x 256 10.8 -> 9.7; eight: 7411 x 512 19.7 -> 18.6, 2000 x 2048 17.9 -> 17.0).  Beyond, the blocks that wait would keep
+  // others of either pass from the SMs (65 536 x 512 100 -> 113).
   const int64_t sms = sm_count() > 0 ? sm_count() : kDefaultSms;
-  const int64_t grid = want < sms * 8 ? want : sms * 8;
-  const bool beside = want <= sms * 4;
+  const int64_t want8 = ceil_div(n4, kQuantThreads * 2 * kTensorVec);
+  const bool beside = want <= sms * 4, beside8 = !beside && want8 <= sms * 4;
+  const int64_t grid = beside8 ? want8 : (want < sms * 8 ? want : sms * 8);
   int rc;
   if (partial == nullptr) {
     rc = launch_pdl(clear_scale_kernel, dim3(1, 1, 1), dim3(1, 1, 1), 0, st, 1, scale_out);
     if (rc != AQT_OK) return rc;
   }
   rc = launch_pdl(absmax_tensor_vec_kernel, dim3((unsigned)blocks, 1, 1), dim3(kQuantThreads, 1, 1), 0, st, 1, x, n4, cols / 4, ld / 4, qmax,
-                  partial, scale_out, beside);
+                  partial, scale_out, beside || beside8);
   if (rc != AQT_OK) return rc;
-  auto kernel = beside ? quantize_tensor_vec_kernel<ROUNDING, PACK, true> : quantize_tensor_vec_kernel<ROUNDING, PACK, false>;
+  auto kernel = beside8 ? quantize_tensor_vec_kernel<ROUNDING, PACK, true, 2 * kTensorVec>
+                        : (beside ? quantize_tensor_vec_kernel<ROUNDING, PACK, true, kTensorVec> : quantize_tensor_vec_kernel<ROUNDING, PACK, false, kTensorVec>);
   return launch_pdl(kernel, dim3((unsigned)grid, 1, 1), dim3(kQuantThreads, 1, 1), 0, st, 1, x, n4,
                     cols / 4, ld / 4, qmax, (const float*)partial, (int)blocks, scale_out, q_out);
 }

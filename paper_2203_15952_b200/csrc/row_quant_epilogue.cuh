@@ -100,7 +100,7 @@ __device__ __forceinline__ float numbers_max(float m, const uint32_t (&u)[NV]) {
 // NV (32 or 16) values of one row -> NV / 4 words of int8 codes (PACK: NV / 8 words of nibbles).
 template <int ROUNDING, bool PACK, int NV>
 __device__ __forceinline__ void codes_of(const uint32_t (&u)[NV], const ScaleCtx& c, int qmax, uint32_t (&w)[NV / 4]) {
-  if (c.fast) {
+  if (__builtin_expect(c.fast, 1)) {
     const float2 s_neg = make_float2(-c.s, -c.s), r2 = make_float2(c.r, c.r);
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j) {
@@ -111,10 +111,8 @@ __device__ __forceinline__ void codes_of(const uint32_t (&u)[NV], const ScaleCtx
   } else {
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j)
-      w[j] = low_bytes((uint32_t)quantize_elem<ROUNDING>(__uint_as_float(u[4 * j]), c, qmax),
-                       (uint32_t)quantize_elem<ROUNDING>(__uint_as_float(u[4 * j + 1]), c, qmax),
-                       (uint32_t)quantize_elem<ROUNDING>(__uint_as_float(u[4 * j + 2]), c, qmax),
-                       (uint32_t)quantize_elem<ROUNDING>(__uint_as_float(u[4 * j + 3]), c, qmax));
+      w[j] = codes4_general(__uint_as_float(u[4 * j]), __uint_as_float(u[4 * j + 1]), __uint_as_float(u[4 * j + 2]), __uint_as_float(u[4 * j + 3]), c.s,
+                            qmax, ROUNDING);
   }
   if (PACK) {
 #pragma unroll
