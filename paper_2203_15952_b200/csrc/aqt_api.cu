@@ -317,7 +317,9 @@ int qmatmul_i8a(const int8_t* a_codes, const float* s_x, int s_x_kind, const voi
   if (is_packed(bits_w)) {
     const int sms = sm_count();
     if (sms <= 0) return AQT_ERR_CUDA;
-    const int plan = forced_plan != kPlanNone ? forced_plan : plan_qgemm(GemmShape{M, N, K, act, 0, false}, sms);
+    GemmShape g = {M, N, K, act, 0, false, residual != nullptr};
+    g.packed = true;
+    const int plan = forced_plan != kPlanNone ? forced_plan : plan_qgemm(g, sms);
     const bool ws_plan = plan == kPlanWs128E16 || plan == kPlanWs128E8;
     if (ws_plan && K % 32 == 0) {  // the packed rows must keep the 16-byte pitch bulk copies need
       b_packed = true;

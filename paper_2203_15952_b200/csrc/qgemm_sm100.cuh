@@ -1294,6 +1294,7 @@ struct GemmShape {
   bool batched;  // stacked batches: streaming kernel, one CTA per tile
   bool residual = false;
   bool beside = false;  // float kind: the next launch runs beside this one (GemmParams::early_trigger)
+  bool packed = false;  // packed weights, which only the weight-stationary kernel expands
 };
 
 // True if the weight-stationary kernel takes this shape (and can therefore unpack 4-bit weights itself).
@@ -1349,8 +1350,15 @@ static int plan_qgemm_pairs(const GemmShape& g, int pairs, int64_t pair_tiles) {
 static int plan_qgemm(const GemmShape& g, int sms) {
   const bool glu = (g.act == AQT_ACT_GLU) || (g.act == AQT_ACT_GLU_SWISH);
   const bool f32 = g.kind == 1;
-  if (!g.batched && qgemm_uses_ws(g.N, g.K, sms)) return glu ? kPlanWs128E8 : kPlanWs128E16;  // a GLU tile has 64 output columns
   const int pairs = sms / 2;
+  if (!g.batched && qgemm_uses_ws(g.N, g.K, sms)) {
+    // With a residual, whose rows every tile waits for, the slab that a CTA loads first and its place in shared memory give
+    // nothing back: single-CTA tiles that stream both operands, and pairs of 128 columns from some 28 M outputs on (us,
+    // weight-stationary / streamed / pairs, inputs not in L2: 7411 x 512 -> 512 12.3 / 11.5 / 11.7, 25 600 rows 24.0 / 23.7 / 24.8,
+    // 65 536 rows 55.3 / 52.7 / 50.4, 65 536 x 512 -> 2048 206 / 188 / 176; without a residual the slab is the better use).
+    if (g.residual && !g.packed && !f32 && g.act == AQT_ACT_NONE) return g.M * g.N >= (28ll << 20) ? kPlanPair128S6E8 : kPlanStream128S4E16;
+    return glu ? kPlanWs128E8 : kPlanWs128E16;  // a GLU tile has 64 output columns
+  }
   const int64_t pair_tiles = ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256);  // 256 x 256 tiles
   if (!f32 && !g.batched) {
     const int plan = plan_qgemm_pairs(g, pairs, pair_tiles);
@@ -1522,7 +1530,8 @@ static int launch_qgemm(const int8_t* a, const void* b, bool b_packed, float* y,
                         int forced_plan = kPlanNone) {
   const int sms = sm_count();
   if (sms <= 0) return AQT_ERR_CUDA;
-  const GemmShape g = gemm_shape_of(p);
+  GemmShape g = gemm_shape_of(p);
+  g.packed = b_packed;
   int plan = forced_plan;
   if (plan != kPlanNone) {
     if (!gemm_plan_takes(plan, g, sms)) return AQT_ERR_UNSUPPORTED;
