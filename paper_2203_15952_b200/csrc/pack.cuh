@@ -28,6 +28,8 @@ __device__ __forceinline__ uint32_t pack_words(uint32_t w0, uint32_t w1) {
 // n_bytes packed bytes -> 2 * n_bytes codes.  vec path: 8 packed bytes per thread per step.
 __global__ void __launch_bounds__(256) unpack_int4_kernel(const uint8_t* __restrict__ packed, int64_t n_bytes,
                                                           int8_t* __restrict__ q, bool vec) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (vec) {
@@ -80,6 +82,8 @@ __global__ void __launch_bounds__(256) pack_int4_kernel(const int8_t* __restrict
 // of 4: dense int8, or nibble pairs if `packed`.  Four codes per thread and step.
 __global__ void __launch_bounds__(256) codes_to_float_kernel(const uint8_t* __restrict__ codes, bool packed, int64_t n,
                                                              float* __restrict__ out) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n >> 2); i += stride) {
     uint32_t w;
@@ -104,6 +108,8 @@ __global__ void __launch_bounds__(256) codes_to_float_kernel(const uint8_t* __re
 // sums x . w with about twenty-one significant bits per activation.  K % 4 == 0, ldx % 4 == 0.
 __global__ void __launch_bounds__(256) split_hi_lo_kernel(const float* __restrict__ x, int64_t ldx, int64_t M, int64_t K,
                                                           float* __restrict__ out) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int64_t k4 = K >> 2, total = M * k4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -127,6 +133,8 @@ __global__ void __launch_bounds__(256) split_hi_lo_kernel(const float* __restric
 // The weight codes as floats, each row written twice: out [rows, 2K] = [w | w].
 __global__ void __launch_bounds__(256) codes_to_float_twice_kernel(const uint8_t* __restrict__ codes, bool packed, int64_t rows,
                                                                    int64_t K, float* __restrict__ out) {
+  grid_dependency_wait();
+  grid_dependents_launch();
   const int64_t k4 = K >> 2, total = rows * k4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -156,23 +164,20 @@ static unsigned flat_grid(int64_t work_items) {
 
 static int launch_unpack_int4(const uint8_t* packed, int64_t n_bytes, int8_t* q, cudaStream_t st) {
   const bool vec = is_aligned(packed, 8) && is_aligned(q, 16);
-  unpack_int4_kernel<<<flat_grid(vec ? n_bytes / 8 + 8 : n_bytes), 256, 0, st>>>(packed, n_bytes, q, vec);
-  return AQT_LAUNCH_STATUS();
+  return launch_pdl(unpack_int4_kernel, dim3(flat_grid(vec ? n_bytes / 8 + 8 : n_bytes), 1, 1), dim3(256, 1, 1), 0, st, 1, packed, n_bytes, q, vec);
 }
 
 // codes: int8 [n] or packed nibbles [n / 2], 4-byte (2-byte if packed) aligned; out: float [n], 16-byte aligned; n % 4 == 0.
 static int launch_codes_to_float(const void* codes, bool packed, int64_t n, float* out, cudaStream_t st) {
-  codes_to_float_kernel<<<flat_grid(n / 4), 256, 0, st>>>(reinterpret_cast<const uint8_t*>(codes), packed, n, out);
-  return AQT_LAUNCH_STATUS();
+  return launch_pdl(codes_to_float_kernel, dim3(flat_grid(n / 4), 1, 1), dim3(256, 1, 1), 0, st, 1, reinterpret_cast<const uint8_t*>(codes), packed, n, out);
 }
 
 static int launch_split_hi_lo(const float* x, int64_t ldx, int64_t M, int64_t K, float* out, cudaStream_t st) {
-  split_hi_lo_kernel<<<flat_grid(M * K / 4), 256, 0, st>>>(x, ldx, M, K, out);
-  return AQT_LAUNCH_STATUS();
+  return launch_pdl(split_hi_lo_kernel, dim3(flat_grid(M * K / 4), 1, 1), dim3(256, 1, 1), 0, st, 1, x, ldx, M, K, out);
 }
 static int launch_codes_to_float_twice(const void* codes, bool packed, int64_t rows, int64_t K, float* out, cudaStream_t st) {
-  codes_to_float_twice_kernel<<<flat_grid(rows * K / 4), 256, 0, st>>>(reinterpret_cast<const uint8_t*>(codes), packed, rows, K, out);
-  return AQT_LAUNCH_STATUS();
+  return launch_pdl(codes_to_float_twice_kernel, dim3(flat_grid(rows * K / 4), 1, 1), dim3(256, 1, 1), 0, st, 1, reinterpret_cast<const uint8_t*>(codes), packed,
+                    rows, K, out);
 }
 
 static int launch_pack_int4(const int8_t* q, int64_t n_bytes, uint8_t* packed, cudaStream_t st) {
