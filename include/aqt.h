@@ -343,6 +343,10 @@ int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer*
  * therefore within 2^-10 * s_w[n] * sum_k |x[m][k] * wq[n][k]| (plus binary32 summation error) of
  * the exact value of the formula, and equals it bit for bit when every x is a tf32 value and no
  * partial sum needs more than 24 bits.
+ * Larger calls (256 <= K <= 1024, K % 8 == 0, N >= 1024, M >= 1024, M * N * K >= 1.3e9) take the same eleven
+ * significant bits, rounded to nearest, as binary16 operands at twice the rate: each row is scaled by a power of two
+ * (undone exactly afterwards), and blocks of 256 rows with a value that is not finite, smaller than 2^-28 of its row's
+ * largest and not zero, or in a row whose largest is below 2^-100 or above 2^100, keep the tf32 operands.
  * precision AQT_FLOAT_TF32: as just described.  AQT_FLOAT_TF32X2: every activation is split
  *           exactly into hi (its tf32 part) + lo, and one matmul over [hi | lo] against the
  *           weights repeated sums both terms: the operand error drops from 2^-10 to 2^-20 of
@@ -351,7 +355,8 @@ int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer*
  * wq, s_w, bias, residual, ldr, residual_scale, act, y, ldy: as for aqt_qmatmul.
  * workspace at least aqt_workspace_bytes(AQT_OP_LINEAR_WEIGHT_ONLY or .._X2, M, N, K, 0, bits_w)
  *           bytes, 256-byte aligned: the weight codes as floats (4 * N * K bytes; X2: 8 * N * K
- *           and the split activations, 8 * M * K), rewritten every call.
+ *           and the split activations, 8 * M * K; calls with binary16 operands 2 * N * K + 2 * M * K + 4 * M
+ *           more, and with the former size alone they take the tf32 operands), rewritten every call.
  * Limits: K % 4 == 0, ldx % 4 == 0, N % 4 == 0 (N % 8 == 0 for GLU), ldy % 4 == 0, ldr % 4 == 0;
  * x, wq, y, residual, s_w, bias 16-byte aligned.  M == 0 or N == 0 is a no-op.
  */

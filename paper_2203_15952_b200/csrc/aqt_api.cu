@@ -51,6 +51,19 @@ size_t ws_weight_only(int64_t M, int64_t N, int64_t K, int precision) {
   return round_up((size_t)N * (size_t)K * 4, 256);
 }
 
+// Half kind of the one-term form: [weights as floats | weights as halves | rows as halves | inverse row scales].
+struct HalfLayout {
+  size_t w_h, x_h, inv, total;
+};
+HalfLayout half_layout(int64_t M, int64_t N, int64_t K) {
+  HalfLayout L;
+  L.w_h = ws_weight_only(0, N, K, AQT_FLOAT_TF32);
+  L.x_h = L.w_h + round_up((size_t)N * (size_t)K * 2, 256);
+  L.inv = L.x_h + round_up((size_t)M * (size_t)K * 2, 256);
+  L.total = L.inv + round_up((size_t)M * 4, 256);
+  return L;
+}
+
 // Backward workspace of the tf32 form: [column-sum partials | s_w-scaled W^T [K, N] | dy^T | s_x-scaled xq^T | dw partials].
 // The weight gradient is an [N, K] output with a contraction of M: few, very deep tiles.  Its
 // contraction is therefore cut into `batches` chunks of `chunk` rows (a multiple of 32), each
@@ -161,6 +174,16 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
   p.small_acc = 0;
   p.early_trigger = early_trigger ? 1 : 0;
   return launch_qgemm(reinterpret_cast<const int8_t*>(a), b, false, y, ldy, p, st);
+}
+
+// True if the one-term weight-only layer's matmul runs on binary16 operands, twice the rate and half the bytes of tf32 ones for a
+// pass that scales and writes the rows first (6 bytes an element).  CTA pairs on 256 x 256 tiles; us in a replayed graph, tf32 /
+// binary16, both with their passes: 12 800 x 512 -> 2048 Swish 51.7 / 45.2, 5000 x 768 -> 3072 47.1 / 37.3, 30 000 x 1024 -> 2048
+// gated 162 / 130, 30 000 x 1024 -> 1024 98.4 / 95.7.  Not where the pass is much of the call (30 000 x 512 -> 512 39.7 / 41.0, 30 000 x
+// 2048 -> 512 98.6 / 117, 30 000 x 4096 -> 1024 321 / 348), the epilogue most of a tile (12 800 x 128 -> 1280 21.1 / 25.4), or the
+// work small (2000 x 512 -> 1024 11.2 / 12.0, 1024 x 512 -> 2048 12.5 / 13.9; but 3000 x 512 -> 1024 14.6 / 13.5).
+bool half_kind_applies(int64_t M, int64_t N, int64_t K) {
+  return K % 8 == 0 && K >= 256 && K <= kHalfMaxK && N >= 1024 && M >= 1024 && M * N * K >= 1300000000ll && tuning_env("AQT_NO_HALF") == nullptr;
 }
 
 // True if the CTA-pair kernel with the row-quantizing epilogue takes the call: deep K, no GLU, int8
@@ -392,7 +415,7 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   bits_w &= ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
   if (op == AQT_OP_QMATMUL) return ws_qmatmul(M, N, K, bits_a, bits_w);
   if (op == AQT_OP_LINEAR_FWD) return ws_linear(M, N, K, bits_w);
-  if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return ws_weight_only(0, N, K, AQT_FLOAT_TF32);
+  if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return half_kind_applies(M, N, K) ? half_layout(M, N, K).total : ws_weight_only(0, N, K, AQT_FLOAT_TF32);
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY_X2) return ws_weight_only(M, N, K, AQT_FLOAT_TF32X2);
   if (op == AQT_OP_LINEAR_BWD) return bwd_workspace(M, N, K);
   if (op == AQT_OP_FFN_FWD) return ffn_layout(M, K, N, bits_w, bits_w).total;
@@ -978,7 +1001,17 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
     a_f = x2;
     k_mm = 2 * K;
     a_pitch = 8 * K;
-  } else {
+  }
+  const HalfLayout H = half_layout(M, N, K);
+  const bool half = precision == AQT_FLOAT_TF32 && half_kind_applies(M, N, K) && workspace_bytes >= H.total;
+  uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
+  const void* b_mm = w_f;
+  if (half) {
+    rc = launch_half_operands(x, ldx, M, K, reinterpret_cast<__half*>(ws + H.x_h), reinterpret_cast<float*>(ws + H.inv), wq, is_packed(bits_w), N * K, w_f,
+                              reinterpret_cast<__half*>(ws + H.w_h), st);
+    if (rc != AQT_OK) return rc;
+    b_mm = ws + H.w_h;
+  } else if (precision == AQT_FLOAT_TF32) {
     rc = launch_codes_to_float(wq, is_packed(bits_w), N * K, w_f, st);
     if (rc != AQT_OK) return rc;
   }
@@ -1000,7 +1033,17 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
   p.n_out = (int)n_out;
   p.tiles_m = p.tiles_n = p.k_blocks = 0;
   p.small_acc = 0;
-  return launch_qgemm(reinterpret_cast<const int8_t*>(a_f), w_f, false, y, ldy, p, st);
+  if (half) {
+    p.kind = 2;
+    p.s_x = reinterpret_cast<const float*>(ws + H.inv);
+    p.K = (int)(2 * K);
+    p.a_pitch = 2 * K;
+    p.wide_a = x;
+    p.wide_a_pitch = 4 * ldx;
+    p.wide_b = w_f;
+    return launch_qgemm_plan(kPlanPair256S4E8, reinterpret_cast<const int8_t*>(ws + H.x_h), b_mm, false, y, ldy, p, st);
+  }
+  return launch_qgemm(reinterpret_cast<const int8_t*>(a_f), b_mm, false, y, ldy, p, st);
 }
 
 // The weight gradient takes the split operands wherever its contraction fills a K-block of 32 rows and the output a fair

@@ -2,6 +2,8 @@
 // Rows are dense, so a [rows, cols] tensor with even cols is one flat stream of byte pairs.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "aqt_common.cuh"
 
 namespace aqt {
@@ -157,6 +159,97 @@ __global__ void __launch_bounds__(256) codes_to_float_twice_kernel(const uint8_t
   }
 }
 
+// Operands of the half kind of the matmul (K % 8 == 0, K <= 16 G, G 32 or 64).  Blocks 0 .. row_blocks - 1: rows of x as binary16, scaled by the
+// power of two that brings a row's largest magnitude into [2^14, 2^15): eleven significant bits of every value down to 2^-28 of
+// the largest, rounded to nearest (a tf32 operand has the same eleven, cut off).  inv[m]: the inverse of the scale, or -1 for a
+// row with values that are smaller and not zero, not finite, or near the ends of binary32's range.  G threads to a row.  The other
+// blocks: the weights' codes as binary16 and as binary32, which tiles with such a row read.
+template <int G>
+__global__ void __launch_bounds__(256) half_operands_kernel(const float* __restrict__ x, int64_t ldx, int M, int K, __half* __restrict__ xh,
+                                                            float* __restrict__ inv, int row_blocks, const uint8_t* __restrict__ codes, bool packed, int64_t n,
+                                                            float* __restrict__ w_f, __half* __restrict__ w_h) {
+  constexpr int VEC = 2;  // pairs of float4s held per thread
+  __shared__ float warp_max[8];
+  __shared__ int warp_wide[8];
+  grid_dependency_wait();
+  grid_dependents_launch();
+  if ((int)blockIdx.x >= row_blocks) {
+    const int64_t stride = (int64_t)((int)gridDim.x - row_blocks) * blockDim.x;
+    for (int64_t i = (int64_t)((int)blockIdx.x - row_blocks) * blockDim.x + threadIdx.x; i < (n >> 2); i += stride) {
+      uint32_t w;
+      if (packed) {
+        uint32_t o1;
+        unpack_word((uint32_t)__ldg(reinterpret_cast<const uint16_t*>(codes) + i), w, o1);
+      } else {
+        w = __ldg(reinterpret_cast<const uint32_t*>(codes) + i);
+      }
+      const float4 f = make_float4((float)(int8_t)(w & 0xFF), (float)(int8_t)((w >> 8) & 0xFF), (float)(int8_t)((w >> 16) & 0xFF), (float)(int8_t)(w >> 24));
+      reinterpret_cast<float4*>(w_f)[i] = f;
+      const __half2 h[2] = {__floats2half2_rn(f.x, f.y), __floats2half2_rn(f.z, f.w)};
+      reinterpret_cast<uint2*>(w_h)[i] = *reinterpret_cast<const uint2*>(h);
+    }
+    return;
+  }
+  const int t = threadIdx.x % G, r_in_cta = threadIdx.x / G, warp = threadIdx.x >> 5;
+  const int m = (int)blockIdx.x * (256 / G) + r_in_cta;
+  const bool live = m < M;
+  const int n8 = K >> 3;
+  const float4* row = reinterpret_cast<const float4*>(x + (int64_t)(live ? m : 0) * ldx);
+  float4 v[VEC][2];
+  float amax = 0.0f;
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) {
+    const int c = t + i * G;
+    v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live && c < n8) {
+      v[i][0] = __ldg(row + 2 * c);
+      v[i][1] = __ldg(row + 2 * c + 1);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {  // NaN wins, so that a row with one is found
+      const float4 f = v[i][j];
+      asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(amax) : "f"(fabsf(f.x)), "f"(fabsf(f.y)));
+      asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(amax) : "f"(fabsf(f.z)), "f"(fabsf(f.w)));
+    }
+  }
+  uint32_t bits = __reduce_max_sync(0xffffffffu, __float_as_uint(amax) & 0x7FFFFFFFu);  // non-negative floats order like their bit patterns
+  if (G > 32) {
+    if ((threadIdx.x & 31) == 0) warp_max[warp] = __uint_as_float(bits);
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < G / 32; ++w) bits = max(bits, __float_as_uint(warp_max[r_in_cta * (G / 32) + w]));
+  }
+  // 2^(14 - exponent of the largest); rows of zeros: 1
+  const int e = (int)(bits >> 23);  // biased
+  const bool in_range = bits == 0 || (e >= 27 && e <= 227);
+  const float scale = bits == 0 || !in_range ? 1.0f : __uint_as_float((uint32_t)(127 + 14 + 127 - e) << 23);
+  bool wide = !in_range;
+#pragma unroll
+  for (int i = 0; i < VEC; ++i) {
+    const int c = t + i * G;
+    if (c >= n8 || !live) continue;
+    uint32_t h[4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const float f[4] = {v[i][j].x * scale, v[i][j].y * scale, v[i][j].z * scale, v[i][j].w * scale};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) wide = wide || (fabsf(f[k]) < 6.103515625e-05f && f[k] != 0.0f);
+      const __half2 a = __floats2half2_rn(f[0], f[1]), b = __floats2half2_rn(f[2], f[3]);
+      h[2 * j] = *reinterpret_cast<const uint32_t*>(&a);
+      h[2 * j + 1] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    reinterpret_cast<uint4*>(xh + (int64_t)m * K)[c] = make_uint4(h[0], h[1], h[2], h[3]);
+  }
+  int any_wide = __any_sync(0xffffffffu, wide);
+  if (G > 32) {
+    if ((threadIdx.x & 31) == 0) warp_wide[warp] = any_wide;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < G / 32; ++w) any_wide |= warp_wide[r_in_cta * (G / 32) + w];
+  }
+  if (live && t == 0) inv[m] = any_wide ? -1.0f : (bits == 0 ? 1.0f : __uint_as_float((uint32_t)(e - 14) << 23));
+}
+
 static unsigned flat_grid(int64_t work_items) {
   const int64_t want = ceil_div(work_items, 256);
   return (unsigned)(want < 1 ? 1 : (want > 148 * 32 ? 148 * 32 : want));
@@ -170,6 +263,18 @@ static int launch_unpack_int4(const uint8_t* packed, int64_t n_bytes, int8_t* q,
 // codes: int8 [n] or packed nibbles [n / 2], 4-byte (2-byte if packed) aligned; out: float [n], 16-byte aligned; n % 4 == 0.
 static int launch_codes_to_float(const void* codes, bool packed, int64_t n, float* out, cudaStream_t st) {
   return launch_pdl(codes_to_float_kernel, dim3(flat_grid(n / 4), 1, 1), dim3(256, 1, 1), 0, st, 1, reinterpret_cast<const uint8_t*>(codes), packed, n, out);
+}
+
+constexpr int kHalfMaxK = 1024;
+// xh: [M, K] halves; inv: [M]; w_f, w_h: [N, K] (n = N * K codes).
+static int launch_half_operands(const float* x, int64_t ldx, int64_t M, int64_t K, __half* xh, float* inv, const void* codes, bool packed, int64_t n,
+                                float* w_f, __half* w_h, cudaStream_t st) {
+  const int g = K <= 512 ? 32 : 64;
+  const int64_t row_blocks = ceil_div(M, 256 / g), want = ceil_div(n / 4, 256 * 2);
+  const int64_t w_blocks = want < 1 ? 1 : (want > 148 * 8 ? 148 * 8 : want);
+  auto kernel = g == 32 ? half_operands_kernel<32> : half_operands_kernel<64>;
+  return launch_pdl(kernel, dim3((unsigned)(row_blocks + w_blocks), 1, 1), dim3(256, 1, 1), 0, st, 1, x, ldx, (int)M, (int)K, xh, inv, (int)row_blocks,
+                    reinterpret_cast<const uint8_t*>(codes), packed, n, w_f, w_h);
 }
 
 static int launch_split_hi_lo(const float* x, int64_t ldx, int64_t M, int64_t K, float* out, cudaStream_t st) {

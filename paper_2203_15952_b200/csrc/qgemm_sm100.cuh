@@ -94,7 +94,7 @@ struct GemmParams {
   int s_x_kind;
   int act;
   int M, N, K;  // K: bytes of contraction per operand row (= elements for 8-bit codes, 4 x elements for the float kind)
-  int kind = 0;       // 0: signed 8-bit codes, int32 accumulators; 1: binary32 operands used as tf32, binary32 accumulators
+  int kind = 0;       // 0: signed 8-bit codes, int32 accumulators; 1: binary32 operands used as tf32, binary32 accumulators; 2: below
   int64_t a_pitch = 0;  // bytes between rows of A; 0 = dense (K)
   // Batched form (streaming kernel, one CTA per tile): every batch_tiles_m consecutive m-tiles form
   // one batch with its own block of batch_b_rows rows of B, stacked below one another (b_rows rows
@@ -125,6 +125,20 @@ struct GemmParams {
   // Float kind: the next launch on the stream does not read what this one writes and may start on SMs that fall free (it
   // sees to it that it does not end first, see DwParams::beside_previous).
   int early_trigger = 0;
+  // Half kind (kind 2): operands are binary16, the rows of A scaled by powers of two (s_x: their inverses).  A row whose values
+  // span more than binary16 holds has a negative entry in s_x; tiles with such a row take the float kind's operands.
+  const float* wide_a = nullptr;
+  const float* wide_b = nullptr;
+  int64_t wide_a_pitch = 0;  // bytes
+  int wide_k_blocks = 0;
+};
+
+// Operands of the half kind's wide tiles, as floats; nothing for the other kinds.
+template <bool HALF_KIND>
+struct WideMaps {};
+template <>
+struct WideMaps<true> {
+  CUtensorMap a, b;
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -297,6 +311,15 @@ __device__ __forceinline__ void tc_mma_tf32_pair(uint32_t d_tmem, uint64_t a_des
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Half kind: A and B hold binary16 values (K = 16 elements = 32 bytes per instruction), binary32 accumulators.
+__device__ __forceinline__ void tc_mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base + i).
 __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -330,6 +353,11 @@ __host__ __device__ constexpr uint32_t idesc_i8(int bn, int m = kBM) {
 // The same for the float kind: D binary32, A and B tf32, both K-major.
 __host__ __device__ constexpr uint32_t idesc_tf32(int bn, int m = kBM) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
+// D binary32, A and B binary16.
+__host__ __device__ constexpr uint32_t idesc_f16(int bn, int m) {
+  return (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -366,10 +394,11 @@ __device__ __forceinline__ float sigmoid_f(float z) {
 //                  -> 512 Swish 89.3 us, 91.2 with conversions); sixteen warps on 128 columns are shorter of issue slots
 //                  than of conversions (feed-forward pair on 12 800 rows 56.4 / 55.5, 12 800 x 512 -> 2048 gated 39.0 / 37.9)
 //   kAccFloat      binary32 already (the float matmul of the weight-only layer)
-constexpr int kAccInt32 = 0, kAccInt32Small = 1, kAccFloat = 2;
+//   kAccHalf       binary32 already, of the half kind
+constexpr int kAccInt32 = 0, kAccInt32Small = 1, kAccFloat = 2, kAccHalf = 3;
 template <int ACCK>
 __device__ __forceinline__ float acc_to_float(uint32_t acc) {
-  if (ACCK == kAccFloat) return __uint_as_float(acc);
+  if (ACCK == kAccFloat || ACCK == kAccHalf) return __uint_as_float(acc);
   if (ACCK == kAccInt32Small) return __int_as_float(0x4B400000 + (int)acc) - 12582912.0f;
   return __int2float_rn((int)acc);
 }
@@ -377,7 +406,7 @@ __device__ __forceinline__ float acc_to_float(uint32_t acc) {
 // Two accumulators -> two floats (see acc_to_float); the subtraction is one packed add.
 template <int ACCK>
 __device__ __forceinline__ float2 acc_to_float2(uint32_t a0, uint32_t a1) {
-  if (ACCK == kAccFloat) return make_float2(__uint_as_float(a0), __uint_as_float(a1));
+  if (ACCK == kAccFloat || ACCK == kAccHalf) return make_float2(__uint_as_float(a0), __uint_as_float(a1));
   if (ACCK == kAccInt32Small)
     return __fadd2_rn(make_float2(__int_as_float(0x4B400000 + (int)a0), __int_as_float(0x4B400000 + (int)a1)),
                       make_float2(-12582912.0f, -12582912.0f));
@@ -520,6 +549,25 @@ __device__ __forceinline__ bool unit_at(const GemmParams& p, int i, int& tm, int
   return tile < p.tiles_m * p.tiles_n;
 }
 
+// Half kind: true if one of the ROWS rows from `row0` on is wide (GemmParams::wide_a).  The same answer in every lane of the warp.
+template <int ROWS>
+__device__ __forceinline__ bool rows_wide(const GemmParams& p, int row0) {
+  constexpr int PER = ROWS / 32;  // rows per lane
+  const int m = row0 + (int)(threadIdx.x & 31) * PER;
+  float least = 0.0f;
+#pragma unroll
+  for (int i = 0; i < PER; i += 4) {
+    if (m + i + 3 < p.M) {
+      const float4 v = __ldg(reinterpret_cast<const float4*>(p.s_x + m + i));
+      least = fminf(least, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+    } else {
+      for (int j = i; j < i + 4; ++j)
+        if (m + j < p.M) least = fminf(least, __ldg(p.s_x + m + j));
+    }
+  }
+  return __any_sync(0xffffffffu, least < 0.0f) != 0;
+}
+
 // RQ (CTA pairs, no GLU): the epilogue also quantizes the output rows for the next layer (Fig. 2 of
 // the paper on u = what the plain epilogue writes): pass 1 is the plain epilogue, which also keeps
 // the row maxima and writes u back over its accumulators; every thread then publishes the maximum
@@ -531,8 +579,11 @@ __device__ __forceinline__ bool unit_at(const GemmParams& p, int i, int& tm, int
 template <int BN, int STAGES, int EW, bool WS, bool BPACK, int ACCK, bool DEBUG, bool CTA2 = false, bool RQ = false, bool HALVES = false>
 __global__ void __launch_bounds__(32 * (2 + EW), 1)
 qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_r, const GemmParams p) {
+                const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_r, const GemmParams p,
+                const __grid_constant__ WideMaps<ACCK == kAccHalf> wm) {
   using Cfg = GemmCfg<BN, STAGES, EW, WS, CTA2>;
+  constexpr bool HALFK = ACCK == kAccHalf;
+  static_assert(!HALFK || (CTA2 && BN == 256 && !DEBUG && !RQ), "the half kind is a form of the CTA-pair kernel");
   constexpr int HALF = BN / 2;
   constexpr int SBUFS = Cfg::kStageBufs;
   constexpr int TILE_M = CTA2 ? 2 * kBM : kBM;  // rows of a tile (of the pair's tile)
@@ -633,7 +684,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (HALFK || lane == 0) {  // (half kind: the whole warp looks for wide rows, one thread issues)
       uint32_t it = 0;
       bool ok = true;
       if (WS) {
@@ -663,7 +714,16 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         const int half_cols = part == 0 ? HALF : HALF / 2;
         const int row0 = (glu ? tn * HALF : tn * BN) + (part == 2 ? (glu ? HALF / 2 : HALF) : 0);
         const int row1 = glu ? p.N / 2 + row0 : row0 + half_cols;
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
+        const CUtensorMap *map_a = &tm_a, *map_b = &tm_b;
+        int k_blocks = p.k_blocks;
+        if constexpr (HALFK) {
+          if (rows_wide<TILE_M>(p, tm * TILE_M)) {
+            map_a = &wm.a;
+            map_b = &wm.b;
+            k_blocks = p.wide_k_blocks;
+          }
+        }
+        for (int kb = 0; (!HALFK || lane == 0) && kb < k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1, &abort_flag, t_start)) { ok = false; break; }
           const uint32_t bar = smem_u32(&full_bar[s]);
@@ -672,47 +732,61 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             // The leader's barrier counts both CTAs' bytes; each CTA loads its 128 rows of A and
             // its half of the weight rows (leader: first half / values, peer: second half / gates).
             if (pair_rank == 0) mbar_arrive_expect_tx(bar, HALVES && part != 0 ? 2 * (Cfg::kABytes + Cfg::kBBytes / 2) : 2 * Cfg::kStageBytes);
-            tma_load_2d_pair(stage, &tm_a, kb * kBK, tm * TILE_M + row_in_tile, bar);
+            tma_load_2d_pair(stage, map_a, kb * kBK, tm * TILE_M + row_in_tile, bar);
             if (BN == 512) {
               // two MMAs of 256 columns per k-step: this CTA supplies 128 weight rows to each
               const int r = tn * BN + (int)pair_rank * 128;
-              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
-              tma_load_2d_pair(stage + Cfg::kABytes + 128 * kBK, &tm_b, kb * kBK, r + 256, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes, map_b, kb * kBK, r, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes + 128 * kBK, map_b, kb * kBK, r + 256, bar);
             } else {
               const int r = pair_rank == 0 ? row0 : row1;
-              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes, map_b, kb * kBK, r, bar);
               // (boxes of half a CTA's rows, so that half a tile is one of them)
-              if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, &tm_b, kb * kBK, r + HALF / 2, bar);
+              if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, map_b, kb * kBK, r + HALF / 2, bar);
             }
             continue;
           }
           mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-          tma_load_2d(stage, &tm_a, kb * kBK, tm * kBM, bar);
+          tma_load_2d(stage, map_a, kb * kBK, tm * kBM, bar);
           if (!WS) {
             const int b_batch = p.batch_tiles_m > 0 ? (tm / p.batch_tiles_m) * p.batch_b_rows : 0;  // this batch's rows of B
-            tma_load_2d(stage + Cfg::kABytes, &tm_b, kb * kBK, row0 + b_batch, bar);
-            tma_load_2d(stage + Cfg::kABytes + HALF * kBK, &tm_b, kb * kBK, row1 + b_batch, bar);
+            tma_load_2d(stage + Cfg::kABytes, map_b, kb * kBK, row0 + b_batch, bar);
+            tma_load_2d(stage + Cfg::kABytes + HALF * kBK, map_b, kb * kBK, row1 + b_batch, bar);
           }
         }
+        if constexpr (HALFK) ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
       grid_dependents_launch();  // every load of this CTA has been issued: the next kernel may be scheduled behind it
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && pair_rank == 0) {
-      constexpr uint32_t idesc_whole = TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M);
-      constexpr uint32_t idesc_half = TF32 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_i8(Cfg::kMmaN / 2, TILE_M);
+    if ((HALFK || lane == 0) && pair_rank == 0) {
+      constexpr uint32_t idesc_whole = HALFK ? idesc_f16(Cfg::kMmaN, TILE_M) : (TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M));
+      constexpr uint32_t idesc_half = HALFK ? idesc_f16(Cfg::kMmaN / 2, TILE_M) : (TF32 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_i8(Cfg::kMmaN / 2, TILE_M));
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       if (WS) ok = mbar_wait(smem_u32(BPACK ? &b_ready_bar : &b_loaded_bar), 0, &abort_flag, t_start);
       int tm, tn, part;
       for (int i = 0; ok && unit_at<WS, CTA2, HALVES>(p, i, tm, tn, part); ++i, ++tcount) {
-        const uint32_t idesc = HALVES && part != 0 ? idesc_half : idesc_whole;
+        uint32_t idesc = HALVES && part != 0 ? idesc_half : idesc_whole;
+        int k_blocks = p.k_blocks;
+        bool wide = false;
+        if constexpr (HALFK) {
+          wide = rows_wide<TILE_M>(p, tm * TILE_M);
+          if (wide) {
+            k_blocks = p.wide_k_blocks;
+            idesc = HALVES && part != 0 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_tf32(Cfg::kMmaN, TILE_M);
+          }
+        }
         const uint32_t buf = tcount % Cfg::kAccBufs, aph = (tcount / Cfg::kAccBufs) & 1;
-        if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
+        if constexpr (HALFK) {
+          if (lane == 0) ok = mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start);
+        } else {
+          if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
+        }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
+        for (int kb = 0; (!HALFK || (lane == 0 && ok)) && kb < k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&full_bar[s]), ph, &abort_flag, t_start)) { ok = false; break; }
           tc_fence_after();
@@ -723,7 +797,9 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           for (int kk = 0; kk < kBK / kMmaK; ++kk) {
             // advancing K inside the 128-byte swizzle row: +32 bytes = +2 in the 16-byte address field
             const uint32_t accumulate = (kb | kk) != 0 ? 1u : 0u;
-            if (TF32) {
+            if (HALFK && !wide) {
+              tc_mma_f16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+            } else if (TF32 || HALFK) {
               if (CTA2) tc_mma_tf32_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
               else tc_mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
             } else {
@@ -737,10 +813,11 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           if (CTA2) tc_commit_pair(smem_u32(&empty_bar[s]));
           else tc_commit(smem_u32(&empty_bar[s]));
         }
-        if (ok) {  // accumulator complete (in both CTAs' TMEM)
+        if (ok && (!HALFK || lane == 0)) {  // accumulator complete (in both CTAs' TMEM)
           if (CTA2) tc_commit_pair(smem_u32(&tmem_full_bar[buf]));
           else tc_commit(smem_u32(&tmem_full_bar[buf]));
         }
+        if constexpr (HALFK) ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
     }
   } else {
@@ -800,7 +877,10 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         }
       }
       const int pm = ptm * TILE_M + row_in_tile + quad * 32 + lane;
-      if constexpr (!TF32) {
+      if constexpr (HALFK) {
+        const bool wide = rows_wide<TILE_M>(p, ptm * TILE_M);
+        pre_sx = pm < p.M && !wide ? __ldg(p.s_x + pm) : 1.0f;
+      } else if constexpr (!TF32) {
         pre_sx = p.s_x_kind == AQT_SCALE_ROW ? (pm < p.M ? __ldg(p.s_x + pm) : 0.0f) : __ldg(p.s_x);
       }
     };
@@ -1224,6 +1304,14 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
   } else {
     tm_r = tm_y;  // never dereferenced
   }
+  WideMaps<ACCK == kAccHalf> wm;
+  if constexpr (ACCK == kAccHalf) {
+    p.wide_k_blocks = (int)ceil_div(2 * (int64_t)p.K, kBK);
+    rc = make_map_2d(&wm.a, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.wide_a, (uint64_t)p.M, (uint64_t)p.K * 2, (uint64_t)p.wide_a_pitch, kBM, kBK);
+    if (rc != AQT_OK) return rc;
+    rc = make_map_2d(&wm.b, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.wide_b, (uint64_t)p.N, (uint64_t)p.K * 2, (uint64_t)p.K * 2, HALVES ? BN / 4 : BN / 2, kBK);
+    if (rc != AQT_OK) return rc;
+  }
   auto kernel = qgemm_i8_kernel<BN, STAGES, EW, WS, BPACK, ACCK, DEBUG, CTA2, RQ, HALVES>;
   static std::atomic<uint64_t> smem_opted_in{0};
   rc = ensure_dynamic_smem(kernel, Cfg::kSmemBytes, smem_opted_in);
@@ -1242,13 +1330,19 @@ static int launch_qgemm_inst(const int8_t* a, const void* b, float* y, int64_t l
     }
     if (HALVES) p.whole_tiles = (int)whole_pair_tiles(tiles, pairs, p.early_trigger != 0);
     grid = 2u * (unsigned)(tiles < pairs ? tiles : pairs);
-    return launch_pdl(kernel, dim3(grid, 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 2, tm_a, tm_b, tm_y, tm_r, p);
+    return launch_pdl(kernel, dim3(grid, 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 2, tm_a, tm_b, tm_y, tm_r, p, wm);
   }
-  return launch_pdl(kernel, dim3(grid, 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 1, tm_a, tm_b, tm_y, tm_r, p);
+  return launch_pdl(kernel, dim3(grid, 1, 1), dim3(Cfg::kThreads, 1, 1), Cfg::kSmemBytes, st, 1, tm_a, tm_b, tm_y, tm_r, p, wm);
 }
 
 template <int BN, int STAGES, int EW, bool WS, bool BPACK, bool CTA2 = false>
 static int launch_qgemm_cfg(const int8_t* a, const void* b, float* y, int64_t ldy, const GemmParams& p, cudaStream_t st) {
+  if (p.kind == 2) {
+    if constexpr (CTA2 && BN == 256 && EW == 8) {
+      if (p.acc_debug == nullptr) return launch_qgemm_inst<BN, STAGES, EW, WS, false, kAccHalf, false, CTA2>(a, b, y, ldy, p, st);
+    }
+    return AQT_ERR_UNSUPPORTED;
+  }
   if (p.kind == 1) {
     if constexpr (!BPACK && BN != 512) {
       if (p.acc_debug == nullptr) return launch_qgemm_inst<BN, STAGES, EW, WS, false, kAccFloat, false, CTA2>(a, b, y, ldy, p, st);
