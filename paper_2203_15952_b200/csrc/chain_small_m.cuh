@@ -23,8 +23,8 @@
 // cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
 // scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
 // wait of the library.
-// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 337 vs 1250 us, 32 rows
-// 346 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 507 vs 1340; beyond, a
+// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 312 vs 1250 us, 32 rows
+// 320 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 488 vs 1340; beyond, a
 // second wave of clusters or 32 rows per cluster lose to the per-layer kernels at d = 1024 (860 vs 700
 // us for 8 blocks at 113 rows), which is where AQT_CHAIN_MAX_ROWS lies.
 // What a layer then costs (2000 to 2600 ns; clock stamps in a copy) is a chain of latencies and of instructions that every warp
@@ -34,6 +34,7 @@
 //     for the rows of the layer before (445 -> 383 us);
 //   * what is not always run stands aside: the general code sequence in a function, the wide form's second words behind a
 //     branch, the loop over pieces left at the last one (383 -> 344 us); stores of a layer's outputs wait until its maxima are on their way;
+//   * layers that read the same input and look alike run as one (chain_group; 343 -> 319 us);
 //   * no integer division and no dependent parameter load in the loops (the step table sits in shared memory with everything
 //     derived from the sizes), and packed weights are used as sixteen times their codes (a nibble in the upper half of a
 //     byte; the sums are shifted back, exact), two instructions per four codes instead of eleven per eight, against
@@ -69,7 +70,9 @@ struct ChainStep {
   float rs;           // residual scale
   uint32_t flags;
   // derived by the host (chain_derive)
-  uint16_t tiles, ks_n;          // 16-channel tiles per CTA, shares of K
+  uint16_t tiles;                // 16-channel tiles per CTA
+  uint8_t ks_n;                  // shares of K
+  uint8_t parts;                 // this step and those behind it that run as one (see chain_group)
   uint32_t inv_tiles;            // ceil(65536 / tiles), ceil(65536 / ks_n): quotients of small numbers by a multiply and a shift
   uint16_t inv_ks_lo, units;     // (ks_n == 1 is not divided by)
 };
@@ -157,8 +160,8 @@ __device__ __forceinline__ float chain_max4(float m, const float (&v)[4]) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
 }
 
-// NT: 8-row tiles per cluster.
-template <int NT, int MAXS>
+// NT: 8-row tiles per cluster.  GROUPED: some steps run as one (chain_group); other chains are 2 to 5 % faster without the code for it.
+template <int NT, int MAXS, bool GROUPED>
 __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const __grid_constant__ ChainParams<MAXS> p) {
   constexpr int R = 8 * NT;
   constexpr int SETS = NT == 1 ? 2 : 1;  // independent accumulators per row tile (the products of one set depend on one another)
@@ -205,13 +208,13 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     uint4 nxt[kChainChunk][2];
     auto open_unit = [&]() {  // the iterator's unit, or the first one of a later step
       while (it_step < n_steps && it_u >= steps[it_step].units) {
-        ++it_step;
+        it_step += GROUPED ? steps[it_step].parts : 1;
         it_u = warp;
       }
       u_left = 0;
       if (it_step >= n_steps) return;
       const ChainStep& st = steps[it_step];
-      const int k128 = st.K >> 7, per_cta = st.N >> 4;
+      const int k128 = st.K >> 7, per_part = st.N >> 4, per_cta = GROUPED ? per_part * st.parts : per_part;
       const int shift = (st.flags & kChainPacked) ? 1 : 0;
       int tile = it_u, kb0 = 0, kb1 = k128, ks = 0;  // tiles fastest, then shares of K
       if (st.ks_n > 1) {
@@ -223,16 +226,29 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       const int c0 = tile * 16 + g;  // this lane's channels among the CTA's: c0 and c0 + 8
       u_both = tile * 16 + 8 < per_cta;
       const int c1 = u_both ? c0 + 8 : c0;
-      int n0 = rank * per_cta + c0, n1 = rank * per_cta + c1;
+      const uint8_t *w0 = st.w, *w1 = st.w;
+      int n0 = rank * per_part + c0, n1 = rank * per_part + c1;
+      if (GROUPED && st.parts > 1) {  // eight channels are of one part
+        for (int i = 1; i < st.parts; ++i) {
+          if (c0 >= i * per_part) {
+            n0 -= per_part;
+            w0 = steps[it_step + i].w;
+          }
+          if (c1 >= i * per_part) {
+            n1 -= per_part;
+            w1 = steps[it_step + i].w;
+          }
+        }
+      }
       if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {  // value channels, then the gate channels of the same output columns
         const int cols = per_cta >> 1, gate_off = (st.N >> 1) - cols;
         n0 = rank * cols + c0 + (c0 >= cols ? gate_off : 0);
         n1 = rank * cols + c1 + (c1 >= cols ? gate_off : 0);
       }
       u_left = (kb1 - kb0) << (1 - shift);
-      const uint8_t* w = st.w + (kb0 << (7 - shift)) + kq * 16;
-      u_src0 = w + (int64_t)n0 * (st.K >> shift);
-      u_src1 = w + (int64_t)n1 * (st.K >> shift);
+      const int k_off = (kb0 << (7 - shift)) + kq * 16;
+      u_src0 = w0 + (int64_t)n0 * (st.K >> shift) + k_off;
+      u_src1 = w1 + (int64_t)n1 * (st.K >> shift) + k_off;
       u_a = g * chain_pitch(st.K, shift != 0) + kb0 * 128 + kq * (16 << shift);
       u_part = (ks * R + 2 * kq) * (per_cta + 4) + c0;
       u_first = true;
@@ -244,7 +260,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         nxt[j][1] = __ldg(reinterpret_cast<const uint4*>(u_src1 + j * 64));
       }
     };
-    auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2 
+    auto prefetch_slice = [&](int s) {  // one step's share of the weights -> L2
       if (threadIdx.x != kChainThreads - 1 || s >= n_steps || blockIdx.x >= kChainCtas) return;
       const ChainStep& st = steps[s];
       const bool glu = (st.flags & kChainActMask) >= AQT_ACT_GLU;
@@ -254,24 +270,29 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((uint32_t)(rows_here * row_bytes)) : "memory");
     };
 
+    auto prefetch_group = [&](int s) {
+      for (int i = 0; s < n_steps && i < (GROUPED ? steps[s].parts : 1); ++i) prefetch_slice(s + i);
+    };
+
     open_unit();
 #pragma unroll
     for (int j = 0; j < kChainChunk; ++j) load_piece(j);
-    prefetch_slice(1);
+    prefetch_group(GROUPED ? steps[0].parts : 1);
     chain_cluster_sync();  // the input's codes are ready; every CTA's barriers exist
 
     uint32_t codes_parity = 0;  // of the codes that the next step with a new input reads
     bool fresh = false;         // the codes of this step's input come from the exchange before it
-    for (int s = 0; s < n_steps; ++s) {
+    for (int s = 0, round = 0, parts; s < n_steps; s += parts, ++round) {
       const ChainStep& st = steps[s];
+      parts = GROUPED ? st.parts : 1;
       const bool packed = (st.flags & kChainPacked) != 0;
-      const int units = st.units, pitch = chain_pitch(st.K, packed), part_pitch = (st.N >> 4) + 4;
-      int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + (s & 1) * p.part_bytes);
+      const int units = st.units, pitch = chain_pitch(st.K, packed), part_pitch = (st.N >> 4) * parts + 4, slot = round & 1;
+      int* part = reinterpret_cast<int*>(chain_smem + p.code_bytes + slot * p.part_bytes);
       if (fresh) {
         mbar_wait(smem_u32(&codes_bar), codes_parity, &abort_flag, t_start);
         codes_parity ^= 1u;
       }
-      if (s >= 2) chain_bar_sync(3 + (s & 1));  // the sums of two steps ago have been read
+      if (round >= 2) chain_bar_sync(3 + slot);  // the sums of two rounds ago have been read
       bool used = false;
       int acc[NT][SETS][4];
       while (it_step == s) {
@@ -354,30 +375,36 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
         }
         if (!more) break;
       }
-      chain_bar_arrive(1 + (s & 1));
+      chain_bar_arrive(1 + slot);
       // the next step's weights are asked for while the rows of this one are worked on
       if (used) {
         open_unit();
 #pragma unroll
         for (int j = 0; j < kChainChunk; ++j) load_piece(j);
       }
-      prefetch_slice(s + 2);
-      fresh = (st.flags & kChainSide) == 0;
+      const int s1 = s + parts;
+      prefetch_group(s1 < n_steps && GROUPED ? s1 + steps[s1].parts : s1 + 1);
+      fresh = (steps[s1 - 1].flags & kChainSide) == 0;
     }
   } else {
     auto load_scales = [&](int s, float& wv, float& bv) {  // this thread's channel of step s
       wv = bv = 0.0f;
       if (s >= n_steps) return;
       const ChainStep& st = steps[s];
-      const int per_cta = st.N >> 4, c = threadIdx.x;
+      const int per_part = st.N >> 4, per_cta = GROUPED ? per_part * st.parts : per_part, c = threadIdx.x;
       if (c - lane >= per_cta || c >= per_cta) return;
-      int n = rank * per_cta + c;
+      int n = rank * per_part + c, of = s;
       if ((st.flags & kChainActMask) >= AQT_ACT_GLU) {
         const int cols = per_cta >> 1, gate = c >= cols ? 1 : 0;
         n = gate * (st.N >> 1) + rank * cols + c - gate * cols;
+      } else if (GROUPED) {
+        for (int i = 1; i < st.parts && c >= i * per_part; ++i) {
+          n -= per_part;
+          ++of;
+        }
       }
-      wv = __ldg(st.s_w + n);
-      if (st.bias != nullptr) bv = __ldg(st.bias + n);
+      wv = __ldg(steps[of].s_w + n);
+      if (steps[of].bias != nullptr) bv = __ldg(steps[of].bias + n);
     };
     float wv, bv;  // scale and bias of this thread's channel of the next step, on their way to sw_s / bias_s
     load_scales(0, wv, bv);
@@ -421,16 +448,19 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
     const uint32_t codes_first = chain_mapa(smem_u32(codes), 0), codes_bar_first = chain_mapa(smem_u32(&codes_bar), 0);
     const uint32_t window = chain_mapa(smem_u32(codes), 1) - codes_first;
     uint32_t exchange_parity = 0;  // of the exchange in progress (steps that are no side steps)
-    for (int s = 0; s < n_steps; ++s) {
+    for (int s = 0, round = 0; s < n_steps; s += GROUPED ? steps[s].parts : 1, ++round) {
       const ChainStep st = steps[s];
-      const uint32_t act = st.flags & kChainActMask;
+      const int parts = GROUPED ? st.parts : 1;
+      const uint32_t act = st.flags & kChainActMask, end_flags = GROUPED ? steps[s + parts - 1].flags : st.flags;
       const bool glu = act >= AQT_ACT_GLU;
-      const int per_cta = st.N >> 4, ks_n = st.ks_n;
+      const int per_part = st.N >> 4, per_cta = per_part * parts, ks_n = st.ks_n;
       const int cols = glu ? per_cta >> 1 : per_cta;  // output columns of this CTA
       const int n_out = glu ? st.N >> 1 : st.N;
       const int part_pitch = per_cta + 4;
-      const bool side = (st.flags & kChainSide) != 0, last = s + 1 == n_steps;
-      const int slot = s & 1;  // of the partial sums and of sw_s / bias_s
+      const int q0 = (parts - 1) * per_part, q_cols = cols - q0;  // the columns that the next step reads
+      const int s1 = s + parts, s2 = s1 < n_steps && GROUPED ? s1 + steps[s1].parts : s1 + 1;
+      const bool side = (end_flags & kChainSide) != 0, last = s1 == n_steps;
+      const int slot = round & 1;  // of the partial sums and of sw_s / bias_s
       const int* part = reinterpret_cast<const int*>(chain_smem + p.code_bytes + slot * p.part_bytes);
       sw_s[slot][threadIdx.x] = wv;
       bias_s[slot][threadIdx.x] = bv;
@@ -493,7 +523,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
             o[2] = __fmaf_rn(st.rs, o[2], r4.z);
             o[3] = __fmaf_rn(st.rs, o[3], r4.w);
           }
-          amax = chain_max4(amax, o);
+          if (!GROUPED || c >= q0) amax = chain_max4(amax, o);
         }
         if (side || last) continue;
         const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(amax));  // non-negative floats order like their bit patterns
@@ -502,7 +532,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
       }
       // what else is to be done, while the maxima are under way
       if (threadIdx.x == 0 && !side && !last) mbar_arrive_expect_tx(smem_u32(&codes_bar), (uint32_t)(rows * n_out));
-      if ((st.flags & kChainAdd) || st.y != nullptr) {
+      if ((st.flags & kChainAdd) || st.y != nullptr || (GROUPED && parts > 1)) {
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
@@ -511,19 +541,28 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
             if (r >= rows || c >= cols) continue;
             const float4 o = make_float4(v[t][j][0], v[t][j][1], v[t][j][2], v[t][j][3]);
             if (st.flags & kChainAdd) *reinterpret_cast<float4*>(h + r * h_cols + c) = o;
-            if (st.y != nullptr) *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + rank * cols + c) = o;
+            if (!GROUPED || parts == 1) {
+              if (st.y != nullptr) *reinterpret_cast<float4*>(st.y + (int64_t)(row0 + r) * st.ldy + rank * cols + c) = o;
+            } else {
+              int of = s, first = 0;
+              while (c >= first + per_part) {
+                first += per_part;
+                ++of;
+              }
+              if (steps[of].y != nullptr) *reinterpret_cast<float4*>(steps[of].y + (int64_t)(row0 + r) * steps[of].ldy + rank * per_part + c - first) = o;
+            }
           }
       }
-      if (s + 2 < n_steps) chain_bar_arrive(3 + slot);
+      if (s2 < n_steps) chain_bar_arrive(3 + slot);
       if (last) break;
 
-      load_scales(s + 1, wv, bv);  // while the maxima are under way
+      load_scales(s1, wv, bv);  // while the maxima are under way
       if (side) continue;
 
       // ---- quantize the output rows for the next step.  All sixteen maxima of a row are here only when every
       // CTA has finished its products, so nobody reads the old codes any more.
-      const int qmax = (st.flags & kChainOut4) ? 7 : 127;
-      const bool next_packed = (steps[s + 1].flags & kChainPacked) != 0;
+      const int qmax = (end_flags & kChainOut4) ? 7 : 127;
+      const bool next_packed = (steps[s1].flags & kChainPacked) != 0;
       const int out_pitch = chain_pitch(n_out, next_packed);
 #pragma unroll
       for (int t = 0; t < NT; ++t) {
@@ -537,17 +576,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (j > 0 && __builtin_expect(cols <= 128, 1)) break;
-          if (4 * lane + 128 * j >= cols) continue;
+          if (4 * lane + 128 * j >= cols || (GROUPED && 4 * lane + 128 * j < q0)) continue;
           word[j] = chain_codes4(v[t][j], sc, qmax, rounding);
         }
         // to all sixteen CTAs, eight codes per lane and store: `span` lanes (a power of two) cover the row's share,
         // so a store instruction is 32 / span runs of consecutive bytes (the interconnect is paid per run: 250 clocks
         // for a store scattered over sixteen CTAs)
-        const int span_bits = cols <= 16 ? 1 : 32 - __clz((cols >> 3) - 1), span = 1 << span_bits, i = lane & (span - 1);
+        const int span_bits = q_cols <= 16 ? 1 : 32 - __clz((q_cols >> 3) - 1), span = 1 << span_bits, i = lane & (span - 1);
         uint32_t w0, w1;
-        if (__builtin_expect(cols <= 128, 1)) {
-          w0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31);
-          w1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
+        if (__builtin_expect(q_cols <= 128, 1)) {
+          const int from = GROUPED ? q0 >> 2 : 0;  // first lane with columns of the last part
+          w0 = __shfl_sync(0xffffffffu, word[0], (from + 2 * i) & 31);
+          w1 = __shfl_sync(0xffffffffu, word[0], (from + 2 * i + 1) & 31);
         } else {  // columns from 128 on sit in the lanes' second word
           const uint32_t x0 = __shfl_sync(0xffffffffu, word[0], (2 * i) & 31), x1 = __shfl_sync(0xffffffffu, word[0], (2 * i + 1) & 31);
           const uint32_t y0 = __shfl_sync(0xffffffffu, word[1], (2 * i) & 31), y1 = __shfl_sync(0xffffffffu, word[1], (2 * i + 1) & 31);
@@ -555,10 +595,10 @@ __global__ void __launch_bounds__(kChainThreads, 1) chain_small_m_kernel(const _
           w1 = i < 16 ? x1 : y1;
         }
         chain_order8(next_packed, w0, w1);
-        const uint32_t dst = codes_first + (uint32_t)(r * out_pitch + rank * cols + 8 * i);
+        const uint32_t dst = codes_first + (uint32_t)(r * out_pitch + rank * q_cols + 8 * i);
         for (int to = lane >> span_bits; to < kChainCtas; to += 32 >> span_bits) {
           const uint32_t at = ((uint32_t)(rank + to) & (kChainCtas - 1)) * window;
-          if (8 * i < cols) chain_st_async_v2(dst + at, w0, w1, codes_bar_first + at);
+          if (8 * i < q_cols) chain_st_async_v2(dst + at, w0, w1, codes_bar_first + at);
         }
       }
       exchange_parity ^= 1u;
@@ -579,12 +619,32 @@ static bool chain_step_ok(const ChainStep& st) {
   return st.N <= kChainMaxN && n_out <= kChainMaxCols * kChainCtas && st.K <= 8192;
 }
 
-static void chain_derive(ChainStep& st) {
-  st.tiles = (uint16_t)chain_tiles(st.N);
-  st.ks_n = (uint16_t)chain_ksplit(st.tiles, st.K);
+// Steps that run as one: side steps and the one behind them that read the same input and look alike (the attention projections).
+// Their channels make up a CTA's tiles together, their rows go through one epilogue (of at most 128 columns: of more, a step is
+// long enough by itself), and the last one's columns are exchanged.  Eight rows through 17 blocks at d = 512 343 -> 317 us, 384
+// 325 -> 304, 256 277 -> 252.
+static int chain_group(const ChainStep* steps, int n) {
+  const ChainStep& a = steps[0];
+  int parts = 1;
+  while (parts < n && (steps[parts - 1].flags & kChainSide)) {
+    const ChainStep& b = steps[parts];
+    if (b.N != a.N || b.K != a.K || ((a.flags ^ b.flags) & (kChainActMask | kChainPacked)) || ((a.flags | b.flags) & kChainAdd)) return 1;
+    ++parts;
+  }
+  const bool takes = (a.flags & kChainActMask) == AQT_ACT_NONE && parts * (a.N / kChainCtas) <= 128 && !(steps[parts - 1].flags & kChainSide);
+  return takes ? parts : 1;
+}
+
+// Fills in what is derived of the next group of steps; returns how many they are.
+static int chain_derive(ChainStep* steps, int n) {
+  ChainStep& st = steps[0];
+  st.parts = (uint8_t)chain_group(steps, n);
+  st.tiles = (uint16_t)chain_tiles(st.N * st.parts);
+  st.ks_n = (uint8_t)chain_ksplit(st.tiles, st.K);
   st.inv_tiles = (65536u + st.tiles - 1) / st.tiles;  // exact: dividends < 16 * 64, divisors <= 16
   st.inv_ks_lo = (uint16_t)((65536u + st.ks_n - 1) / st.ks_n);
   st.units = (uint16_t)(st.tiles * st.ks_n);
+  return st.parts;
 }
 
 struct ChainSizes {
@@ -593,10 +653,9 @@ struct ChainSizes {
 };
 static ChainSizes chain_sizes(const ChainStep* steps, int n, int R) {
   int code = 0, part = 0, h = 0;
-  for (int i = 0; i < n; ++i) {
+  for (int i = 0; i < n; i += steps[i].parts) {
     const ChainStep& st = steps[i];
-    const int tiles = chain_tiles(st.N);
-    const int c = R * (st.K + 64), q = chain_ksplit(tiles, st.K) * R * (st.N / kChainCtas + 4) * 4;
+    const int c = R * (st.K + 64), q = st.ks_n * R * (st.N * st.parts / kChainCtas + 4) * 4;
     if (c > code) code = c;
     if (q > part) part = q;
     if ((st.flags & kChainAdd) && R * (st.N / kChainCtas) * 4 > h) h = R * (st.N / kChainCtas) * 4;
@@ -613,11 +672,11 @@ constexpr int kChainMaxSmem = 180 * 1024;  // beside the step table and the exch
 // Clusters that run at the same time (the part schedules seven or eight of sixteen CTAs each).
 constexpr int kChainClusters = 7;
 
-template <int NT, int MAXS>
-static int launch_chain_inst(const ChainParams<kChainMaxSteps>& full, int smem, cudaStream_t st) {
+template <int NT, int MAXS, bool GROUPED>
+static int launch_chain_form(const ChainParams<kChainMaxSteps>& full, int smem, cudaStream_t st) {
   ChainParams<MAXS> p;
   memcpy(static_cast<void*>(&p), &full, offsetof(ChainParams<MAXS>, steps) + (size_t)full.n_steps * sizeof(ChainStep));
-  auto kernel = chain_small_m_kernel<NT, MAXS>;
+  auto kernel = chain_small_m_kernel<NT, MAXS, GROUPED>;
   static std::atomic<uint64_t> opted_in{0}, wide{0};
   int rc = ensure_dynamic_smem(kernel, kChainMaxSmem, opted_in);
   if (rc != AQT_OK) return rc;
@@ -625,6 +684,12 @@ static int launch_chain_inst(const ChainParams<kChainMaxSteps>& full, int smem, 
   if (rc != AQT_OK) return rc;
   const unsigned clusters = (unsigned)ceil_div(full.M, 8 * NT);
   return launch_pdl(kernel, dim3(clusters * kChainCtas, 1, 1), dim3(kChainThreads, 1, 1), (size_t)smem, st, kChainCtas, p);
+}
+template <int NT, int MAXS>
+static int launch_chain_inst(const ChainParams<kChainMaxSteps>& p, int smem, cudaStream_t st) {
+  bool grouped = false;
+  for (int i = 0; i < p.n_steps; i += p.steps[i].parts) grouped = grouped || p.steps[i].parts > 1;
+  return grouped ? launch_chain_form<NT, MAXS, true>(p, smem, st) : launch_chain_form<NT, MAXS, false>(p, smem, st);
 }
 template <int NT>
 static int launch_chain_rows(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
@@ -638,7 +703,7 @@ static int launch_chain_rows(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
 // p: everything but the shared-memory sizes.  AQT_ERR_UNSUPPORTED if the kernel cannot take the chain.
 static int launch_chain(ChainParams<kChainMaxSteps>& p, cudaStream_t st) {
   if (p.M <= 0 || p.n_steps <= 0 || p.n_steps > kChainMaxSteps) return AQT_ERR_UNSUPPORTED;
-  for (int i = 0; i < p.n_steps; ++i) chain_derive(p.steps[i]);
+  for (int i = 0; i < p.n_steps;) i += chain_derive(p.steps + i, p.n_steps - i);
   // the fewest rows per cluster with which all clusters run at once
   if (p.M <= 8 * kChainClusters) return launch_chain_rows<1>(p, st);
   return launch_chain_rows<2>(p, st);
