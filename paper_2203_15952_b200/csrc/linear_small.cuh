@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(LinSmallCfg<NT>::kThreads) linear_small_kernel
             const float v1[4] = {f[t][u][1].x, f[t][u][1].y, f[t][u][1].z, f[t][u][1].w};
             uint32_t q0 = 0u, q1 = 0u;
             if (c < K8) {
-              q0 = chain_codes4(v0, sc[t], p.qmax, p.rounding);
-              q1 = chain_codes4(v1, sc[t], p.qmax, p.rounding);
+              q0 = chain_codes4<false>(v0, sc[t], p.qmax, p.rounding);
+              q1 = chain_codes4<false>(v1, sc[t], p.qmax, p.rounding);
               chain_order8(PACKED, q0, q1);
             }
             *reinterpret_cast<uint2*>(codes + r * pitch + 8 * c) = make_uint2(q0, q1);
