@@ -155,7 +155,7 @@ int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, 
  * the same matmul) would launch for a shape without a residual: "small_m", "few64", "ws128e16", "pair256s6e4", ...  Host-only:
  * sm_count_or_0 > 0 plans for a device with that many multiprocessors, 0 for the current device
  * (148 if there is none).  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
- * aqt_linear_bwd with K in elements.  (No counterpart in the paper: the choice of tile shapes is
+ * aqt_linear_bwd with K in elements (tf32 operands; calls that take binary16 ones run "pair256s4e8").  (No counterpart in the paper: the choice of tile shapes is
  * this library's.)  name_out receives a NUL-terminated string of at most name_bytes bytes.
  */
 int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int float_kind,

@@ -829,6 +829,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     const int out_cols_tile = glu ? HALF : BN;               // output columns per tile
     const int chunks_whole = out_cols_tile / 32 / (EW / 4);  // 32-column chunks per epilogue warp and tile
     const bool has_res = p.residual != nullptr;
+    const int n_value_limit = glu ? p.N / 2 : p.N;
     // where the scales of this warp's chunk c start: per-CTA slab (WS) or per-warp slab
     const uint32_t slab_sw = WS ? smem_scale + (uint32_t)(chalf * chunks_whole * 32) * 4 : smem_scale + ew * 2 * Cfg::kSlabFloats * 4;
     const uint32_t slab_bias = WS ? slab_sw + BN * 4 : slab_sw + Cfg::kSlabFloats * 4;
@@ -852,16 +853,17 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     }
 
     int tm, tn, part;
-    // Scales and biases of this warp's columns (GLU: of a chunk's values, then of its gates) and the scale of this thread's row of the
-    // i-th unit, fetched while the unit ahead of it is worked on: their latency between two units was 1300 of a unit's 8800
-    // clocks (pair tiles of 256 columns, Swish).  Sixteen warps have no registers for that.
-    constexpr bool AHEAD = EW <= 8;
-    constexpr int PRE = Cfg::kScaleSlab && !WS ? BN / 32 / (EW / 4) : 1;
+    // Pair tiles: scales and biases of this warp's columns (GLU: of a chunk's values, then of its gates) and the scale of this thread's row
+    // of the i-th unit.  Where the epilogue is what bounds a unit they are fetched while the unit ahead of it is worked on: their
+    // latency between two units was 1300 of a unit's 8800 clocks (256 columns, Swish).
+    constexpr bool AHEAD = CTA2 && EW == 8;
+    const bool ahead = AHEAD && (RQ || p.act != AQT_ACT_NONE);
+    constexpr int PRE = AHEAD && Cfg::kScaleSlab ? BN / 32 / (EW / 4) : 1;
     float pre_w[PRE], pre_b[PRE], pre_sx = 1.0f;
     const auto prefetch_scales = [&](int i) {
       int ptm, ptn, ppart;
       if (!unit_at<WS, CTA2, HALVES>(p, i, ptm, ptn, ppart)) return;
-      if (!WS && Cfg::kScaleSlab) {
+      if (AHEAD && Cfg::kScaleSlab) {
         const int chunks = ppart == 0 ? chunks_whole : chunks_whole / 2;
         const int n0 = ptn * out_cols_tile + (ppart == 2 ? out_cols_tile / 2 : 0) + chalf * chunks * 32 + lane;
 #pragma unroll
@@ -884,7 +886,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         pre_sx = p.s_x_kind == AQT_SCALE_ROW ? (pm < p.M ? __ldg(p.s_x + pm) : 0.0f) : __ldg(p.s_x);
       }
     };
-    if (AHEAD) prefetch_scales(0);
+    if (ahead) prefetch_scales(0);
     // residual prefetch for the very first chunk of this warp
     if (ok && has_res && lane == 0 && unit_at<WS, CTA2, HALVES>(p, 0, tm, tn, part)) {
       const int oc0 = tn * out_cols_tile + (part == 2 ? out_cols_tile / 2 : 0) + chalf * (part == 0 ? chunks_whole : chunks_whole / 2) * 32, r0 = tm * TILE_M + row_in_tile + quad * 32;
@@ -901,19 +903,50 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
       const int m = row0_warp + lane;
       const bool row_ok = m < p.M;
 
-      if (!AHEAD) prefetch_scales(i);
-      if (!WS && Cfg::kScaleSlab) {
-        // this warp's s_w / bias slices for the tile -> shared memory (before the accumulator is ready)
+      float sx;
+      if constexpr (AHEAD) {
+        if (!ahead) prefetch_scales(i);
         __syncwarp();
+        if (Cfg::kScaleSlab) {
 #pragma unroll
-        for (int c = 0; c < PRE; ++c) {
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + c * 128 + lane * 4), "f"(pre_w[c]) : "memory");
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + c * 128 + lane * 4), "f"(pre_b[c]) : "memory");
+          for (int c = 0; c < PRE; ++c) {
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + c * 128 + lane * 4), "f"(pre_w[c]) : "memory");
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + c * 128 + lane * 4), "f"(pre_b[c]) : "memory");
+          }
         }
+        sx = pre_sx;
+        __syncwarp();
+        if (ahead) prefetch_scales(i + 1);
+      } else {
+        if (!WS && Cfg::kScaleSlab) {
+          // this warp's s_w / bias slices for the tile -> shared memory (before the accumulator is ready)
+          __syncwarp();
+          for (int c = 0; c < chunks; ++c) {
+            const int col = (chalf * chunks + c) * 32;
+            const int nv = out0 + col + lane;  // value channel of this lane
+            const uint32_t off = c * slab_chunk_stride + lane * 4;
+            float wv = 0.0f, bv = 0.0f;
+            if (nv < n_value_limit) {
+              wv = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + nv);
+              if (p.bias != nullptr) bv = __ldg(p.bias + nv);
+            }
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + off), "f"(wv) : "memory");
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + off), "f"(bv) : "memory");
+            if (glu) {
+              const int ng = p.N / 2 + out0 + col + lane;  // gate channel
+              float wg = 0.0f, bg = 0.0f;
+              if (ng < p.N) {
+                wg = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + ng);
+                if (p.bias != nullptr) bg = __ldg(p.bias + ng);
+              }
+              asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + off + slab_gate_off), "f"(wg) : "memory");
+              asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + off + slab_gate_off), "f"(bg) : "memory");
+            }
+          }
+        }
+        sx = TF32 ? 1.0f : ((p.s_x_kind == AQT_SCALE_ROW) ? (row_ok ? __ldg(p.s_x + m) : 0.0f) : __ldg(p.s_x));
+        __syncwarp();
       }
-      const float sx = pre_sx;
-      __syncwarp();
-      if (AHEAD) prefetch_scales(i + 1);
       float rq_amax = 0.0f;  // RQ: maximum of this thread's row over this warp's columns
 
       if (!mbar_wait(smem_u32(&tmem_full_bar[buf]), aph, &abort_flag, t_start)) break;
