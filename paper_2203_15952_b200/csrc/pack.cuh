@@ -231,9 +231,10 @@ __global__ void __launch_bounds__(256) half_operands_kernel(const float* __restr
     uint32_t h[4];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const float f[4] = {v[i][j].x * scale, v[i][j].y * scale, v[i][j].z * scale, v[i][j].w * scale};
+      const float u[4] = {v[i][j].x, v[i][j].y, v[i][j].z, v[i][j].w};
+      const float f[4] = {u[0] * scale, u[1] * scale, u[2] * scale, u[3] * scale};
 #pragma unroll
-      for (int k = 0; k < 4; ++k) wide = wide || (fabsf(f[k]) < 6.103515625e-05f && f[k] != 0.0f);
+      for (int k = 0; k < 4; ++k) wide = wide || (fabsf(f[k]) < 6.103515625e-05f && u[k] != 0.0f);  // (f itself may have become zero)
       const __half2 a = __floats2half2_rn(f[0], f[1]), b = __floats2half2_rn(f[2], f[3]);
       h[2 * j] = *reinterpret_cast<const uint32_t*>(&a);
       h[2 * j + 1] = *reinterpret_cast<const uint32_t*>(&b);
