@@ -568,6 +568,50 @@ __device__ __forceinline__ bool rows_wide(const GemmParams& p, int row0) {
   return __any_sync(0xffffffffu, least < 0.0f) != 0;
 }
 
+// Scales and biases of an epilogue warp's columns (GLU: of a chunk's values, then of its gates) and the scale of a thread's row, for
+// one unit of a CTA-pair tile: their latency between two units was 1300 of a unit's 8800 clocks (256 columns, Swish).  A struct and
+// a function that other forms do not instantiate: the same lines as a lambda in the kernel cost the sixteen-warp tiles, which never
+// called it, 32 bytes of spills (65 536 x 1024 -> 4096 Swish 368 -> 405 us, 25 033 x 1408 -> 3808 168.2 -> 171.4).
+template <int COUNT>
+struct UnitScales {
+  static constexpr int kCount = COUNT;
+  float w[COUNT], b[COUNT], sx = 1.0f;
+};
+template <>
+struct UnitScales<0> {};
+
+// The i-th unit's (COUNT chunks of 32 columns a warp, eight epilogue warps; row: this thread's in the tile); nothing beyond the last unit.
+template <int BN, bool SLAB, int ACCK, bool HALVES, int COUNT>
+__device__ __forceinline__ void unit_scales(const GemmParams& p, int i, int chalf, int row, UnitScales<COUNT>& pre) {
+  constexpr int TILE_M = 2 * kBM;
+  const bool glu = (p.act == AQT_ACT_GLU) || (p.act == AQT_ACT_GLU_SWISH);
+  int tm, tn, part;
+  if (!unit_at<false, true, HALVES>(p, i, tm, tn, part)) return;
+  if (SLAB) {
+    const int out_cols_tile = glu ? BN / 2 : BN, chunks_whole = out_cols_tile / 32 / 2;
+    const int chunks = part == 0 ? chunks_whole : chunks_whole / 2;
+    const int n0 = tn * out_cols_tile + (part == 2 ? out_cols_tile / 2 : 0) + chalf * chunks * 32 + (int)(threadIdx.x & 31);
+#pragma unroll
+    for (int c = 0; c < COUNT; ++c) {
+      const int n = glu ? n0 + (c >> 1) * 32 + ((c & 1) ? p.N / 2 : 0) : n0 + c * 32;
+      const int limit = glu && !(c & 1) ? p.N / 2 : p.N;
+      const bool there = c < (glu ? 2 * chunks : chunks) && n < limit;
+      pre.w[c] = pre.b[c] = 0.0f;
+      if (there) {
+        pre.w[c] = ACCK == kAccFloat && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + n);
+        if (p.bias != nullptr) pre.b[c] = __ldg(p.bias + n);
+      }
+    }
+  }
+  const int m = tm * TILE_M + row;
+  if constexpr (ACCK == kAccHalf) {
+    const bool wide = rows_wide<TILE_M>(p, tm * TILE_M);
+    pre.sx = m < p.M && !wide ? __ldg(p.s_x + m) : 1.0f;
+  } else if constexpr (ACCK != kAccFloat) {
+    pre.sx = p.s_x_kind == AQT_SCALE_ROW ? (m < p.M ? __ldg(p.s_x + m) : 0.0f) : __ldg(p.s_x);
+  }
+}
+
 // RQ (CTA pairs, no GLU): the epilogue also quantizes the output rows for the next layer (Fig. 2 of
 // the paper on u = what the plain epilogue writes): pass 1 is the plain epilogue, which also keeps
 // the row maxima and writes u back over its accumulators; every thread then publishes the maximum
@@ -616,7 +660,8 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const uint64_t t_start = global_timer_ns();
-  const bool glu = (p.act == AQT_ACT_GLU) || (p.act == AQT_ACT_GLU_SWISH);
+  // (512 columns: no gates, which the host sees to; known here, it takes 36 bytes of spills from their sixteen warps)
+  const bool glu = BN != 512 && ((p.act == AQT_ACT_GLU) || (p.act == AQT_ACT_GLU_SWISH));
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -853,40 +898,14 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
     }
 
     int tm, tn, part;
-    // Pair tiles: scales and biases of this warp's columns (GLU: of a chunk's values, then of its gates) and the scale of this thread's row
-    // of the i-th unit.  Where the epilogue is what bounds a unit they are fetched while the unit ahead of it is worked on: their
-    // latency between two units was 1300 of a unit's 8800 clocks (256 columns, Swish).
+    // Pair tiles, where the epilogue is what bounds a unit: scales and biases are fetched while the unit ahead of it is worked on
+    // (see UnitScales).
     constexpr bool AHEAD = CTA2 && EW == 8;
     const bool ahead = AHEAD && (RQ || p.act != AQT_ACT_NONE);
-    constexpr int PRE = AHEAD && Cfg::kScaleSlab ? BN / 32 / (EW / 4) : 1;
-    float pre_w[PRE], pre_b[PRE], pre_sx = 1.0f;
-    const auto prefetch_scales = [&](int i) {
-      int ptm, ptn, ppart;
-      if (!unit_at<WS, CTA2, HALVES>(p, i, ptm, ptn, ppart)) return;
-      if (AHEAD && Cfg::kScaleSlab) {
-        const int chunks = ppart == 0 ? chunks_whole : chunks_whole / 2;
-        const int n0 = ptn * out_cols_tile + (ppart == 2 ? out_cols_tile / 2 : 0) + chalf * chunks * 32 + lane;
-#pragma unroll
-        for (int c = 0; c < PRE; ++c) {
-          const int n = glu ? n0 + (c >> 1) * 32 + ((c & 1) ? p.N / 2 : 0) : n0 + c * 32;
-          const int limit = glu && !(c & 1) ? p.N / 2 : p.N;
-          const bool there = c < (glu ? 2 * chunks : chunks) && n < limit;
-          pre_w[c] = pre_b[c] = 0.0f;
-          if (there) {
-            pre_w[c] = TF32 && p.s_w == nullptr ? 1.0f : __ldg(p.s_w + n);
-            if (p.bias != nullptr) pre_b[c] = __ldg(p.bias + n);
-          }
-        }
-      }
-      const int pm = ptm * TILE_M + row_in_tile + quad * 32 + lane;
-      if constexpr (HALFK) {
-        const bool wide = rows_wide<TILE_M>(p, ptm * TILE_M);
-        pre_sx = pm < p.M && !wide ? __ldg(p.s_x + pm) : 1.0f;
-      } else if constexpr (!TF32) {
-        pre_sx = p.s_x_kind == AQT_SCALE_ROW ? (pm < p.M ? __ldg(p.s_x + pm) : 0.0f) : __ldg(p.s_x);
-      }
-    };
-    if (ahead) prefetch_scales(0);
+    UnitScales<AHEAD ? (Cfg::kScaleSlab ? BN / 32 / (EW / 4) : 1) : 0> pre;
+    if constexpr (AHEAD) {
+      if (ahead) unit_scales<BN, Cfg::kScaleSlab, ACCK, HALVES>(p, 0, chalf, row_in_tile + quad * 32 + lane, pre);
+    }
     // residual prefetch for the very first chunk of this warp
     if (ok && has_res && lane == 0 && unit_at<WS, CTA2, HALVES>(p, 0, tm, tn, part)) {
       const int oc0 = tn * out_cols_tile + (part == 2 ? out_cols_tile / 2 : 0) + chalf * (part == 0 ? chunks_whole : chunks_whole / 2) * 32, r0 = tm * TILE_M + row_in_tile + quad * 32;
@@ -905,18 +924,18 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
 
       float sx;
       if constexpr (AHEAD) {
-        if (!ahead) prefetch_scales(i);
+        if (!ahead) unit_scales<BN, Cfg::kScaleSlab, ACCK, HALVES>(p, i, chalf, row_in_tile + quad * 32 + lane, pre);
         __syncwarp();
         if (Cfg::kScaleSlab) {
 #pragma unroll
-          for (int c = 0; c < PRE; ++c) {
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + c * 128 + lane * 4), "f"(pre_w[c]) : "memory");
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + c * 128 + lane * 4), "f"(pre_b[c]) : "memory");
+          for (int c = 0; c < pre.kCount; ++c) {
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_sw + c * 128 + lane * 4), "f"(pre.w[c]) : "memory");
+            asm volatile("st.shared.f32 [%0], %1;" ::"r"(slab_bias + c * 128 + lane * 4), "f"(pre.b[c]) : "memory");
           }
         }
-        sx = pre_sx;
+        sx = pre.sx;
         __syncwarp();
-        if (ahead) prefetch_scales(i + 1);
+        if (ahead) unit_scales<BN, Cfg::kScaleSlab, ACCK, HALVES>(p, i + 1, chalf, row_in_tile + quad * 32 + lane, pre);
       } else {
         if (!WS && Cfg::kScaleSlab) {
           // this warp's s_w / bias slices for the tile -> shared memory (before the accumulator is ready)
