@@ -519,8 +519,11 @@ qgemm_requant_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_cons
           for (int s = 1; s < split; ++s) amax = fmaxf(amax, part_amax[set + s][row_in_tile]);
         }
       }
+      // (Where sets share tiles and y is written, a register held for the tag is one too many beside the call of the general
+      // sequence, 8 bytes of spills: it is read again.)
       if (part == 0)
-        st_relaxed_gpu_64(rp.exchange + ((size_t)tm * p.tiles_n + tn) * kBM + row_in_tile, ((uint64_t)tag << 32) | __float_as_uint(amax));
+        st_relaxed_gpu_64(rp.exchange + ((size_t)tm * p.tiles_n + tn) * kBM + row_in_tile,
+                          ((uint64_t)(SHARED && WITH_Y ? *(volatile uint32_t*)&tag_slot : tag) << 32) | __float_as_uint(amax));
 
       // -------------------------------------------------------------- pass 2: scale, codes
       if (!mbar_wait(smem_u32(&ctx_ready_bar[buf][quad >> 1]), aph, &abort_flag, t_start)) { ok = false; break; }
