@@ -384,11 +384,14 @@ __global__ void __launch_bounds__(kQuantThreads) quantize_tensor_vec_kernel(cons
       const int64_t i = i0 + j * kQuantThreads;
       if (i >= n4) break;
       uint32_t w;
-      if (__builtin_expect(c.fast, 1))
+      if (__builtin_expect(c.fast, 1)) {
         w = pack4_i8(quantize_fast<ROUNDING>(v[j].x, c.s, c.r), quantize_fast<ROUNDING>(v[j].y, c.s, c.r), quantize_fast<ROUNDING>(v[j].z, c.s, c.r),
                      quantize_fast<ROUNDING>(v[j].w, c.s, c.r));
-      else
-        w = codes4_general(v[j].x, v[j].y, v[j].z, v[j].w, c.s, qmax, ROUNDING);
+      } else {
+        // (eight float4s held across the call are 24 bytes of spills at 64 registers; read again, 51 registers and none)
+        const float4 g = VEC > kTensorVec ? __ldg(tensor_vec(x, i, nvec, ld4)) : v[j];
+        w = codes4_general(g.x, g.y, g.z, g.w, c.s, qmax, ROUNDING);
+      }
       if (PACK) reinterpret_cast<uint16_t*>(q_out)[i] = (uint16_t)nibbles4(w);
       else reinterpret_cast<uint32_t*>(q_out)[i] = w;
     }
