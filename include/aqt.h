@@ -79,6 +79,11 @@ extern "C" {
 #define AQT_MAY_WAIT 0x200 /* may be OR-ed into bits_w of aqt_qmatmul_requant: whatever the shape, the call may run in a kernel
                               whose CTAs wait on one another (see there), and q_out and s_out are not xq and s_x. */
 
+/* may be OR-ed into bits_w of aqt_plan_qmatmul */
+#define AQT_PLAN_RESIDUAL 0x400    /* the call has a residual */
+#define AQT_PLAN_WEIGHT_ONLY 0x800 /* float_kind != 0: the call is aqt_linear_fwd_weight_only, precision AQT_FLOAT_TF32, more rows than its
+                                      one-launch form takes, with the workspace that the query asks for */
+
 /* operations for aqt_workspace_bytes */
 #define AQT_OP_QMATMUL 1
 #define AQT_OP_LINEAR_FWD 2
@@ -152,10 +157,11 @@ int aqt_qmatmul(const void* xq, const float* s_x, int s_x_kind, const void* wq, 
 
 /*
  * aqt_plan_qmatmul -- names the kernel configuration aqt_qmatmul (and every entry point that runs
- * the same matmul) would launch for a shape without a residual: "small_m", "few64", "ws128e16", "pair256s6e4", ...  Host-only:
+ * the same matmul) would launch for a shape: "small_m", "few64", "ws128e16", "pair256s6e4", ...  Host-only:
  * sm_count_or_0 > 0 plans for a device with that many multiprocessors, 0 for the current device
- * (148 if there is none).  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
- * aqt_linear_bwd with K in elements (tf32 operands; calls that take binary16 ones run "pair256s4e8").  (No counterpart in the paper: the choice of tile shapes is
+ * (148 if there is none).  bits_w may carry AQT_PLAN_RESIDUAL.  float_kind != 0 plans the float matmul of aqt_linear_fwd_weight_only /
+ * aqt_linear_bwd with K in elements (tf32 operands; with AQT_PLAN_WEIGHT_ONLY "pair256s4e8f16" for calls that take binary16
+ * ones).  (No counterpart in the paper: the choice of tile shapes is
  * this library's.)  name_out receives a NUL-terminated string of at most name_bytes bytes.
  */
 int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int float_kind,

@@ -29,6 +29,7 @@ FLOAT_TF32, FLOAT_TF32X2 = 0, 1
 BITS_4_UNPACKED = 48  # 4-bit codes, one per int8 container
 MAY_WAIT = 0x200  # OR into bits_w of aqt_qmatmul_requant: its CTAs may wait on one another whatever the shape
 STATIC_WEIGHTS = 0x100  # OR into bits_w: the weights were complete before the preceding work on the stream was enqueued
+PLAN_RESIDUAL, PLAN_WEIGHT_ONLY = 0x400, 0x800  # OR into bits_w of aqt_plan_qmatmul: the call has a residual; it is aqt_linear_fwd_weight_only
 
 EXPORTS = ("aqt_version", "aqt_status_string", "aqt_quantize", "aqt_pack_int4", "aqt_unpack_int4", "aqt_qmatmul",
            "aqt_linear_fwd", "aqt_linear_fwd_host", "aqt_workspace_bytes", "aqt_device_status", "aqt_qmatmul_w4_noalloc",

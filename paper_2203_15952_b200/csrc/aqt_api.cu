@@ -176,14 +176,31 @@ int float_gemm_nt(const float* a, int64_t lda, const float* b, int64_t rows, int
   return launch_qgemm(reinterpret_cast<const int8_t*>(a), b, false, y, ldy, p, st);
 }
 
-// True if the one-term weight-only layer's matmul runs on binary16 operands, twice the rate and half the bytes of tf32 ones for a
-// pass that scales and writes the rows first (6 bytes an element).  CTA pairs on 256 x 256 tiles; us in a replayed graph, tf32 /
-// binary16, both with their passes: 12 800 x 512 -> 2048 Swish 51.7 / 45.2, 5000 x 768 -> 3072 47.1 / 37.3, 30 000 x 1024 -> 2048
-// gated 162 / 130, 30 000 x 1024 -> 1024 98.4 / 95.7.  Not where the pass is much of the call (30 000 x 512 -> 512 39.7 / 41.0, 30 000 x
-// 2048 -> 512 98.6 / 117, 30 000 x 4096 -> 1024 321 / 348), the epilogue most of a tile (12 800 x 128 -> 1280 21.1 / 25.4), or the
-// work small (2000 x 512 -> 1024 11.2 / 12.0, 1024 x 512 -> 2048 12.5 / 13.9; but 3000 x 512 -> 1024 14.6 / 13.5).
-bool half_kind_applies(int64_t M, int64_t N, int64_t K) {
-  return K % 8 == 0 && K >= 256 && K <= kHalfMaxK && N >= 1024 && M >= 1024 && M * N * K >= 1300000000ll && tuning_env("AQT_NO_HALF") == nullptr;
+// Sizes at which calls of the one-term weight-only layer may run on binary16 operands, twice the rate and half the bytes of tf32 ones for
+// a pass that scales and writes the rows first (6 bytes an element).  What the workspace query goes by.  Not smaller outputs or deeper
+// rows, of which the pass is too much (us in a replayed graph, tf32 / binary16: 30 000 x 512 -> 512 39.7 / 41.0, 30 000 x 2048 -> 512 98.6 /
+// 117, 30 000 x 4096 -> 1024 321 / 348), nor less work (2000 x 512 -> 1024 11.2 / 12.0).
+bool half_kind_sizes(int64_t M, int64_t N, int64_t K) {
+  return K % 8 == 0 && K >= 256 && K <= kHalfMaxK && N >= 1024 && M >= 1024 && M * N >= ceil_div(1300000000ll, K) && tuning_env("AQT_NO_HALF") == nullptr;
+}
+
+// True if a call of such sizes does.  CTA pairs on 256 x 256 tiles; us in a replayed graph, tf32 / binary16, both with their passes:
+// 12 800 x 512 -> 2048 Swish 51.9 / 45.7, 5000 x 768 -> 3072 Swish 45.7 / 36.5, 30 000 x 1024 -> 2048 gated 158 / 129, 30 000 x 1024 -> 1024
+// 98.3 / 95.6.  Not where what a tile saves does not pay for the pass (over 480 sizes and activations; the line lies where both are equal):
+//   - one round of pairs saves once: K below 448, with gates 512 (1614 x 408 -> 2432 13.3 / 14.5, 3102 x 488 -> 1216 gated 14.3 / 15.4), and of
+//     fewer than 40 tiles, where tf32 ones run on narrow single-CTA tiles, below 900 (1024 x 640 -> 2048 Swish 14.0 / 14.7, 1698 x 840 ->
+//     1096 Swish 16.0 / 17.3; but 1254 x 1024 -> 1024, 20 tiles, 16.4 / 15.1);
+//   - an activation's epilogue is most of a tile: Swish below K = 320 (18 359 x 296 -> 1824 53.2 / 55.6); gates in two rounds below 416 (2629 x 344 ->
+//     2440 15.3 / 16.0), in more below 352 and N = 1536 (43 495 x 264 -> 1064 54.8 / 60.3; but 7122 x 304 -> 3192 0.865 of the time);
+//   - few columns to a row, whose pass is the larger part, and full rounds, in which pairs of tf32 tiles lose nothing: 31 595 x 648 -> 1096
+//     87.4 / 89.1 (with rounds less full 15 311 x 256 -> 1064 0.869, rows that L2 holds 5062 x 768 -> 1024 24.5 / 21.7).
+bool half_kind_applies(int64_t M, int64_t N, int64_t K, int act, int sms) {
+  if (!half_kind_sizes(M, N, K)) return false;
+  const int64_t pairs = sms / 2, tiles = ceil_div(M, 2 * kBM) * ceil_div(N, 256), rounds = ceil_div(tiles, pairs);
+  if (rounds == 1 && K < (tiles < 40 ? 900 : (is_glu(act) ? 512 : 448))) return false;
+  if (act == AQT_ACT_SWISH && K < 320) return false;
+  if (is_glu(act) && (rounds == 2 ? K < 416 : K < 352 && N < 1536)) return false;
+  return !(N < 1152 && K < 704 && M * K > (2 << 20) && 20 * tiles > 17 * rounds * pairs);
 }
 
 // True if the CTA-pair kernel with the row-quantizing epilogue takes the call: deep K, no GLU, int8
@@ -415,7 +432,7 @@ size_t aqt_workspace_bytes(int op, int64_t M, int64_t N, int64_t K, int bits_a, 
   bits_w &= ~(AQT_STATIC_WEIGHTS | AQT_MAY_WAIT);
   if (op == AQT_OP_QMATMUL) return ws_qmatmul(M, N, K, bits_a, bits_w);
   if (op == AQT_OP_LINEAR_FWD) return ws_linear(M, N, K, bits_w);
-  if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return half_kind_applies(M, N, K) ? half_layout(M, N, K).total : ws_weight_only(0, N, K, AQT_FLOAT_TF32);
+  if (op == AQT_OP_LINEAR_WEIGHT_ONLY) return half_kind_sizes(M, N, K) ? half_layout(M, N, K).total : ws_weight_only(0, N, K, AQT_FLOAT_TF32);
   if (op == AQT_OP_LINEAR_WEIGHT_ONLY_X2) return ws_weight_only(M, N, K, AQT_FLOAT_TF32X2);
   if (op == AQT_OP_LINEAR_BWD) return bwd_workspace(M, N, K);
   if (op == AQT_OP_FFN_FWD) return ffn_layout(M, K, N, bits_w, bits_w).total;
@@ -528,8 +545,10 @@ int aqt_qmatmul_with_plan(const char* plan, const void* xq, const float* s_x, in
 
 int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, int act, int float_kind, int sm_count_or_0,
                      char* name_out, size_t name_bytes) {
+  const bool residual = (bits_w & AQT_PLAN_RESIDUAL) != 0, weight_only = (bits_w & AQT_PLAN_WEIGHT_ONLY) != 0;
+  bits_w &= ~(AQT_PLAN_RESIDUAL | AQT_PLAN_WEIGHT_ONLY);
   if (name_out == nullptr || name_bytes == 0 || M <= 0 || N <= 0 || K <= 0 || !act_ok(act)) return AQT_ERR_BADARG;
-  if (!float_kind && (!bits_ok(bits_a) || !bits_ok(bits_w))) return AQT_ERR_BADARG;
+  if (!float_kind && (!bits_ok(bits_a) || !bits_ok(bits_w) || weight_only)) return AQT_ERR_BADARG;
   int sms = sm_count_or_0;
   if (sms <= 0) sms = sm_count();
   if (sms <= 0) sms = kDefaultSms;
@@ -538,8 +557,12 @@ int aqt_plan_qmatmul(int64_t M, int64_t N, int64_t K, int bits_a, int bits_w, in
     name = "small_m";
   } else if (const int bn = float_kind ? 0 : few_tiles_bn(M, N, K, act, -1, sms)) {
     name = gemm_plan_name(bn == 32 ? kPlanFew32 : (bn == 64 ? kPlanFew64 : kPlanFew128));
+  } else if (weight_only && half_kind_applies(M, N, K, act, sms)) {
+    name = "pair256s4e8f16";
   } else {
-    name = gemm_plan_name(plan_qgemm(GemmShape{M, N, float_kind ? 4 * K : K, act, float_kind ? 1 : 0, false}, sms));
+    GemmShape g = {M, N, float_kind ? 4 * K : K, act, float_kind ? 1 : 0, false, residual};
+    g.packed = !float_kind && is_packed(bits_w) && K % 32 == 0;  // (other rows of packed codes are expanded first, and then int8 ones)
+    name = gemm_plan_name(plan_qgemm(g, sms));
   }
   if (strlen(name) + 1 > name_bytes) return AQT_ERR_BADARG;
   memcpy(name_out, name, strlen(name) + 1);
@@ -1003,7 +1026,9 @@ int aqt_linear_fwd_weight_only(const float* x, int64_t ldx, const void* wq, cons
     a_pitch = 8 * K;
   }
   const HalfLayout H = half_layout(M, N, K);
-  const bool half = precision == AQT_FLOAT_TF32 && half_kind_applies(M, N, K) && workspace_bytes >= H.total;
+  const int sms = sm_count();
+  if (sms <= 0) return AQT_ERR_CUDA;
+  const bool half = precision == AQT_FLOAT_TF32 && workspace_bytes >= H.total && half_kind_applies(M, N, K, act, sms);
   uint8_t* ws = reinterpret_cast<uint8_t*>(workspace);
   const void* b_mm = w_f;
   if (half) {

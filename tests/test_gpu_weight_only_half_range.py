@@ -11,9 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("large,small", [(100, -70), (100, -60), (70, -100), (14, -120), (0, -120), (-90, -120), (100, -140), (40, -149)])
-@pytest.mark.parametrize("M,N,K", [(1024, 2048, 640), (2605, 1024, 520)])
+@pytest.mark.parametrize("M,N,K", [(1281, 4096, 256), (2605, 1024, 520)])
 def test_small_values_beside_a_large_one(M, N, K, large, small):
     """One large value a row, in channels whose code for it is zero: what is left are the small ones."""
+    assert aqt.aqt_plan_qmatmul(M, N, K, 0, 8 | aqt.PLAN_WEIGHT_ONLY, float_kind=True) == "pair256s4e8f16"
     g = torch.Generator(device="cuda").manual_seed(K)
     x = torch.randint(1, 4, (M, K), generator=g, device="cuda").double() * 2.0 ** small
     x[:, 0] = 2.0 ** large
