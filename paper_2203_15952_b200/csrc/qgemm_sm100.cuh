@@ -568,6 +568,53 @@ __device__ __forceinline__ bool rows_wide(const GemmParams& p, int row0) {
   return __any_sync(0xffffffffu, least < 0.0f) != 0;
 }
 
+// The half kind's inner loops, one for each sort of operands and apart from the other kinds' loop.  With all in one (maps by pointer, a
+// choice of instruction for each MMA) the matmul of 12 800 x 512 -> 2048 Swish by itself took 38.5 us, 59.2 with all tiles wide where
+// the float kind takes 51.1, and other kinds lost by the pointers (dx of 68 x 1792 -> 2464 24.7 -> 25.2); with these 37.6 and 52.0.
+template <int STAGES>
+struct PairRing {
+  static constexpr int kStages = STAGES;
+  uint32_t smem, full_bar, empty_bar;  // shared-memory addresses: the stages, and their barriers (eight bytes each)
+  int* abort_flag;
+  uint64_t t_start;
+};
+// Loads of one unit by this CTA (one thread).  False: a wait ran out.
+template <class Cfg, bool HALVES, int STAGES>
+__device__ __forceinline__ bool load_half_unit(const PairRing<STAGES>& ring, const CUtensorMap& map_a, const CUtensorMap& map_b, int k_blocks, int row_a,
+                                               int row_b, int part, uint32_t pair_rank, uint32_t& it) {
+  const uint32_t bytes = HALVES && part != 0 ? 2 * (Cfg::kABytes + Cfg::kBBytes / 2) : 2 * Cfg::kStageBytes;
+  for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
+    if (!mbar_wait(ring.empty_bar + 8 * s, ph ^ 1, ring.abort_flag, ring.t_start)) return false;
+    const uint32_t bar = ring.full_bar + 8 * s, stage = ring.smem + s * Cfg::kStageBytes;
+    if (pair_rank == 0) mbar_arrive_expect_tx(bar, bytes);
+    tma_load_2d_pair(stage, &map_a, kb * kBK, row_a, bar);
+    tma_load_2d_pair(stage + Cfg::kABytes, &map_b, kb * kBK, row_b, bar);
+    if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, &map_b, kb * kBK, row_b + 64, bar);
+  }
+  return true;
+}
+// MMAs of one unit (one thread of the leader).
+template <class Cfg, bool WIDE, int STAGES>
+__device__ __forceinline__ bool contract_half_unit(const PairRing<STAGES>& ring, int k_blocks, int mma_n, uint32_t d_tmem, uint32_t& it) {
+  const uint32_t idesc = WIDE ? idesc_tf32(mma_n, 2 * kBM) : idesc_f16(mma_n, 2 * kBM);
+  for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
+    if (!mbar_wait(ring.full_bar + 8 * s, ph, ring.abort_flag, ring.t_start)) return false;
+    tc_fence_after();
+    const uint32_t stage = ring.smem + s * Cfg::kStageBytes;
+    const uint64_t a_desc = smem_desc_k_major_sw128(stage), b_desc = smem_desc_k_major_sw128(stage + Cfg::kABytes);
+#pragma unroll
+    for (int kk = 0; kk < kBK / kMmaK; ++kk) {
+      const uint32_t accumulate = (kb | kk) != 0 ? 1u : 0u;
+      if (WIDE) tc_mma_tf32_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+      else tc_mma_f16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
+    }
+    tc_commit_pair(ring.empty_bar + 8 * s);
+  }
+  return true;
+}
+
 // Scales and biases of an epilogue warp's columns (GLU: of a chunk's values, then of its gates) and the scale of a thread's row, for
 // one unit of a CTA-pair tile: their latency between two units was 1300 of a unit's 8800 clocks (256 columns, Swish).  A struct and
 // a function that other forms do not instantiate: the same lines as a lambda in the kernel cost the sixteen-warp tiles, which never
@@ -759,16 +806,18 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
         const int half_cols = part == 0 ? HALF : HALF / 2;
         const int row0 = (glu ? tn * HALF : tn * BN) + (part == 2 ? (glu ? HALF / 2 : HALF) : 0);
         const int row1 = glu ? p.N / 2 + row0 : row0 + half_cols;
-        const CUtensorMap *map_a = &tm_a, *map_b = &tm_b;
-        int k_blocks = p.k_blocks;
         if constexpr (HALFK) {
-          if (rows_wide<TILE_M>(p, tm * TILE_M)) {
-            map_a = &wm.a;
-            map_b = &wm.b;
-            k_blocks = p.wide_k_blocks;
+          const bool wide = rows_wide<TILE_M>(p, tm * TILE_M);
+          if (lane == 0) {
+            const int row_b = pair_rank == 0 ? row0 : row1;
+            const PairRing<STAGES> ring = {smem_ring, smem_u32(full_bar), smem_u32(empty_bar), &abort_flag, t_start};
+            ok = wide ? load_half_unit<Cfg, HALVES>(ring, wm.a, wm.b, p.wide_k_blocks, tm * TILE_M + row_in_tile, row_b, part, pair_rank, it)
+                      : load_half_unit<Cfg, HALVES>(ring, tm_a, tm_b, p.k_blocks, tm * TILE_M + row_in_tile, row_b, part, pair_rank, it);
           }
+          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          continue;
         }
-        for (int kb = 0; (!HALFK || lane == 0) && kb < k_blocks; ++kb, ++it) {
+        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1, &abort_flag, t_start)) { ok = false; break; }
           const uint32_t bar = smem_u32(&full_bar[s]);
@@ -777,61 +826,61 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             // The leader's barrier counts both CTAs' bytes; each CTA loads its 128 rows of A and
             // its half of the weight rows (leader: first half / values, peer: second half / gates).
             if (pair_rank == 0) mbar_arrive_expect_tx(bar, HALVES && part != 0 ? 2 * (Cfg::kABytes + Cfg::kBBytes / 2) : 2 * Cfg::kStageBytes);
-            tma_load_2d_pair(stage, map_a, kb * kBK, tm * TILE_M + row_in_tile, bar);
+            tma_load_2d_pair(stage, &tm_a, kb * kBK, tm * TILE_M + row_in_tile, bar);
             if (BN == 512) {
               // two MMAs of 256 columns per k-step: this CTA supplies 128 weight rows to each
               const int r = tn * BN + (int)pair_rank * 128;
-              tma_load_2d_pair(stage + Cfg::kABytes, map_b, kb * kBK, r, bar);
-              tma_load_2d_pair(stage + Cfg::kABytes + 128 * kBK, map_b, kb * kBK, r + 256, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes + 128 * kBK, &tm_b, kb * kBK, r + 256, bar);
             } else {
               const int r = pair_rank == 0 ? row0 : row1;
-              tma_load_2d_pair(stage + Cfg::kABytes, map_b, kb * kBK, r, bar);
+              tma_load_2d_pair(stage + Cfg::kABytes, &tm_b, kb * kBK, r, bar);
               // (boxes of half a CTA's rows, so that half a tile is one of them)
-              if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, map_b, kb * kBK, r + HALF / 2, bar);
+              if (HALVES && part == 0) tma_load_2d_pair(stage + Cfg::kABytes + Cfg::kBBytes / 2, &tm_b, kb * kBK, r + HALF / 2, bar);
             }
             continue;
           }
           mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-          tma_load_2d(stage, map_a, kb * kBK, tm * kBM, bar);
+          tma_load_2d(stage, &tm_a, kb * kBK, tm * kBM, bar);
           if (!WS) {
             const int b_batch = p.batch_tiles_m > 0 ? (tm / p.batch_tiles_m) * p.batch_b_rows : 0;  // this batch's rows of B
-            tma_load_2d(stage + Cfg::kABytes, map_b, kb * kBK, row0 + b_batch, bar);
-            tma_load_2d(stage + Cfg::kABytes + HALF * kBK, map_b, kb * kBK, row1 + b_batch, bar);
+            tma_load_2d(stage + Cfg::kABytes, &tm_b, kb * kBK, row0 + b_batch, bar);
+            tma_load_2d(stage + Cfg::kABytes + HALF * kBK, &tm_b, kb * kBK, row1 + b_batch, bar);
           }
         }
-        if constexpr (HALFK) ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
       grid_dependents_launch();  // every load of this CTA has been issued: the next kernel may be scheduled behind it
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if ((HALFK || lane == 0) && pair_rank == 0) {
-      constexpr uint32_t idesc_whole = HALFK ? idesc_f16(Cfg::kMmaN, TILE_M) : (TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M));
-      constexpr uint32_t idesc_half = HALFK ? idesc_f16(Cfg::kMmaN / 2, TILE_M) : (TF32 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_i8(Cfg::kMmaN / 2, TILE_M));
+      constexpr uint32_t idesc_whole = TF32 ? idesc_tf32(Cfg::kMmaN, TILE_M) : idesc_i8(Cfg::kMmaN, TILE_M);
+      constexpr uint32_t idesc_half = TF32 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_i8(Cfg::kMmaN / 2, TILE_M);
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       if (WS) ok = mbar_wait(smem_u32(BPACK ? &b_ready_bar : &b_loaded_bar), 0, &abort_flag, t_start);
       int tm, tn, part;
       for (int i = 0; ok && unit_at<WS, CTA2, HALVES>(p, i, tm, tn, part); ++i, ++tcount) {
-        uint32_t idesc = HALVES && part != 0 ? idesc_half : idesc_whole;
-        int k_blocks = p.k_blocks;
-        bool wide = false;
-        if constexpr (HALFK) {
-          wide = rows_wide<TILE_M>(p, tm * TILE_M);
-          if (wide) {
-            k_blocks = p.wide_k_blocks;
-            idesc = HALVES && part != 0 ? idesc_tf32(Cfg::kMmaN / 2, TILE_M) : idesc_tf32(Cfg::kMmaN, TILE_M);
-          }
-        }
+        const uint32_t idesc = HALVES && part != 0 ? idesc_half : idesc_whole;
         const uint32_t buf = tcount % Cfg::kAccBufs, aph = (tcount / Cfg::kAccBufs) & 1;
         if constexpr (HALFK) {
-          if (lane == 0) ok = mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start);
-        } else {
-          if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
+          const bool wide = rows_wide<TILE_M>(p, tm * TILE_M);
+          if (lane == 0) {
+            const PairRing<STAGES> ring = {smem_ring, smem_u32(full_bar), smem_u32(empty_bar), &abort_flag, t_start};
+            const int mma_n = HALVES && part != 0 ? Cfg::kMmaN / 2 : Cfg::kMmaN;
+            ok = mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start);
+            tc_fence_after();
+            if (ok) ok = wide ? contract_half_unit<Cfg, true>(ring, p.wide_k_blocks, mma_n, tmem_base + buf * BN, it)
+                              : contract_half_unit<Cfg, false>(ring, p.k_blocks, mma_n, tmem_base + buf * BN, it);
+            if (ok) tc_commit_pair(smem_u32(&tmem_full_bar[buf]));  // accumulator complete in both CTAs' TMEM
+          }
+          ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+          continue;
         }
+        if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = 0; (!HALFK || (lane == 0 && ok)) && kb < k_blocks; ++kb, ++it) {
+        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&full_bar[s]), ph, &abort_flag, t_start)) { ok = false; break; }
           tc_fence_after();
@@ -842,9 +891,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           for (int kk = 0; kk < kBK / kMmaK; ++kk) {
             // advancing K inside the 128-byte swizzle row: +32 bytes = +2 in the 16-byte address field
             const uint32_t accumulate = (kb | kk) != 0 ? 1u : 0u;
-            if (HALFK && !wide) {
-              tc_mma_f16_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
-            } else if (TF32 || HALFK) {
+            if (TF32) {
               if (CTA2) tc_mma_tf32_pair(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
               else tc_mma_tf32(d_tmem, a_desc + 2 * kk, b_desc + 2 * kk, idesc, accumulate);
             } else {
@@ -858,11 +905,10 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           if (CTA2) tc_commit_pair(smem_u32(&empty_bar[s]));
           else tc_commit(smem_u32(&empty_bar[s]));
         }
-        if (ok && (!HALFK || lane == 0)) {  // accumulator complete (in both CTAs' TMEM)
+        if (ok) {  // accumulator complete (in both CTAs' TMEM)
           if (CTA2) tc_commit_pair(smem_u32(&tmem_full_bar[buf]));
           else tc_commit(smem_u32(&tmem_full_bar[buf]));
         }
-        if constexpr (HALFK) ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       }
     }
   } else {
