@@ -187,7 +187,7 @@ bool half_kind_sizes(int64_t M, int64_t N, int64_t K) {
 // True if a call of such sizes does.  CTA pairs on 256 x 256 tiles; us in a replayed graph, tf32 / binary16, both with their passes:
 // 12 800 x 512 -> 2048 Swish 51.7 / 44.2, 5000 x 768 -> 3072 Swish 48.3 / 37.2, 30 000 x 1024 -> 2048 gated 161 / 128, 30 000 x 1024 -> 1024
 // 100 / 96.  An input with a wide row in every block of 256 (GemmParams::wide_a) pays for the pass and gains nothing: 51.9 / 59.2, 47.5 / 51.7,
-// 173 / 214, 104 / 138; of normal values every 600th such block of 512 columns has one.
+// 173 / 214, 104 / 138; of normal values one block in 800 has one (512 columns).
 // Not where what a tile saves does not pay for the pass (over 480 sizes and activations; the line lies where both are equal):
 //   - one round of pairs saves once: K below 448, with gates 512 (1614 x 408 -> 2432 13.3 / 14.5, 3102 x 488 -> 1216 gated 14.3 / 15.4), and of
 //     fewer than 40 tiles, where tf32 ones run on narrow single-CTA tiles, below 900 (1024 x 640 -> 2048 Swish 14.0 / 14.7, 1698 x 840 ->

@@ -815,9 +815,8 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
                       : load_half_unit<Cfg, HALVES>(ring, tm_a, tm_b, p.k_blocks, tm * TILE_M + row_in_tile, row_b, part, pair_rank, it);
           }
           ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-          continue;
         }
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
+        for (int kb = 0; !HALFK && kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1, &abort_flag, t_start)) { ok = false; break; }
           const uint32_t bar = smem_u32(&full_bar[s]);
@@ -875,12 +874,11 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
             if (ok) tc_commit_pair(smem_u32(&tmem_full_bar[buf]));  // accumulator complete in both CTAs' TMEM
           }
           ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-          continue;
         }
-        if (!mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
+        if (!HALFK && !mbar_wait(smem_u32(&tmem_empty_bar[buf]), aph ^ 1, &abort_flag, t_start)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * BN;
-        for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
+        for (int kb = 0; !HALFK && kb < p.k_blocks; ++kb, ++it) {
           const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
           if (!mbar_wait(smem_u32(&full_bar[s]), ph, &abort_flag, t_start)) { ok = false; break; }
           tc_fence_after();
@@ -905,7 +903,7 @@ qgemm_i8_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant_
           if (CTA2) tc_commit_pair(smem_u32(&empty_bar[s]));
           else tc_commit(smem_u32(&empty_bar[s]));
         }
-        if (ok) {  // accumulator complete (in both CTAs' TMEM)
+        if (!HALFK && ok) {  // accumulator complete (in both CTAs' TMEM)
           if (CTA2) tc_commit_pair(smem_u32(&tmem_full_bar[buf]));
           else tc_commit(smem_u32(&tmem_full_bar[buf]));
         }
