@@ -1557,10 +1557,13 @@ static int plan_qgemm(const GemmShape& g, int sms) {
   const int pairs = sms / 2;
   if (!g.batched && qgemm_uses_ws(g.N, g.K, sms)) {
     // With a residual, whose rows every tile waits for, the slab that a CTA loads first and its place in shared memory give
-    // nothing back: single-CTA tiles that stream both operands, and pairs of 128 columns from some 28 M outputs on (us,
-    // weight-stationary / streamed / pairs, inputs not in L2: 7411 x 512 -> 512 12.3 / 11.5 / 11.7, 25 600 rows 24.0 / 23.7 / 24.8,
-    // 65 536 rows 55.3 / 52.7 / 50.4, 65 536 x 512 -> 2048 206 / 188 / 176; without a residual the slab is the better use).
-    if (g.residual && !g.packed && !f32 && g.act == AQT_ACT_NONE) return g.M * g.N >= (28ll << 20) ? kPlanPair128S6E8 : kPlanStream128S4E16;
+    // nothing back: single-CTA tiles that stream both operands, and pairs of 128 columns from some 28 M outputs on, below K = 256, where
+    // a tile is little more than its epilogue, from some 88 M (us, weight-stationary / streamed / pairs, inputs not in L2: 7411 x 512 ->
+    // 512 11.8 / 11.3 / 11.3, 25 600 rows 25.0 / 24.6 / 25.5, 65 536 rows 56.0 / 56.0 / 53.9; 32 768 x 512 -> 1024 55.0 / 51.2 / 50.5;
+    // 65 536 x 64 -> 512 48.5 / 48.1 / 50.5, 22 356 x 64 -> 2208 72.4 / 71.0 / 77.1, 33 685 x 128 -> 3904 201 / 180 / 169; without a
+    // residual the slab is the better use).
+    if (g.residual && !g.packed && !f32 && g.act == AQT_ACT_NONE)
+      return g.M * g.N >= ((g.K >= 256 ? 28ll : 88ll) << 20) ? kPlanPair128S6E8 : kPlanStream128S4E16;
     return glu ? kPlanWs128E8 : kPlanWs128E16;  // a GLU tile has 64 output columns
   }
   const int64_t pair_tiles = ceil_div(g.M, 2 * kBM) * ceil_div(g.N, 256);  // 256 x 256 tiles
