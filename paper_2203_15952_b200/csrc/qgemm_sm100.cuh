@@ -368,11 +368,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // sigmoid(z) = 1 / (1 + e^-z) with e^-z = 2^(-z log2 e): one multiply, the special-function
 // unit's 2^t, one add, its reciprocal.  Five instructions with the caller's final multiply, two of
