@@ -29,3 +29,51 @@ def test_small_values_beside_a_large_one(M, N, K, large, small):
         z, mag = x.double() @ wq.double().t(), x.double().abs() @ wq.double().abs().t()
         assert ((y.double() - z).abs() <= (2.0 ** -10 + K * 2.0 ** -24) * mag + 2.0 ** -23 * z.abs()).all()
     assert aqt.aqt_device_status() == 0
+
+
+def _pair(x, wq, N, K):
+    """The call with the workspace asked for, and with room for tf32 operands alone."""
+    s_w = torch.ones(N, device="cuda")
+    ws = torch.empty(aqt.aqt_workspace_bytes(aqt.OP_LINEAR_WEIGHT_ONLY, x.shape[0], N, K, 0, 8), dtype=torch.uint8, device="cuda")
+    out = [aqt.aqt_linear_fwd_weight_only(x, wq, s_w, None, bits_w=8, y=torch.empty(x.shape[0], N, device="cuda"), workspace=w)
+           for w in (ws, ws[:4 * N * K])]
+    assert aqt.aqt_device_status() == 0
+    return out
+
+
+@pytest.mark.parametrize("M,N,K", [(2605, 1024, 520), (1281, 4096, 256)])
+def test_a_wide_row_changes_its_block_of_rows_alone(M, N, K):
+    """Blocks without one run on binary16: rounded to nearest, where tf32 operands are cut off, so half the error (0.29 and 0.58 units rms)."""
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn(M, K, generator=g, device="cuda")
+    x[x.abs() < 1e-6] = 0.0
+    wq = torch.randint(-127, 128, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    plain, tf32 = _pair(x, wq, N, K)
+    z = x.double() @ wq.double().t()
+    blocks = range(0, M, 256)
+    for b in blocks:
+        e, e32 = ((y[b:b + 256].double() - z[b:b + 256]).square().mean().sqrt() for y in (plain, tf32))
+        assert e < 0.75 * e32
+    x[700, 5] = 1e-12
+    x[M - 1, 1] = -1e-30
+    marked, tf32 = _pair(x, wq, N, K)
+    for b in blocks:
+        want = tf32 if b in (512, (M - 1) // 256 * 256) else plain
+        assert torch.equal(marked[b:b + 256].view(torch.int32), want[b:b + 256].view(torch.int32))
+
+
+def test_rows_at_the_ends_of_the_scales():
+    """Blocks of rows whose values are all of one size: from 2^-100 up to 2^101 they run on binary16, beyond on tf32 operands."""
+    g = torch.Generator(device="cuda").manual_seed(3)
+    exps, N, K = [-100, -101, 100, 101, 0, -126, 127 - 20], 4096, 256
+    x = torch.cat([(1 + torch.rand(256, K, generator=g, device="cuda")) * torch.randn(256, K, generator=g, device="cuda").sign() * 2.0 ** e for e in exps])
+    assert (x.abs() < 2 * 2.0 ** torch.tensor(exps, device="cuda").repeat_interleave(256)[:, None]).all()
+    wq = torch.randint(-127, 128, (N, K), generator=g, device="cuda", dtype=torch.int8)
+    y, tf32 = _pair(x, wq, N, K)
+    z, mag = x.double() @ wq.double().t(), x.double().abs() @ wq.double().abs().t()
+    for i, e in enumerate(exps):
+        r = slice(256 * i, 256 * i + 256)
+        half = -100 <= e <= 100
+        assert torch.equal(y[r], tf32[r]) == (not half)
+        bound = ((2.0 ** -11 if half else 2.0 ** -10) + K * 2.0 ** -24) * mag[r] + 2.0 ** -23 * z[r].abs()
+        assert ((y[r].double() - z[r]).abs() <= bound).all()
