@@ -350,13 +350,13 @@ int aqt_chain_fwd(const float* x, int64_t ldx, int64_t M, const aqt_chain_layer*
  * the exact value of the formula, and equals it bit for bit when every x is a tf32 value and no
  * partial sum needs more than 24 bits.
  * Larger calls (256 <= K <= 1024, K % 8 == 0, N >= 1024, M >= 1024, M * N * K >= 1.3e9, of those the ones that are faster so:
- * aqt_plan_qmatmul with AQT_PLAN_WEIGHT_ONLY tells) take the same eleven significant bits, rounded to nearest, as binary16
- * operands at twice the rate: each row is scaled by a power of two (undone exactly afterwards), and blocks of 256 rows (counted from
- * row 0) with a value that is not finite, smaller than 2^-28 of its row's largest and not zero, or in a row whose largest is not zero and
- * below 2^-100 or at least 2^101, keep the tf32 operands.  So the bits of a row's result depend on whether a row of its block is such a
- * row, as they do on M, N, K, act and the workspace through the choice of the form; its error is within the bound above in each
- * form.  A caller that wants a row's result to be the same bits whatever the other rows hold passes a workspace of
- * the size that the query gives for M = 0, with which no call takes the binary16 operands.
+ * aqt_plan_qmatmul with AQT_PLAN_WEIGHT_ONLY tells) take the same eleven significant bits, cut off as the tensor core cuts tf32
+ * operands, as binary16 operands at twice the rate: each row is scaled by a power of two (undone exactly afterwards), and blocks
+ * of 256 rows (counted from row 0) with a value that is not finite, smaller than 2^-28 of its row's largest and not zero, or in a row
+ * whose largest is not zero and below 2^-100 or at least 2^101, keep the tf32 operands.  The products are the same in either form, and
+ * so are the results up to the order in which binary32 sums are formed (2e-8 of their norm, one result in thirty by a last
+ * bit).  A caller that wants a row's result to be the same bits whatever the other rows hold, and whatever M, N and act are, passes a
+ * workspace of the size that the query gives for M = 0, with which no call takes the binary16 operands.
  * precision AQT_FLOAT_TF32: as just described.  AQT_FLOAT_TF32X2: every activation is split
  *           exactly into hi (its tf32 part) + lo, and one matmul over [hi | lo] against the
  *           weights repeated sums both terms: the operand error drops from 2^-10 to 2^-20 of

@@ -160,10 +160,11 @@ __global__ void __launch_bounds__(256) codes_to_float_twice_kernel(const uint8_t
 }
 
 // Operands of the half kind of the matmul (K % 8 == 0, K <= 16 G, G 32 or 64).  Blocks 0 .. row_blocks - 1: rows of x as binary16, scaled by the
-// power of two that brings a row's largest magnitude into [2^14, 2^15): eleven significant bits of every value down to 2^-28 of
-// the largest, rounded to nearest (a tf32 operand has the same eleven, cut off).  inv[m]: the inverse of the scale, or -1 for a
-// row with values that are smaller and not zero, not finite, or near the ends of binary32's range.  G threads to a row.  The other
-// blocks: the weights' codes as binary16 and as binary32, which tiles with such a row read.
+// power of two that brings a row's largest magnitude into [2^14, 2^15): the upper eleven significant bits of every value down to 2^-28 of
+// the largest, cut off as the tensor core cuts tf32 operands, so that products are the same whichever of the two a tile takes
+// (rounded to nearest they have half the error, and results that are 6e-4 from the tf32 form's).  inv[m]: the inverse of the scale, or -1
+// for a row with values that are smaller and not zero, not finite, or near the ends of binary32's range.  G threads to a row.  The
+// other blocks: the weights' codes as binary16 and as binary32, which tiles with such a row read.
 template <int G>
 __global__ void __launch_bounds__(256) half_operands_kernel(const float* __restrict__ x, int64_t ldx, int M, int K, __half* __restrict__ xh,
                                                             float* __restrict__ inv, int row_blocks, const uint8_t* __restrict__ codes, bool packed, int64_t n,
@@ -235,9 +236,8 @@ __global__ void __launch_bounds__(256) half_operands_kernel(const float* __restr
       const float f[4] = {u[0] * scale, u[1] * scale, u[2] * scale, u[3] * scale};
 #pragma unroll
       for (int k = 0; k < 4; ++k) wide = wide || (fabsf(f[k]) < 6.103515625e-05f && u[k] != 0.0f);  // (f itself may have become zero)
-      const __half2 a = __floats2half2_rn(f[0], f[1]), b = __floats2half2_rn(f[2], f[3]);
-      h[2 * j] = *reinterpret_cast<const uint32_t*>(&a);
-      h[2 * j + 1] = *reinterpret_cast<const uint32_t*>(&b);
+      asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(h[2 * j]) : "f"(f[1]), "f"(f[0]));  // (the first source is the upper half)
+      asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(h[2 * j + 1]) : "f"(f[3]), "f"(f[2]));
     }
     reinterpret_cast<uint4*>(xh + (int64_t)m * K)[c] = make_uint4(h[0], h[1], h[2], h[3]);
   }
