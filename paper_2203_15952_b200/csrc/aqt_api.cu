@@ -189,20 +189,22 @@ bool half_kind_sizes(int64_t M, int64_t N, int64_t K) {
 // 100 / 96.  An input with a wide row in every block of 256 (GemmParams::wide_a) pays for the pass and gains nothing: 51.9 / 59.2, 47.5 / 51.7,
 // 173 / 214, 104 / 138; of normal values one block in 800 has one (512 columns).
 // Not where what a tile saves does not pay for the pass (over 480 sizes and activations; the line lies where both are equal):
-//   - one round of pairs saves once: K below 448, with gates 512 (1614 x 408 -> 2432 13.3 / 14.5, 3102 x 488 -> 1216 gated 14.3 / 15.4), and of
+//   - one round of pairs saves once: K below 496, with gates 512 (1614 x 408 -> 2432 13.3 / 14.5, 3102 x 488 -> 1216 gated 14.3 / 15.4), and of
 //     fewer than 40 tiles, where tf32 ones run on narrow single-CTA tiles, below 900 (1024 x 640 -> 2048 Swish 14.0 / 14.7, 1698 x 840 ->
 //     1096 Swish 16.0 / 17.3; but 1254 x 1024 -> 1024, 20 tiles, 16.4 / 15.1);
 //   - an activation's epilogue is most of a tile: Swish below K = 320 (18 359 x 296 -> 1824 53.2 / 55.6); gates in two rounds below 416 (2629 x 344 ->
 //     2440 15.3 / 16.0), in more below 352 and N = 1536 (43 495 x 264 -> 1064 54.8 / 60.3; but 7122 x 304 -> 3192 0.865 of the time);
-//   - few columns to a row, whose pass is the larger part, and full rounds, in which pairs of tf32 tiles lose nothing: 31 595 x 648 -> 1096
-//     87.4 / 89.1 (with rounds less full 15 311 x 256 -> 1064 0.869, rows that L2 holds 5062 x 768 -> 1024 24.5 / 21.7).
+//   - few columns to a row (up to 1152, or a sixth column of tiles that is mostly padding), whose pass is the larger part, and full rounds,
+//     in which pairs of tf32 tiles lose nothing: 31 595 x 648 -> 1096 87.4 / 89.1, 31 324 x 280 -> 1304 58.7 / 61.1 (with rounds less full
+//     15 311 x 256 -> 1064 0.869, rows that L2 holds 5062 x 768 -> 1024 24.5 / 21.7).
 bool half_kind_applies(int64_t M, int64_t N, int64_t K, int act, int sms) {
   if (!half_kind_sizes(M, N, K)) return false;
   const int64_t pairs = sms / 2, tiles = ceil_div(M, 2 * kBM) * ceil_div(N, 256), rounds = ceil_div(tiles, pairs);
-  if (rounds == 1 && K < (tiles < 40 ? 900 : (is_glu(act) ? 512 : 448))) return false;
+  if (rounds == 1 && K < (tiles < 40 ? 900 : (is_glu(act) ? 512 : 496))) return false;
   if (act == AQT_ACT_SWISH && K < 320) return false;
   if (is_glu(act) && (rounds == 2 ? K < 416 : K < 352 && N < 1536)) return false;
-  return !(N < 1152 && K < 704 && M * K > (2 << 20) && 20 * tiles > 17 * rounds * pairs);
+  const bool few_columns = N < 1152 || (N > 1280 && N < 1344);
+  return !(few_columns && K < 704 && M * K > (2 << 20) && 20 * tiles > 17 * rounds * pairs);
 }
 
 // True if the CTA-pair kernel with the row-quantizing epilogue takes the call: deep K, no GLU, int8
