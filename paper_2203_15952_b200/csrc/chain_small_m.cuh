@@ -144,27 +144,18 @@ __device__ __forceinline__ void chain_order8(bool packed, uint32_t& w0, uint32_t
   w1 = packed ? odd : w1;
 }
 
-// Four codes of a row as one word.  SELECT: both roundings of every value and a choice, which is less code (the chain runs through it
-// once a layer); else a branch around either, which is fewer conversions (loops over many rows).
-template <bool SELECT = true>
+// Four codes of a row as one word: both roundings of every value and a choice, which is less code than a branch around either (the chain
+// runs through it once a layer).
 __device__ __forceinline__ uint32_t chain_codes4(const float (&v)[4], const ScaleCtx& c, int qmax, int rounding) {
   if (__builtin_expect(!c.fast, 0)) return codes4_general(v[0], v[1], v[2], v[3], c.s, qmax, rounding);
   const bool half_up = rounding == AQT_ROUND_HALF_UP_FLOOR;
-  if constexpr (!SELECT) {
-    if (half_up)
-      return pack4_i8(quantize_fast<AQT_ROUND_HALF_UP_FLOOR>(v[0], c.s, c.r), quantize_fast<AQT_ROUND_HALF_UP_FLOOR>(v[1], c.s, c.r),
-                      quantize_fast<AQT_ROUND_HALF_UP_FLOOR>(v[2], c.s, c.r), quantize_fast<AQT_ROUND_HALF_UP_FLOOR>(v[3], c.s, c.r));
-    return pack4_i8(quantize_fast<AQT_ROUND_NEAREST_EVEN>(v[0], c.s, c.r), quantize_fast<AQT_ROUND_NEAREST_EVEN>(v[1], c.s, c.r),
-                    quantize_fast<AQT_ROUND_NEAREST_EVEN>(v[2], c.s, c.r), quantize_fast<AQT_ROUND_NEAREST_EVEN>(v[3], c.s, c.r));
-  } else {
-    int q[4];
+  int q[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float q0 = __fmul_rn(v[e], c.r), t = __fmaf_rn(__fmaf_rn(-q0, c.s, v[e]), c.r, q0);  // as quantize_fast
-      q[e] = half_up ? __float2int_rd(__fadd_rn(t, 0.5f)) : __float2int_rn(t);
-    }
-    return pack4_i8(q[0], q[1], q[2], q[3]);
+  for (int e = 0; e < 4; ++e) {
+    const float q0 = __fmul_rn(v[e], c.r), t = __fmaf_rn(__fmaf_rn(-q0, c.s, v[e]), c.r, q0);  // as quantize_fast
+    q[e] = half_up ? __float2int_rd(__fadd_rn(t, 0.5f)) : __float2int_rn(t);
   }
+  return pack4_i8(q[0], q[1], q[2], q[3]);
 }
 __device__ __forceinline__ float chain_max4(float m, const float (&v)[4]) {
   return fmaxf(m, fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))));
