@@ -23,10 +23,10 @@
 // cost 1000 to 1300 clocks a time with their round trip and the skew of sixteen CTAs), and a cluster is
 // scheduled as a whole, so nothing has to be resident beside it.  The waits are bounded like every
 // wait of the library.
-// Measured, a step through 17 blocks at d = 512, against layer by layer: 8 rows 312 vs 1250 us, 32 rows
-// 320 vs 1285, 112 rows (seven clusters of sixteen rows, all that run at once) 488 vs 1340; beyond, a
-// second wave of clusters or 32 rows per cluster lose to the per-layer kernels at d = 1024 (860 vs 700
-// us for 8 blocks at 113 rows), which is where AQT_CHAIN_MAX_ROWS lies.
+// Measured, against layer by layer, both in a replayed graph: a step through 17 blocks at d = 512 8 rows 318 vs 827 us, 32 rows 322 vs
+// 836, 112 rows (seven clusters of sixteen rows, all that run at once) 489 vs 866.  Beyond, a second wave of clusters: 113 rows 793 vs 866,
+// 128 rows 963 vs 868, 224 rows 971 vs 871; d = 256 656 vs 673, 801 vs 669, 803 vs 687; 8 blocks at d = 1024 815 vs 575, 909 vs 575, 887
+// vs 582.  So AQT_CHAIN_MAX_ROWS lies where the second wave begins.
 // What a layer then costs (2000 to 2600 ns; clock stamps in a copy) is a chain of latencies and of instructions that every warp
 // issues once, at the pace at which their lines are fetched:
 //   * eight warps form the products and eight take the rows from there, so that the next weights are asked for while the rows
@@ -34,7 +34,7 @@
 //     for the rows of the layer before (445 -> 383 us);
 //   * what is not always run stands aside: the general code sequence in a function, the wide form's second words behind a
 //     branch, the loop over pieces left at the last one (383 -> 344 us); stores of a layer's outputs wait until its maxima are on their way;
-//   * layers that read the same input and look alike run as one (chain_group; 343 -> 319 us);
+//   * layers that read the same input and look alike run as one (chain_group);
 //   * no integer division and no dependent parameter load in the loops (the step table sits in shared memory with everything
 //     derived from the sizes), and packed weights are used as sixteen times their codes (a nibble in the upper half of a
 //     byte; the sums are shifted back, exact), two instructions per four codes instead of eleven per eight, against
@@ -622,8 +622,8 @@ static bool chain_step_ok(const ChainStep& st) {
 
 // Steps that run as one: side steps and the one behind them that read the same input and look alike (the attention projections).
 // Their channels make up a CTA's tiles together, their rows go through one epilogue (of at most 128 columns: of more, a step is
-// long enough by itself), and the last one's columns are exchanged.  Eight rows through 17 blocks at d = 512 343 -> 317 us, 384
-// 325 -> 304, 256 277 -> 252.
+// long enough by itself), and the last one's columns are exchanged.  Eight rows through 17 blocks in a replayed graph, without and with
+// it: d = 512 342 -> 318 us, 384 312 -> 291, 256 277 -> 254.
 static int chain_group(const ChainStep* steps, int n) {
   const ChainStep& a = steps[0];
   int parts = 1;
