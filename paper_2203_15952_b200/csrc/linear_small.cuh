@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(LinSmallCfg<NT>::kThreads) linear_small_kernel
     const bool again = K8 > 32 * U;  // the loads above were more than the registers hold: once more, from L1
     // A loop for each rounding, and one for rows whose scale is not fast.  With a call of the general sequence, and a branch around either
     // rounding, for each word the loads of a step are not all in flight at once: 16 x 4096 -> 512 11.2 us, 10.15 so; 4 x 512 -> 2048, one
-    // step, 2.86 and 2.77.  (Both roundings of every value and a choice: 10.03, 1 to 4 % faster at 9 to 16 rows beyond K = 1024, and 3.11.)
+    // step, 2.86 and 2.77.  (The general sequence inline and both roundings of every value: 10.03, at 9 to 16 rows beyond K = 1024 1 to 4 %
+    // faster, and 3.11.)
     constexpr int kGeneral = -1;
     const auto convert = [&](auto mode) {
       for (int c0 = 0; c0 < pieces * (kPieceK / 8); c0 += 32 * U) {
